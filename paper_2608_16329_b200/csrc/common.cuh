@@ -75,7 +75,7 @@ struct mlip_ctx {
     int n_sm = 0;
 
     // model
-    float *head_w = nullptr;     // per-species head weights packed in MMA fragment order (megakernel.cu)
+    uint32_t *head_w = nullptr;  // per-species head weights as the tensor-memory image (megakernel.cu)
     float *table = nullptr;      // spline coefficients
     double *mass = nullptr;      // [C] dev
     double *nhc = nullptr;       // thermostat state {v_eta[3], eta[3], scale, -} (integrate.cu)

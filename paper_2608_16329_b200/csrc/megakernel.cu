@@ -17,16 +17,16 @@
 //               radial values g being evaluated straight into the B fragments.  P_i stays in
 //               the accumulator registers until the derivation.
 //   Invariants  Eq. 5 from the accumulator fragments by three xor-shuffles.
-//   Regression  Eq. 6 forward and reverse for the 8 atoms of the tile at once as W X^T on the tensor
-//               pipe (weights pre-packed in A-fragment order, 2-way split over the reduction
-//               dimension across the group's warps, elementwise epilogue over the group's threads).
-//               The current species' weights live in tensor memory (tcgen05.alloc / st / ld): a warp
-//               fetches the 32 registers of its next contraction in one instruction, off the
-//               L1/shared-memory pipe; the hidden layers are stored already split into hi + lo.
+//   Regression  Eq. 6 forward and reverse for the 8 atoms of the tile at once as W X^T on the tensor pipe
+//               (mma.sync m16n8k16, fp16 operands in hi + lo pairs: 22 significant bits, fp32 accumulate); a
+//               warp keeps its 16 neurons x 8 atoms in accumulator fragments from layer to layer and passes
+//               the activations on through shared memory in B-fragment order, one barrier per layer.
+//               The current species' weights live in tensor memory (tcgen05.alloc / st / ld), split already: a
+//               warp fetches 32 registers of A fragments in one instruction, off the L1/shared-memory pipe.
 //   Derivation  W_i (Eq. 7) is the accumulator fragment of P_i scaled in place: by construction
 //               of the channel permutation it already is the B fragment of the next contraction.
 //               [V; T] = [G; G'] W^T (Eq. 9 and the re-associated Eq. 8 term, U_i never formed)
-//               on the tensor pipe, 16 pairs per tile; results are transposed through shared
+//               on the tensor pipe, 16 pairs per tile; results are transposed through tensor
 //               memory to lane = pair for the projection of Eq. 10 and the scatter.
 // Everything that is not a contraction (geometry, harmonics, splines, projection) stays on the
 // fp32 pipe; positions are differenced in fp64.
@@ -35,6 +35,8 @@
 // integrator raises far_flag.
 // Operand splits for the three-term TF32 products are packed fp32 arithmetic (two values per instruction): a
 // Veltkamp split where the result feeds energies, a truncating split where it feeds forces only.
+#include <cuda_fp16.h>
+
 #include <algorithm>
 
 #include "common.cuh"
@@ -49,47 +51,52 @@ constexpr int PB_CAP = 160;   // queued pairs per warp: up to 31 left over + fou
 constexpr int J_BITS = 28;    // queue entries pack the neighbor index (low 28 bits) with its species
 constexpr int ST_STRIDE = 24; // encoding hand-over: 16 h, 4 b, table offset (bank-conflict-free for the fragment reads)
 constexpr int BS_STRIDE = 12; // derivation hand-over: 4 b, 4 b', table offset
-constexpr int VT_STRIDE = 40; // 16 v + 16 t per pair
-constexpr int X_STRIDE = 132; // invariants / dE/dG per atom
-constexpr int Z_STRIDE = 68;  // head activations per atom
+constexpr int X_STRIDE = 132; // dE/dG per atom
 #ifndef MLIP_TAB_STRIDE
 #define MLIP_TAB_STRIDE 36
 #endif
 constexpr int TAB_STRIDE_SMEM = MLIP_TAB_STRIDE;   // padded table row in shared memory
 
 constexpr int Q_WORDS = 4 * PB_CAP;                             // pair queue of a warp: kept from encoding to derivation
-constexpr int SCR_WORDS = 32 * BS_STRIDE + 32 * VT_STRIDE;      // scratch of a warp: 384 + 1280
-static_assert(32 * ST_STRIDE <= SCR_WORDS, "encoding stage must fit the derivation buffers");
-constexpr int SX_WORDS = TILE * X_STRIDE;                       // per group
-// head buffers of a group (alias of the scratch of the group's warps)
-constexpr int HB_XS = 0;                                   // split invariants  [8][2 * X_STRIDE]
-constexpr int HB_ZS = HB_XS + TILE * 2 * X_STRIDE;         // split activations [2][8][2 * Z_STRIDE]
-constexpr int HB_DP = HB_ZS + 2 * TILE * 2 * Z_STRIDE;     // split dE/dpre     [8][2 * Z_STRIDE]
-constexpr int HB_PART = HB_DP + TILE * 2 * Z_STRIDE;       // split-K partials  [2][8][Z_STRIDE]
-constexpr int HB_WORDS = HB_PART + 2 * TILE * Z_STRIDE;
-static_assert(HB_WORDS <= TILE * SCR_WORDS, "head buffers alias the scratch of the group's warps");
-constexpr int HC_WORDS = HEAD_L * HEAD_H + HEAD_H + 16;         // biases, w_out, b_out of the current species
+constexpr int SCR_WORDS = 32 * ST_STRIDE;                       // scratch of a warp
+static_assert(32 * BS_STRIDE <= SCR_WORDS && N_INV <= SCR_WORDS, "the derivation's hand-over and the invariants must fit the encoding's");
+// Regression buffers of a group.  Activations are kept as B fragments: per 16-input k-step, atom row and quad lane one
+// 16-byte vector {b0 hi, b0 lo, b1 hi, b1 lo} of fp16 pairs (see act_store).
+constexpr int ACT_KSTEP = 32 * 4;                               // words per k-step
+constexpr int XS_WORDS = (N_INV / 16) * ACT_KSTEP;              // split invariants (written before the group's barrier: space of their own)
+constexpr int ZS_WORDS = (HEAD_H / 16) * ACT_KSTEP;             // one layer's activations
+constexpr int SX_WORDS = TILE * X_STRIDE;                       // dE/dG
+constexpr int SC_WORDS = 8 * TILE;                              // per-atom scales (see below)
+constexpr int EP_WORDS = 4 * TILE;                              // E_i partial sums of the four m-tiles
+constexpr int GROUP_WORDS = XS_WORDS + SX_WORDS + SC_WORDS + EP_WORDS;
+static_assert(2 * ZS_WORDS <= TILE * SCR_WORDS, "layer activations alias the scratch of the group's warps");
+// Head constants of the current species: biases, w_out, b_out, then the powers of two and bounds of the fp16 scaling:
+//   pre-activation of layer L (input scaled by a per-atom 2^s): acc * (2^-s * HC_WS[L]) + bias
+//   |input of layer L| <= HC_BND[2L-2] * max|G| + HC_BND[2L-1]  (L = 1..3; row-sum norms of the weights)
+//   dE/dpre of layer L is stored times HC_SR[L]; its product with the weights is unscaled by HC_UR[L]
+constexpr int HC_WOUT = HEAD_L * HEAD_H, HC_BOUT = HC_WOUT + HEAD_H, HC_WS = HC_BOUT + 1, HC_BND = HC_WS + HEAD_L;
+constexpr int HC_SR = HC_BND + 2 * (HEAD_L - 1), HC_UR = HC_SR + HEAD_L, HC_USED = HC_UR + HEAD_L;
+constexpr int HC_WORDS = (HC_USED + 15) / 16 * 16;
 constexpr int64_t STAGGER_BELOW_ATOMS = 200000;                 // systems below this size start their CTAs on different species
 constexpr int PF_IDX = 160;                                     // neighbor indices prefetched per warp for its next atom
 constexpr int PF_CS = 96;                                       // compact lists: the codes take 81 words at most, the 27 cell bases sit here
 static_assert(PF_IDX / 2 + 1 <= PF_CS && PF_CS + 27 <= PF_IDX, "prefetch buffer layout for compact lists");
 constexpr int PF_WORDS = PF_IDX + 4;                            // + {atom, list start (2 words), list length}
-constexpr int FIXED_WORDS = NG * SX_WORDS + NW * (Q_WORDS + SCR_WORDS + PF_WORDS) + HC_WORDS + 16;
+constexpr int FIXED_WORDS = NG * GROUP_WORDS + NW * (Q_WORDS + SCR_WORDS + PF_WORDS) + HC_WORDS + 16;
 constexpr int SMEM_LIMIT_WORDS = 227 * 1024 / 4 - 256;
 
-// Pre-packed head weights per species (floats).  A record holds the A operand of one
-// (m-tile, k-step): per lane {a0, a1, a2, a3}, i.e. 128 floats (split into hi + lo in registers).
-//   forward  layer L: A[m][k] = W_L[m][k]   (m = neuron)    4 m-tiles, K_L / 8 k-steps
-//   reverse  layer L: A[m][k] = W_L[k][m]   (m = input)     K_L / 16 m-tiles, 8 k-steps
-// followed by biases [4][64], w_out[64], b_out, pad.
-constexpr int KS0 = N_INV / 8, KS1 = HEAD_H / 8;
-constexpr int FWD_RECORDS = 4 * KS0 + (HEAD_L - 1) * 4 * KS1;
-constexpr int BWD_RECORDS = (N_INV / 16) * 8 + (HEAD_L - 1) * 4 * 8;
-constexpr int HP_FWD = 0;
-constexpr int HP_BWD = HP_FWD + FWD_RECORDS * 128;
-constexpr int HP_BIAS = HP_BWD + BWD_RECORDS * 128;
-constexpr int HP_WOUT = HP_BIAS + HEAD_L * HEAD_H;
-constexpr int HP_TOTAL = HP_WOUT + HEAD_H + 4;
+// Pre-packed head weights per species (32-bit words): the tensor-memory image, [quarter][column / 4][lane][4], followed by
+// the HC_USED constants (as fp32).  Quarter q holds m-tile q (16 neurons) of every forward layer and of the hidden layers'
+// reverse pass, and m-tiles q, q + 4 (16 inputs each) of the first layer's reverse pass.  A 16-wide k-step of one m-tile
+// takes eight columns: the A fragment's four registers of fp16 pairs, hi then lo.
+//   columns [  0,  64)  forward, first layer: 8 k-steps
+//           [ 64, 160)  forward, hidden layers: 3 x 4 k-steps
+//           [160, 256)  reverse, hidden layers: 3 x 4 k-steps
+//           [256, 320)  reverse, first layer: 2 m-tiles x 4 k-steps
+//           [320, 448)  V and T on their way from fragments to lane = pair: 32 columns per warp of the quarter
+constexpr int TM_FWD0 = 0, TM_FWD = 64, TM_BWD = 160, TM_BWD0 = 256, TM_VT = 320;
+constexpr int HP_TMEM = 4 * TM_VT * 32;
+constexpr int HP_TOTAL = HP_TMEM + (HC_USED + 3) / 4 * 4;
 
 // SiLU and its derivative.  exp through the fast exponential: its error scales with |x| 2^-24 and
 // enters the sigmoid damped by s (1 - s), far below fp32 rounding of the surrounding sums.
@@ -175,6 +182,32 @@ __device__ __forceinline__ void mma_tf32_z(float (&d)[4], uint32_t a0, uint32_t 
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
 }
 
+// x, y -> fp16 pairs hi, lo with hi + lo = x to 22 significant bits (x in the lower half; |x| must stay inside fp16's
+// range, which the callers' power-of-two scales see to: below 2^-3 of a scaled unit lo loses bits, an absolute 2^-25).
+__device__ __forceinline__ void split_h2(float x, float y, uint32_t &hi, uint32_t &lo) {
+    float lx, ly;
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(y), "f"(x));
+    asm("{.reg .b16 h0, h1, m1; mov.b32 {h0, h1}, %2; mov.b16 m1, 0xBC00; fma.rn.f32.f16 %0, h0, m1, %3; fma.rn.f32.f16 %1, h1, m1, %4;}"
+        : "=f"(lx), "=f"(ly) : "r"(hi), "f"(x), "f"(y));
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(ly), "f"(lx));
+}
+__device__ __forceinline__ void mma_f16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_f16_z(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+}
+// The power of two 2^s with |x| 2^s < 2^15 for every |x| <= bound, and its inverse.
+__device__ __forceinline__ float scale_for(float bound) {
+    const int e = 268 - (int)(__float_as_uint(bound) >> 23);
+    return __uint_as_float((uint32_t)(e > 253 ? 253 : e) << 23);
+}
+__device__ __forceinline__ float inverse_pow2(float s) { return __uint_as_float((254u << 23) - __float_as_uint(s)); }
+
 // Every product A B below has both operands split: A_hi B_hi + A_lo B_hi + A_hi B_lo.  The tensor
 // pipe truncates when it adds into its fp32 accumulator, so the energy path keeps accumulation
 // chains short (a fresh accumulator per k-step, folded into the running sum by a rounded fp32
@@ -209,7 +242,7 @@ struct KernelArgs {
     const int32_t *cell_id;    // build-time cell of each atom (L16)
     const int32_t *cell_start; // first atom of each cell (L16)
     int64_t nbr_cap;           // entries the list array holds (range-checked builds)
-    const float *head_pack;
+    const uint32_t *head_pack;
     float4 *force;
     long long *force_fx;   // deterministic mode: forces as 2^-32 eV/Angstrom integers [N][3]
     long long *acc_fx;     // deterministic mode: energy (2^-32 eV) and virial (2^-28 eV) integers [10]
@@ -428,24 +461,73 @@ __device__ __forceinline__ int encode_atom(const KernelArgs &k, const TableView 
     return total;
 }
 
+// ---------------- Tensor memory (TMEM) ----------------
+// The SM's 256 KB of tensor memory (128 lanes x 512 columns of 32 bits) is otherwise idle in this kernel (the
+// contractions are per-atom products too small for tcgen05.mma), and it is the one on-chip store large enough for a
+// species' head: 41 k weights in MMA-fragment order for the forward and the reverse pass, as fp16 hi + lo pairs (the layout
+// is given at TM_FWD0 above).  A warp reaches the 32 lanes of quarter (warp % 4); all four warps of a quarter read the
+// same 320 columns.  tcgen05.ld / st bypass the L1/shared-memory data pipe, which is this kernel's busiest unit.
+constexpr uint32_t TM_COLS = 512;
+
+__device__ __forceinline__ void tmem_st4(uint32_t addr, uint4 v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t addr, uint32_t (&r)[32]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+                   "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
+                   "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
+                   "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(addr) : "memory");
+}
+// Accumulator fragments of a 16-pair tile -> 16 lanes x 32 columns: the 16x256b shape's register layout is the m16n8
+// accumulator's, eight columns per n-tile.
+__device__ __forceinline__ void tmem_st_vt(uint32_t addr, const float (&V)[2][4], const float (&T)[2][4]) {
+    asm volatile("tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(addr),
+                 "f"(V[0][0]), "f"(V[0][1]), "f"(V[0][2]), "f"(V[0][3]), "f"(V[1][0]), "f"(V[1][1]), "f"(V[1][2]), "f"(V[1][3]),
+                 "f"(T[0][0]), "f"(T[0][1]), "f"(T[0][2]), "f"(T[0][3]), "f"(T[1][0]), "f"(T[1][1]), "f"(T[1][2]), "f"(T[1][3]) : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tmem_fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// A warp copies its fourth of its quarter's weight columns for the species whose packed weights start at hp (ten 16-byte
+// loads in flight at a time: a small system's kernel time is made of such round trips).
+__device__ __forceinline__ void tmem_fill(uint32_t quarter_base, const uint32_t *__restrict__ hp, int warp, int lane) {
+    constexpr int VECS = TM_VT / 4 / (NW / 4), STEP = 10;   // 16-byte vectors per lane and warp
+    static_assert(VECS % STEP == 0 && NW % 4 == 0, "weight columns divide evenly over the warps of a quarter");
+    const int v0 = (warp >> 2) * VECS;
+    const uint4 *src = reinterpret_cast<const uint4 *>(hp) + ((size_t)(warp & 3) * (TM_VT / 4) + v0) * 32 + lane;
+#pragma unroll
+    for (int v = 0; v < VECS; v += STEP) {
+        uint4 r[STEP];
+#pragma unroll
+        for (int q = 0; q < STEP; ++q) r[q] = __ldg(src + (size_t)(v + q) * 32);
+#pragma unroll
+        for (int q = 0; q < STEP; ++q) tmem_st4(quarter_base + 4 * (v0 + v + q), r[q]);
+    }
+    tmem_wait_st();
+}
+
 // ---------------- Derivation of one atom (Eq. 8-10) ----------------
 template <bool TAB_SMEM, bool DET, bool L16>
 __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView &tv, int i,
                                             float4 *pq, float *scr, int queued, int lane, const uint32_t (&Wh)[4][4],
-                                            const uint32_t (&Wl)[4][4], float (&vir)[9], PhaseClock &pc) {
+                                            const uint32_t (&Wl)[4][4], float (&vir)[9], uint32_t tm_vt, PhaseClock &pc) {
     const int g = lane >> 2, t = lane & 3;
-    float *bs = scr, *vt = scr + 32 * BS_STRIDE;
+    float *bs = scr;
     constexpr int rs = TAB_SMEM ? TAB_STRIDE_SMEM : K_RADIAL;
     float fx = 0.f, fy = 0.f, fz = 0.f;
 
     auto batch = [&](int first, int n) {
         {   // lane = pair: spline basis and its derivative
-            float4 ent = make_float4(1.f, 0.f, 0.f, 0.f);
             float b[4] = {0.f, 0.f, 0.f, 0.f}, db[4] = {0.f, 0.f, 0.f, 0.f};
             int off = 0, row_index = 0;
             const bool live = lane < n;
             if (live) {
-                ent = pq[first + lane];
+                const float4 ent = pq[first + lane];
                 const float d2 = ent.x * ent.x + ent.y * ent.y + ent.z * ent.z, r = d2 * rsqrtf(d2);
                 const int iv = spline_basis<true, float>(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, b, db, k.status);
                 row_index = (__float_as_int(ent.w) >> J_BITS) * (k.tab.knots + 3) + iv;
@@ -456,9 +538,6 @@ __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView
             row[0] = make_float4(b[0], b[1], b[2], b[3]);
             row[1] = make_float4(db[0], db[1], db[2], db[3]);
             reinterpret_cast<int *>(bs)[slot * BS_STRIDE + 8] = off;
-            // geometry for the projection, which runs with lane = slot (spare chunk of the V/T row; the row's
-            // 16-byte chunks are stored at chunk ^ ((slot >> 2) & 1) so that lane = row reads hit eight bank groups)
-            *reinterpret_cast<float4 *>(vt + slot * VT_STRIDE + 32 + 4 * ((slot >> 2) & 1)) = ent;
         }
         __syncwarp();
         pc.mark(4);
@@ -526,28 +605,21 @@ __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView
                 mma_tf32(T[0], dh[0], dh[1], dh[2], dh[3], Wh[ks][0], Wh[ks][1]);
                 mma_tf32(T[1], dh[0], dh[1], dh[2], dh[3], Wh[ks][2], Wh[ks][3]);
             }
-            float *va = vt + (16 * mt + g) * VT_STRIDE + ((2 * t) ^ (g & 4)), *vb = va + 8 * VT_STRIDE;   // chunk ^ ((row >> 2) & 1)
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                *reinterpret_cast<float2 *>(va + 8 * q) = make_float2(V[q][0], V[q][1]);
-                *reinterpret_cast<float2 *>(vb + 8 * q) = make_float2(V[q][2], V[q][3]);
-                *reinterpret_cast<float2 *>(va + 16 + 8 * q) = make_float2(T[q][0], T[q][1]);
-                *reinterpret_cast<float2 *>(vb + 16 + 8 * q) = make_float2(T[q][2], T[q][3]);
-            }
+            // The accumulator fragments of the 16 pairs go to tensor memory as 16 lanes (pair) x 32 columns (V, T); read back
+            // below with lane = pair.  (Through shared memory the same exchange was 188 of the kernel's 1,958 L1 wavefronts per
+            // atom.)
+            tmem_st_vt(tm_vt + ((uint32_t)(16 * mt) << 16), V, T);
         }
-        __syncwarp();
+        tmem_wait_st();
         pc.mark(5);
+        uint32_t vt[32];
+        tmem_ld32(tm_vt, vt);
+        tmem_wait_ld();
         if (lane < n) {   // lane = pair: projection onto the pair vector (Eq. 10) and scatter
             float v[D_ANG], tt[D_ANG];
-            const int sw = (lane >> 2) & 1;
-            const float4 *src = reinterpret_cast<const float4 *>(vt + lane * VT_STRIDE);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float4 a = src[q ^ sw], b = src[(4 + q) ^ sw];
-                v[4 * q] = a.x; v[4 * q + 1] = a.y; v[4 * q + 2] = a.z; v[4 * q + 3] = a.w;
-                tt[4 * q] = b.x; tt[4 * q + 1] = b.y; tt[4 * q + 2] = b.z; tt[4 * q + 3] = b.w;
-            }
-            const float4 ent = src[8 ^ sw];
+            for (int q = 0; q < D_ANG; ++q) { v[q] = __uint_as_float(vt[q]); tt[q] = __uint_as_float(vt[16 + q]); }
+            const float4 ent = pq[first + lane];
             const float x = ent.x, y = ent.y, z = ent.z;
             const float rinv = rsqrtf(x * x + y * y + z * z);
             const int j = __float_as_int(ent.w) & ((1 << J_BITS) - 1);
@@ -594,146 +666,36 @@ __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView
     }
 }
 
-// ---------------- Tensor memory (TMEM) as the home of the regression network's weights ----------------
-// The SM's 256 KB of tensor memory (128 lanes x 512 columns of 32 bits) is otherwise idle in this kernel (the
-// contractions are per-atom products too small for tcgen05.mma), and it is the one on-chip store large enough for a
-// species' head: 41 k weights in MMA-fragment order for the forward and the reverse pass, 27 k of them with their hi/lo
-// split already taken.  A warp reaches the 32 lanes of quarter (warp % 4); a "record" is one A fragment = 4 consecutive
-// columns (a0..a3 of each lane).  The four warps of a quarter are the two roles (m-tile = quarter, k-half 0 / 1) of
-// the two groups, so each role's region is written once per species (by group 0) and read by both groups.
-//   region of role kh: columns 256 kh + ...
-//     [  0,  32)  forward, first layer: 8 records as they are (split on the fly)
-//     [ 32, 128)  forward, hidden layers 2-4: per layer 4 records hi, then 4 records lo (rounded split: energy path)
-//     [128, 224)  reverse, hidden layers: per layer 4 records as they are, then 4 records lo of the truncating split
-//     [224, 256)  reverse, first layer: 8 records as they are
-// tcgen05.ld / st move 4, 16 or 32 consecutive columns between a thread's registers and its lane; they bypass the
-// L1/shared-memory data pipe, which is this kernel's busiest unit.
-constexpr uint32_t TM_COLS = 512;
-constexpr int TM_ROLE = 256, TM_FWD0 = 0, TM_FWD = 32, TM_BWD = 128, TM_BWD0 = 224;
-
-__device__ __forceinline__ void tmem_st4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t addr, uint32_t (&r)[32]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-                   "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-                   "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-                   "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                 : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tmem_fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// One warp of group 0 writes its role's region (wg = m-tile + 4 k-half) for the species whose packed weights start at hp.
-__device__ __forceinline__ void tmem_fill_role(uint32_t region, const float *__restrict__ hp, int wg, int lane) {
-    const float4 *fwd = reinterpret_cast<const float4 *>(hp + HP_FWD), *bwd = reinterpret_cast<const float4 *>(hp + HP_BWD);
-    const int mt4 = wg & 3, kh = wg >> 2;
-    auto as_is = [&](uint32_t col, const float4 *rec) {
-        const float4 v = __ldg(rec + lane);
-        tmem_st4(region + col, __float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w));
-    };
-    // (the loops are unrolled so that a warp has 8 to 16 loads in flight: one L2 round trip per group of records instead of
-    // one per record, which is what a small system's kernel time is made of)
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        as_is(TM_FWD0 + 4 * q, fwd + (size_t)(mt4 * KS0 + kh * 8 + q) * 32);
-        as_is(TM_BWD0 + 4 * q, bwd + (size_t)(wg * 8 + q) * 32);
-    }
-#pragma unroll 1
-    for (int b = 0; b < HEAD_L - 1; ++b)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            {   // forward: hi, lo of the rounded split
-                const float4 v = __ldg(fwd + (size_t)(4 * KS0 + b * 4 * KS1 + mt4 * KS1 + kh * 4 + q) * 32 + lane);
-                uint32_t h[4], l[4];
-                split_tf32(v.x, h[0], l[0]); split_tf32(v.y, h[1], l[1]); split_tf32(v.z, h[2], l[2]); split_tf32(v.w, h[3], l[3]);
-                tmem_st4(region + TM_FWD + 32 * b + 4 * q, h[0], h[1], h[2], h[3]);
-                tmem_st4(region + TM_FWD + 32 * b + 16 + 4 * q, l[0], l[1], l[2], l[3]);
-            }
-            {   // reverse: the value itself (the tensor pipe truncates it), lo of the truncating split
-                const float4 v = __ldg(bwd + (size_t)((N_INV / 16) * 8 + b * 32 + mt4 * 8 + kh * 4 + q) * 32 + lane);
-                uint32_t h[4], l[4];
-                split2_force(v.x, v.y, h[0], h[1], l[0], l[1]);
-                split2_force(v.z, v.w, h[2], h[3], l[2], l[3]);
-                tmem_st4(region + TM_BWD + 32 * b + 4 * q, h[0], h[1], h[2], h[3]);
-                tmem_st4(region + TM_BWD + 32 * b + 16 + 4 * q, l[0], l[1], l[2], l[3]);
-            }
-        }
-    tmem_wait_st();
-}
-
 // Barrier among the 256 threads of one group (hardware barrier 1 + group).
 __device__ __forceinline__ void group_sync(int group) {
     asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(TILE * 32) : "memory");
 }
 
-// Head contraction on the tensor pipe: C^T[16 rows of W x 8 atoms] over NKS k-steps from ks0.
-// A records come from tensor memory (32 columns = 8 records as stored, or 4 records hi + 4 records lo when PRE);
-// B = activations (hi, lo interleaved) from shared memory with `bstride` floats per atom.
-// FRESH: every k-step gets its own accumulator, folded in by a rounded add (energy path);
-// otherwise one accumulation chain (reverse pass: feeds forces only).
-template <int NKS, bool FRESH, bool PRE>
-__device__ __forceinline__ void head_gemm(float (&c)[4], const uint32_t (&wr)[32], int ks0, const float *__restrict__ act, int bstride, int lane) {
-    static_assert(NKS % 4 == 0, "k-steps are processed four at a time (four independent MMA chains in flight)");
-    static_assert(!PRE || NKS == 4, "a pre-split load holds four records");
-    const int g = lane >> 2, t = lane & 3;
-    float acc[4][4];   // FRESH: per-k-step products; otherwise four accumulation chains
+// Head contraction on the tensor pipe: C^T[16 rows of W x 8 atoms] over four 16-wide k-steps.  A = wr (32 columns of tensor
+// memory), B = activations in fragment order from shared memory; every k-step gets its own accumulator (four independent
+// chains of three products), summed in fp32.
+__device__ __forceinline__ void head_gemm(float (&c)[4], const uint32_t (&wr)[32], const uint4 *__restrict__ act) {
+    float acc[4][4];
+    uint4 b[4];
 #pragma unroll
-    for (int q = 0; q < NKS; q += 4) {
-        uint32_t ah[4][4], al[4][4];
-        float2 x0[4], x1[4];
+    for (int u = 0; u < 4; ++u) b[u] = act[32 * u];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const float *r0 = act + g * bstride + 2 * (8 * (ks0 + q + u) + t);
-            x0[u] = *reinterpret_cast<const float2 *>(r0);
-            x1[u] = *reinterpret_cast<const float2 *>(r0 + 8);
-        }
+    for (int u = 0; u < 4; ++u) mma_f16_z(acc[u], wr[8 * u + 4], wr[8 * u + 5], wr[8 * u + 6], wr[8 * u + 7], b[u].x, b[u].z);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int o = 4 * (q + u);
-            if (PRE) {
+    for (int u = 0; u < 4; ++u) mma_f16(acc[u], wr[8 * u], wr[8 * u + 1], wr[8 * u + 2], wr[8 * u + 3], b[u].y, b[u].w);
 #pragma unroll
-                for (int e = 0; e < 4; ++e) { ah[u][e] = wr[o + e]; al[u][e] = wr[16 + o + e]; }
-            } else if (FRESH) {
-                split2_rn(__uint_as_float(wr[o]), __uint_as_float(wr[o + 1]), ah[u][0], ah[u][1], al[u][0], al[u][1]);
-                split2_rn(__uint_as_float(wr[o + 2]), __uint_as_float(wr[o + 3]), ah[u][2], ah[u][3], al[u][2], al[u][3]);
-            } else {
-                split2_force(__uint_as_float(wr[o]), __uint_as_float(wr[o + 1]), ah[u][0], ah[u][1], al[u][0], al[u][1]);
-                split2_force(__uint_as_float(wr[o + 2]), __uint_as_float(wr[o + 3]), ah[u][2], ah[u][3], al[u][2], al[u][3]);
-            }
-        }
+    for (int u = 0; u < 4; ++u) mma_f16(acc[u], wr[8 * u], wr[8 * u + 1], wr[8 * u + 2], wr[8 * u + 3], b[u].x, b[u].z);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (FRESH || q == 0) mma_tf32_z(acc[u], al[u][0], al[u][1], al[u][2], al[u][3], __float_as_uint(x0[u].x), __float_as_uint(x1[u].x));
-            else mma_tf32(acc[u], al[u][0], al[u][1], al[u][2], al[u][3], __float_as_uint(x0[u].x), __float_as_uint(x1[u].x));
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) mma_tf32(acc[u], ah[u][0], ah[u][1], ah[u][2], ah[u][3], __float_as_uint(x0[u].y), __float_as_uint(x1[u].y));
-#pragma unroll
-        for (int u = 0; u < 4; ++u) mma_tf32(acc[u], ah[u][0], ah[u][1], ah[u][2], ah[u][3], __float_as_uint(x0[u].x), __float_as_uint(x1[u].x));
-        if (FRESH) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float s4 = (acc[0][e] + acc[1][e]) + (acc[2][e] + acc[3][e]);
-                c[e] = q == 0 ? s4 : c[e] + s4;
-            }
-        }
-    }
-    if (!FRESH) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) c[e] = (acc[0][e] + acc[1][e]) + (acc[2][e] + acc[3][e]);
-    }
+    for (int e = 0; e < 4; ++e) c[e] = (acc[0][e] + acc[1][e]) + (acc[2][e] + acc[3][e]);
 }
 
-// c fragment (rows = 16 m + g, g + 8; columns = atoms 2t, 2t + 1) -> part[atom][row] with `pstride` floats per atom
-__device__ __forceinline__ void store_partial(const float (&c)[4], float *part, int pstride, int m_tile, int lane) {
-    const int g = lane >> 2, t = lane & 3;
-    float *p = part + 2 * t * pstride + 16 * m_tile + g;
-    p[0] = c[0]; p[pstride] = c[1]; p[8] = c[2]; p[pstride + 8] = c[3];
+// Activations in B-fragment order.  k-step s covers neurons (or inputs) 16 s .. 16 s + 15, its k-index 2 j + h standing for
+// neuron 16 s + j + 8 h, so that the two values a lane of an accumulator fragment holds for one atom (neurons g, g + 8) are one
+// fp16 pair.  Fragment lane (atom a, quad lane q) reads {pair q, pair q + 4}; atom rows are stored in the order
+// act_row(a), which spreads a store over all banks.
+__device__ __forceinline__ int act_row(int a) { return (a & 4) | ((a & 1) << 1) | ((a >> 1) & 1); }
+__device__ __forceinline__ void act_store(float *act, int kstep, int atom, int j, uint32_t hi, uint32_t lo) {
+    *reinterpret_cast<uint2 *>(act + kstep * ACT_KSTEP + (act_row(atom) * 4 + (j & 3)) * 4 + 2 * (j >> 2)) = make_uint2(hi, lo);
 }
 
 // Prefetch of the warp's atom in the group's NEXT tile, spread over three points of the head so
@@ -792,112 +754,126 @@ struct NextAtom {
 };
 
 // ---------------- Regression (Eq. 6) forward and reverse for the group's tile ----------------
-// In: sX = invariants [atom][128].  Out: sX = dE/dG; per-atom energies written.
-// hc = biases [4][64], w_out [64], b_out of the species in shared memory.  wg = warp within the group.
-template <bool DET, bool L16>
-__device__ __forceinline__ void head_tile(const KernelArgs &k, float *sX, float *hb, const float *hc, uint32_t tm_role, int count, int first,
-                                          int group, int wg, int lane, double &e_sum, NextAtom &nx, PhaseClock &pc) {
-    float *xs = hb + HB_XS, *zs = hb + HB_ZS, *dp = hb + HB_DP, *part = hb + HB_PART;
-    const int mt4 = wg & 3, kh = wg >> 2;   // forward / reverse hidden layers: 4 m-tiles x 2 k-halves
-    const int atom = wg;                    // elementwise phases: warp = atom, lane = neuron (and neuron + 32)
-    uint32_t w[32];   // A records of the coming contraction, fetched from tensor memory just before it
-
-    // split the invariants once
-#pragma unroll
-    for (int f = lane; f < N_INV; f += 64) {
-        uint32_t h0, h1, l0, l1;
-        split2_rn(sX[atom * X_STRIDE + f], sX[atom * X_STRIDE + f + 32], h0, h1, l0, l1);
-        *reinterpret_cast<float2 *>(xs + atom * 2 * X_STRIDE + 2 * f) = make_float2(__uint_as_float(h0), __uint_as_float(l0));
-        *reinterpret_cast<float2 *>(xs + atom * 2 * X_STRIDE + 2 * (f + 32)) = make_float2(__uint_as_float(h1), __uint_as_float(l1));
+// One atom's invariants (warp = atom) -> scaled fp16 pairs in fragment order, and the atom's scales for all layers:
+// sc[2 L][atom] = 2^s of layer L's input, sc[2 L + 1][atom] = the factor that takes layer L's product back.
+__device__ __forceinline__ void split_invariants(const float *xrow, float *xs, float *sc, const float *hc, int atom, int lane) {
+    // lane handles the pairs (c, c + 8) number lane and lane + 32 of the 64: k-step p / 8, j = p % 8
+    const int j = lane & 7, s0 = lane >> 3, s1 = s0 + 4;
+    const float a0 = xrow[16 * s0 + j], a1 = xrow[16 * s0 + 8 + j], b0 = xrow[16 * s1 + j], b1 = xrow[16 * s1 + 8 + j];
+    const float most = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fmaxf(fabsf(a0), fabsf(a1)), fmaxf(fabsf(b0), fabsf(b1))))));
+    const float sx = scale_for(most);
+    uint32_t hi, lo;
+    split_h2(a0 * sx, a1 * sx, hi, lo);
+    act_store(xs, s0, atom, j, hi, lo);
+    split_h2(b0 * sx, b1 * sx, hi, lo);
+    act_store(xs, s1, atom, j, hi, lo);
+    if (lane < HEAD_L) {
+        const float s = lane == 0 ? sx : scale_for(hc[HC_BND + 2 * (lane - 1)] * most + hc[HC_BND + 2 * (lane - 1) + 1]);
+        sc[2 * lane * TILE + atom] = s;
+        sc[(2 * lane + 1) * TILE + atom] = inverse_pow2(s) * hc[HC_WS + lane];
     }
-    nx.stage_a();
-    pc.mark(3);
-    group_sync(group);
-    pc.mark(14);
+}
 
-    float e_i = 0.f;
-    float ya = 0.f, yb = 0.f;   // running activations of this thread's two neurons (the skip path)
-    float2 dzn = make_float2(0.f, 0.f);   // dE/dy of the same two neurons in the reverse pass
-    float2 sdr[HEAD_L];                    // SiLU' of their pre-activations, layer by layer
+// In: xs = split invariants.  Out: sX = dE/dG [atom][128]; per-atom energies written.  wg = warp within the group; warps
+// 0..3 own m-tile wg (16 neurons) of the eight atoms through all layers, all eight take part in the first layer's reverse.
+template <bool DET, bool L16>
+__device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, float *sX, const float *sc, float *ep, float *zs, const float *hc,
+                                          uint32_t tm, int count, int first, int group, int wg, int lane, double &e_sum, NextAtom &nx, PhaseClock &pc) {
+    const int g = lane >> 2, t = lane & 3, mt = wg & 3;
+    const int frag = act_row(g) * 4 + t;        // this lane's vector of a k-step
+    const bool owner = wg < 4;
+    const int n0 = 16 * mt + g, n1 = n0 + 8;    // the lane's neurons; its atoms are 2t, 2t + 1: values {n0 2t, n0 2t+1, n1 2t, n1 2t+1}
+    float y[4] = {0.f, 0.f, 0.f, 0.f};          // running activations (the skip path)
+    float dz[4];                                // dE/dy in the reverse pass
+    float sd[HEAD_L][4];                        // SiLU' of the pre-activations, layer by layer
+    uint32_t w[32];                             // A fragments of the coming contraction
 #pragma unroll
     for (int L = 0; L < HEAD_L; ++L) {
-        const float *zin = zs + ((L + 1) & 1) * TILE * 2 * Z_STRIDE;
-        float *zout = zs + (L & 1) * TILE * 2 * Z_STRIDE;
-        float c[4];
-        tmem_ld32(tm_role + (L == 0 ? TM_FWD0 : TM_FWD + 32 * (L - 1)), w);
-        tmem_wait_ld();
-        if (L == 0) head_gemm<KS0 / 2, true, false>(c, w, kh * (KS0 / 2), xs, 2 * X_STRIDE, lane);
-        else head_gemm<KS1 / 2, true, true>(c, w, kh * (KS1 / 2), zin, 2 * Z_STRIDE, lane);
-        pc.mark(12);
-        store_partial(c, part + kh * TILE * Z_STRIDE, Z_STRIDE, mt4, lane);
-        if (L == 0) nx.template stage_b<L16>();
-        if (L == 1) nx.template stage_c<L16>(lane);
+        const float *zin = zs + ((L + 1) & 1) * ZS_WORDS;
+        float *zout = zs + (L & 1) * ZS_WORDS;
+        if (owner) {
+            float c[4];
+            tmem_ld32(tm + (L == 0 ? TM_FWD0 : TM_FWD + 32 * (L - 1)), w);
+            tmem_wait_ld();
+            head_gemm(c, w, reinterpret_cast<const uint4 *>(L == 0 ? xs : zin) + frag);
+            if (L == 0) {
+                float c2[4];
+                tmem_ld32(tm + TM_FWD0 + 32, w);
+                tmem_wait_ld();
+                head_gemm(c2, w, reinterpret_cast<const uint4 *>(xs + 4 * ACT_KSTEP) + frag);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) c[e] += c2[e];
+            }
+            pc.mark(12);
+            const float2 u = *reinterpret_cast<const float2 *>(sc + (2 * L + 1) * TILE + 2 * t);
+            const float bias0 = hc[L * HEAD_H + n0], bias1 = hc[L * HEAD_H + n1];
+            y[0] += silu_f(c[0] * u.x + bias0, sd[L][0]); y[1] += silu_f(c[1] * u.y + bias0, sd[L][1]);
+            y[2] += silu_f(c[2] * u.x + bias1, sd[L][2]); y[3] += silu_f(c[3] * u.y + bias1, sd[L][3]);
+            float m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f;   // what goes to the next contraction
+            if (L < HEAD_L - 1) {
+                const float2 s = *reinterpret_cast<const float2 *>(sc + 2 * (L + 1) * TILE + 2 * t);
+                m0 = y[0] * s.x; m1 = y[1] * s.y; m2 = y[2] * s.x; m3 = y[3] * s.y;
+            } else {   // output layer and the start of the reverse pass: dE/dy = w_out
+                const float wo0 = hc[HC_WOUT + n0], wo1 = hc[HC_WOUT + n1], s = hc[HC_SR + L];
+                float e0 = wo0 * y[0] + wo1 * y[2], e1 = wo0 * y[1] + wo1 * y[3];
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) {
+                    e0 += __shfl_xor_sync(0xffffffffu, e0, o);
+                    e1 += __shfl_xor_sync(0xffffffffu, e1, o);
+                }
+                if (g == 0) *reinterpret_cast<float2 *>(ep + mt * TILE + 2 * t) = make_float2(e0, e1);
+                dz[0] = dz[1] = wo0; dz[2] = dz[3] = wo1;
+                m0 = (wo0 * s) * sd[L][0]; m1 = (wo0 * s) * sd[L][1]; m2 = (wo1 * s) * sd[L][2]; m3 = (wo1 * s) * sd[L][3];
+            }
+            uint32_t hi, lo;
+            split_h2(m0, m2, hi, lo);
+            act_store(zout, mt, 2 * t, g, hi, lo);
+            split_h2(m1, m3, hi, lo);
+            act_store(zout, mt, 2 * t + 1, g, hi, lo);
+        }
+        if (L == 0) nx.stage_a();
+        if (L == 1) nx.template stage_b<L16>();
+        if (L == 2) nx.template stage_c<L16>(lane);
         pc.mark(13);
         group_sync(group);
         pc.mark(14);
-        // elementwise: bias, SiLU, residual; this thread owns neurons 2 lane, 2 lane + 1 of its atom
-        {
-            const int n0 = 2 * lane;
-            const float2 p0 = *reinterpret_cast<const float2 *>(part + atom * Z_STRIDE + n0);
-            const float2 p1 = *reinterpret_cast<const float2 *>(part + (TILE + atom) * Z_STRIDE + n0);
-            const float2 bb = *reinterpret_cast<const float2 *>(hc + L * HEAD_H + n0);
-            float d0, d1;
-            ya += silu_f((p0.x + p1.x) + bb.x, d0);
-            yb += silu_f((p0.y + p1.y) + bb.y, d1);
-            const float y0 = ya, y1 = yb;
-            sdr[L] = make_float2(d0, d1);
-            if (L < HEAD_L - 1) {
-                uint32_t h0, h1, l0, l1;
-                split2_rn(y0, y1, h0, h1, l0, l1);
-                *reinterpret_cast<uint4 *>(zout + atom * 2 * Z_STRIDE + 2 * n0) = make_uint4(h0, l0, h1, l1);
-            } else {   // output layer and the start of the reverse pass: dE/dz = w_out
-                const float2 wo = *reinterpret_cast<const float2 *>(hc + HEAD_L * HEAD_H + n0);
-                e_i += wo.x * y0 + wo.y * y1;
-                dzn = wo;
-                uint32_t h0, h1, l0, l1;
-                split2_rn(wo.x * d0, wo.y * d1, h0, h1, l0, l1);
-                *reinterpret_cast<uint4 *>(dp + atom * 2 * Z_STRIDE + 2 * n0) = make_uint4(h0, l0, h1, l1);
-            }
-        }
-        pc.mark(15);
-        group_sync(group);
-        pc.mark(14);
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) e_i += __shfl_xor_sync(0xffffffffu, e_i, o);
-    e_i += hc[HEAD_L * HEAD_H + HEAD_H];
-    if (lane == 0 && atom < count) {
-        k.e_atom[__ldg(k.center_order + first + atom)] = e_i;
+    if (wg == 7 && lane < count) {
+        const float e_i = ((ep[lane] + ep[TILE + lane]) + (ep[2 * TILE + lane] + ep[3 * TILE + lane])) + hc[HC_BOUT];
+        k.e_atom[__ldg(k.center_order + first + lane)] = e_i;
         e_sum += DET ? rint((double)e_i * ENERGY_FX) : (double)e_i;   // DET: exact integer sums
     }
 
-    // reverse through the hidden layers 3, 2, 1 (each with its skip path)
+    // reverse through the hidden layers 3, 2, 1 (each with its skip path); dE/dpre_3 sits where layer 3 put it
 #pragma unroll
     for (int L = HEAD_L - 1; L >= 1; --L) {
-        float c[4];
-        tmem_ld32(tm_role + TM_BWD + 32 * (L - 1), w);
-        tmem_wait_ld();
-        head_gemm<4, false, true>(c, w, kh * 4, dp, 2 * Z_STRIDE, lane);
-        store_partial(c, part + kh * TILE * Z_STRIDE, Z_STRIDE, mt4, lane);
-        group_sync(group);
-        {
-            const int n0 = 2 * lane;
-            const float2 p0 = *reinterpret_cast<const float2 *>(part + atom * Z_STRIDE + n0);
-            const float2 p1 = *reinterpret_cast<const float2 *>(part + (TILE + atom) * Z_STRIDE + n0);
-            dzn.x += p0.x + p1.x; dzn.y += p0.y + p1.y;
-            const float2 da = sdr[L - 1];
-            uint32_t h0, h1, l0, l1;
-            split2_rn(dzn.x * da.x, dzn.y * da.y, h0, h1, l0, l1);
-            *reinterpret_cast<uint4 *>(dp + atom * 2 * Z_STRIDE + 2 * n0) = make_uint4(h0, l0, h1, l1);
+        const float *zin = zs + (L & 1) * ZS_WORDS;
+        float *zout = zs + ((L + 1) & 1) * ZS_WORDS;
+        if (owner) {
+            float c[4];
+            tmem_ld32(tm + TM_BWD + 32 * (L - 1), w);
+            tmem_wait_ld();
+            head_gemm(c, w, reinterpret_cast<const uint4 *>(zin) + frag);
+            const float u = hc[HC_UR + L], s = hc[HC_SR + L - 1];
+            float m[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) { dz[e] += c[e] * u; m[e] = dz[e] * sd[L - 1][e] * s; }
+            uint32_t hi, lo;
+            split_h2(m[0], m[2], hi, lo);
+            act_store(zout, mt, 2 * t, g, hi, lo);
+            split_h2(m[1], m[3], hi, lo);
+            act_store(zout, mt, 2 * t + 1, g, hi, lo);
         }
         group_sync(group);
     }
-    {   // first layer: dE/dG [128 x 8], warp = m-tile (16 inputs), written over the invariants
+    {   // first layer: dE/dG [128 x 8], warp = m-tile (16 inputs)
         float c[4];
-        tmem_ld32(tm_role + TM_BWD0, w);   // warp = m-tile, all 8 k-steps
+        tmem_ld32(tm + TM_BWD0 + 32 * (wg >> 2), w);
         tmem_wait_ld();
-        head_gemm<8, false, false>(c, w, 0, dp, 2 * Z_STRIDE, lane);
-        store_partial(c, sX, X_STRIDE, wg, lane);
+        head_gemm(c, w, reinterpret_cast<const uint4 *>(zs) + frag);   // layer 0's dE/dpre: buffer 0
+        const float u = hc[HC_UR];
+        float *p = sX + 2 * t * X_STRIDE + 16 * wg + g;
+        p[0] = c[0] * u; p[X_STRIDE] = c[1] * u; p[8] = c[2] * u; p[X_STRIDE + 8] = c[3] * u;
     }
     group_sync(group);
 }
@@ -909,9 +885,10 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
     const int group = warp / TILE, wg = warp % TILE;
     const int g = lane >> 2, t = lane & 3;
     float *s_tab = smem;                                   // [C][rows][TAB_STRIDE_SMEM] when TAB_SMEM
-    float *sX = smem + (TAB_SMEM ? tab_words : 0) + group * SX_WORDS;
-    float *scr_all = smem + (TAB_SMEM ? tab_words : 0) + NG * SX_WORDS;
-    float *hb = scr_all + group * TILE * SCR_WORDS;        // head buffers = the scratch of the group's warps
+    float *xs = smem + (TAB_SMEM ? tab_words : 0) + group * GROUP_WORDS;
+    float *sX = xs + XS_WORDS, *sc = sX + SX_WORDS, *ep = sc + SC_WORDS;
+    float *scr_all = smem + (TAB_SMEM ? tab_words : 0) + NG * GROUP_WORDS;
+    float *zs = scr_all + group * TILE * SCR_WORDS;        // layer activations = the scratch of the group's warps
     float *scr = scr_all + warp * SCR_WORDS;
     float4 *pq = reinterpret_cast<float4 *>(scr_all + NW * SCR_WORDS + warp * Q_WORDS);
     int *pf = reinterpret_cast<int *>(scr_all + NW * (SCR_WORDS + Q_WORDS)) + warp * PF_WORDS;
@@ -933,7 +910,8 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
     __syncthreads();
     tmem_fence_after_sync();
     const uint32_t tm_base = *reinterpret_cast<volatile uint32_t *>(ctl + 4);
-    const uint32_t tm_role = tm_base + ((uint32_t)(32 * (wg & 3)) << 16) + TM_ROLE * (wg >> 2);
+    const uint32_t tm_quarter = tm_base + ((uint32_t)(32 * (warp & 3)) << 16);
+    const uint32_t tm_vt = tm_quarter + TM_VT + 32 * (warp >> 2);
 
     double e_sum = 0.0;
     float vir[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -966,9 +944,9 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
             tv.base = k.tab.coef + (size_t)species * k.n_species * rows * K_RADIAL;
             tv.row_stride = K_RADIAL; tv.table_stride = rows * K_RADIAL;
         }
-        for (int idx = threadIdx.x; idx < HEAD_L * HEAD_H + HEAD_H + 1; idx += NW * 32)
-            hc[idx] = __ldg(k.head_pack + (size_t)species * HP_TOTAL + HP_BIAS + idx);
-        if (group == 0) tmem_fill_role(tm_role, k.head_pack + (size_t)species * HP_TOTAL, wg, lane);
+        const uint32_t *hp = k.head_pack + (size_t)species * HP_TOTAL;
+        for (int idx = threadIdx.x; idx < HC_USED; idx += NW * 32) hc[idx] = __uint_as_float(__ldg(hp + HP_TMEM + idx));
+        tmem_fill(tm_quarter, hp, warp, lane);
         tmem_fence_before_sync();
         __syncthreads();
         tmem_fence_after_sync();
@@ -994,7 +972,8 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
             int64_t beg = 0, end = 0;
             float Pf[4][4];
             int queued = -1;
-            float *xrow = sX + wg * X_STRIDE;
+            const float *drow = sX + wg * X_STRIDE;   // dE/dG of this warp's atom
+            float *xrow = scr;                        // its invariants (the encoding is done with the scratch)
             if (have) {
                 if (prefetched) {
                     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -1040,6 +1019,8 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
             } else {   // empty slot of a ragged tile: feed zeros to the head
                 for (int c = lane; c < N_INV; c += 32) xrow[c] = 0.f;
             }
+            __syncwarp();
+            split_invariants(xrow, xs, sc, hc, wg, lane);
             if (wg == 0 && lane == 0) ctl[2 * group + 1] = look_ahead;
             pc.mark(7);
             group_sync(group);
@@ -1051,7 +1032,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
             nx.k = &k; nx.sidx = pf; nx.meta = pf + PF_IDX;
             nx.slot = (tile_next < n_tiles && s_beg + tile_next * TILE + wg < s_end) ? s_beg + tile_next * TILE + wg : -1;
             nx.i = 0; nx.beg = 0; nx.end = 0; nx.use_far = use_far; nx.cid = 0;
-            head_tile<DET, L16>(k, sX, hb, hc, tm_role, count, first, group, wg, lane, e_sum, nx, pc);
+            head_tile<DET, L16>(k, xs, sX, sc, ep, zs, hc, tm_quarter, count, first, group, wg, lane, e_sum, nx, pc);
             prefetched = nx.slot >= 0;
             pc.mark(9);
 
@@ -1061,8 +1042,8 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
                 const int la = g == 0 ? 0 : (g <= 3 ? 1 : 2), lb = g == 0 ? 2 : 3;
                 float da[8], db[8];
                 {
-                    const float4 a0 = *reinterpret_cast<const float4 *>(xrow + 32 * la + 8 * t), a1 = *reinterpret_cast<const float4 *>(xrow + 32 * la + 8 * t + 4);
-                    const float4 b0 = *reinterpret_cast<const float4 *>(xrow + 32 * lb + 8 * t), b1 = *reinterpret_cast<const float4 *>(xrow + 32 * lb + 8 * t + 4);
+                    const float4 a0 = *reinterpret_cast<const float4 *>(drow + 32 * la + 8 * t), a1 = *reinterpret_cast<const float4 *>(drow + 32 * la + 8 * t + 4);
+                    const float4 b0 = *reinterpret_cast<const float4 *>(drow + 32 * lb + 8 * t), b1 = *reinterpret_cast<const float4 *>(drow + 32 * lb + 8 * t + 4);
                     da[0] = a0.x; da[1] = a0.y; da[2] = a0.z; da[3] = a0.w; da[4] = a1.x; da[5] = a1.y; da[6] = a1.z; da[7] = a1.w;
                     db[0] = b0.x; db[1] = b0.y; db[2] = b0.z; db[3] = b0.w; db[4] = b1.x; db[5] = b1.y; db[6] = b1.z; db[7] = b1.w;
                 }
@@ -1076,7 +1057,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
                     split2_rn(w0, w1, Wh[ks][0], Wh[ks][1], Wl[ks][0], Wl[ks][1]);   // once per atom: the rounded split
                     split2_rn(w2, w3, Wh[ks][2], Wh[ks][3], Wl[ks][2], Wl[ks][3]);
                 }
-                derive_atom<TAB_SMEM, DET, L16>(k, tv, i, pq, scr, queued, lane, Wh, Wl, vir, pc);
+                derive_atom<TAB_SMEM, DET, L16>(k, tv, i, pq, scr, queued, lane, Wh, Wl, vir, tm_vt, pc);
                 if (DET) {   // fold this atom's virial in now: lane sums in a fixed order, then integers
 #pragma unroll
                     for (int q = 0; q < 9; ++q) {
@@ -1097,7 +1078,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
     // per-warp totals -> global accumulators
     if (DET) {
         if (lane < 9) atomicAdd(reinterpret_cast<unsigned long long *>(k.acc_fx + 1 + lane), (unsigned long long)(long long)vir_fx);
-        if (lane == 0) atomicAdd(reinterpret_cast<unsigned long long *>(k.acc_fx), (unsigned long long)(long long)e_sum);
+        if (wg == 7 && lane < TILE) atomicAdd(reinterpret_cast<unsigned long long *>(k.acc_fx), (unsigned long long)(long long)e_sum);
     } else {
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
@@ -1106,7 +1087,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
             for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
             if (lane == 0) atomicAdd(&k.acc[ACC_VIRIAL + q], (double)x);
         }
-        if (lane == 0) atomicAdd(&k.acc[ACC_ENERGY], e_sum);
+        if (wg == 7 && lane < TILE) atomicAdd(&k.acc[ACC_ENERGY], e_sum);
     }
     if (lane == 0) atomicAdd(k.pair_counter, n_pairs);
     tmem_fence_before_sync();
@@ -1118,53 +1099,99 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
 int table_smem_words(const mlip_ctx *c) { return c->cfg.n_species * (c->cfg.table_knots + 3) * TAB_STRIDE_SMEM; }
 bool tables_fit_smem(const mlip_ctx *c) { return FIXED_WORDS + table_smem_words(c) <= SMEM_LIMIT_WORDS; }
 
+static float pow2f(int e) { return ldexpf(1.f, e); }
+
 int upload_head(mlip_ctx *c, const double *w) {
     const int C = c->cfg.n_species;
-    float *host = (float *)calloc((size_t)C * HP_TOTAL, sizeof(float));
+    uint32_t *host = (uint32_t *)calloc((size_t)C * HP_TOTAL, sizeof(uint32_t));
     if (!host) return MLIP_ERR_OOM;
     for (int s = 0; s < C; ++s) {
-        const double *src = w + (size_t)s * HEAD_NET;
-        float *hp = host + (size_t)s * HP_TOTAL;
-        float *fwd = hp + HP_FWD, *bwd = hp + HP_BWD;
-        int in = N_INV;
+        const double *layer[HEAD_L], *out = w + (size_t)s * HEAD_NET;
+        int in_of[HEAD_L];
+        for (int L = 0, in = N_INV; L < HEAD_L; ++L, in = HEAD_H) { layer[L] = out; in_of[L] = in; out += in * HEAD_H + HEAD_H; }
+        uint32_t *hp = host + (size_t)s * HP_TOTAL;
+        float *hc = reinterpret_cast<float *>(hp + HP_TMEM);
+        // powers of two: weights of a layer to below 2^14; bounds of the layers' inputs from row sums, of dE/dpre from column sums
+        // (both a little enlarged for the device's fp32 arithmetic)
+        float wscale[HEAD_L];
+        double row_sum[HEAD_L], bias_max[HEAD_L], col_sum[HEAD_L], wout_max = 0.0;
         for (int L = 0; L < HEAD_L; ++L) {
-            const int nks = in / 8;
-            // forward: A[m][k] = W[m][k]; record (mt, ks), lane (g, t):
-            //   a0 = W[16mt+g][8ks+t], a1 = W[16mt+g+8][8ks+t], a2 = W[16mt+g][8ks+t+4], a3 = W[16mt+g+8][8ks+t+4]
-            for (int mt = 0; mt < 4; ++mt)
-                for (int ks = 0; ks < nks; ++ks)
-                    for (int lane = 0; lane < 32; ++lane) {
-                        const int g = lane >> 2, t = lane & 3;
-                        float *rec = fwd + ((size_t)(mt * nks + ks) * 32 + lane) * 4;
-                        rec[0] = (float)src[(16 * mt + g) * in + 8 * ks + t];
-                        rec[1] = (float)src[(16 * mt + g + 8) * in + 8 * ks + t];
-                        rec[2] = (float)src[(16 * mt + g) * in + 8 * ks + t + 4];
-                        rec[3] = (float)src[(16 * mt + g + 8) * in + 8 * ks + t + 4];
-                    }
-            // reverse: A[m][k] = W[k][m] (m = input, k = neuron); record (mt, ks)
-            for (int mt = 0; mt < in / 16; ++mt)
-                for (int ks = 0; ks < 8; ++ks)
-                    for (int lane = 0; lane < 32; ++lane) {
-                        const int g = lane >> 2, t = lane & 3;
-                        float *rec = bwd + ((size_t)(mt * 8 + ks) * 32 + lane) * 4;
-                        rec[0] = (float)src[(8 * ks + t) * in + 16 * mt + g];
-                        rec[1] = (float)src[(8 * ks + t) * in + 16 * mt + g + 8];
-                        rec[2] = (float)src[(8 * ks + t + 4) * in + 16 * mt + g];
-                        rec[3] = (float)src[(8 * ks + t + 4) * in + 16 * mt + g + 8];
-                    }
-            for (int o = 0; o < HEAD_H; ++o) hp[HP_BIAS + L * HEAD_H + o] = (float)src[in * HEAD_H + o];
-            src += in * HEAD_H + HEAD_H;
-            fwd += (size_t)4 * nks * 128;
-            bwd += (size_t)(in / 16) * 8 * 128;
-            in = HEAD_H;
+            const int in = in_of[L];
+            double most = 0.0;
+            row_sum[L] = bias_max[L] = col_sum[L] = 0.0;
+            for (int o = 0; o < HEAD_H; ++o) {
+                double r = 0.0;
+                for (int q = 0; q < in; ++q) { const double a = fabs(layer[L][(size_t)o * in + q]); r += a; most = std::max(most, a); }
+                row_sum[L] = std::max(row_sum[L], r);
+                bias_max[L] = std::max(bias_max[L], fabs(layer[L][(size_t)in * HEAD_H + o]));
+            }
+            for (int q = 0; q < in; ++q) {
+                double r = 0.0;
+                for (int o = 0; o < HEAD_H; ++o) r += fabs(layer[L][(size_t)o * in + q]);
+                col_sum[L] = std::max(col_sum[L], r);
+            }
+            int e = 0;
+            if (most > 0.0) frexp(most, &e);
+            wscale[L] = pow2f(std::min(14 - e, 60));
         }
-        for (int o = 0; o < HEAD_H + 1; ++o) hp[HP_WOUT + o] = (float)src[o];
+        for (int o = 0; o < HEAD_H; ++o) wout_max = std::max(wout_max, fabs(out[o]));
+        // |SiLU(x)| <= |x|, |SiLU'(x)| < 1.1: |y_0| <= A max|G| + B, |y_L| <= (1 + r_L) |y_{L-1}| + b_L
+        double A = row_sum[0], B = bias_max[0];
+        for (int L = 1; L < HEAD_L; ++L) {
+            hc[HC_BND + 2 * (L - 1)] = (float)(1.001 * A);
+            hc[HC_BND + 2 * (L - 1) + 1] = (float)(1.001 * B);
+            A *= 1.0 + row_sum[L];
+            B = B * (1.0 + row_sum[L]) + bias_max[L];
+        }
+        double dz = wout_max;
+        for (int L = HEAD_L - 1; L >= 0; --L) {
+            int e = 0;
+            if (dz > 0.0) frexp(1.101 * dz, &e);
+            const float sr = pow2f(std::min(15 - e, 60));
+            hc[HC_SR + L] = sr;
+            hc[HC_UR + L] = 1.f / (sr * wscale[L]);
+            hc[HC_WS + L] = 1.f / wscale[L];
+            dz *= 1.0 + 1.1 * col_sum[L];
+        }
+        for (int L = 0; L < HEAD_L; ++L)
+            for (int o = 0; o < HEAD_H; ++o) hc[L * HEAD_H + o] = (float)layer[L][(size_t)in_of[L] * HEAD_H + o];
+        for (int o = 0; o < HEAD_H; ++o) hc[HC_WOUT + o] = (float)out[o];
+        hc[HC_BOUT] = (float)out[HEAD_H];
+        // A fragments: k-step ks, lane (g, t), register r holds row 16 m + g + 8 (r & 1) and the k pair (n, n + 8) with
+        // n = 16 ks + t + 4 (r >> 1)  (see act_store)
+        auto put = [&](int quarter, int col, int lane, double lo_k, double hi_k, float sc) {
+            auto half_bits = [](float x) { const __half h = __float2half_rn(x); return (uint32_t)__half_as_ushort(h); };
+            auto rest = [](float x) { return x - __half2float(__float2half_rn(x)); };
+            const float x = (float)lo_k * sc, y = (float)hi_k * sc;
+            const auto word = [&](int cc) -> uint32_t & { return hp[(((size_t)quarter * (TM_VT / 4) + cc / 4) * 32 + lane) * 4 + cc % 4]; };
+            word(col) = half_bits(x) | half_bits(y) << 16;
+            word(col + 4) = half_bits(rest(x)) | half_bits(rest(y)) << 16;
+        };
+        for (int L = 0; L < HEAD_L; ++L) {
+            const int in = in_of[L];
+            const double *W = layer[L];
+            for (int lane = 0; lane < 32; ++lane)
+                for (int r = 0; r < 4; ++r) {
+                    const int g = lane >> 2, t = lane & 3, row = g + 8 * (r & 1), n = t + 4 * (r >> 1);
+                    for (int mt = 0; mt < 4; ++mt)   // forward: A[m][k] = W[m][k]
+                        for (int ks = 0; ks < in / 16; ++ks) {
+                            const double *src = W + (size_t)(16 * mt + row) * in + 16 * ks + n;
+                            put(mt, (L == 0 ? TM_FWD0 : TM_FWD + 32 * (L - 1)) + 8 * ks + r, lane, src[0], src[8], wscale[L]);
+                        }
+                    for (int m = 0; m < in / 16; ++m)   // reverse: A[m][k] = W[k][m]
+                        for (int ks = 0; ks < HEAD_H / 16; ++ks) {
+                            const double *src = W + (size_t)(16 * ks + n) * in + 16 * m + row;
+                            put(m & 3, (L == 0 ? TM_BWD0 + 32 * (m >> 2) : TM_BWD + 32 * (L - 1)) + 8 * ks + r, lane, src[0], src[(size_t)8 * in], wscale[L]);
+                        }
+                }
+        }
     }
-    cudaError_t e = cudaMalloc(&c->head_w, sizeof(float) * (size_t)C * HP_TOTAL);
-    if (e == cudaSuccess) e = cudaMemcpy(c->head_w, host, sizeof(float) * (size_t)C * HP_TOTAL, cudaMemcpyHostToDevice);
+    const size_t bytes = sizeof(uint32_t) * (size_t)C * HP_TOTAL;
+    cudaError_t e = cudaMalloc(&c->head_w, bytes);
+    if (e == cudaSuccess) e = cudaMemcpy(c->head_w, host, bytes, cudaMemcpyHostToDevice);
     free(host);
     if (e != cudaSuccess) { c->err = cudaGetErrorString(e); return MLIP_ERR_CUDA; }
-    c->resident += sizeof(float) * (size_t)C * HP_TOTAL;
+    c->resident += bytes;
     return MLIP_OK;
 }
 
