@@ -268,13 +268,15 @@ int mlip_create(mlip_ctx **out, const mlip_config *cfg, const double *enc_w, siz
             cudaMemset(c->nhc, 0, sizeof(double) * 8) != cudaSuccess || cudaMemset(c->launch_block, 0, sizeof(double) * LB_COUNT) != cudaSuccess) {
             rc = MLIP_ERR_CUDA; c->err = "initial upload failed"; break;
         }
-        if ((rc = f64 ? upload_head_f64(c, head_w) : upload_head(c, head_w)) != MLIP_OK) break;
         rc = build_tables(c, enc_w, n_enc);
         // automatic knot count: double until the spline meets the tolerance
         while (auto_knots && rc == MLIP_ERR_TABLE_TOLERANCE && c->cfg.table_knots < (f64 ? 8192 : 2048)) {
             c->cfg.table_knots *= 2;
             rc = build_tables(c, enc_w, n_enc);
         }
+        if (rc != MLIP_OK && rc != MLIP_ERR_TABLE_TOLERANCE) break;
+        const int head_rc = f64 ? upload_head_f64(c, head_w) : upload_head(c, head_w);   // (the fp32 form depends on the tables' scales)
+        if (head_rc != MLIP_OK) rc = head_rc;
     } while (0);
     if (rc != MLIP_OK && rc != MLIP_ERR_TABLE_TOLERANCE) {
         g_last_error = c->err;

@@ -58,9 +58,12 @@ struct CellGrid {
     int n_cells;
 };
 
+// The 16-byte chunk c of row r of a species' radial tables is stored at position c ^ table_swizzle(r) (0, 3, 4, 7 for r mod 4).
+__host__ __device__ constexpr int table_swizzle(int r) { return 2 * (r & 3) + (r & 1); }
+
 // Radial table: uniform cubic B-spline per ordered species pair and channel.
 struct TableDesc {
-    const float *coef;   // [C*C][knots + 3][K_RADIAL]
+    const float *coef;   // [C*C][knots + 3][K_RADIAL], scaled by 2^table_exp, chunks permuted (table_swizzle)
     int knots;           // number of intervals
     float r_min;
     float inv_h;         // 1 / interval width
@@ -77,6 +80,7 @@ struct mlip_ctx {
     // model
     uint32_t *head_w = nullptr;  // per-species head weights as the tensor-memory image (megakernel.cu)
     float *table = nullptr;      // spline coefficients
+    int table_exp[mlip::MAX_SPECIES * mlip::K_RADIAL] = {0};   // fp32 tables: power-of-two exponents per (central species, channel)
     double *mass = nullptr;      // [C] dev
     double *nhc = nullptr;       // thermostat state {v_eta[3], eta[3], scale, -} (integrate.cu)
     double nhc_nf = 0, nhc_kT = 0, nhc_q1 = 0, nhc_qk = 0;   // parameters of the last NVT call

@@ -12,8 +12,8 @@
 //   Encoding    The warp scans the atom's list (lane = entry), queues the pairs inside r_cut in
 //               shared memory, and every 32 queued pairs evaluates harmonics (Eq. 3) and the
 //               spline basis with lane = pair.  The moment P_i = H^T G (Eq. 4, 16 x n times
-//               n x 32) is accumulated on the tensor pipe: mma.sync m16n8k8 TF32 with a
-//               three-term hi/lo split of both operands (~2^-21 relative, fp32 accumulate), the
+//               n x 32) is accumulated on the tensor pipe: mma.sync m16n8k16 with both operands as fp16
+//               hi + lo pairs (three products, ~2^-22 relative, fp32 accumulate), the
 //               radial values g being evaluated straight into the B fragments.  P_i stays in
 //               the accumulator registers until the derivation.
 //   Invariants  Eq. 5 from the accumulator fragments by three xor-shuffles.
@@ -33,11 +33,17 @@
 // Lists come in two parts (neighbor.cu): entries that were within r_cut + skin / 2 at build time first, the rest
 // behind them; the far part cannot reach r_cut before some atom has moved skin / 4, and is skipped until the
 // integrator raises far_flag.
-// Operand splits for the three-term TF32 products are packed fp32 arithmetic (two values per instruction): a
-// Veltkamp split where the result feeds energies, a truncating split where it feeds forces only.
+// Three-term products: both operands of every contraction are split into fp16 hi + lo (22 significant bits, the same as two
+// TF32 terms) and A_lo B_hi + A_hi B_lo + A_hi B_hi is accumulated in fp32.  fp16 halves the tensor instructions and the fragment
+// registers of TF32.  Its narrow exponent range (full precision over 2^18 below the largest scaled value, an absolute error of 2^-40
+// of it further down) is met by exact powers of two: the radial tables are stored scaled per central species and channel
+// (tables.cu) with the regression's first layer scaled to match and equalised per input (upload_head), and the activations and
+// W_i carry per-atom scales that are taken back in fp32.
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <new>
+#include <vector>
 
 #include "common.cuh"
 #include "pair_math.cuh"
@@ -49,17 +55,19 @@ constexpr int NG = 2;         // groups per CTA
 constexpr int NW = NG * TILE; // warps per CTA
 constexpr int PB_CAP = 160;   // queued pairs per warp: up to 31 left over + four list chunks of 32
 constexpr int J_BITS = 28;    // queue entries pack the neighbor index (low 28 bits) with its species
-constexpr int ST_STRIDE = 24; // encoding hand-over: 16 h, 4 b, table offset (bank-conflict-free for the fragment reads)
-constexpr int BS_STRIDE = 12; // derivation hand-over: 4 b, 4 b', table offset
+constexpr int ST_STRIDE = 20; // encoding hand-over: h as 8 words hi + 8 words lo (fp16 pairs), 4 b (80 bytes: conflict-free for ldmatrix and STS.128)
+constexpr int BS_STRIDE = 12; // derivation hand-over: 4 b, 4 b', row addresses
 constexpr int X_STRIDE = 132; // dE/dG per atom
-#ifndef MLIP_TAB_STRIDE
-#define MLIP_TAB_STRIDE 36
-#endif
-constexpr int TAB_STRIDE_SMEM = MLIP_TAB_STRIDE;   // padded table row in shared memory
 
+// Radial table rows (32 channels, 128 bytes, read by both pair loops) are stored with their eight 16-byte chunks permuted: chunk
+// c of row r sits at position c ^ table_swizzle(r).  Lanes that read the same chunk of rows with different r mod 4 then hit
+// different bank groups; every pair uses four consecutive rows, one of each residue, and the pair loops take them in an
+// order that gives the lanes of a load different residues (RowOffsets).  Without that the rows of a load are random and
+// collide: 6 instead of 4 wavefronts per pair in the derivation, and a shuffle per value in the encoding.
+static_assert(K_RADIAL == 32, "a table row is eight 16-byte chunks");
 constexpr int Q_WORDS = 4 * PB_CAP;                             // pair queue of a warp: kept from encoding to derivation
-constexpr int SCR_WORDS = 32 * ST_STRIDE;                       // scratch of a warp
-static_assert(32 * BS_STRIDE <= SCR_WORDS && N_INV <= SCR_WORDS, "the derivation's hand-over and the invariants must fit the encoding's");
+constexpr int SCR_WORDS = 32 * ST_STRIDE + 32 * 4;              // scratch of a warp: hand-over rows, table row addresses
+static_assert(32 * BS_STRIDE <= SCR_WORDS && N_INV <= 32 * ST_STRIDE, "the derivation's hand-over and the invariants must fit the encoding's");
 // Regression buffers of a group.  Activations are kept as B fragments: per 16-input k-step, atom row and quad lane one
 // 16-byte vector {b0 hi, b0 lo, b1 hi, b1 lo} of fp16 pairs (see act_store).
 constexpr int ACT_KSTEP = 32 * 4;                               // words per k-step
@@ -74,8 +82,9 @@ static_assert(2 * ZS_WORDS <= TILE * SCR_WORDS, "layer activations alias the scr
 //   pre-activation of layer L (input scaled by a per-atom 2^s): acc * (2^-s * HC_WS[L]) + bias
 //   |input of layer L| <= HC_BND[2L-2] * max|G| + HC_BND[2L-1]  (L = 1..3; row-sum norms of the weights)
 //   dE/dpre of layer L is stored times HC_SR[L]; its product with the weights is unscaled by HC_UR[L]
+//   the invariants enter, and dE/dG leaves, times HC_CS[input]: the powers of two that equalise the first layer's columns
 constexpr int HC_WOUT = HEAD_L * HEAD_H, HC_BOUT = HC_WOUT + HEAD_H, HC_WS = HC_BOUT + 1, HC_BND = HC_WS + HEAD_L;
-constexpr int HC_SR = HC_BND + 2 * (HEAD_L - 1), HC_UR = HC_SR + HEAD_L, HC_USED = HC_UR + HEAD_L;
+constexpr int HC_SR = HC_BND + 2 * (HEAD_L - 1), HC_UR = HC_SR + HEAD_L, HC_CS = HC_UR + HEAD_L, HC_USED = HC_CS + N_INV;
 constexpr int HC_WORDS = (HC_USED + 15) / 16 * 16;
 constexpr int64_t STAGGER_BELOW_ATOMS = 200000;                 // systems below this size start their CTAs on different species
 constexpr int PF_IDX = 160;                                     // neighbor indices prefetched per warp for its next atom
@@ -119,28 +128,6 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
     return d;
 }
 
-__device__ __forceinline__ void split_tf32(float x, uint32_t &hi, uint32_t &lo) {
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hi) : "f"(x));
-    lo = __float_as_uint(x - __uint_as_float(hi));
-}
-__device__ __forceinline__ float2 split_pair(float x) {
-    uint32_t hi, lo;
-    split_tf32(x, hi, lo);
-    return make_float2(__uint_as_float(hi), __uint_as_float(lo));
-}
-
-// Two-at-a-time variant for operands that feed forces only.  The tensor pipe reads the upper 19 bits of a TF32 operand
-// and ignores the rest, so the fp32 value itself serves as "hi" (= its truncation) and lo = x - trunc(x), taken for two
-// values by one packed subtract: 1.5 instructions per value instead of 2, at one bit less in the lo term.
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
-    unsigned long long ra, rb, rd;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(ra) : "f"(a.x), "f"(a.y));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(rb) : "f"(b.x), "f"(b.y));
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
-    float2 d;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(rd));
-    return d;
-}
 __device__ __forceinline__ float2 add2(float2 a, float2 b) {
     unsigned long long ra, rb, rd;
     asm("mov.b64 %0, {%1, %2};" : "=l"(ra) : "f"(a.x), "f"(a.y));
@@ -150,38 +137,6 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
     asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(rd));
     return d;
 }
-// Rounded hi/lo split of two values in four packed fp32 operations (Veltkamp's splitting with the constant 2^13 + 1:
-// hi keeps 11 significant bits, rounded to nearest, so it is exact in TF32; lo = x - hi exactly).  Same result as
-// split_tf32 up to ties, but on the FMA pipe and two values at a time -- the conversion instruction expands into integer
-// operations on the half-rate pipe.  For the energy path, where the truncating split's bias would show.
-// The product is written as an explicit fused multiply-add with a zero addend: given a separate packed multiply, the
-// assembler contracts it with the subtraction that follows (even with .rn on both), which turns the split into hi = x.
-__device__ __forceinline__ void split2_rn(float x, float y, uint32_t &xh, uint32_t &yh, uint32_t &xl, uint32_t &yl) {
-    const float2 v = make_float2(x, y);
-    const float2 c = ffma2(v, make_float2(8193.f, 8193.f), make_float2(0.f, 0.f));
-    const float2 hi = sub2(c, sub2(c, v));
-    const float2 lo = sub2(v, hi);
-    xh = __float_as_uint(hi.x); yh = __float_as_uint(hi.y); xl = __float_as_uint(lo.x); yl = __float_as_uint(lo.y);
-}
-__device__ __forceinline__ void split2_force(float x, float y, uint32_t &xh, uint32_t &yh, uint32_t &xl, uint32_t &yl) {
-    xh = __float_as_uint(x); yh = __float_as_uint(y);
-    const float2 lo = sub2(make_float2(x, y), make_float2(__uint_as_float(xh & 0xffffe000u), __uint_as_float(yh & 0xffffe000u)));
-    xl = __float_as_uint(lo.x); yl = __float_as_uint(lo.y);
-}
-
-__device__ __forceinline__ void mma_tf32(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-// d = A B (zero accumulator input: saves initialising the accumulator registers)
-__device__ __forceinline__ void mma_tf32_z(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
-        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
-}
-
 // x, y -> fp16 pairs hi, lo with hi + lo = x to 22 significant bits (x in the lower half; |x| must stay inside fp16's
 // range, which the callers' power-of-two scales see to: below 2^-3 of a scaled unit lo loses bits, an absolute 2^-25).
 __device__ __forceinline__ void split_h2(float x, float y, uint32_t &hi, uint32_t &lo) {
@@ -208,10 +163,14 @@ __device__ __forceinline__ float scale_for(float bound) {
 }
 __device__ __forceinline__ float inverse_pow2(float s) { return __uint_as_float((254u << 23) - __float_as_uint(s)); }
 
-// Every product A B below has both operands split: A_hi B_hi + A_lo B_hi + A_hi B_lo.  The tensor
-// pipe truncates when it adds into its fp32 accumulator, so the energy path keeps accumulation
-// chains short (a fresh accumulator per k-step, folded into the running sum by a rounded fp32
-// add): a long chain of same-sign terms otherwise drifts by ~1e-6 relative.
+// The tensor pipe truncates when it adds into its fp32 accumulator, so the energy path keeps accumulation chains short (a fresh
+// accumulator per k-step, folded into the running sum by a rounded fp32 add): a long chain of same-sign terms otherwise drifts
+// by ~1e-6 relative.
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // Deterministic mode (force_mode = 1): every sum whose order depends on scheduling -- the force scatter across
 // warps, the energy and virial totals -- is taken in integer arithmetic, which is associative, so two runs on the
@@ -261,13 +220,55 @@ __device__ __forceinline__ double4 load_pos4(const double4 *p) {
     return v;
 }
 
-// Where the radial tables of the current central species live: shared memory (rows padded to
-// TAB_STRIDE_SMEM, table index = neighbor species) or, when they do not fit, global memory.
+// The radial tables of the current central species: in shared memory or, when they do not fit, in global memory (same
+// layout).  Rows are numbered through the neighbor species.
 struct TableView {
     const float *base;
-    int row_stride;     // floats per row
-    int table_stride;   // floats per neighbor species
+    uint32_t saddr;   // shared-memory address of the first row (TAB_SMEM), a multiple of 128
 };
+template <bool TAB_SMEM>
+__device__ __forceinline__ float4 table_load(const TableView &tv, uint32_t off) {   // off: row address | chunk position, see RowOffsets
+    float4 v;
+    if (TAB_SMEM) asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(off));
+    else v = __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(tv.base) + off));
+    return v;
+}
+template <bool TAB_SMEM> constexpr int OFF_WORDS = TAB_SMEM ? 2 : 4;
+// Byte addresses of a pair's four rows in the order they are taken, handed from the lane that owns the pair to the lanes that
+// evaluate it: 16-bit shared-memory addresses (the tables come first in shared memory and end below 64 KB) or 32-bit offsets.
+template <bool TAB_SMEM> struct RowOffsets;
+template <> struct RowOffsets<true> {
+    uint2 o;
+    // rows first + ((turn + s) & 3), s = 0..3
+    __device__ __forceinline__ void make(const TableView &tv, int first, int turn) {
+        const uint32_t order = __funnelshift_r(0x03020100u, 0x03020100u, 8 * turn);   // bytes turn, turn + 1, .. mod 4
+        const uint32_t both = (tv.saddr + 128u * first) * 0x10001u;
+        o.x = __byte_perm(order, 0, 0x4140) * 128u + both;
+        o.y = __byte_perm(order, 0, 0x4342) * 128u + both;
+    }
+    __device__ __forceinline__ void store(float *p) const { *reinterpret_cast<uint2 *>(p) = o; }
+    __device__ __forceinline__ void load(const float *p) { o = *reinterpret_cast<const uint2 *>(p); }
+    // address of step s's row with the chunk position (a multiple of 16 below 128) put into its free low bits
+    __device__ __forceinline__ uint32_t at(int s, uint32_t chunk) const {
+        const uint32_t w = s < 2 ? o.x : o.y;
+        return s & 1 ? (w >> 16) | chunk : (w & 0xffffu) | chunk;
+    }
+};
+template <> struct RowOffsets<false> {
+    uint4 o;
+    __device__ __forceinline__ void make(const TableView &, int first, int turn) {
+        o = make_uint4(128u * (first + (turn & 3)), 128u * (first + ((turn + 1) & 3)), 128u * (first + ((turn + 2) & 3)), 128u * (first + ((turn + 3) & 3)));
+    }
+    __device__ __forceinline__ void store(float *p) const { *reinterpret_cast<uint4 *>(p) = o; }
+    __device__ __forceinline__ void load(const float *p) { o = *reinterpret_cast<const uint4 *>(p); }
+    __device__ __forceinline__ uint32_t at(int s, uint32_t chunk) const { return (s == 0 ? o.x : s == 1 ? o.y : s == 2 ? o.z : o.w) | chunk; }
+};
+// b[0..3] -> b[turn], b[turn + 1], .. (mod 4): spline weights in the order the rows are taken
+__device__ __forceinline__ float4 rotate4(const float (&b)[4], int turn) {
+    const bool r1 = turn & 1, r2 = turn & 2;
+    const float c0 = r1 ? b[1] : b[0], c1 = r1 ? b[2] : b[1], c2 = r1 ? b[3] : b[2], c3 = r1 ? b[0] : b[3];
+    return make_float4(r2 ? c2 : c0, r2 ? c3 : c1, r2 ? c0 : c2, r2 ? c1 : c3);
+}
 
 // Fill the warp's pair queue from list position `cur` on (lane = entry), up to five 32-entry chunks
 // at a time with all index loads, then all position gathers, in flight together (a typical list
@@ -339,7 +340,14 @@ __device__ __forceinline__ int encode_atom(const KernelArgs &k, const TableView 
                                            float4 *pq, float *stage, int lane, float (&Pf)[4][4], int &queued, const int *sidx, int n_pref,
                                            int cs, PhaseClock &pc) {
     const int g = lane >> 2, t = lane & 3;
-    constexpr int rs = TAB_SMEM ? TAB_STRIDE_SMEM : K_RADIAL;   // = tv.row_stride, known here so that row offsets fold into the loads
+    float *offs = stage + 32 * ST_STRIDE;
+    // k-step fragments: lane (g, t) evaluates chunk g (channels 4g ..) of pairs 2t, 2t + 1, 2t + 8, 2t + 9 of the k-step.  A pair
+    // in slot p takes its rows in the residue order p / 2, p / 2 + 1, .. (mod 4): the eight lanes of a load phase, two chunks of
+    // four pairs, then fall into eight bank groups.
+    uint32_t chunk[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) chunk[q] = 16u * (g ^ table_swizzle((t + q) & 3));
+    const uint32_t a_addr = smem_addr(stage) + ((lane & 7) + ((lane >> 4) << 3)) * (ST_STRIDE * 4) + ((lane >> 3) & 1) * 16;
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -348,96 +356,74 @@ __device__ __forceinline__ int encode_atom(const KernelArgs &k, const TableView 
     auto batch = [&](int first, int n) {
         {   // lane = pair: harmonics (Eq. 3) and spline basis
             float h[D_ANG], b[4];
-            int off = 0;
+            int row = 0;
             if (lane < n) {
                 const float4 e = pq[first + lane];
                 const float d2 = e.x * e.x + e.y * e.y + e.z * e.z, rinv = rsqrtf(d2), r = d2 * rinv;
                 harmonics(e.x * rinv, e.y * rinv, e.z * rinv, h);
                 const int iv = spline_basis<false, float>(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, b, nullptr, k.status);
-                const int sj = __float_as_int(e.w) >> J_BITS;
-                off = sj * tv.table_stride + iv * rs;
+                row = (__float_as_int(e.w) >> J_BITS) * (k.tab.knots + 3) + iv;
             } else {
 #pragma unroll
                 for (int a = 0; a < D_ANG; ++a) h[a] = 0.f;
                 b[0] = b[1] = b[2] = b[3] = 0.f;
             }
-            // 16-byte chunk c of row r is stored at chunk c ^ ((r >> 2) & 1): the eight rows of a store phase
-            // then fall into eight different bank groups (the row stride alone gives only four)
-            const int sw = (lane >> 2) & 1;
-            float4 *row = reinterpret_cast<float4 *>(stage + lane * ST_STRIDE);
-            row[0 ^ sw] = make_float4(h[0], h[1], h[2], h[3]);
-            row[1 ^ sw] = make_float4(h[4], h[5], h[6], h[7]);
-            row[2 ^ sw] = make_float4(h[8], h[9], h[10], h[11]);
-            row[3 ^ sw] = make_float4(h[12], h[13], h[14], h[15]);
-            row[4 ^ sw] = make_float4(b[0], b[1], b[2], b[3]);
-            reinterpret_cast<int *>(stage)[lane * ST_STRIDE + 4 * (5 ^ sw)] = off;
+            uint32_t hi[8], lo[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) split_h2(h[2 * q], h[2 * q + 1], hi[q], lo[q]);
+            uint4 *dst = reinterpret_cast<uint4 *>(stage + lane * ST_STRIDE);
+            dst[0] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            dst[1] = make_uint4(hi[4], hi[5], hi[6], hi[7]);
+            dst[2] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            dst[3] = make_uint4(lo[4], lo[5], lo[6], lo[7]);
+            const int turn = ((lane >> 1) - row) & 3;
+            *reinterpret_cast<float4 *>(dst + 4) = rotate4(b, turn);
+            RowOffsets<TAB_SMEM> ro;
+            ro.make(tv, row, turn);
+            ro.store(offs + lane * OFF_WORDS<TAB_SMEM>);
         }
         __syncwarp();
         pc.mark(1);
-        const int nks = (n + 7) >> 3;
-#ifndef MLIP_KSTEP_UNROLL
-#define MLIP_KSTEP_UNROLL 4
-#endif
-        constexpr int kstep_unroll = MLIP_KSTEP_UNROLL;
-#pragma unroll kstep_unroll
-        for (int ks = 0; ks < nks; ++ks) {
-            // A = H^T (16 x 8 pairs): rows a = g, g + 8; columns pairs t, t + 4 of this k-step
-            const float *ra = stage + (8 * ks + t) * ST_STRIDE, *rb = ra + 4 * ST_STRIDE;
-            uint32_t ah[4], al[4];
-            split2_rn(ra[g], ra[g + 8], ah[0], ah[1], al[0], al[1]);
-            split2_rn(rb[g ^ 4], rb[(g ^ 4) + 8], ah[2], ah[3], al[2], al[3]);   // rows t + 4 are stored with their chunk pairs swapped
-            // B = G (8 pairs x 8 channels per n-tile).  Evaluation pattern: quarter-warp q reads the table
-            // rows of ONE pair (8 lanes x 16 bytes = a full row per access: no bank conflicts), i.e. lane
-            // (q, c) evaluates channels 4c .. 4c+3 of pairs q and q + 4 of this k-step; a fixed shuffle
-            // then hands the values to the lane that owns them in the B fragment (pair t, channels 4g .. 4g+3).
-            const int q = lane >> 3, cch = lane & 7;
-            const float *qa = stage + (8 * ks + q) * ST_STRIDE, *qb = qa + 4 * ST_STRIDE;
-            const float4 ba = *reinterpret_cast<const float4 *>(qa + 16), bb = *reinterpret_cast<const float4 *>(qb + 20);
-            const float *ta = tv.base + reinterpret_cast<const int *>(qa)[20] + 4 * cch;
-            const float *tb = tv.base + reinterpret_cast<const int *>(qb)[16] + 4 * cch;
-            const float4 a0 = *reinterpret_cast<const float4 *>(ta), a1 = *reinterpret_cast<const float4 *>(ta + rs);
-            const float4 a2 = *reinterpret_cast<const float4 *>(ta + 2 * rs), a3 = *reinterpret_cast<const float4 *>(ta + 3 * rs);
-            const float4 b0 = *reinterpret_cast<const float4 *>(tb), b1 = *reinterpret_cast<const float4 *>(tb + rs);
-            const float4 b2 = *reinterpret_cast<const float4 *>(tb + 2 * rs), b3 = *reinterpret_cast<const float4 *>(tb + 3 * rs);
-            float ga[4], gb[4];
-            {   // g = sum_m b_m c_m for the four channels of each pair, two channels per packed FMA
-                float2 lo, hi;
-                lo = ffma2(make_float2(ba.x, ba.x), make_float2(a0.x, a0.y), make_float2(0.f, 0.f));
-                hi = ffma2(make_float2(ba.x, ba.x), make_float2(a0.z, a0.w), make_float2(0.f, 0.f));
-                lo = ffma2(make_float2(ba.y, ba.y), make_float2(a1.x, a1.y), lo);
-                hi = ffma2(make_float2(ba.y, ba.y), make_float2(a1.z, a1.w), hi);
-                lo = ffma2(make_float2(ba.z, ba.z), make_float2(a2.x, a2.y), lo);
-                hi = ffma2(make_float2(ba.z, ba.z), make_float2(a2.z, a2.w), hi);
-                lo = ffma2(make_float2(ba.w, ba.w), make_float2(a3.x, a3.y), lo);
-                hi = ffma2(make_float2(ba.w, ba.w), make_float2(a3.z, a3.w), hi);
-                ga[0] = lo.x; ga[1] = lo.y; ga[2] = hi.x; ga[3] = hi.y;
-                lo = ffma2(make_float2(bb.x, bb.x), make_float2(b0.x, b0.y), make_float2(0.f, 0.f));
-                hi = ffma2(make_float2(bb.x, bb.x), make_float2(b0.z, b0.w), make_float2(0.f, 0.f));
-                lo = ffma2(make_float2(bb.y, bb.y), make_float2(b1.x, b1.y), lo);
-                hi = ffma2(make_float2(bb.y, bb.y), make_float2(b1.z, b1.w), hi);
-                lo = ffma2(make_float2(bb.z, bb.z), make_float2(b2.x, b2.y), lo);
-                hi = ffma2(make_float2(bb.z, bb.z), make_float2(b2.z, b2.w), hi);
-                lo = ffma2(make_float2(bb.w, bb.w), make_float2(b3.x, b3.y), lo);
-                hi = ffma2(make_float2(bb.w, bb.w), make_float2(b3.z, b3.w), hi);
-                gb[0] = lo.x; gb[1] = lo.y; gb[2] = hi.x; gb[3] = hi.y;
-            }
-            const int owner_src = 8 * t + g;   // lane (g, t) takes (pair t, chunk g) from lane (q = t, c = g)
+        const int nks = (n + 15) >> 4;
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                ga[nt] = __shfl_sync(0xffffffffu, ga[nt], owner_src);
-                gb[nt] = __shfl_sync(0xffffffffu, gb[nt], owner_src);
-            }
-            // Eq. 4 for eight pairs; the three terms of each n-tile are issued interleaved over the n-tiles
+        for (int ks = 0; ks < 2; ++ks) {
+            if (ks >= nks) break;
+            // A = H^T (16 x 16 pairs), stored pair by pair: transposed on the way in
+            uint32_t ah[4], al[4];
+            ldmatrix_x4_trans(ah, a_addr + ks * (16 * ST_STRIDE * 4));
+            ldmatrix_x4_trans(al, a_addr + ks * (16 * ST_STRIDE * 4) + 32);
+            // B = G (16 pairs x 8 channels per n-tile; column g of n-tile c is channel 4 g + c): g = sum_m b_m c_m (Eq. 2)
             uint32_t bh[4][2], bl[4][2];
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                float gv[2][4];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int slot = 16 * ks + 8 * half + 2 * t + u;
+                    const float4 b = *reinterpret_cast<const float4 *>(stage + slot * ST_STRIDE + 16);
+                    RowOffsets<TAB_SMEM> ro;
+                    ro.load(offs + slot * OFF_WORDS<TAB_SMEM>);
+                    const float bw[4] = {b.x, b.y, b.z, b.w};
+                    float2 lo = make_float2(0.f, 0.f), hi = lo;
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {
+                        const float4 c = table_load<TAB_SMEM>(tv, ro.at(m, chunk[m]));
+                        lo = ffma2(make_float2(bw[m], bw[m]), make_float2(c.x, c.y), lo);
+                        hi = ffma2(make_float2(bw[m], bw[m]), make_float2(c.z, c.w), hi);
+                    }
+                    gv[u][0] = lo.x; gv[u][1] = lo.y; gv[u][2] = hi.x; gv[u][3] = hi.y;
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) split_h2(gv[0][c], gv[1][c], bh[c][half], bl[c][half]);
+            }
+            // Eq. 4 for sixteen pairs; the three terms of each n-tile are issued interleaved over the n-tiles
             float c[4][4];
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt) split2_rn(ga[nt], gb[nt], bh[nt][0], bh[nt][1], bl[nt][0], bl[nt][1]);
+            for (int nt = 0; nt < 4; ++nt) mma_f16_z(c[nt], al[0], al[1], al[2], al[3], bh[nt][0], bh[nt][1]);
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt) mma_tf32_z(c[nt], al[0], al[1], al[2], al[3], bh[nt][0], bh[nt][1]);
+            for (int nt = 0; nt < 4; ++nt) mma_f16(c[nt], ah[0], ah[1], ah[2], ah[3], bl[nt][0], bl[nt][1]);
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt) mma_tf32(c[nt], ah[0], ah[1], ah[2], ah[3], bl[nt][0], bl[nt][1]);
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) mma_tf32(c[nt], ah[0], ah[1], ah[2], ah[3], bh[nt][0], bh[nt][1]);
+            for (int nt = 0; nt < 4; ++nt) mma_f16(c[nt], ah[0], ah[1], ah[2], ah[3], bh[nt][0], bh[nt][1]);
 #pragma unroll
             for (int nt = 0; nt < 4; ++nt) {
                 const float2 s01 = add2(make_float2(Pf[nt][0], Pf[nt][1]), make_float2(c[nt][0], c[nt][1]));
@@ -514,30 +500,35 @@ __device__ __forceinline__ void tmem_fill(uint32_t quarter_base, const uint32_t 
 // ---------------- Derivation of one atom (Eq. 8-10) ----------------
 template <bool TAB_SMEM, bool DET, bool L16>
 __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView &tv, int i,
-                                            float4 *pq, float *scr, int queued, int lane, const uint32_t (&Wh)[4][4],
-                                            const uint32_t (&Wl)[4][4], float (&vir)[9], uint32_t tm_vt, PhaseClock &pc) {
+                                            float4 *pq, float *scr, int queued, int lane, const uint32_t (&Wh)[2][2][2],
+                                            const uint32_t (&Wl)[2][2][2], float w_scale_inv, float (&vir)[9], uint32_t tm_vt, PhaseClock &pc) {
+    // Wh, Wl [k-step][n-tile][b0, b1]: B fragments of W_i^T times 1 / w_scale_inv; k-step q holds channels 8t + 4q .. + 3 of lane (g, t)
     const int g = lane >> 2, t = lane & 3;
     float *bs = scr;
-    constexpr int rs = TAB_SMEM ? TAB_STRIDE_SMEM : K_RADIAL;
+    // tile fragments: lane (g, t) evaluates chunks 2t, 2t + 1 of pairs g, g + 8.  A pair in slot p takes its rows in the residue
+    // order p, p + 1, .. (mod 4): of the two pairs in a load phase one reads the even, the other the odd chunk positions.
+    uint32_t chunk[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) chunk[q] = 16u * ((2 * t) ^ table_swizzle((g + q) & 3));
     float fx = 0.f, fy = 0.f, fz = 0.f;
 
     auto batch = [&](int first, int n) {
         {   // lane = pair: spline basis and its derivative
             float b[4] = {0.f, 0.f, 0.f, 0.f}, db[4] = {0.f, 0.f, 0.f, 0.f};
-            int off = 0, row_index = 0;
-            const bool live = lane < n;
-            if (live) {
+            int row = 0;
+            if (lane < n) {
                 const float4 ent = pq[first + lane];
                 const float d2 = ent.x * ent.x + ent.y * ent.y + ent.z * ent.z, r = d2 * rsqrtf(d2);
-                const int iv = spline_basis<true, float>(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, b, db, k.status);
-                row_index = (__float_as_int(ent.w) >> J_BITS) * (k.tab.knots + 3) + iv;
-                off = row_index * rs;
+                const int iv = spline_basis<true, float, true>(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, b, db, k.status);
+                row = (__float_as_int(ent.w) >> J_BITS) * (k.tab.knots + 3) + iv;
             }
-            const int slot = lane;
-            float4 *row = reinterpret_cast<float4 *>(bs + slot * BS_STRIDE);
-            row[0] = make_float4(b[0], b[1], b[2], b[3]);
-            row[1] = make_float4(db[0], db[1], db[2], db[3]);
-            reinterpret_cast<int *>(bs)[slot * BS_STRIDE + 8] = off;
+            const int turn = (lane - row) & 3;
+            float *dst = bs + lane * BS_STRIDE;
+            *reinterpret_cast<float4 *>(dst) = rotate4(b, turn);
+            *reinterpret_cast<float4 *>(dst + 4) = rotate4(db, turn);
+            RowOffsets<TAB_SMEM> ro;
+            ro.make(tv, row, turn);
+            ro.store(dst + 8);
         }
         __syncwarp();
         pc.mark(4);
@@ -550,60 +541,58 @@ __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView
         for (int mt = 0; mt < nmt; ++mt) {
             // A = [G; G'] (16 pairs x 32 channels): rows pairs g, g + 8; this lane evaluates channels 8t .. 8t+7
             // (one accumulator per output here: the truncating accumulation costs ~1e-6 relative on a
-            // 12-term chain, irrelevant for forces, and the registers are needed elsewhere)
+            // short chain, irrelevant for forces, and the registers are needed elsewhere).  G' is the derivative per knot interval.
             float V[2][4], T[2][4];
-            float G[2][8], dG[2][8];
+            uint32_t ah[2][4], al[2][4], dh[2][4], dl[2][4];   // [k-step][fragment register]
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const float *rp = bs + (16 * mt + g + 8 * q) * BS_STRIDE;
                 const float4 b = *reinterpret_cast<const float4 *>(rp), db = *reinterpret_cast<const float4 *>(rp + 4);
-                const float *tc = tv.base + reinterpret_cast<const int *>(rp)[8] + 8 * t;
+                RowOffsets<TAB_SMEM> ro;
+                ro.load(rp + 8);
                 const float bw[4] = {b.x, b.y, b.z, b.w}, dbw[4] = {db.x, db.y, db.z, db.w};
                 float2 G2[4], dG2[4];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) { G2[c] = make_float2(0.f, 0.f); dG2[c] = make_float2(0.f, 0.f); }
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
-                    const float4 c0 = *reinterpret_cast<const float4 *>(tc + m * rs), c1 = *reinterpret_cast<const float4 *>(tc + m * rs + 4);
+                    const uint32_t at = ro.at(m, chunk[m]);
+                    const float4 c0 = table_load<TAB_SMEM>(tv, at), c1 = table_load<TAB_SMEM>(tv, at ^ 16u);
                     const float2 cv[4] = {make_float2(c0.x, c0.y), make_float2(c0.z, c0.w), make_float2(c1.x, c1.y), make_float2(c1.z, c1.w)};
                     const float2 b2 = make_float2(bw[m], bw[m]), db2 = make_float2(dbw[m], dbw[m]);
 #pragma unroll
                     for (int c = 0; c < 4; ++c) { G2[c] = ffma2(b2, cv[c], G2[c]); dG2[c] = ffma2(db2, cv[c], dG2[c]); }
                 }
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    G[q][2 * c] = G2[c].x; G[q][2 * c + 1] = G2[c].y;
-                    dG[q][2 * c] = dG2[c].x; dG[q][2 * c + 1] = dG2[c].y;
+                for (int c = 0; c < 4; ++c) {   // channel pair c: k-step c / 2, fragment register q + 2 (c % 2)
+                    split_h2(G2[c].x, G2[c].y, ah[c >> 1][q + 2 * (c & 1)], al[c >> 1][q + 2 * (c & 1)]);
+                    split_h2(dG2[c].x, dG2[c].y, dh[c >> 1][q + 2 * (c & 1)], dl[c >> 1][q + 2 * (c & 1)]);
                 }
             }
+            // Eq. 9 (rows of V: a = 0..7 and 8..15) and W g' (Eq. 8 re-associated); cross terms first, the four
+            // independent accumulators interleaved
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-                uint32_t ah[4], al[4], dh[4], dl[4];
-                split2_force(G[0][ks], G[1][ks], ah[0], ah[1], al[0], al[1]);
-                split2_force(G[0][4 + ks], G[1][4 + ks], ah[2], ah[3], al[2], al[3]);
-                split2_force(dG[0][ks], dG[1][ks], dh[0], dh[1], dl[0], dl[1]);
-                split2_force(dG[0][4 + ks], dG[1][4 + ks], dh[2], dh[3], dl[2], dl[3]);
-                // Eq. 9 (rows of V: a = 0..7 and 8..15) and W g' (Eq. 8 re-associated); cross terms first, the
-                // four independent accumulators interleaved
-                if (ks == 0) {
-                    mma_tf32_z(V[0], al[0], al[1], al[2], al[3], Wh[ks][0], Wh[ks][1]);
-                    mma_tf32_z(V[1], al[0], al[1], al[2], al[3], Wh[ks][2], Wh[ks][3]);
-                    mma_tf32_z(T[0], dl[0], dl[1], dl[2], dl[3], Wh[ks][0], Wh[ks][1]);
-                    mma_tf32_z(T[1], dl[0], dl[1], dl[2], dl[3], Wh[ks][2], Wh[ks][3]);
-                } else {
-                    mma_tf32(V[0], al[0], al[1], al[2], al[3], Wh[ks][0], Wh[ks][1]);
-                    mma_tf32(V[1], al[0], al[1], al[2], al[3], Wh[ks][2], Wh[ks][3]);
-                    mma_tf32(T[0], dl[0], dl[1], dl[2], dl[3], Wh[ks][0], Wh[ks][1]);
-                    mma_tf32(T[1], dl[0], dl[1], dl[2], dl[3], Wh[ks][2], Wh[ks][3]);
+            for (int ks = 0; ks < 2; ++ks) {
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt) {
+                    if (ks == 0) {
+                        mma_f16_z(V[nt], al[ks][0], al[ks][1], al[ks][2], al[ks][3], Wh[ks][nt][0], Wh[ks][nt][1]);
+                        mma_f16_z(T[nt], dl[ks][0], dl[ks][1], dl[ks][2], dl[ks][3], Wh[ks][nt][0], Wh[ks][nt][1]);
+                    } else {
+                        mma_f16(V[nt], al[ks][0], al[ks][1], al[ks][2], al[ks][3], Wh[ks][nt][0], Wh[ks][nt][1]);
+                        mma_f16(T[nt], dl[ks][0], dl[ks][1], dl[ks][2], dl[ks][3], Wh[ks][nt][0], Wh[ks][nt][1]);
+                    }
                 }
-                mma_tf32(V[0], ah[0], ah[1], ah[2], ah[3], Wl[ks][0], Wl[ks][1]);
-                mma_tf32(V[1], ah[0], ah[1], ah[2], ah[3], Wl[ks][2], Wl[ks][3]);
-                mma_tf32(T[0], dh[0], dh[1], dh[2], dh[3], Wl[ks][0], Wl[ks][1]);
-                mma_tf32(T[1], dh[0], dh[1], dh[2], dh[3], Wl[ks][2], Wl[ks][3]);
-                mma_tf32(V[0], ah[0], ah[1], ah[2], ah[3], Wh[ks][0], Wh[ks][1]);
-                mma_tf32(V[1], ah[0], ah[1], ah[2], ah[3], Wh[ks][2], Wh[ks][3]);
-                mma_tf32(T[0], dh[0], dh[1], dh[2], dh[3], Wh[ks][0], Wh[ks][1]);
-                mma_tf32(T[1], dh[0], dh[1], dh[2], dh[3], Wh[ks][2], Wh[ks][3]);
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt) {
+                    mma_f16(V[nt], ah[ks][0], ah[ks][1], ah[ks][2], ah[ks][3], Wl[ks][nt][0], Wl[ks][nt][1]);
+                    mma_f16(T[nt], dh[ks][0], dh[ks][1], dh[ks][2], dh[ks][3], Wl[ks][nt][0], Wl[ks][nt][1]);
+                }
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt) {
+                    mma_f16(V[nt], ah[ks][0], ah[ks][1], ah[ks][2], ah[ks][3], Wh[ks][nt][0], Wh[ks][nt][1]);
+                    mma_f16(T[nt], dh[ks][0], dh[ks][1], dh[ks][2], dh[ks][3], Wh[ks][nt][0], Wh[ks][nt][1]);
+                }
             }
             // The accumulator fragments of the 16 pairs go to tensor memory as 16 lanes (pair) x 32 columns (V, T); read back
             // below with lane = pair.  (Through shared memory the same exchange was 188 of the kernel's 1,958 L1 wavefronts per
@@ -626,10 +615,11 @@ __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView
             const float ux = x * rinv, uy = y * rinv, uz = z * rinv;
             float s, tx, ty, tz, tu;
             harmonics_project(ux, uy, uz, v, tt, s, tx, ty, tz, tu);
-            // f_ij = (g' . u_ij) r^ + J_ang^T v_ij,  J_ang = (grad_u h)(I - u u^T) / r
-            const float qx = s * ux + (tx - tu * ux) * rinv;
-            const float qy = s * uy + (ty - tu * uy) * rinv;
-            const float qz = s * uz + (tz - tu * uz) * rinv;
+            // f_ij = (g' . u_ij) r^ + J_ang^T v_ij,  J_ang = (grad_u h)(I - u u^T) / r, the scales taken back
+            const float sr = s * (w_scale_inv * k.tab.inv_h), vr = rinv * w_scale_inv;
+            const float qx = sr * ux + (tx - tu * ux) * vr;
+            const float qy = sr * uy + (ty - tu * uy) * vr;
+            const float qz = sr * uz + (tz - tu * uz) * vr;
             fx += qx; fy += qy; fz += qz;
             if (DET) fixed_add3(k.force_fx + 3 * (size_t)j, -qx, -qy, -qz);
             else atomicAdd(&k.force[j], make_float4(-qx, -qy, -qz, 0.f));   // one 128-bit reduction per pair
@@ -759,7 +749,9 @@ struct NextAtom {
 __device__ __forceinline__ void split_invariants(const float *xrow, float *xs, float *sc, const float *hc, int atom, int lane) {
     // lane handles the pairs (c, c + 8) number lane and lane + 32 of the 64: k-step p / 8, j = p % 8
     const int j = lane & 7, s0 = lane >> 3, s1 = s0 + 4;
-    const float a0 = xrow[16 * s0 + j], a1 = xrow[16 * s0 + 8 + j], b0 = xrow[16 * s1 + j], b1 = xrow[16 * s1 + 8 + j];
+    const float *cs = hc + HC_CS;
+    const float a0 = xrow[16 * s0 + j] * cs[16 * s0 + j], a1 = xrow[16 * s0 + 8 + j] * cs[16 * s0 + 8 + j];
+    const float b0 = xrow[16 * s1 + j] * cs[16 * s1 + j], b1 = xrow[16 * s1 + 8 + j] * cs[16 * s1 + 8 + j];
     const float most = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fmaxf(fabsf(a0), fabsf(a1)), fmaxf(fabsf(b0), fabsf(b1))))));
     const float sx = scale_for(most);
     uint32_t hi, lo;
@@ -871,20 +863,20 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
         tmem_ld32(tm + TM_BWD0 + 32 * (wg >> 2), w);
         tmem_wait_ld();
         head_gemm(c, w, reinterpret_cast<const uint4 *>(zs) + frag);   // layer 0's dE/dpre: buffer 0
-        const float u = hc[HC_UR];
+        const float u = hc[HC_UR], ua = u * hc[HC_CS + 16 * wg + g], ub = u * hc[HC_CS + 16 * wg + g + 8];
         float *p = sX + 2 * t * X_STRIDE + 16 * wg + g;
-        p[0] = c[0] * u; p[X_STRIDE] = c[1] * u; p[8] = c[2] * u; p[X_STRIDE + 8] = c[3] * u;
+        p[0] = c[0] * ua; p[X_STRIDE] = c[1] * ua; p[8] = c[2] * ub; p[X_STRIDE + 8] = c[3] * ub;
     }
     group_sync(group);
 }
 
 template <bool TAB_SMEM, bool DET, bool L16, bool STAGGER>
 __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words) {
-    extern __shared__ __align__(16) float smem[];
+    extern __shared__ __align__(128) float smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int group = warp / TILE, wg = warp % TILE;
     const int g = lane >> 2, t = lane & 3;
-    float *s_tab = smem;                                   // [C][rows][TAB_STRIDE_SMEM] when TAB_SMEM
+    float *s_tab = smem;                                   // [C][rows][K_RADIAL] when TAB_SMEM
     float *xs = smem + (TAB_SMEM ? tab_words : 0) + group * GROUP_WORDS;
     float *sX = xs + XS_WORDS, *sc = sX + SX_WORDS, *ep = sc + SC_WORDS;
     float *scr_all = smem + (TAB_SMEM ? tab_words : 0) + NG * GROUP_WORDS;
@@ -934,15 +926,14 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
         if (threadIdx.x == 0) ctl[6 + (ss & 1)] = *reinterpret_cast<volatile int *>(k.tile_counter + species);
         __syncthreads();   // both groups are done with the previous species' tables
         if (ctl[6 + (ss & 1)] >= n_tiles) continue;
+        const float *tab = k.tab.coef + (size_t)species * k.n_species * rows * K_RADIAL;
         if (TAB_SMEM) {
-            const float4 *src = reinterpret_cast<const float4 *>(k.tab.coef + (size_t)species * k.n_species * rows * K_RADIAL);
+            const float4 *src = reinterpret_cast<const float4 *>(tab);
             const int n4 = k.n_species * rows * (K_RADIAL / 4);
-            for (int idx = threadIdx.x; idx < n4; idx += NW * 32)
-                *reinterpret_cast<float4 *>(s_tab + (idx >> 3) * TAB_STRIDE_SMEM + 4 * (idx & 7)) = __ldg(src + idx);
-            tv.base = s_tab; tv.row_stride = TAB_STRIDE_SMEM; tv.table_stride = rows * TAB_STRIDE_SMEM;
+            for (int idx = threadIdx.x; idx < n4; idx += NW * 32) reinterpret_cast<float4 *>(s_tab)[idx] = __ldg(src + idx);
+            tv.base = s_tab; tv.saddr = smem_addr(s_tab);
         } else {
-            tv.base = k.tab.coef + (size_t)species * k.n_species * rows * K_RADIAL;
-            tv.row_stride = K_RADIAL; tv.table_stride = rows * K_RADIAL;
+            tv.base = tab; tv.saddr = 0;
         }
         const uint32_t *hp = k.head_pack + (size_t)species * HP_TOTAL;
         for (int idx = threadIdx.x; idx < HC_USED; idx += NW * 32) hc[idx] = __uint_as_float(__ldg(hp + HP_TMEM + idx));
@@ -1047,17 +1038,26 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
                     da[0] = a0.x; da[1] = a0.y; da[2] = a0.z; da[3] = a0.w; da[4] = a1.x; da[5] = a1.y; da[6] = a1.z; da[7] = a1.w;
                     db[0] = b0.x; db[1] = b0.y; db[2] = b0.z; db[3] = b0.w; db[4] = b1.x; db[5] = b1.y; db[6] = b1.z; db[7] = b1.w;
                 }
-                uint32_t Wh[4][4], Wl[4][4];
+                float w[4][4];   // [nt][0, 1]: row a = g, channels 8t + nt and 8t + 4 + nt; [2, 3]: row g + 8
+                float most = 0.f;
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks) {
-                    const float w0 = g == 0 ? da[ks] : 2.f * da[ks] * Pf[ks][0];          // row a = g,     channel 8t + ks
-                    const float w1 = g == 0 ? da[4 + ks] : 2.f * da[4 + ks] * Pf[ks][1];  // row a = g,     channel 8t + 4 + ks
-                    const float w2 = 2.f * db[ks] * Pf[ks][2];                            // row a = g + 8, channel 8t + ks
-                    const float w3 = 2.f * db[4 + ks] * Pf[ks][3];                        // row a = g + 8, channel 8t + 4 + ks
-                    split2_rn(w0, w1, Wh[ks][0], Wh[ks][1], Wl[ks][0], Wl[ks][1]);   // once per atom: the rounded split
-                    split2_rn(w2, w3, Wh[ks][2], Wh[ks][3], Wl[ks][2], Wl[ks][3]);
+                for (int nt = 0; nt < 4; ++nt) {
+                    w[nt][0] = g == 0 ? da[nt] : 2.f * da[nt] * Pf[nt][0];
+                    w[nt][1] = g == 0 ? da[4 + nt] : 2.f * da[4 + nt] * Pf[nt][1];
+                    w[nt][2] = 2.f * db[nt] * Pf[nt][2];
+                    w[nt][3] = 2.f * db[4 + nt] * Pf[nt][3];
+                    most = fmaxf(fmaxf(most, fmaxf(fabsf(w[nt][0]), fabsf(w[nt][1]))), fmaxf(fabsf(w[nt][2]), fabsf(w[nt][3])));
                 }
-                derive_atom<TAB_SMEM, DET, L16>(k, tv, i, pq, scr, queued, lane, Wh, Wl, vir, tm_vt, pc);
+                const float sw = scale_for(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(most))));
+                uint32_t Wh[2][2][2], Wl[2][2][2];
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+                    for (int nt = 0; nt < 2; ++nt) {
+                        split_h2(w[0][2 * nt + ks] * sw, w[1][2 * nt + ks] * sw, Wh[ks][nt][0], Wl[ks][nt][0]);
+                        split_h2(w[2][2 * nt + ks] * sw, w[3][2 * nt + ks] * sw, Wh[ks][nt][1], Wl[ks][nt][1]);
+                    }
+                derive_atom<TAB_SMEM, DET, L16>(k, tv, i, pq, scr, queued, lane, Wh, Wl, inverse_pow2(sw), vir, tm_vt, pc);
                 if (DET) {   // fold this atom's virial in now: lane sums in a fixed order, then integers
 #pragma unroll
                     for (int q = 0; q < 9; ++q) {
@@ -1096,40 +1096,78 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
 }
 
 // ---------------- host side ----------------
-int table_smem_words(const mlip_ctx *c) { return c->cfg.n_species * (c->cfg.table_knots + 3) * TAB_STRIDE_SMEM; }
-bool tables_fit_smem(const mlip_ctx *c) { return FIXED_WORDS + table_smem_words(c) <= SMEM_LIMIT_WORDS; }
+int table_smem_words(const mlip_ctx *c) { return c->cfg.n_species * (c->cfg.table_knots + 3) * K_RADIAL; }
+bool tables_fit_smem(const mlip_ctx *c) {   // (the rows' 16-bit addresses, with room for a reserved kilobyte in front, are the tighter limit)
+    return FIXED_WORDS + table_smem_words(c) <= SMEM_LIMIT_WORDS && 4 * table_smem_words(c) + 2048 <= 65536;
+}
 
 static float pow2f(int e) { return ldexpf(1.f, e); }
 
+// The tensor-memory image of the weights, one thread per word: A fragments; k-step ks, lane (g, t), register r holds row
+// 16 m + g + 8 (r & 1) and the k pair (n, n + 8) with n = 16 ks + t + 4 (r >> 1)  (see act_store).
+struct HeadScales { float w[MAX_SPECIES][HEAD_L]; };
+__global__ void k_pack_head(const double *__restrict__ nets, HeadScales sc, uint32_t *__restrict__ image) {
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x, s = blockIdx.y;
+    const int lane = (idx >> 2) & 31, col = 4 * ((idx >> 7) % (TM_VT / 4)) + (idx & 3), quarter = (idx >> 7) / (TM_VT / 4);
+    const int g = lane >> 2, t = lane & 3, r = col & 3, row = g + 8 * (r & 1), n = t + 4 * (r >> 1);
+    int L, m = quarter, ks;
+    bool reverse = col >= TM_BWD;
+    if (col < TM_FWD) { L = 0; ks = col >> 3; }
+    else if (col < TM_BWD) { L = 1 + (col - TM_FWD) / 32; ks = ((col - TM_FWD) & 31) >> 3; }
+    else if (col < TM_BWD0) { L = 1 + (col - TM_BWD) / 32; ks = ((col - TM_BWD) & 31) >> 3; }
+    else { L = 0; m += 4 * ((col - TM_BWD0) / 32); ks = ((col - TM_BWD0) & 31) >> 3; }
+    const int in = L == 0 ? N_INV : HEAD_H;
+    const double *W = nets + (size_t)s * HEAD_NET + (L == 0 ? 0 : N_INV * HEAD_H + HEAD_H + (L - 1) * (HEAD_H * HEAD_H + HEAD_H));
+    // forward: A[m][k] = W[m][k]; reverse: A[m][k] = W[k][m]
+    const double *src = reverse ? W + (size_t)(16 * ks + n) * in + 16 * m + row : W + (size_t)(16 * m + row) * in + 16 * ks + n;
+    uint32_t hi, lo;
+    split_h2((float)src[0] * sc.w[s][L], (float)src[reverse ? 8 * in : 8] * sc.w[s][L], hi, lo);
+    image[(size_t)s * HP_TOTAL + idx] = col & 4 ? lo : hi;
+}
+
+// (after build_tables: the first layer is scaled to match the tables)
 int upload_head(mlip_ctx *c, const double *w) {
     const int C = c->cfg.n_species;
-    uint32_t *host = (uint32_t *)calloc((size_t)C * HP_TOTAL, sizeof(uint32_t));
-    if (!host) return MLIP_ERR_OOM;
+    std::vector<double> scaled;    // the networks with the first layer's columns equalised
+    std::vector<float> consts;     // [C][HC_USED]
+    try { scaled.assign(w, w + (size_t)C * HEAD_NET); consts.resize((size_t)C * HC_USED); } catch (const std::bad_alloc &) { return MLIP_ERR_OOM; }
+    HeadScales scales;
     for (int s = 0; s < C; ++s) {
-        const double *layer[HEAD_L], *out = w + (size_t)s * HEAD_NET;
+        const double *layer[HEAD_L], *out = scaled.data() + (size_t)s * HEAD_NET;
         int in_of[HEAD_L];
         for (int L = 0, in = N_INV; L < HEAD_L; ++L, in = HEAD_H) { layer[L] = out; in_of[L] = in; out += in * HEAD_H + HEAD_H; }
-        uint32_t *hp = host + (size_t)s * HP_TOTAL;
-        float *hc = reinterpret_cast<float *>(hp + HP_TMEM);
+        float *hc = consts.data() + (size_t)s * HC_USED;
+        // The tables carry 2^table_exp per channel, the moments too, the invariants once (l = 0) or squared: the weights take the
+        // inverse.  Then every column is brought to a largest weight in [1/2, 1) and its invariant multiplied by what was
+        // divided out, so that the values in one contraction are compared by what they contribute.
+        double *first = scaled.data() + (size_t)s * HEAD_NET, most_of[N_INV] = {0.0};
+        for (int o = 0; o < HEAD_H; ++o)
+            for (int q = 0; q < N_INV; ++q) most_of[q] = std::max(most_of[q], fabs(first[(size_t)o * N_INV + q]));
+        for (int q = 0; q < N_INV; ++q) {
+            int e = 0;
+            if (most_of[q] > 0.0) frexp(most_of[q], &e);
+            const int te = c->table_exp[s * K_RADIAL + q % K_RADIAL] * (q < K_RADIAL ? 1 : 2);
+            const int ce = std::max(-126, std::min(126, e - te));
+            hc[HC_CS + q] = pow2f(ce);
+            most_of[q] = ldexp(1.0, -te - ce);
+        }
+        for (int o = 0; o < HEAD_H; ++o)
+            for (int q = 0; q < N_INV; ++q) first[(size_t)o * N_INV + q] *= most_of[q];
         // powers of two: weights of a layer to below 2^14; bounds of the layers' inputs from row sums, of dE/dpre from column sums
         // (both a little enlarged for the device's fp32 arithmetic)
-        float wscale[HEAD_L];
+        float *wscale = scales.w[s];
         double row_sum[HEAD_L], bias_max[HEAD_L], col_sum[HEAD_L], wout_max = 0.0;
         for (int L = 0; L < HEAD_L; ++L) {
             const int in = in_of[L];
-            double most = 0.0;
+            double most = 0.0, col[N_INV] = {0.0};
             row_sum[L] = bias_max[L] = col_sum[L] = 0.0;
             for (int o = 0; o < HEAD_H; ++o) {
                 double r = 0.0;
-                for (int q = 0; q < in; ++q) { const double a = fabs(layer[L][(size_t)o * in + q]); r += a; most = std::max(most, a); }
+                for (int q = 0; q < in; ++q) { const double a = fabs(layer[L][(size_t)o * in + q]); r += a; col[q] += a; most = std::max(most, a); }
                 row_sum[L] = std::max(row_sum[L], r);
                 bias_max[L] = std::max(bias_max[L], fabs(layer[L][(size_t)in * HEAD_H + o]));
             }
-            for (int q = 0; q < in; ++q) {
-                double r = 0.0;
-                for (int o = 0; o < HEAD_H; ++o) r += fabs(layer[L][(size_t)o * in + q]);
-                col_sum[L] = std::max(col_sum[L], r);
-            }
+            for (int q = 0; q < in; ++q) col_sum[L] = std::max(col_sum[L], col[q]);
             int e = 0;
             if (most > 0.0) frexp(most, &e);
             wscale[L] = pow2f(std::min(14 - e, 60));
@@ -1157,39 +1195,18 @@ int upload_head(mlip_ctx *c, const double *w) {
             for (int o = 0; o < HEAD_H; ++o) hc[L * HEAD_H + o] = (float)layer[L][(size_t)in_of[L] * HEAD_H + o];
         for (int o = 0; o < HEAD_H; ++o) hc[HC_WOUT + o] = (float)out[o];
         hc[HC_BOUT] = (float)out[HEAD_H];
-        // A fragments: k-step ks, lane (g, t), register r holds row 16 m + g + 8 (r & 1) and the k pair (n, n + 8) with
-        // n = 16 ks + t + 4 (r >> 1)  (see act_store)
-        auto put = [&](int quarter, int col, int lane, double lo_k, double hi_k, float sc) {
-            auto half_bits = [](float x) { const __half h = __float2half_rn(x); return (uint32_t)__half_as_ushort(h); };
-            auto rest = [](float x) { return x - __half2float(__float2half_rn(x)); };
-            const float x = (float)lo_k * sc, y = (float)hi_k * sc;
-            const auto word = [&](int cc) -> uint32_t & { return hp[(((size_t)quarter * (TM_VT / 4) + cc / 4) * 32 + lane) * 4 + cc % 4]; };
-            word(col) = half_bits(x) | half_bits(y) << 16;
-            word(col + 4) = half_bits(rest(x)) | half_bits(rest(y)) << 16;
-        };
-        for (int L = 0; L < HEAD_L; ++L) {
-            const int in = in_of[L];
-            const double *W = layer[L];
-            for (int lane = 0; lane < 32; ++lane)
-                for (int r = 0; r < 4; ++r) {
-                    const int g = lane >> 2, t = lane & 3, row = g + 8 * (r & 1), n = t + 4 * (r >> 1);
-                    for (int mt = 0; mt < 4; ++mt)   // forward: A[m][k] = W[m][k]
-                        for (int ks = 0; ks < in / 16; ++ks) {
-                            const double *src = W + (size_t)(16 * mt + row) * in + 16 * ks + n;
-                            put(mt, (L == 0 ? TM_FWD0 : TM_FWD + 32 * (L - 1)) + 8 * ks + r, lane, src[0], src[8], wscale[L]);
-                        }
-                    for (int m = 0; m < in / 16; ++m)   // reverse: A[m][k] = W[k][m]
-                        for (int ks = 0; ks < HEAD_H / 16; ++ks) {
-                            const double *src = W + (size_t)(16 * ks + n) * in + 16 * m + row;
-                            put(m & 3, (L == 0 ? TM_BWD0 + 32 * (m >> 2) : TM_BWD + 32 * (L - 1)) + 8 * ks + r, lane, src[0], src[(size_t)8 * in], wscale[L]);
-                        }
-                }
-        }
     }
-    const size_t bytes = sizeof(uint32_t) * (size_t)C * HP_TOTAL;
-    cudaError_t e = cudaMalloc(&c->head_w, bytes);
-    if (e == cudaSuccess) e = cudaMemcpy(c->head_w, host, bytes, cudaMemcpyHostToDevice);
-    free(host);
+    const size_t bytes = sizeof(uint32_t) * (size_t)C * HP_TOTAL, net_bytes = sizeof(double) * (size_t)C * HEAD_NET;
+    double *nets = nullptr;
+    MLIP_CUDA_TRY(c, cudaMalloc(&c->head_w, bytes));
+    MLIP_CUDA_TRY(c, cudaMalloc(&nets, net_bytes));
+    cudaError_t e = cudaMemcpy(nets, scaled.data(), net_bytes, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        k_pack_head<<<dim3(4 * TM_VT * 32 / 256, C), 256>>>(nets, scales, c->head_w);
+        c->launches += 1;
+        e = cudaMemcpy2D(c->head_w + HP_TMEM, sizeof(uint32_t) * HP_TOTAL, consts.data(), sizeof(float) * HC_USED, sizeof(float) * HC_USED, C, cudaMemcpyHostToDevice);
+    }
+    cudaFree(nets);
     if (e != cudaSuccess) { c->err = cudaGetErrorString(e); return MLIP_ERR_CUDA; }
     c->resident += bytes;
     return MLIP_OK;

@@ -65,7 +65,8 @@ __device__ __forceinline__ void harmonics_project(T x, T y, T z, const T *v, con
 
 // Spline interval and cubic B-spline basis (and its r-derivative) at distance r for a table of
 // `knots` intervals of width 1 / inv_h starting at r_min.
-template <bool DERIV, typename T>
+// PER_KNOT: the derivative per knot interval instead of per Angstrom (without the factor inv_h).
+template <bool DERIV, typename T, bool PER_KNOT = false>
 __device__ __forceinline__ int spline_basis(T r, T r_min, T inv_h, int knots, T *b, T *db, int *status) {
     T xk = (r - r_min) * inv_h;
     if (xk < T(0)) { atomicOr(status, FLAG_TABLE_RANGE); xk = T(0); }
@@ -78,10 +79,11 @@ __device__ __forceinline__ int spline_basis(T r, T r_min, T inv_h, int knots, T 
     b[2] = (T(-3) * u3 + T(3) * u2 + T(3) * u + T(1)) * sixth;
     b[3] = u3 * sixth;
     if (DERIV) {
-        db[0] = T(-0.5) * w * w * inv_h;
-        db[1] = (T(1.5) * u2 - T(2) * u) * inv_h;
-        db[2] = (T(-1.5) * u2 + u + T(0.5)) * inv_h;
-        db[3] = T(0.5) * u2 * inv_h;
+        const T per = PER_KNOT ? T(1) : inv_h;
+        db[0] = T(-0.5) * w * w * per;
+        db[1] = (T(1.5) * u2 - T(2) * u) * per;
+        db[2] = (T(-1.5) * u2 + u + T(0.5)) * per;
+        db[3] = T(0.5) * u2 * per;
     }
     return i;
 }

@@ -4,6 +4,9 @@
 // by a C^2 cubic B-spline with clamped (first-derivative) ends on [r_min, r_cut].  g'(r) used
 // by the force (Eq. 10) is the exact derivative of that spline, so energies and forces stay
 // consistent.  The spline is then compared with the network between the knots.
+#include <math.h>
+#include <string.h>
+
 #include "common.cuh"
 
 namespace mlip {
@@ -138,6 +141,28 @@ __global__ void k_table_check(const double *__restrict__ val, const double *__re
     for (int q = 0; q < 4; ++q) atomic_max_pos(out + q, m[q]);
 }
 
+// Finish the fp32 tables for the fused kernel: find max |coefficient| of every (central species, channel); then scale each by a
+// power of two (so that table values and their derivatives per knot fit fp16 hi + lo pairs at full precision) and put the rows'
+// chunks into their bank order.  Rows are numbered through each central species' block of `rows_per_species`.
+__global__ void k_table_max(const float *__restrict__ coef, int rows_per_species, unsigned int *__restrict__ out) {
+    const int species = blockIdx.x, channel = threadIdx.x & (K_RADIAL - 1);
+    unsigned int m = 0;
+    for (int r = threadIdx.x / K_RADIAL; r < rows_per_species; r += blockDim.x / K_RADIAL)
+        m = max(m, __float_as_uint(fabsf(coef[((size_t)species * rows_per_species + r) * K_RADIAL + channel])));
+    atomicMax(out + species * K_RADIAL + channel, m);
+}
+__global__ void k_table_finish(float *__restrict__ coef, int n_rows, int rows_per_species, const float *__restrict__ scale) {
+    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    if (row >= n_rows) return;
+    float4 *p = reinterpret_cast<float4 *>(coef) + (size_t)row * (K_RADIAL / 4), v[K_RADIAL / 4];
+    const float4 *sc = reinterpret_cast<const float4 *>(scale) + (size_t)(row / rows_per_species) * (K_RADIAL / 4);
+    const int sw = table_swizzle(row % rows_per_species);
+#pragma unroll
+    for (int q = 0; q < K_RADIAL / 4; ++q) v[q] = p[q];
+#pragma unroll
+    for (int q = 0; q < K_RADIAL / 4; ++q) { const float4 f = sc[q]; p[q ^ sw] = make_float4(v[q].x * f.x, v[q].y * f.y, v[q].z * f.z, v[q].w * f.w); }
+}
+
 int build_tables(mlip_ctx *c, const double *enc_w_host, size_t n_enc) {
     const mlip_config &cfg = c->cfg;
     const int C = cfg.n_species, n_nets = C * C, K = cfg.table_knots, k = cfg.k, H = cfg.enc_hidden;
@@ -180,6 +205,26 @@ int build_tables(mlip_ctx *c, const double *enc_w_host, size_t n_enc) {
     if (f64) k_table_check<double><<<(nt + 63) / 64, 64>>>(val, der, c->table_d, n_nets, n_chk, K, k, r_min, r0, step, h, stats);
     else k_table_check<float><<<(nt + 63) / 64, 64>>>(val, der, c->table, n_nets, n_chk, K, k, r_min, r0, step, h, stats);
     c->launches += 4;
+    if (!f64) {
+        // (the solver's scratch is free: 2 (K + 1) doubles for every (pair, channel))
+        unsigned int *most_dev = reinterpret_cast<unsigned int *>(work), most_bits[MAX_SPECIES * K_RADIAL];
+        float scale[MAX_SPECIES * K_RADIAL];
+        const size_t bytes = sizeof(float) * C * K_RADIAL;
+        MLIP_CUDA_TRY(c, cudaMemset(most_dev, 0, bytes));
+        k_table_max<<<C, 1024>>>(c->table, C * (K + 3), most_dev);
+        MLIP_CUDA_TRY(c, cudaMemcpy(most_bits, most_dev, bytes, cudaMemcpyDeviceToHost));
+        for (int q = 0; q < C * K_RADIAL; ++q) {
+            float most;
+            memcpy(&most, &most_bits[q], sizeof most);
+            int e = 14;
+            if (most > 0.f && isfinite(most)) frexpf(most, &e);
+            c->table_exp[q] = e < -100 ? 114 : 14 - e;   // |coefficient| < 2^14; |derivative per knot| <= 1.5 times that
+            scale[q] = ldexpf(1.f, c->table_exp[q]);
+        }
+        MLIP_CUDA_TRY(c, cudaMemcpy(most_dev, scale, bytes, cudaMemcpyHostToDevice));
+        k_table_finish<<<(n_nets * (K + 3) + 63) / 64, 64>>>(c->table, n_nets * (K + 3), C * (K + 3), reinterpret_cast<const float *>(most_dev));
+        c->launches += 2;
+    }
     unsigned long long host_stats[4];
     MLIP_CUDA_TRY(c, cudaMemcpy(host_stats, stats, sizeof host_stats, cudaMemcpyDeviceToHost));
     MLIP_CUDA_TRY(c, cudaDeviceSynchronize());
