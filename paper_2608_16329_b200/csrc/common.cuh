@@ -15,7 +15,6 @@ constexpr int N_INV = 128;     // (l_max + 1) * k invariants (Eq. 5)
 constexpr int HEAD_H = 64;     // head width (Section 4.1.3)
 constexpr int HEAD_L = 4;      // head hidden layers
 constexpr int MAX_SPECIES = 8;
-constexpr int MAX_K = 64;      // widest radial feature vector of the fp64 path's shape variants
 constexpr size_t head_net_size(int n_inv) {   // doubles per regression network in the caller's layout
     return (size_t)n_inv * HEAD_H + HEAD_H + (size_t)(HEAD_L - 1) * (HEAD_H * HEAD_H + HEAD_H) + HEAD_H + 1;
 }

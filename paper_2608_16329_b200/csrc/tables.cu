@@ -18,64 +18,73 @@ struct EncShape { int hidden, layers, k, n_species; double r_cut; int envelope; 
 __device__ inline double d_sigmoid(double x) { return 1.0 / (1.0 + exp(-x)); }
 
 // Encoder value and derivative (forward mode) times the smooth cutoff.
-__device__ void eval_radial(const double *__restrict__ w, EncShape sh, double r, double *g, double *dg) {
-    const int H = sh.hidden;
-    double a[MAX_ENC_H], da[MAX_ENC_H], pre[MAX_ENC_H], dpre[MAX_ENC_H];
-    for (int o = 0; o < H; ++o) {
-        double p = w[o] * r + w[H + o], s = d_sigmoid(p);
-        a[o] = p * s;
-        da[o] = s * (1.0 + p * (1.0 - s)) * w[o];
+// samples: [net][point][k] values and derivatives at r = r0 + point * step
+// A block takes SAMPLE_PTS points of one net, thread = neuron: a weight is read once for all of them and the activations come
+// from shared memory.  (One thread per point with the activations in local memory kept 37 of the chip's SMs busy for 2.3 ms on
+// the 6-species model's 36 x 65 points; the sums run in the same order, so the tables are the same.)
+constexpr int SAMPLE_PTS = 8;
+__global__ void k_table_sample(const double *__restrict__ enc_w, size_t net_size, EncShape sh, int n_points,
+                               double r0, double step, double r_last, double *__restrict__ val, double *__restrict__ der) {
+    extern __shared__ double s_act[];   // a, da [H][SAMPLE_PTS]
+    const int H = sh.hidden, o = threadIdx.x, net = blockIdx.y, first = blockIdx.x * SAMPLE_PTS;
+    double *a = s_act, *da = s_act + H * SAMPLE_PTS;
+    auto radius = [&](int q) { const int p = first + q; return p >= n_points - 1 ? r_last : r0 + p * step; };
+    const double *w = enc_w + (size_t)net * net_size;
+    if (o < H) {
+#pragma unroll
+        for (int q = 0; q < SAMPLE_PTS; ++q) {
+            const double p = w[o] * radius(q) + w[H + o], s = d_sigmoid(p);
+            a[o * SAMPLE_PTS + q] = p * s;
+            da[o * SAMPLE_PTS + q] = s * (1.0 + p * (1.0 - s)) * w[o];
+        }
     }
     w += 2 * H;
+    __syncthreads();
     for (int layer = 1; layer < sh.layers; ++layer) {
-        const double *b = w + (size_t)H * H;
-        for (int o = 0; o < H; ++o) {
-            double p = b[o], dp = 0.0;
-            const double *row = w + (size_t)o * H;
-            for (int i = 0; i < H; ++i) { p += row[i] * a[i]; dp += row[i] * da[i]; }
-            pre[o] = p; dpre[o] = dp;
+        double p[SAMPLE_PTS], dp[SAMPLE_PTS];
+        if (o < H) {
+            const double b = w[(size_t)H * H + o], *row = w + (size_t)o * H;
+#pragma unroll
+            for (int q = 0; q < SAMPLE_PTS; ++q) { p[q] = b; dp[q] = 0.0; }
+            for (int i = 0; i < H; ++i) {
+                const double wi = row[i];
+#pragma unroll
+                for (int q = 0; q < SAMPLE_PTS; ++q) { p[q] += wi * a[i * SAMPLE_PTS + q]; dp[q] += wi * da[i * SAMPLE_PTS + q]; }
+            }
         }
-        for (int o = 0; o < H; ++o) {
-            double p = pre[o], s = d_sigmoid(p);
-            a[o] += p * s;
-            da[o] += s * (1.0 + p * (1.0 - s)) * dpre[o];
+        __syncthreads();
+        if (o < H) {
+#pragma unroll
+            for (int q = 0; q < SAMPLE_PTS; ++q) {
+                const double s = d_sigmoid(p[q]);
+                a[o * SAMPLE_PTS + q] += p[q] * s;
+                da[o * SAMPLE_PTS + q] += s * (1.0 + p[q] * (1.0 - s)) * dp[q];
+            }
         }
+        __syncthreads();
         w += (size_t)H * H + H;
     }
-    double fc = 0.0, dfc = 0.0;   // smooth cutoff: cosine or quintic polynomial
-    if (r < sh.r_cut) {
-        if (sh.envelope == 1) {
-            const double x = r / sh.r_cut, x2 = x * x;
-            fc = 1.0 + x2 * x * (-10.0 + x * (15.0 - 6.0 * x));
-            dfc = x2 * (-30.0 + x * (60.0 - 30.0 * x)) / sh.r_cut;
-        } else {
-            const double x = M_PI * r / sh.r_cut;
-            fc = 0.5 * (1.0 + cos(x));
-            dfc = -0.5 * (M_PI / sh.r_cut) * sin(x);
+    for (int item = threadIdx.x; item < sh.k * SAMPLE_PTS; item += blockDim.x) {
+        const int c = item % sh.k, q = item / sh.k;
+        if (first + q >= n_points) break;
+        const double r = radius(q), *row = w + (size_t)c * H;
+        double fc = 0.0, dfc = 0.0;   // smooth cutoff: cosine or quintic polynomial
+        if (r < sh.r_cut) {
+            if (sh.envelope == 1) {
+                const double x = r / sh.r_cut, x2 = x * x;
+                fc = 1.0 + x2 * x * (-10.0 + x * (15.0 - 6.0 * x));
+                dfc = x2 * (-30.0 + x * (60.0 - 30.0 * x)) / sh.r_cut;
+            } else {
+                const double x = M_PI * r / sh.r_cut;
+                fc = 0.5 * (1.0 + cos(x));
+                dfc = -0.5 * (M_PI / sh.r_cut) * sin(x);
+            }
         }
-    }
-    const double *b = w + (size_t)sh.k * H;
-    for (int c = 0; c < sh.k; ++c) {
-        double y = b[c], dy = 0.0;
-        const double *row = w + (size_t)c * H;
-        for (int i = 0; i < H; ++i) { y += row[i] * a[i]; dy += row[i] * da[i]; }
-        g[c] = fc * y;
-        dg[c] = dfc * y + fc * dy;
-    }
-}
-
-// samples: [net][point][k] values and derivatives at r = r0 + point * step
-__global__ void k_table_sample(const double *__restrict__ enc_w, size_t net_size, EncShape sh, int n_nets, int n_points,
-                               double r0, double step, double r_last, double *__restrict__ val, double *__restrict__ der) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n_nets * n_points) return;
-    int net = t / n_points, p = t % n_points;
-    double r = p == n_points - 1 ? r_last : r0 + p * step;
-    double g[MAX_K], dg[MAX_K];
-    eval_radial(enc_w + (size_t)net * net_size, sh, r, g, dg);
-    for (int c = 0; c < sh.k; ++c) {
-        val[((size_t)net * n_points + p) * sh.k + c] = g[c];
-        der[((size_t)net * n_points + p) * sh.k + c] = dg[c];
+        double y = w[(size_t)sh.k * H + c], dy = 0.0;
+        for (int i = 0; i < H; ++i) { y += row[i] * a[i * SAMPLE_PTS + q]; dy += row[i] * da[i * SAMPLE_PTS + q]; }
+        const size_t out = ((size_t)net * n_points + first + q) * sh.k + c;
+        val[out] = fc * y;
+        der[out] = dfc * y + fc * dy;
     }
 }
 
@@ -195,13 +204,14 @@ int build_tables(mlip_ctx *c, const double *enc_w_host, size_t n_enc) {
     MLIP_CUDA_TRY(c, cudaMemcpy(w, enc_w_host, sizeof(double) * n_enc, cudaMemcpyHostToDevice));
     MLIP_CUDA_TRY(c, cudaMemset(stats, 0, sizeof(unsigned long long) * 4));
 
-    int nt = n_nets * n_knot_pts;
-    k_table_sample<<<(nt + 63) / 64, 64>>>(w, net_size, sh, n_nets, n_knot_pts, r_min, h, cfg.r_cut, val, der);
+    const int threads = (H + 31) / 32 * 32;
+    const size_t smem = sizeof(double) * 2 * H * SAMPLE_PTS;   // at most 32 KB
+    k_table_sample<<<dim3((n_knot_pts + SAMPLE_PTS - 1) / SAMPLE_PTS, n_nets), threads, smem>>>(w, net_size, sh, n_knot_pts, r_min, h, cfg.r_cut, val, der);
     if (f64) k_table_solve<double><<<(n_nets * k + 63) / 64, 64>>>(val, der, n_nets, K, k, h, work, c->table_d);
     else k_table_solve<float><<<(n_nets * k + 63) / 64, 64>>>(val, der, n_nets, K, k, h, work, c->table);
-    nt = n_nets * n_chk;
+    const int nt = n_nets * n_chk;
     const double step = h / 4.0, r0 = r_min + 0.37 * step;
-    k_table_sample<<<(nt + 63) / 64, 64>>>(w, net_size, sh, n_nets, n_chk, r0, step, r0 + (n_chk - 1) * step, val, der);
+    k_table_sample<<<dim3((n_chk + SAMPLE_PTS - 1) / SAMPLE_PTS, n_nets), threads, smem>>>(w, net_size, sh, n_chk, r0, step, r0 + (n_chk - 1) * step, val, der);
     if (f64) k_table_check<double><<<(nt + 63) / 64, 64>>>(val, der, c->table_d, n_nets, n_chk, K, k, r_min, r0, step, h, stats);
     else k_table_check<float><<<(nt + 63) / 64, 64>>>(val, der, c->table, n_nets, n_chk, K, k, r_min, r0, step, h, stats);
     c->launches += 4;
