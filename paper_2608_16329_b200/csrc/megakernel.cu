@@ -6,7 +6,8 @@
 //   One persistent CTA of 16 warps per SM, organised as two independent groups of 8 warps.  The CTA
 //   walks through the central species in order; for each it stages that species' radial tables
 //   (one per neighbor species) and head constants in shared memory, then each group takes tiles of
-//   8 central atoms of that species from a global counter (warp = atom) and runs them on its own,
+//   16 (small systems: 8) central atoms of that species from a global counter (each warp encodes and
+//   derives two of them, one after the other) and runs them on its own,
 //   synchronising only inside the group (named barriers), so that one group's latency-bound head
 //   overlaps the other group's pair loops.
 //   Encoding    The warp scans the atom's list (lane = entry), queues the pairs inside r_cut in
@@ -14,10 +15,10 @@
 //               spline basis with lane = pair.  The moment P_i = H^T G (Eq. 4, 16 x n times
 //               n x 32) is accumulated on the tensor pipe: mma.sync m16n8k16 with both operands as fp16
 //               hi + lo pairs (three products, ~2^-22 relative, fp32 accumulate), the
-//               radial values g being evaluated straight into the B fragments.  P_i stays in
-//               the accumulator registers until the derivation.
+//               radial values g being evaluated straight into the B fragments.  P_i waits
+//               in tensor memory for the derivation.
 //   Invariants  Eq. 5 from the accumulator fragments by three xor-shuffles.
-//   Regression  Eq. 6 forward and reverse for the 8 atoms of the tile at once as W X^T on the tensor pipe
+//   Regression  Eq. 6 forward and reverse for the atoms of the tile at once as W X^T on the tensor pipe
 //               (mma.sync m16n8k16, fp16 operands in hi + lo pairs: 22 significant bits, fp32 accumulate); a
 //               warp keeps its 16 neurons x 8 atoms in accumulator fragments from layer to layer and passes
 //               the activations on through shared memory in B-fragment order, one barrier per layer.
@@ -50,10 +51,9 @@
 
 namespace mlip {
 
-constexpr int TILE = 8;       // atoms per tile = warps per group
+constexpr int GW = 8;         // warps per group; a tile is GW x APW atoms, APW = atoms per warp (1 or 2)
 constexpr int NG = 2;         // groups per CTA
-constexpr int NW = NG * TILE; // warps per CTA
-constexpr int PB_CAP = 160;   // queued pairs per warp: up to 31 left over + four list chunks of 32
+constexpr int NW = NG * GW;   // warps per CTA
 constexpr int J_BITS = 28;    // queue entries pack the neighbor index (low 28 bits) with its species
 constexpr int ST_STRIDE = 20; // encoding hand-over: h as 8 words hi + 8 words lo (fp16 pairs), 4 b (80 bytes: conflict-free for ldmatrix and STS.128)
 constexpr int BS_STRIDE = 12; // derivation hand-over: 4 b, 4 b', row addresses
@@ -65,19 +65,18 @@ constexpr int X_STRIDE = 132; // dE/dG per atom
 // order that gives the lanes of a load different residues (RowOffsets).  Without that the rows of a load are random and
 // collide: 6 instead of 4 wavefronts per pair in the derivation, and a shuffle per value in the encoding.
 static_assert(K_RADIAL == 32, "a table row is eight 16-byte chunks");
-constexpr int Q_WORDS = 4 * PB_CAP;                             // pair queue of a warp: kept from encoding to derivation
 constexpr int SCR_WORDS = 32 * ST_STRIDE + 32 * 4;              // scratch of a warp: hand-over rows, table row addresses
 static_assert(32 * BS_STRIDE <= SCR_WORDS && N_INV <= 32 * ST_STRIDE, "the derivation's hand-over and the invariants must fit the encoding's");
 // Regression buffers of a group.  Activations are kept as B fragments: per 16-input k-step, atom row and quad lane one
 // 16-byte vector {b0 hi, b0 lo, b1 hi, b1 lo} of fp16 pairs (see act_store).
 constexpr int ACT_KSTEP = 32 * 4;                               // words per k-step
-constexpr int XS_WORDS = (N_INV / 16) * ACT_KSTEP;              // split invariants (written before the group's barrier: space of their own)
-constexpr int ZS_WORDS = (HEAD_H / 16) * ACT_KSTEP;             // one layer's activations
-constexpr int SX_WORDS = TILE * X_STRIDE;                       // dE/dG
-constexpr int SC_WORDS = 8 * TILE;                              // per-atom scales (see below)
-constexpr int EP_WORDS = 4 * TILE;                              // E_i partial sums of the four m-tiles
-constexpr int GROUP_WORDS = XS_WORDS + SX_WORDS + SC_WORDS + EP_WORDS;
-static_assert(2 * ZS_WORDS <= TILE * SCR_WORDS, "layer activations alias the scratch of the group's warps");
+constexpr int XS_WORDS = (N_INV / 16) * ACT_KSTEP;              // split invariants of eight atoms (written before the group's barrier: space of their own)
+constexpr int ZS_WORDS = (HEAD_H / 16) * ACT_KSTEP;             // one layer's activations of eight atoms
+constexpr int PF_IDX = 160;                                     // neighbor indices prefetched per coming atom
+constexpr int PF_CS = 96;                                       // compact lists: the codes take 81 words at most, the 27 cell bases sit here
+static_assert(PF_IDX / 2 + 1 <= PF_CS && PF_CS + 27 <= PF_IDX, "prefetch buffer layout for compact lists");
+constexpr int PF_WORDS = PF_IDX + 4;                            // + {atom, list start (2 words), list length}
+static_assert(2 * 2 * ZS_WORDS <= GW * SCR_WORDS, "layer activations alias the scratch of the group's warps");
 // Head constants of the current species: biases, w_out, b_out, then the powers of two and bounds of the fp16 scaling:
 //   pre-activation of layer L (input scaled by a per-atom 2^s): acc * (2^-s * HC_WS[L]) + bias
 //   |input of layer L| <= HC_BND[2L-2] * max|G| + HC_BND[2L-1]  (L = 1..3; row-sum norms of the weights)
@@ -86,12 +85,27 @@ static_assert(2 * ZS_WORDS <= TILE * SCR_WORDS, "layer activations alias the scr
 constexpr int HC_WOUT = HEAD_L * HEAD_H, HC_BOUT = HC_WOUT + HEAD_H, HC_WS = HC_BOUT + 1, HC_BND = HC_WS + HEAD_L;
 constexpr int HC_SR = HC_BND + 2 * (HEAD_L - 1), HC_UR = HC_SR + HEAD_L, HC_CS = HC_UR + HEAD_L, HC_USED = HC_CS + N_INV;
 constexpr int HC_WORDS = (HC_USED + 15) / 16 * 16;
+// Systems below this size take tiles of 8 atoms, one per warp: with few tiles per SM the chain through one tile is what counts
+// (kernel us with 8- / 16-atom tiles, 6 species: 864 atoms 47 / 53, 6,912 96 / 97, 16,384 174 / 166, 55,296 499 / 474, 131,072
+// 1119 / 1046; one species: 4,394 63 / 66, 16,000 140 / 135, 65,536 476 / 441).
+constexpr int64_t ONE_PER_WARP_BELOW_ATOMS = 12000;
 constexpr int64_t STAGGER_BELOW_ATOMS = 200000;                 // systems below this size start their CTAs on different species
-constexpr int PF_IDX = 160;                                     // neighbor indices prefetched per warp for its next atom
-constexpr int PF_CS = 96;                                       // compact lists: the codes take 81 words at most, the 27 cell bases sit here
-static_assert(PF_IDX / 2 + 1 <= PF_CS && PF_CS + 27 <= PF_IDX, "prefetch buffer layout for compact lists");
-constexpr int PF_WORDS = PF_IDX + 4;                            // + {atom, list start (2 words), list length}
-constexpr int FIXED_WORDS = NG * GROUP_WORDS + NW * (Q_WORDS + SCR_WORDS + PF_WORDS) + HC_WORDS + 16;
+// Shared memory per tile shape.  Two atoms per warp halve the regression's barriers, weight fetches and idle time per atom
+// (each warp owns 16 neurons x 8 atoms of a 16-atom tile instead of half of the warps owning an 8-atom tile); one atom per warp
+// spreads a small system over more SMs.
+template <int APW>
+struct Layout {
+    static constexpr int NA = GW * APW;                         // atoms per tile
+    static constexpr int POOL = APW == 1 ? 160 : 256;           // pair queue of a warp, shared by its atoms, kept from encoding to derivation
+    static constexpr int Q_WORDS = 4 * POOL;
+    static constexpr int SX = NA * X_STRIDE;                    // dE/dG
+    static constexpr int SC = 2 * HEAD_L * NA;                  // per-atom scales (see split_invariants)
+    static constexpr int EP = 4 * NA;                           // E_i partial sums of the four m-tiles
+    static constexpr int GROUP = APW * XS_WORDS + SX + SC + EP;
+    static constexpr int INFO = 4 * APW;                        // per warp: {atom, queued pairs, queue start, -} of its atoms, from encoding to derivation
+    static constexpr int WARP = Q_WORDS + SCR_WORDS + APW * PF_WORDS + INFO;
+    static constexpr int FIXED = NG * GROUP + NW * WARP + HC_WORDS + 16;
+};
 constexpr int SMEM_LIMIT_WORDS = 227 * 1024 / 4 - 256;
 
 // Pre-packed head weights per species (32-bit words): the tensor-memory image, [quarter][column / 4][lane][4], followed by
@@ -102,8 +116,10 @@ constexpr int SMEM_LIMIT_WORDS = 227 * 1024 / 4 - 256;
 //           [ 64, 160)  forward, hidden layers: 3 x 4 k-steps
 //           [160, 256)  reverse, hidden layers: 3 x 4 k-steps
 //           [256, 320)  reverse, first layer: 2 m-tiles x 4 k-steps
-//           [320, 448)  V and T on their way from fragments to lane = pair: 32 columns per warp of the quarter
-constexpr int TM_FWD0 = 0, TM_FWD = 64, TM_BWD = 160, TM_BWD0 = 256, TM_VT = 320;
+//           [320, 448)  V and T on their way from fragments to lane = pair: 32 columns per warp of the quarter; before that
+//                       the moment P of the warp's second atom waits there for its derivation
+//           [448, 512)  P of the warp's first atom: 16 columns per warp of the quarter
+constexpr int TM_FWD0 = 0, TM_FWD = 64, TM_BWD = 160, TM_BWD0 = 256, TM_VT = 320, TM_P = 448;
 constexpr int HP_TMEM = 4 * TM_VT * 32;
 constexpr int HP_TOTAL = HP_TMEM + (HC_USED + 3) / 4 * 4;
 
@@ -270,23 +286,25 @@ __device__ __forceinline__ float4 rotate4(const float (&b)[4], int turn) {
     return make_float4(r2 ? c2 : c0, r2 ? c3 : c1, r2 ? c0 : c2, r2 ? c1 : c3);
 }
 
-// Fill the warp's pair queue from list position `cur` on (lane = entry), up to five 32-entry chunks
+// Fill the warp's pair queue (room for `cap` pairs at pq) from list position `cur` on (lane = entry), up to five 32-entry chunks
 // at a time with all index loads, then all position gathers, in flight together (a typical list
 // of ~134 entries is one round trip).  Pairs inside r_cut are queued as {x, y, z, j | species << 28}.
 // Stops when the list ends or the next group might not fit; returns the number of queued pairs
 // and advances `cur`.  The first n_pref indices of the list may come from shared memory (sidx).
-constexpr int SCAN_CHUNKS = 5;
-static_assert(SCAN_CHUNKS * 32 <= PB_CAP, "a full group must fit an empty queue");
+constexpr int WIDE_CHUNKS = 5, NARROW_CHUNKS = 3;
+static_assert(WIDE_CHUNKS * 32 <= Layout<1>::POOL, "a full group must fit an empty queue");
+// (a tile's second atom finds at least this much room: the first keeps at most POOL - SECOND_ROOM pairs)
+constexpr int SECOND_ROOM = NARROW_CHUNKS * 32;
 // Compact lists: lane q < 27 holds the first atom of the q-th cell around atom i's build-time cell; an entry's index is
 // that base (one shuffle) plus the position coded in its low bits.
 __device__ __forceinline__ int cell_base_of_lane(const KernelArgs &k, int i, int lane) {
     return lane < 27 ? __ldg(k.cell_start + neighbor_cell(k.grid, __ldg(k.cell_id + i), lane)) : 0;
 }
 template <int SCAN_CHUNKS, bool L16>
-__device__ __forceinline__ int collect_pairs_n(const KernelArgs &k, const double4 &pi, int64_t beg, int64_t &cur, int64_t end, float4 *pq, int lane,
+__device__ __forceinline__ int collect_pairs_n(const KernelArgs &k, const double4 &pi, int64_t beg, int64_t &cur, int64_t end, float4 *pq, int cap, int lane,
                                                const int *sidx, int n_pref, int cs) {
     int nq = 0;
-    while (cur < end && nq + (int)min((int64_t)(SCAN_CHUNKS * 32), end - cur) <= PB_CAP) {
+    while (cur < end && nq + (int)min((int64_t)(SCAN_CHUNKS * 32), end - cur) <= cap) {
         int jj[SCAN_CHUNKS];
 #pragma unroll
         for (int c = 0; c < SCAN_CHUNKS; ++c) {
@@ -326,10 +344,10 @@ __device__ __forceinline__ int collect_pairs_n(const KernelArgs &k, const double
 // Short lists (the usual case while the far entries are skipped) take the three-chunk form: fewer loads in flight,
 // fewer registers.
 template <bool L16>
-__device__ __forceinline__ int collect_pairs(const KernelArgs &k, const double4 &pi, int64_t beg, int64_t &cur, int64_t end, float4 *pq, int lane,
+__device__ __forceinline__ int collect_pairs(const KernelArgs &k, const double4 &pi, int64_t beg, int64_t &cur, int64_t end, float4 *pq, int cap, int lane,
                                              const int *sidx, int n_pref, int cs) {
-    if (end - beg <= 96) return collect_pairs_n<3, L16>(k, pi, beg, cur, end, pq, lane, sidx, n_pref, cs);
-    return collect_pairs_n<5, L16>(k, pi, beg, cur, end, pq, lane, sidx, n_pref, cs);
+    if (end - beg <= NARROW_CHUNKS * 32 || cap < WIDE_CHUNKS * 32) return collect_pairs_n<NARROW_CHUNKS, L16>(k, pi, beg, cur, end, pq, cap, lane, sidx, n_pref, cs);
+    return collect_pairs_n<WIDE_CHUNKS, L16>(k, pi, beg, cur, end, pq, cap, lane, sidx, n_pref, cs);
 }
 
 // ---------------- Encoding of one atom: returns the moment as accumulator fragments ----------------
@@ -337,7 +355,7 @@ __device__ __forceinline__ int collect_pairs(const KernelArgs &k, const double4 
 // (the derivation then reuses them), or -1.
 template <bool TAB_SMEM, bool L16>
 __device__ __forceinline__ int encode_atom(const KernelArgs &k, const TableView &tv, const double4 &pi, int64_t beg, int64_t end,
-                                           float4 *pq, float *stage, int lane, float (&Pf)[4][4], int &queued, const int *sidx, int n_pref,
+                                           float4 *pq, int cap, float *stage, int lane, float (&Pf)[4][4], int &queued, const int *sidx, int n_pref,
                                            int cs, PhaseClock &pc) {
     const int g = lane >> 2, t = lane & 3;
     float *offs = stage + 32 * ST_STRIDE;
@@ -437,7 +455,7 @@ __device__ __forceinline__ int encode_atom(const KernelArgs &k, const TableView 
     int total = 0, rounds = 0, n = 0;
     int64_t cur = beg;
     do {
-        n = collect_pairs<L16>(k, pi, beg, cur, end, pq, lane, sidx, n_pref, cs);
+        n = collect_pairs<L16>(k, pi, beg, cur, end, pq, cap, lane, sidx, n_pref, cs);
         pc.mark(0);
         for (int q0 = 0; q0 < n; q0 += 32) batch(q0, min(32, n - q0));
         total += n;
@@ -474,6 +492,18 @@ __device__ __forceinline__ void tmem_st_vt(uint32_t addr, const float (&V)[2][4]
                  "f"(V[0][0]), "f"(V[0][1]), "f"(V[0][2]), "f"(V[0][3]), "f"(V[1][0]), "f"(V[1][1]), "f"(V[1][2]), "f"(V[1][3]),
                  "f"(T[0][0]), "f"(T[0][1]), "f"(T[0][2]), "f"(T[0][3]), "f"(T[1][0]), "f"(T[1][1]), "f"(T[1][2]), "f"(T[1][3]) : "memory");
 }
+// 16 registers of every lane to / from 16 columns (the moment P between encoding and derivation)
+__device__ __forceinline__ void tmem_st16(uint32_t addr, const float (&P)[4][4]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(addr),
+                 "f"(P[0][0]), "f"(P[0][1]), "f"(P[0][2]), "f"(P[0][3]), "f"(P[1][0]), "f"(P[1][1]), "f"(P[1][2]), "f"(P[1][3]),
+                 "f"(P[2][0]), "f"(P[2][1]), "f"(P[2][2]), "f"(P[2][3]), "f"(P[3][0]), "f"(P[3][1]), "f"(P[3][2]), "f"(P[3][3]) : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, float (&P)[4][4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=f"(P[0][0]), "=f"(P[0][1]), "=f"(P[0][2]), "=f"(P[0][3]), "=f"(P[1][0]), "=f"(P[1][1]), "=f"(P[1][2]), "=f"(P[1][3]),
+                   "=f"(P[2][0]), "=f"(P[2][1]), "=f"(P[2][2]), "=f"(P[2][3]), "=f"(P[3][0]), "=f"(P[3][1]), "=f"(P[3][2]), "=f"(P[3][3])
+                 : "r"(addr) : "memory");
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -500,7 +530,7 @@ __device__ __forceinline__ void tmem_fill(uint32_t quarter_base, const uint32_t 
 // ---------------- Derivation of one atom (Eq. 8-10) ----------------
 template <bool TAB_SMEM, bool DET, bool L16>
 __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView &tv, int i,
-                                            float4 *pq, float *scr, int queued, int lane, const uint32_t (&Wh)[2][2][2],
+                                            float4 *pq, int cap, float *scr, int queued, int lane, const uint32_t (&Wh)[2][2][2],
                                             const uint32_t (&Wl)[2][2][2], float w_scale_inv, float (&vir)[9], uint32_t tm_vt, PhaseClock &pc) {
     // Wh, Wl [k-step][n-tile][b0, b1]: B fragments of W_i^T times 1 / w_scale_inv; k-step q holds channels 8t + 4q .. + 3 of lane (g, t)
     const int g = lane >> 2, t = lane & 3;
@@ -639,7 +669,7 @@ __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView
         int64_t cur = beg;
         const int cs = L16 ? cell_base_of_lane(k, i, lane) : 0;
         do {
-            const int n = collect_pairs<L16>(k, pi, beg, cur, end, pq, lane, nullptr, 0, cs);
+            const int n = collect_pairs<L16>(k, pi, beg, cur, end, pq, cap, lane, nullptr, 0, cs);
             pc.mark(3);
             for (int q0 = 0; q0 < n; q0 += 32) batch(q0, min(32, n - q0));
         } while (cur < end);
@@ -658,7 +688,7 @@ __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView
 
 // Barrier among the 256 threads of one group (hardware barrier 1 + group).
 __device__ __forceinline__ void group_sync(int group) {
-    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(TILE * 32) : "memory");
+    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(GW * 32) : "memory");
 }
 
 // Head contraction on the tensor pipe: C^T[16 rows of W x 8 atoms] over four 16-wide k-steps.  A = wr (32 columns of tensor
@@ -688,65 +718,69 @@ __device__ __forceinline__ void act_store(float *act, int kstep, int atom, int j
     *reinterpret_cast<uint2 *>(act + kstep * ACT_KSTEP + (act_row(atom) * 4 + (j & 3)) * 4 + 2 * (j >> 2)) = make_uint2(hi, lo);
 }
 
-// Prefetch of the warp's atom in the group's NEXT tile, spread over three points of the head so
+// Prefetch of the warp's atoms in the group's NEXT tile, spread over three points of the head so
 // that each dependent global load has a barrier's worth of time to arrive: centre index -> list
-// bounds -> the first PF_IDX neighbor indices (cp.async straight into shared memory).  (Pulling the
-// neighbors' positions into L2 as a fourth step cost more issue slots than it saved latency.)
-struct NextAtom {
+// bounds (lane u for the warp's u-th atom) -> the first PF_IDX neighbor indices (cp.async straight into shared memory).
+// (Pulling the neighbors' positions into L2 as a fourth step cost more issue slots than it saved latency.)
+template <int APW>
+struct NextAtoms {
     const KernelArgs *k;
-    int *meta;        // shared: {atom, list start lo, list start hi, list length}
-    int *sidx;        // shared: neighbor indices
-    int slot;         // position in center_order, or -1
+    int *pf;          // shared: per atom PF_IDX neighbor indices, then {atom, list start lo, list start hi, list length}
+    int slot;         // lane u < APW: position in center_order, or -1
     int i;
     bool use_far;     // the lists' far entries have to be scanned as well
-    int64_t beg, end;
+    int64_t beg;
+    int len;
     int cid;          // compact lists: the atom's build-time cell
     __device__ __forceinline__ void stage_a() { if (slot >= 0) i = __ldg(k->center_order + slot); }
     template <bool L16>
     __device__ __forceinline__ void stage_b() {
         if (slot >= 0) {
-            beg = __ldg(k->nbr_off + i); end = use_far ? __ldg(k->nbr_off + i + 1) : beg + __ldg(k->nbr_near + i);
+            beg = __ldg(k->nbr_off + i);
+            len = use_far ? (int)(__ldg(k->nbr_off + i + 1) - beg) : __ldg(k->nbr_near + i);
             if (L16) cid = __ldg(k->cell_id + i);
         }
     }
     template <bool L16>
     __device__ __forceinline__ void stage_c(int lane) {
-        if (slot < 0) return;
-        const int n = (int)min((int64_t)PF_IDX, end - beg);
-        if (L16) {   // codes travel as whole 32-bit words from the even entry at or before `beg`; the 27 cell bases follow them
-            const int odd = (int)(beg & 1), words = (odd + n + 1) >> 1;
-            const int *src = reinterpret_cast<const int *>(k->nbr16 + (beg - odd));
 #pragma unroll
-            for (int c = 0; c < (PF_IDX / 2 + 1 + 31) / 32; ++c) {
-                const int e = 32 * c + lane;
-                if (e < words) {
-                    const unsigned dst = (unsigned)__cvta_generic_to_shared(sidx + e);
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src + e) : "memory");
+        for (int u = 0; u < APW; ++u) {
+            if (__shfl_sync(0xffffffffu, slot, u) < 0) break;   // (a ragged tile's atoms come first)
+            int *sidx = pf + u * PF_WORDS;
+            const int64_t b = __shfl_sync(0xffffffffu, beg, u);
+            const int n = min(PF_IDX, __shfl_sync(0xffffffffu, len, u));
+            if (L16) {   // codes travel as whole 32-bit words from the even entry at or before `b`; the 27 cell bases follow them
+                const int cell = __shfl_sync(0xffffffffu, cid, u);
+                const int odd = (int)(b & 1), words = (odd + n + 1) >> 1;
+                const int *src = reinterpret_cast<const int *>(k->nbr16 + (b - odd));
+#pragma unroll
+                for (int c = 0; c < (PF_IDX / 2 + 1 + 31) / 32; ++c) {
+                    const int e = 32 * c + lane;
+                    if (e < words) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(sidx + e)), "l"(src + e) : "memory");
                 }
-            }
-            if (lane < 27) {
-                const unsigned dst = (unsigned)__cvta_generic_to_shared(sidx + PF_CS + lane);
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(k->cell_start + neighbor_cell(k->grid, cid, lane)) : "memory");
-            }
-        } else {
+                if (lane < 27)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(sidx + PF_CS + lane)), "l"(k->cell_start + neighbor_cell(k->grid, cell, lane)) : "memory");
+            } else {
 #pragma unroll
-            for (int c = 0; c < PF_IDX / 32; ++c) {
-                const int e = 32 * c + lane;
-                if (e < n) {
-                    const unsigned dst = (unsigned)__cvta_generic_to_shared(sidx + e);
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(k->nbr + beg + e) : "memory");
+                for (int c = 0; c < PF_IDX / 32; ++c) {
+                    const int e = 32 * c + lane;
+                    if (e < n) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(sidx + e)), "l"(k->nbr + b + e) : "memory");
                 }
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
-        if (lane == 0) { meta[0] = i; meta[1] = (int)(beg & 0xffffffff); meta[2] = (int)(beg >> 32); meta[3] = (int)(end - beg); }
+        if (lane < APW && slot >= 0) {
+            int *meta = pf + lane * PF_WORDS + PF_IDX;
+            meta[0] = i; meta[1] = (int)(beg & 0xffffffff); meta[2] = (int)(beg >> 32); meta[3] = len;
+        }
     }
 };
 
 // ---------------- Regression (Eq. 6) forward and reverse for the group's tile ----------------
 // One atom's invariants (warp = atom) -> scaled fp16 pairs in fragment order, and the atom's scales for all layers:
 // sc[2 L][atom] = 2^s of layer L's input, sc[2 L + 1][atom] = the factor that takes layer L's product back.
-__device__ __forceinline__ void split_invariants(const float *xrow, float *xs, float *sc, const float *hc, int atom, int lane) {
+__device__ __forceinline__ void split_invariants(const float *xrow, float *xs, float *sc, const float *hc, int atom, int n_atoms, int lane) {
+    xs += (atom >> 3) * XS_WORDS;
     // lane handles the pairs (c, c + 8) number lane and lane + 32 of the 64: k-step p / 8, j = p % 8
     const int j = lane & 7, s0 = lane >> 3, s1 = s0 + 4;
     const float *cs = hc + HC_CS;
@@ -756,25 +790,28 @@ __device__ __forceinline__ void split_invariants(const float *xrow, float *xs, f
     const float sx = scale_for(most);
     uint32_t hi, lo;
     split_h2(a0 * sx, a1 * sx, hi, lo);
-    act_store(xs, s0, atom, j, hi, lo);
+    act_store(xs, s0, atom & 7, j, hi, lo);
     split_h2(b0 * sx, b1 * sx, hi, lo);
-    act_store(xs, s1, atom, j, hi, lo);
+    act_store(xs, s1, atom & 7, j, hi, lo);
     if (lane < HEAD_L) {
         const float s = lane == 0 ? sx : scale_for(hc[HC_BND + 2 * (lane - 1)] * most + hc[HC_BND + 2 * (lane - 1) + 1]);
-        sc[2 * lane * TILE + atom] = s;
-        sc[(2 * lane + 1) * TILE + atom] = inverse_pow2(s) * hc[HC_WS + lane];
+        sc[2 * lane * n_atoms + atom] = s;
+        sc[(2 * lane + 1) * n_atoms + atom] = inverse_pow2(s) * hc[HC_WS + lane];
     }
 }
 
-// In: xs = split invariants.  Out: sX = dE/dG [atom][128]; per-atom energies written.  wg = warp within the group; warps
-// 0..3 own m-tile wg (16 neurons) of the eight atoms through all layers, all eight take part in the first layer's reverse.
-template <bool DET, bool L16>
+// In: xs = split invariants.  Out: sX = dE/dG [atom][128]; per-atom energies written.  wg = warp within the group: it owns
+// m-tile wg % 4 (16 neurons) of the atoms 8 (wg / 4) .. + 7 through all layers (one atom per warp: warps 4..7 own nothing).
+template <int APW, bool DET, bool L16>
 __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, float *sX, const float *sc, float *ep, float *zs, const float *hc,
-                                          uint32_t tm, int count, int first, int group, int wg, int lane, double &e_sum, NextAtom &nx, PhaseClock &pc) {
-    const int g = lane >> 2, t = lane & 3, mt = wg & 3;
+                                          uint32_t tm, int count, int first, int group, int wg, int lane, double &e_sum, NextAtoms<APW> &nx, PhaseClock &pc) {
+    constexpr int NA = GW * APW;
+    const int g = lane >> 2, t = lane & 3, mt = wg & 3, nt = wg >> 2;
     const int frag = act_row(g) * 4 + t;        // this lane's vector of a k-step
-    const bool owner = wg < 4;
-    const int n0 = 16 * mt + g, n1 = n0 + 8;    // the lane's neurons; its atoms are 2t, 2t + 1: values {n0 2t, n0 2t+1, n1 2t, n1 2t+1}
+    const bool owner = APW == 2 || wg < 4;
+    const int a0 = (APW == 2 ? 8 * nt : 0) + 2 * t;   // the lane's atoms: a0, a0 + 1
+    const int n0 = 16 * mt + g, n1 = n0 + 8;    // and neurons: its values are {n0 a0, n0 a0+1, n1 a0, n1 a0+1}
+    if (APW == 2) { xs += nt * XS_WORDS; zs += nt * 2 * ZS_WORDS; }
     float y[4] = {0.f, 0.f, 0.f, 0.f};          // running activations (the skip path)
     float dz[4];                                // dE/dy in the reverse pass
     float sd[HEAD_L][4];                        // SiLU' of the pre-activations, layer by layer
@@ -797,13 +834,13 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
                 for (int e = 0; e < 4; ++e) c[e] += c2[e];
             }
             pc.mark(12);
-            const float2 u = *reinterpret_cast<const float2 *>(sc + (2 * L + 1) * TILE + 2 * t);
+            const float2 u = *reinterpret_cast<const float2 *>(sc + (2 * L + 1) * NA + a0);
             const float bias0 = hc[L * HEAD_H + n0], bias1 = hc[L * HEAD_H + n1];
             y[0] += silu_f(c[0] * u.x + bias0, sd[L][0]); y[1] += silu_f(c[1] * u.y + bias0, sd[L][1]);
             y[2] += silu_f(c[2] * u.x + bias1, sd[L][2]); y[3] += silu_f(c[3] * u.y + bias1, sd[L][3]);
             float m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f;   // what goes to the next contraction
             if (L < HEAD_L - 1) {
-                const float2 s = *reinterpret_cast<const float2 *>(sc + 2 * (L + 1) * TILE + 2 * t);
+                const float2 s = *reinterpret_cast<const float2 *>(sc + 2 * (L + 1) * NA + a0);
                 m0 = y[0] * s.x; m1 = y[1] * s.y; m2 = y[2] * s.x; m3 = y[3] * s.y;
             } else {   // output layer and the start of the reverse pass: dE/dy = w_out
                 const float wo0 = hc[HC_WOUT + n0], wo1 = hc[HC_WOUT + n1], s = hc[HC_SR + L];
@@ -813,7 +850,7 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
                     e0 += __shfl_xor_sync(0xffffffffu, e0, o);
                     e1 += __shfl_xor_sync(0xffffffffu, e1, o);
                 }
-                if (g == 0) *reinterpret_cast<float2 *>(ep + mt * TILE + 2 * t) = make_float2(e0, e1);
+                if (g == 0) *reinterpret_cast<float2 *>(ep + mt * NA + a0) = make_float2(e0, e1);
                 dz[0] = dz[1] = wo0; dz[2] = dz[3] = wo1;
                 m0 = (wo0 * s) * sd[L][0]; m1 = (wo0 * s) * sd[L][1]; m2 = (wo1 * s) * sd[L][2]; m3 = (wo1 * s) * sd[L][3];
             }
@@ -831,7 +868,7 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
         pc.mark(14);
     }
     if (wg == 7 && lane < count) {
-        const float e_i = ((ep[lane] + ep[TILE + lane]) + (ep[2 * TILE + lane] + ep[3 * TILE + lane])) + hc[HC_BOUT];
+        const float e_i = ((ep[lane] + ep[NA + lane]) + (ep[2 * NA + lane] + ep[3 * NA + lane])) + hc[HC_BOUT];
         k.e_atom[__ldg(k.center_order + first + lane)] = e_i;
         e_sum += DET ? rint((double)e_i * ENERGY_FX) : (double)e_i;   // DET: exact integer sums
     }
@@ -858,33 +895,39 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
         }
         group_sync(group);
     }
-    {   // first layer: dE/dG [128 x 8], warp = m-tile (16 inputs)
+    // first layer: dE/dG [128 x atoms], 16 inputs per m-tile: the warp's m-tiles mt, mt + 4 (one atom per warp: m-tile wg)
+#pragma unroll
+    for (int h = 0; h < APW; ++h) {
+        const int m = APW == 2 ? mt + 4 * h : wg;
         float c[4];
-        tmem_ld32(tm + TM_BWD0 + 32 * (wg >> 2), w);
+        tmem_ld32(tm + TM_BWD0 + 32 * (m >> 2), w);
         tmem_wait_ld();
         head_gemm(c, w, reinterpret_cast<const uint4 *>(zs) + frag);   // layer 0's dE/dpre: buffer 0
-        const float u = hc[HC_UR], ua = u * hc[HC_CS + 16 * wg + g], ub = u * hc[HC_CS + 16 * wg + g + 8];
-        float *p = sX + 2 * t * X_STRIDE + 16 * wg + g;
+        const float u = hc[HC_UR], ua = u * hc[HC_CS + 16 * m + g], ub = u * hc[HC_CS + 16 * m + g + 8];
+        float *p = sX + a0 * X_STRIDE + 16 * m + g;
         p[0] = c[0] * ua; p[X_STRIDE] = c[1] * ua; p[8] = c[2] * ub; p[X_STRIDE + 8] = c[3] * ub;
     }
     group_sync(group);
 }
 
-template <bool TAB_SMEM, bool DET, bool L16, bool STAGGER>
+template <int APW, bool TAB_SMEM, bool DET, bool L16, bool STAGGER>
 __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words) {
     extern __shared__ __align__(128) float smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int group = warp / TILE, wg = warp % TILE;
+    using LY = Layout<APW>;
+    constexpr int NA = LY::NA;
+    const int group = warp / GW, wg = warp % GW;
     const int g = lane >> 2, t = lane & 3;
     float *s_tab = smem;                                   // [C][rows][K_RADIAL] when TAB_SMEM
-    float *xs = smem + (TAB_SMEM ? tab_words : 0) + group * GROUP_WORDS;
-    float *sX = xs + XS_WORDS, *sc = sX + SX_WORDS, *ep = sc + SC_WORDS;
-    float *scr_all = smem + (TAB_SMEM ? tab_words : 0) + NG * GROUP_WORDS;
-    float *zs = scr_all + group * TILE * SCR_WORDS;        // layer activations = the scratch of the group's warps
+    float *xs = smem + (TAB_SMEM ? tab_words : 0) + group * LY::GROUP;
+    float *sX = xs + APW * XS_WORDS, *sc = sX + LY::SX, *ep = sc + LY::SC;
+    float *scr_all = smem + (TAB_SMEM ? tab_words : 0) + NG * LY::GROUP;
+    float *zs = scr_all + group * GW * SCR_WORDS;          // layer activations = the scratch of the group's warps
     float *scr = scr_all + warp * SCR_WORDS;
-    float4 *pq = reinterpret_cast<float4 *>(scr_all + NW * SCR_WORDS + warp * Q_WORDS);
-    int *pf = reinterpret_cast<int *>(scr_all + NW * (SCR_WORDS + Q_WORDS)) + warp * PF_WORDS;
-    float *hc = scr_all + NW * (SCR_WORDS + Q_WORDS + PF_WORDS);
+    float4 *pq = reinterpret_cast<float4 *>(scr_all + NW * SCR_WORDS + warp * LY::Q_WORDS);
+    int *pf = reinterpret_cast<int *>(scr_all + NW * (SCR_WORDS + LY::Q_WORDS)) + warp * APW * PF_WORDS;
+    int *info = reinterpret_cast<int *>(scr_all + NW * (SCR_WORDS + LY::Q_WORDS + APW * PF_WORDS)) + warp * LY::INFO;
+    float *hc = scr_all + NW * LY::WARP;
     int *ctl = reinterpret_cast<int *>(hc + HC_WORDS);
     const int rows = k.tab.knots + 3;
     // lists that an in-step rebuild could not complete (capacity, broken configuration) are not evaluated: the outputs
@@ -903,7 +946,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
     tmem_fence_after_sync();
     const uint32_t tm_base = *reinterpret_cast<volatile uint32_t *>(ctl + 4);
     const uint32_t tm_quarter = tm_base + ((uint32_t)(32 * (warp & 3)) << 16);
-    const uint32_t tm_vt = tm_quarter + TM_VT + 32 * (warp >> 2);
+    const uint32_t tm_vt = tm_quarter + TM_VT + 32 * (warp >> 2), tm_p = tm_quarter + TM_P + 16 * (warp >> 2);
 
     double e_sum = 0.0;
     float vir[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -921,7 +964,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
     for (int ss = 0; ss < k.n_species; ++ss) {
         const int species = STAGGER ? (int)((ss + blockIdx.x) % (unsigned)k.n_species) : ss;
         const int s_beg = __ldg(k.species_start + species), s_end = __ldg(k.species_start + species + 1);
-        const int n_tiles = (s_end - s_beg + TILE - 1) / TILE;
+        const int n_tiles = (s_end - s_beg + NA - 1) / NA;
         if (n_tiles == 0) continue;
         if (threadIdx.x == 0) ctl[6 + (ss & 1)] = *reinterpret_cast<volatile int *>(k.tile_counter + species);
         __syncthreads();   // both groups are done with the previous species' tables
@@ -953,65 +996,74 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
         while (tile < n_tiles) {
             if (wg == 0 && lane == 0) look_ahead = atomicAdd(k.tile_counter + species, 1);   // consumed after the encoding
             pc.mark(11);
-            const int first = s_beg + tile * TILE;
-            const int count = min(TILE, s_end - first);
+            const int first = s_beg + tile * NA;
+            const int count = min(NA, s_end - first);
 
-            // ---------------- Encoding + invariants: warp = atom ----------------
-            const bool have = wg < count;
-            int i = 0, n_pref = 0, cs = 0;
-            double4 pi = make_double4(0.0, 0.0, 0.0, 0.0);
-            int64_t beg = 0, end = 0;
-            float Pf[4][4];
-            int queued = -1;
-            const float *drow = sX + wg * X_STRIDE;   // dE/dG of this warp's atom
-            float *xrow = scr;                        // its invariants (the encoding is done with the scratch)
-            if (have) {
-                if (prefetched) {
-                    asm volatile("cp.async.wait_group 0;" ::: "memory");
-                    __syncwarp();
-                    i = pf[PF_IDX];
-                    beg = ((int64_t)pf[PF_IDX + 2] << 32) | (unsigned)pf[PF_IDX + 1];
-                    end = beg + pf[PF_IDX + 3];
-                    n_pref = min(PF_IDX, pf[PF_IDX + 3]);
-                    if (L16) cs = lane < 27 ? pf[PF_CS + lane] : 0;
-                } else {
-                    i = (int)MLIP_CHECK_INDEX(__ldg(k.center_order + first + wg), k.n, k.status);
-                    beg = k.nbr_off[i]; end = use_far ? k.nbr_off[i + 1] : beg + k.nbr_near[i];
-                    if (L16) cs = cell_base_of_lane(k, i, lane);
-                }
-                pi = load_pos4(k.pos4 + i);
-                n_pairs += encode_atom<TAB_SMEM, L16>(k, tv, pi, beg, end, pq, scr, lane, Pf, queued, pf, n_pref, cs, pc);
-                // Eq. 5 (C_l = I): this lane holds rows a = g, g + 8 of channels 8t + j; sum squares over the rows of a block.
-                // Rows 1..3 (l = 1) and 4..7 (l = 2) differ in the top bit of g, so one two-step butterfly over the lower
-                // bits sums both; l = 2 then takes row 8 (held by g = 0) and the upper half's sum, l = 3 is rows 9..15.
-                float part[4][8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float pa = Pf[j & 3][j >> 2], pb = Pf[j & 3][2 + (j >> 2)];
-                    float qa = g >= 1 ? pa * pa : 0.f, qb = g >= 1 ? pb * pb : 0.f;
-                    qa += __shfl_xor_sync(0xffffffffu, qa, 4);
-                    qb += __shfl_xor_sync(0xffffffffu, qb, 4);
-                    qa += __shfl_xor_sync(0xffffffffu, qa, 8);
-                    qb += __shfl_xor_sync(0xffffffffu, qb, 8);
-                    const float upper = __shfl_xor_sync(0xffffffffu, qa, 16);   // g = 0 receives the sum over g = 4..7
-                    qb += __shfl_xor_sync(0xffffffffu, qb, 16);
-                    part[0][j] = pa;                  // (the values below are those of the storing lanes, g = 0)
-                    part[1][j] = qa;
-                    part[2][j] = upper + pb * pb;
-                    part[3][j] = qb;
-                }
-                if (g == 0) {
-#pragma unroll
-                    for (int l = 0; l < 4; ++l) {
-                        *reinterpret_cast<float4 *>(xrow + 32 * l + 8 * t) = make_float4(part[l][0], part[l][1], part[l][2], part[l][3]);
-                        *reinterpret_cast<float4 *>(xrow + 32 * l + 8 * t + 4) = make_float4(part[l][4], part[l][5], part[l][6], part[l][7]);
-                    }
-                }
-            } else {   // empty slot of a ragged tile: feed zeros to the head
-                for (int c = lane; c < N_INV; c += 32) xrow[c] = 0.f;
+            // ---------------- Encoding + invariants: the warp's atoms wg, wg + 8 one after the other ----------------
+            if (prefetched) {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                __syncwarp();
             }
-            __syncwarp();
-            split_invariants(xrow, xs, sc, hc, wg, lane);
+            int q_used = 0;   // pairs of the queue that are kept for the derivation
+#pragma unroll 1
+            for (int u = 0; u < APW; ++u) {
+                float *xrow = scr;                        // the atom's invariants (the encoding is done with the scratch)
+                if (wg + GW * u < count) {
+                    int i, n_pref = 0, cs = 0, queued = -1;
+                    int64_t beg, end;
+                    const int *nidx = pf + u * PF_WORDS;
+                    if (prefetched) {
+                        i = nidx[PF_IDX];
+                        beg = ((int64_t)nidx[PF_IDX + 2] << 32) | (unsigned)nidx[PF_IDX + 1];
+                        end = beg + nidx[PF_IDX + 3];
+                        n_pref = min(PF_IDX, nidx[PF_IDX + 3]);
+                        if (L16) cs = lane < 27 ? nidx[PF_CS + lane] : 0;
+                    } else {
+                        i = (int)MLIP_CHECK_INDEX(__ldg(k.center_order + first + wg + GW * u), k.n, k.status);
+                        beg = k.nbr_off[i]; end = use_far ? k.nbr_off[i + 1] : beg + k.nbr_near[i];
+                        if (L16) cs = cell_base_of_lane(k, i, lane);
+                    }
+                    const double4 pi = load_pos4(k.pos4 + i);
+                    float Pf[4][4];
+                    n_pairs += encode_atom<TAB_SMEM, L16>(k, tv, pi, beg, end, pq + q_used, LY::POOL - q_used, scr, lane, Pf, queued, nidx, n_pref, cs, pc);
+                    if (u + 1 < APW && queued > LY::POOL - SECOND_ROOM) queued = -1;   // leave the next atom room for a scan
+                    if (lane == 0) *reinterpret_cast<int4 *>(info + 4 * u) = make_int4(i, queued, q_used, 0);
+                    q_used += max(queued, 0);
+                    tmem_st16(u == 0 ? tm_p : tm_vt, Pf);
+                    // Eq. 5 (C_l = I): this lane holds rows a = g, g + 8 of channels 8t + j; sum squares over the rows of a block.
+                    // Rows 1..3 (l = 1) and 4..7 (l = 2) differ in the top bit of g, so one two-step butterfly over the lower
+                    // bits sums both; l = 2 then takes row 8 (held by g = 0) and the upper half's sum, l = 3 is rows 9..15.
+                    float part[4][8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float pa = Pf[j & 3][j >> 2], pb = Pf[j & 3][2 + (j >> 2)];
+                        float qa = g >= 1 ? pa * pa : 0.f, qb = g >= 1 ? pb * pb : 0.f;
+                        qa += __shfl_xor_sync(0xffffffffu, qa, 4);
+                        qb += __shfl_xor_sync(0xffffffffu, qb, 4);
+                        qa += __shfl_xor_sync(0xffffffffu, qa, 8);
+                        qb += __shfl_xor_sync(0xffffffffu, qb, 8);
+                        const float upper = __shfl_xor_sync(0xffffffffu, qa, 16);   // g = 0 receives the sum over g = 4..7
+                        qb += __shfl_xor_sync(0xffffffffu, qb, 16);
+                        part[0][j] = pa;                  // (the values below are those of the storing lanes, g = 0)
+                        part[1][j] = qa;
+                        part[2][j] = upper + pb * pb;
+                        part[3][j] = qb;
+                    }
+                    if (g == 0) {
+#pragma unroll
+                        for (int l = 0; l < 4; ++l) {
+                            *reinterpret_cast<float4 *>(xrow + 32 * l + 8 * t) = make_float4(part[l][0], part[l][1], part[l][2], part[l][3]);
+                            *reinterpret_cast<float4 *>(xrow + 32 * l + 8 * t + 4) = make_float4(part[l][4], part[l][5], part[l][6], part[l][7]);
+                        }
+                    }
+                } else {   // empty slot of a ragged tile: feed zeros to the head
+                    for (int c = lane; c < N_INV; c += 32) xrow[c] = 0.f;
+                }
+                __syncwarp();
+                split_invariants(xrow, xs, sc, hc, wg + GW * u, NA, lane);
+                __syncwarp();   // (the next atom's hand-over rows overwrite the invariants)
+            }
+            tmem_wait_st();
             if (wg == 0 && lane == 0) ctl[2 * group + 1] = look_ahead;
             pc.mark(7);
             group_sync(group);
@@ -1019,16 +1071,24 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
             const int tile_next = ctl[2 * group + 1];
 
             // ---------------- Regression (and the prefetch for the next tile) ----------------
-            NextAtom nx;
-            nx.k = &k; nx.sidx = pf; nx.meta = pf + PF_IDX;
-            nx.slot = (tile_next < n_tiles && s_beg + tile_next * TILE + wg < s_end) ? s_beg + tile_next * TILE + wg : -1;
-            nx.i = 0; nx.beg = 0; nx.end = 0; nx.use_far = use_far; nx.cid = 0;
-            head_tile<DET, L16>(k, xs, sX, sc, ep, zs, hc, tm_quarter, count, first, group, wg, lane, e_sum, nx, pc);
-            prefetched = nx.slot >= 0;
+            NextAtoms<APW> nx;
+            nx.k = &k; nx.pf = pf;
+            const int next_slot = s_beg + tile_next * NA + wg + GW * lane;
+            nx.slot = (lane < APW && tile_next < n_tiles && next_slot < s_end) ? next_slot : -1;
+            nx.i = 0; nx.beg = 0; nx.len = 0; nx.use_far = use_far; nx.cid = 0;
+            head_tile<APW, DET, L16>(k, xs, sX, sc, ep, zs, hc, tm_quarter, count, first, group, wg, lane, e_sum, nx, pc);
+            prefetched = tile_next < n_tiles && s_beg + tile_next * NA + wg < s_end;
             pc.mark(9);
 
-            // ---------------- Derivation ----------------
-            if (have) {
+            // ---------------- Derivation: the second atom first (a rescan of the first one's list would overwrite its queue) ----
+#pragma unroll 1
+            for (int u = APW - 1; u >= 0; --u) {
+                if (wg + GW * u >= count) continue;
+                const int4 inf = *reinterpret_cast<const int4 *>(info + 4 * u);
+                const float *drow = sX + (wg + GW * u) * X_STRIDE;   // dE/dG of the atom
+                float Pf[4][4];
+                tmem_ld16(u == 0 ? tm_p : tm_vt, Pf);
+                tmem_wait_ld();
                 // W_i = dE_i/dP_i (Eq. 7), already in B-fragment order
                 const int la = g == 0 ? 0 : (g <= 3 ? 1 : 2), lb = g == 0 ? 2 : 3;
                 float da[8], db[8];
@@ -1057,7 +1117,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
                         split_h2(w[0][2 * nt + ks] * sw, w[1][2 * nt + ks] * sw, Wh[ks][nt][0], Wl[ks][nt][0]);
                         split_h2(w[2][2 * nt + ks] * sw, w[3][2 * nt + ks] * sw, Wh[ks][nt][1], Wl[ks][nt][1]);
                     }
-                derive_atom<TAB_SMEM, DET, L16>(k, tv, i, pq, scr, queued, lane, Wh, Wl, inverse_pow2(sw), vir, tm_vt, pc);
+                derive_atom<TAB_SMEM, DET, L16>(k, tv, inf.x, pq + inf.z, LY::POOL - inf.z, scr, inf.y, lane, Wh, Wl, inverse_pow2(sw), vir, tm_vt, pc);
                 if (DET) {   // fold this atom's virial in now: lane sums in a fixed order, then integers
 #pragma unroll
                     for (int q = 0; q < 9; ++q) {
@@ -1078,7 +1138,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
     // per-warp totals -> global accumulators
     if (DET) {
         if (lane < 9) atomicAdd(reinterpret_cast<unsigned long long *>(k.acc_fx + 1 + lane), (unsigned long long)(long long)vir_fx);
-        if (wg == 7 && lane < TILE) atomicAdd(reinterpret_cast<unsigned long long *>(k.acc_fx), (unsigned long long)(long long)e_sum);
+        if (wg == 7 && lane < NA) atomicAdd(reinterpret_cast<unsigned long long *>(k.acc_fx), (unsigned long long)(long long)e_sum);
     } else {
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
@@ -1087,7 +1147,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
             for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
             if (lane == 0) atomicAdd(&k.acc[ACC_VIRIAL + q], (double)x);
         }
-        if (wg == 7 && lane < TILE) atomicAdd(&k.acc[ACC_ENERGY], e_sum);
+        if (wg == 7 && lane < NA) atomicAdd(&k.acc[ACC_ENERGY], e_sum);
     }
     if (lane == 0) atomicAdd(k.pair_counter, n_pairs);
     tmem_fence_before_sync();
@@ -1098,7 +1158,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
 // ---------------- host side ----------------
 int table_smem_words(const mlip_ctx *c) { return c->cfg.n_species * (c->cfg.table_knots + 3) * K_RADIAL; }
 bool tables_fit_smem(const mlip_ctx *c) {   // (the rows' 16-bit addresses, with room for a reserved kilobyte in front, are the tighter limit)
-    return FIXED_WORDS + table_smem_words(c) <= SMEM_LIMIT_WORDS && 4 * table_smem_words(c) + 2048 <= 65536;
+    return Layout<2>::FIXED + table_smem_words(c) <= SMEM_LIMIT_WORDS && 4 * table_smem_words(c) + 2048 <= 65536;
 }
 
 static float pow2f(int e) { return ldexpf(1.f, e); }
@@ -1233,23 +1293,23 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     if (det) MLIP_CUDA_TRY(c, cudaMemsetAsync(c->force_fx, 0, sizeof(long long) * 3 * n, s));
     MLIP_CUDA_TRY(c, cudaMemsetAsync(c->force, 0, sizeof(float4) * n, s));
     MLIP_CUDA_TRY(c, cudaMemsetAsync(c->launch_block, 0, LAUNCH_CLEAR_BYTES, s));   // tile and pair counters, integer and fp64 accumulators
-    const int64_t tiles_max = (n + TILE - 1) / TILE + c->cfg.n_species;
-    const int blocks = (int)std::min<int64_t>(tiles_max, (int64_t)c->n_sm);
     const bool in_smem = tables_fit_smem(c);
     const int tab_words = in_smem ? table_smem_words(c) : 0;
-    const size_t smem_bytes = sizeof(float) * (size_t)(FIXED_WORDS + tab_words);
-    // instantiations: tables in shared / global memory x floating-point / integer scatter x int32 / 16-bit lists, and the
-    // shared-memory ones again with staggered species for small systems
+    // instantiations: {one, two atoms per warp with staggered species, two without, two with tables in global memory}
+    // x floating-point / integer scatter x int32 / 16-bit lists
     using Kernel = void (*)(KernelArgs, int);
-    static const Kernel kernels[12] = {k_mega<false, false, false, false>, k_mega<false, false, true, false>, k_mega<false, true, false, false>,
-                                       k_mega<false, true, true, false>,   k_mega<true, false, false, false>, k_mega<true, false, true, false>,
-                                       k_mega<true, true, false, false>,   k_mega<true, true, true, false>,   k_mega<true, false, false, true>,
-                                       k_mega<true, false, true, true>,    k_mega<true, true, false, true>,   k_mega<true, true, true, true>};
-    const bool stagger = in_smem && n < STAGGER_BELOW_ATOMS;
+#define MLIP_MEGA4(APW, SMEM, STAG) {k_mega<APW, SMEM, false, false, STAG>, k_mega<APW, SMEM, false, true, STAG>, k_mega<APW, SMEM, true, false, STAG>, k_mega<APW, SMEM, true, true, STAG>}
+    static const Kernel kernels[4][4] = {MLIP_MEGA4(1, true, true), MLIP_MEGA4(2, true, true), MLIP_MEGA4(2, true, false), MLIP_MEGA4(2, false, false)};
+#undef MLIP_MEGA4
+    const int shape = !in_smem ? 3 : n >= STAGGER_BELOW_ATOMS ? 2 : n >= ONE_PER_WARP_BELOW_ATOMS ? 1 : 0;
+    const int apw = shape == 0 ? 1 : 2;
+    const size_t smem_bytes = sizeof(float) * (size_t)((apw == 1 ? Layout<1>::FIXED : Layout<2>::FIXED) + tab_words);
+    const int64_t tiles_max = (n + GW * apw - 1) / (GW * apw) + c->cfg.n_species;
+    const int blocks = (int)std::min<int64_t>(tiles_max, (int64_t)c->n_sm);
     if (!c->kernel_ready) {
-        for (int q = 0; q < 12; ++q) {
-            const size_t bytes = sizeof(float) * (size_t)(FIXED_WORDS + (q >= 4 ? tab_words : 0));
-            cudaError_t e = cudaFuncSetAttribute((const void *)kernels[q], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        for (int q = 0; q < 16; ++q) {
+            const int most = (q < 4 ? Layout<1>::FIXED : Layout<2>::FIXED) + (q < 12 ? tab_words : 0);
+            cudaError_t e = cudaFuncSetAttribute((const void *)kernels[q / 4][q % 4], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(float) * most);
             if (e != cudaSuccess) { c->err = std::string("fused kernel shared memory: ") + cudaGetErrorString(e); return MLIP_ERR_CUDA; }
         }
         c->kernel_ready = true;
@@ -1263,7 +1323,7 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     k.acc = c->acc; k.pair_counter = c->pair_counter; k.status = c->status; k.tile_counter = c->tile_counter;
     const int slot = (int)(c->ev_count % mlip_ctx::EV_POOL);
     MLIP_CUDA_TRY(c, cudaEventRecord(c->ev[2 * slot], s));
-    kernels[(stagger ? 8 : in_smem ? 4 : 0) + (det ? 2 : 0) + (c->list16 ? 1 : 0)]<<<blocks, NW * 32, smem_bytes, s>>>(k, tab_words);
+    kernels[shape][(det ? 2 : 0) + (c->list16 ? 1 : 0)]<<<blocks, NW * 32, smem_bytes, s>>>(k, tab_words);
     if (det) {
         k_fixed_finish<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, c->force_fx, c->acc_fx, c->force, c->acc);
         c->launches += 1;
