@@ -165,12 +165,12 @@ int mlip_get_neighbors(mlip_ctx *ctx, int64_t *seg_ptr, int32_t *nbr, int64_t ca
 /*
  * mlip_get_neighbors without any allocation (the paper has no counterpart: this is a
  * deployment variant, not a step of its method).  Same arguments, same output, same status codes.
- * mlip_get_neighbors takes two temporary device blocks with cudaMalloc on every call; some callers
- * cannot afford that: an MD driver that has handed all device memory to its own pools, a plug-in
- * that must not disturb its host's allocator, code running where an allocation would stall every
- * stream.  This variant keeps those temporaries in a static device array of about 4 MiB that every
- * GPU loading the library holds until the process exits, and calls no cudaMalloc, cudaFree or
- * allocating library routine.
+ * mlip_get_neighbors keeps its temporaries in buffers of the context that list builds use; this variant
+ * leaves those alone and keeps them in a static device array of about 4 MiB that every GPU loading the
+ * library holds until the process exits.  Neither calls cudaMalloc, cudaFree or an allocating library
+ * routine, for the sake of callers that cannot afford one: an MD driver that has handed all device memory
+ * to its own pools, a plug-in that must not disturb its host's allocator, code running where an
+ * allocation would stall every stream.
  *   Limit: n_atoms * n_species <= 1,048,576; larger systems get MLIP_ERR_UNSUPPORTED.
  *   The first call on a device looks up the array's device address (once per device, with that
  *   device current); make that first call before starting any stream capture.

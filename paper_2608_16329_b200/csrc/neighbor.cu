@@ -554,39 +554,74 @@ struct ListView {
     }
 };
 
-__global__ void k_export_count(int64_t n, int n_species, const int64_t *__restrict__ nbr_off, ListView lv,
-                               const double4 *__restrict__ pos4, const int32_t *__restrict__ user_of,
-                               int32_t *__restrict__ seg_count) {
-    const int lane = threadIdx.x & 31;
-    int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (i >= n) return;
-    int cnt[MAX_SPECIES] = {0};
-    for (int64_t e = nbr_off[i] + lane; e < nbr_off[i + 1]; e += 32) cnt[(int)pos4[lv.at(i, e)].w]++;
-    int64_t row = (int64_t)user_of[i] * n_species;
-    for (int s = 0; s < n_species; ++s) {
-        int v = cnt[s];
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) seg_count[row + s] = v;
-    }
+// An atom's place in every canonical list: species, then caller index, in one word (8 species, 2^28 atoms).
+__global__ void k_export_keys(int64_t n, const double4 *__restrict__ pos4, const int32_t *__restrict__ user_of, int32_t *__restrict__ key) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) key[i] = ((int)pos4[i].w << 28) | user_of[i];
 }
 
-__global__ void k_export_fill(int64_t n, int n_species, const int64_t *__restrict__ nbr_off, ListView lv,
-                              const double4 *__restrict__ pos4, const int32_t *__restrict__ user_of,
-                              const int64_t *__restrict__ seg_ptr, int32_t *__restrict__ out) {
+// Warp per atom: entries per species.  Each lane counts in 16-bit fields (a list holds at most 27 x MAX_CELL_ATOMS entries).
+__global__ void __launch_bounds__(256) k_export_count(int64_t n, int n_species, const int64_t *__restrict__ nbr_off, ListView lv,
+                                                      const int32_t *__restrict__ key, int32_t *__restrict__ seg_count) {
+    static_assert(27 * MAX_CELL_ATOMS < 65536 && MAX_SPECIES == 8, "16-bit fields, two to a word");
     const int lane = threadIdx.x & 31;
     int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (i >= n) return;
-    const int64_t beg = nbr_off[i], end = nbr_off[i + 1];
-    const int64_t row = (int64_t)user_of[i] * n_species;
-    for (int64_t e = beg + lane; e < end; e += 32) {
-        int j = lv.at(i, e);
-        int sj = (int)pos4[j].w, uj = user_of[j];
-        int rank = 0;   // entries of the same species with a smaller caller index
-        for (int64_t f = beg; f < end; ++f) {
-            int jf = lv.at(i, f);
-            rank += ((int)pos4[jf].w == sj) && (user_of[jf] < uj);
+    unsigned cnt[4] = {0, 0, 0, 0};
+    for (int64_t e = nbr_off[i] + lane; e < nbr_off[i + 1]; e += 32) {
+        const int s = (int)((unsigned)key[lv.at(i, e)] >> 28);
+#pragma unroll
+        for (int w = 0; w < 4; ++w) cnt[w] += (s >> 1) == w ? 1u << (16 * (s & 1)) : 0u;
+    }
+    const int64_t row = (int64_t)(key[i] & 0x0fffffff) * n_species;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) cnt[w] = __reduce_add_sync(0xffffffffu, cnt[w]);
+    if (lane < n_species) seg_count[row + lane] = (int)((((lane >> 1) == 0 ? cnt[0] : (lane >> 1) == 1 ? cnt[1] : (lane >> 1) == 2 ? cnt[2] : cnt[3]) >> (16 * (lane & 1))) & 0xffffu);
+}
+
+// Warp per atom: an entry's place is the number of smaller keys in the list (keys differ within a list), counted against the keys
+// in shared memory, four per load.  Lists longer than the buffer read them again from global memory.  (Ranking by re-reading
+// list, species and caller index for every pair of entries took 2.0 ms for 108,000 atoms with 134 entries each; this takes
+// a tenth.)
+constexpr int EXPORT_BUF = 256;
+__global__ void __launch_bounds__(256) k_export_fill(int64_t n, int n_species, const int64_t *__restrict__ nbr_off, ListView lv,
+                                                     const int32_t *__restrict__ key, const int64_t *__restrict__ seg_ptr, int32_t *__restrict__ out) {
+    __shared__ __align__(16) int32_t s_keys[8][EXPORT_BUF];
+    const int lane = threadIdx.x & 31;
+    int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= n) return;
+    int32_t *keys = s_keys[threadIdx.x >> 5];
+    const int64_t beg = nbr_off[i];
+    const int m = (int)(nbr_off[i + 1] - beg);
+    out += seg_ptr[(int64_t)(key[i] & 0x0fffffff) * n_species];   // the species' segments of an atom follow one another
+    if (m <= EXPORT_BUF) {
+        constexpr int PER_LANE = EXPORT_BUF / 32;
+        int32_t mine[PER_LANE], rank[PER_LANE];
+#pragma unroll
+        for (int c = 0; c < PER_LANE; ++c) {
+            const int e = 32 * c + lane;
+            mine[c] = e < m ? key[lv.at(i, beg + e)] : 0x7fffffff;
+            rank[c] = 0;
+            keys[e] = mine[c];
         }
-        out[seg_ptr[row + sj] + rank] = uj;
+        __syncwarp();
+        const int chunks = (m + 31) >> 5;
+        for (int q = 0; q < m; q += 4) {
+            const int4 other = *reinterpret_cast<const int4 *>(keys + q);
+#pragma unroll
+            for (int c = 0; c < PER_LANE; ++c)
+                if (c < chunks) rank[c] += (other.x < mine[c]) + (other.y < mine[c]) + (other.z < mine[c]) + (other.w < mine[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < PER_LANE; ++c)
+            if (32 * c + lane < m) out[rank[c]] = mine[c] & 0x0fffffff;
+        return;
+    }
+    for (int e = lane; e < m; e += 32) {
+        const int32_t mine = key[lv.at(i, beg + e)];
+        int rank = 0;
+        for (int f = 0; f < m; ++f) rank += key[lv.at(i, beg + f)] < mine;
+        out[rank] = mine & 0x0fffffff;
     }
 }
 
@@ -736,39 +771,36 @@ static int lists_whole(mlip_ctx *c, cudaStream_t s) {
     return MLIP_OK;
 }
 
-int launch_export(mlip_ctx *c, int64_t *seg_ptr, int32_t *nbr, int64_t capacity, int64_t *n_entries_host, cudaStream_t s) {
+// Keys, counts, scan; then, if the caller's array holds them, the lists.  `seg_count` [n * C] and `tmp` (scan_tmp_items(n * C)) are scratch;
+// the keys go to cell_of, which is read during list builds only.
+static int export_lists(mlip_ctx *c, int64_t *seg_ptr, int32_t *nbr, int64_t capacity, int64_t *n_entries_host, int32_t *seg_count, int64_t *tmp, cudaStream_t s) {
     const int64_t n = c->n;
     const int C = c->cfg.n_species;
-    int whole = lists_whole(c, s);
-    if (whole != MLIP_OK) return whole;
-    int32_t *seg_count = nullptr;
-    MLIP_CUDA_TRY(c, cudaMalloc(&seg_count, sizeof(int32_t) * (size_t)(n * C + 1)));
-    int64_t *tmp = nullptr;
-    if (cudaMalloc(&tmp, sizeof(int64_t) * (size_t)scan_tmp_items(n * C)) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(seg_count);
-        c->err = "neighbor export: cudaMalloc of the scan scratch failed";
-        return MLIP_ERR_OOM;
-    }
-    k_export_count<<<blocks_for(n * 32, 256), 256, 0, s>>>(n, C, c->nbr_off, list_view(c), c->pos4, c->user_of, seg_count);
+    k_export_keys<<<blocks_for(n, 256), 256, 0, s>>>(n, c->pos4, c->user_of, c->cell_of);
+    k_export_count<<<blocks_for(n * 32, 256), 256, 0, s>>>(n, C, c->nbr_off, list_view(c), c->cell_of, seg_count);
     exclusive_scan<int32_t, int64_t>(seg_count, seg_ptr, n * C, tmp, s);
-    int rc = MLIP_OK;
-    cudaError_t e = cudaMemcpyAsync(c->total_host, seg_ptr + n * C, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) {
-        if (n_entries_host) *n_entries_host = *c->total_host;
-        if (*c->total_host > capacity || !nbr) rc = MLIP_ERR_NEIGHBOR_OVERFLOW;
-        else {
-            k_export_fill<<<blocks_for(n * 32, 256), 256, 0, s>>>(n, C, c->nbr_off, list_view(c), c->pos4, c->user_of, seg_ptr, nbr);
-            e = cudaStreamSynchronize(s);
-        }
-    }
+    MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->total_host, seg_ptr + n * C, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
     c->launches += 5;
-    cudaFree(seg_count);
-    cudaFree(tmp);
-    if (e != cudaSuccess) { c->err = cudaGetErrorString(e); return MLIP_ERR_CUDA; }
-    if (rc != MLIP_OK) c->err = "neighbor export: capacity too small";
-    return rc;
+    if (n_entries_host) *n_entries_host = *c->total_host;
+    if (*c->total_host > capacity || !nbr) {
+        c->err = "neighbor export: capacity too small";
+        return MLIP_ERR_NEIGHBOR_OVERFLOW;
+    }
+    k_export_fill<<<blocks_for(n * 32, 256), 256, 0, s>>>(n, C, c->nbr_off, list_view(c), c->cell_of, seg_ptr, nbr);
+    c->launches += 1;
+    MLIP_CUDA_TRY(c, cudaGetLastError());
+    MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
+    return MLIP_OK;
+}
+
+int launch_export(mlip_ctx *c, int64_t *seg_ptr, int32_t *nbr, int64_t capacity, int64_t *n_entries_host, cudaStream_t s) {
+    const int whole = lists_whole(c, s);
+    if (whole != MLIP_OK) return whole;
+    // The source set of the list builds is dead between builds and holds the scratch (device allocations here stalled the call
+    // by up to 10 ms): n * C <= 8 n counts in the 32 n bytes of pos4_src, n * C / 4,096 + 3 sums in the 24 n bytes of vel_src.
+    static_assert(sizeof(double4) >= MAX_SPECIES * sizeof(int32_t) && SCAN_TILE >= 8 * MAX_SPECIES, "export scratch");
+    return export_lists(c, seg_ptr, nbr, capacity, n_entries_host, reinterpret_cast<int32_t *>(c->pos4_src), reinterpret_cast<int64_t *>(c->vel_src), s);
 }
 
 }  // namespace mlip
@@ -809,14 +841,12 @@ static int export_scratch_for_current_device(mlip_ctx *c, void **out) {
     return MLIP_OK;
 }
 
-// Same kernels and the same order as launch_export, with the temporaries taken from the static
+// The same export as launch_export, with the temporaries taken from the static
 // array.  Every scratch word that is read (counts of all n * C segments, the scan's tile sums) is
 // written earlier in the same call, so nothing has to be cleared between calls; two calls whose
 // kernels overlap on the GPU (different streams or contexts on one device) would race on it.
 int launch_export_noalloc(mlip_ctx *c, int64_t *seg_ptr, int32_t *nbr, int64_t capacity, int64_t *n_entries_host, cudaStream_t s) {
-    const int64_t n = c->n;
-    const int C = c->cfg.n_species;
-    if (n * C > NOALLOC_MAX_SEGMENTS) {
+    if (c->n * c->cfg.n_species > NOALLOC_MAX_SEGMENTS) {
         c->err = "mlip_get_neighbors_noalloc: n_atoms * n_species exceeds 1048576 (the static scratch size); use mlip_get_neighbors";
         return MLIP_ERR_UNSUPPORTED;
     }
@@ -824,22 +854,8 @@ int launch_export_noalloc(mlip_ctx *c, int64_t *seg_ptr, int32_t *nbr, int64_t c
     int rc = lists_whole(c, s);
     if (rc != MLIP_OK) return rc;
     if ((rc = export_scratch_for_current_device(c, &base)) != MLIP_OK) return rc;
-    int32_t *seg_count = reinterpret_cast<int32_t *>(base);
-    int64_t *tmp = reinterpret_cast<int64_t *>(static_cast<unsigned char *>(base) + NOALLOC_COUNT_BYTES);
-    k_export_count<<<blocks_for(n * 32, 256), 256, 0, s>>>(n, C, c->nbr_off, list_view(c), c->pos4, c->user_of, seg_count);
-    exclusive_scan<int32_t, int64_t>(seg_count, seg_ptr, n * C, tmp, s);
-    MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->total_host, seg_ptr + n * C, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
-    c->launches += 4;
-    if (n_entries_host) *n_entries_host = *c->total_host;
-    if (*c->total_host > capacity || !nbr) {
-        c->err = "neighbor export: capacity too small";
-        return MLIP_ERR_NEIGHBOR_OVERFLOW;
-    }
-    k_export_fill<<<blocks_for(n * 32, 256), 256, 0, s>>>(n, C, c->nbr_off, list_view(c), c->pos4, c->user_of, seg_ptr, nbr);
-    c->launches += 1;
-    MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
-    return MLIP_OK;
+    return export_lists(c, seg_ptr, nbr, capacity, n_entries_host, reinterpret_cast<int32_t *>(base),
+                        reinterpret_cast<int64_t *>(static_cast<unsigned char *>(base) + NOALLOC_COUNT_BYTES), s);
 }
 
 }  // namespace mlip
