@@ -50,14 +50,14 @@ static void free_atoms(mlip_ctx *c) {
     dev_free(c, &c->nbr_count, n); dev_free(c, &c->nbr_near, n); dev_free(c, &c->nbr_off, n + 1);
     if (c->cfg.precision == 1) { dev_free(c, &c->force_d, 3 * n); dev_free(c, &c->e_atom_d, n); }
     if (c->cfg.force_mode == 1) dev_free(c, &c->force_fx, 3 * n);
-    dev_free(c, &c->tile_state, n / 64 + 2);
+    dev_free(c, &c->tile_state, (size_t)tile_words(c->cap_atoms));
     if (c->cfg.list_format == 1) dev_free(c, &c->cell_id, n);
     c->cap_atoms = 0;
 }
 
 static void free_cells(mlip_ctx *c) {
     const size_t nc = (size_t)c->cap_cells, C = (size_t)c->cfg.n_species;
-    dev_free(c, &c->cell_count, nc + 1); dev_free(c, &c->cell_start, nc + 1); dev_free(c, &c->cell_fill, nc + 1);
+    dev_free(c, &c->cell_count, nc + 1); dev_free(c, &c->cell_start, nc + 1);
     dev_free(c, &c->bin_count, C * nc + 1); dev_free(c, &c->bin_start, C * nc + 1);
     c->cap_cells = 0;
 }
@@ -76,14 +76,16 @@ static int ensure_capacity(mlip_ctx *c, int64_t n, int64_t n_cells) {
         TRY_ALLOC(c->nbr_count, m); TRY_ALLOC(c->nbr_near, m); TRY_ALLOC(c->nbr_off, m + 1);
         if (c->cfg.precision == 1) { TRY_ALLOC(c->force_d, 3 * m); TRY_ALLOC(c->e_atom_d, m); }
         if (c->cfg.force_mode == 1) TRY_ALLOC(c->force_fx, 3 * m);
-        TRY_ALLOC(c->tile_state, m / 64 + 2);
+        TRY_ALLOC(c->tile_state, (size_t)tile_words(n));
         if (c->cfg.list_format == 1) TRY_ALLOC(c->cell_id, m);
         c->cap_atoms = n;
     }
     if (n_cells > c->cap_cells) {
         free_cells(c);
         const size_t nc = (size_t)n_cells, C = (size_t)c->cfg.n_species;
-        TRY_ALLOC(c->cell_count, nc + 1); TRY_ALLOC(c->cell_start, nc + 1); TRY_ALLOC(c->cell_fill, nc + 1);
+        TRY_ALLOC(c->cell_count, nc + 1); TRY_ALLOC(c->cell_start, nc + 1);
+        MLIP_CUDA_TRY(c, cudaMemset(c->cell_count, 0, sizeof(int32_t) * (nc + 1)));   // zero between builds from here on
+        MLIP_CUDA_TRY(c, cudaStreamSynchronize(nullptr));
         TRY_ALLOC(c->bin_count, C * nc + 1); TRY_ALLOC(c->bin_start, C * nc + 1);
         c->cap_cells = n_cells;
     }
@@ -245,17 +247,16 @@ int mlip_create(mlip_ctx **out, const mlip_config *cfg, const double *enc_w, siz
         c->pair_counter = reinterpret_cast<unsigned long long *>(c->launch_block + LB_PAIR);
         c->acc_fx = reinterpret_cast<long long *>(c->launch_block + LB_ACC_FX);
         c->acc = c->launch_block + LB_ACC;
-        if ((rc = dev_alloc(c, &c->status, 1)) != MLIP_OK) break;
-        if ((rc = dev_alloc(c, &c->rebuild_flag, 1)) != MLIP_OK) break;
-        if ((rc = dev_alloc(c, &c->far_flag, 1)) != MLIP_OK) break;
+        if ((rc = dev_alloc(c, &c->build_word, 8)) != MLIP_OK) break;
+        c->status = c->build_word + 4; c->rebuild_flag = c->build_word + 5; c->far_flag = c->build_word + 6;
         if ((rc = dev_alloc(c, &c->nhc, 8)) != MLIP_OK) break;
-        if ((rc = dev_alloc(c, &c->tile_ticket, 2)) != MLIP_OK) break;   // ticket, private overflow flag
         if ((rc = dev_alloc(c, &c->species_start, (size_t)MAX_SPECIES + 1)) != MLIP_OK) break;
         if ((rc = dev_alloc(c, &c->stage_out, 10)) != MLIP_OK) break;
         if ((rc = dev_alloc(c, &c->kin_part, 1184)) != MLIP_OK) break;
         if (cudaMallocHost((void **)&c->status_host, sizeof(int)) != cudaSuccess ||
             cudaMallocHost((void **)&c->total_host, sizeof(int64_t)) != cudaSuccess ||
-            cudaMallocHost((void **)&c->rebuild_host, sizeof(int)) != cudaSuccess) {
+            cudaMallocHost((void **)&c->rebuild_host, sizeof(int)) != cudaSuccess ||
+            cudaMallocHost((void **)&c->build_host, sizeof(int) * 8) != cudaSuccess) {
             rc = MLIP_ERR_CUDA; c->err = "pinned host allocation failed"; break;
         }
         bool ev_ok = true;
@@ -264,7 +265,7 @@ int mlip_create(mlip_ctx **out, const mlip_config *cfg, const double *enc_w, siz
                     cudaEventCreate(&c->ev_integrate[q]) == cudaSuccess;
         if (!ev_ok) { rc = MLIP_ERR_CUDA; c->err = "event creation failed"; break; }
         if (cudaMemcpy(c->mass, mass, sizeof(double) * cfg->n_species, cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemset(c->status, 0, sizeof(int)) != cudaSuccess || cudaMemset(c->rebuild_flag, 0, sizeof(int)) != cudaSuccess ||
+            cudaMemset(c->build_word, 0, sizeof(int) * 8) != cudaSuccess ||
             cudaMemset(c->nhc, 0, sizeof(double) * 8) != cudaSuccess || cudaMemset(c->launch_block, 0, sizeof(double) * LB_COUNT) != cudaSuccess) {
             rc = MLIP_ERR_CUDA; c->err = "initial upload failed"; break;
         }
@@ -318,13 +319,7 @@ int mlip_build_neighbors_ghost(mlip_ctx *c, int64_t n_owned, int64_t n_ghost, co
     c->n_owned = n_owned;
     if (n_ghost > 0) MLIP_CUDA_TRY(c, cudaMemsetAsync(c->e_atom, 0, sizeof(float) * n, s));   // ghosts have no E_i
     if (n_ghost > 0 && c->cfg.precision == 1) MLIP_CUDA_TRY(c, cudaMemsetAsync(c->e_atom_d, 0, sizeof(double) * n, s));
-    if ((rc = launch_pack_source(c, pos, species, s)) != MLIP_OK) return rc;
-    double *keep = c->vel_src;   // a NULL source makes the gather reset velocities to zero
-    c->vel_src = nullptr;
-    rc = launch_build(c, true, s);
-    c->vel_src = keep;
-    if (rc != MLIP_OK) return rc;
-    MLIP_CUDA_TRY(c, cudaMemsetAsync(c->rebuild_flag, 0, sizeof(int), s));
+    if ((rc = launch_build(c, true, pos, species, s)) != MLIP_OK) return rc;
     c->built = true;
     c->forces_current = false;
     c->n_builds += 1;
@@ -438,12 +433,11 @@ static int rebuild_if_due(mlip_ctx *c, int rebuild_every, cudaStream_t s) {
         rebuild = *c->rebuild_host != 0;
     }
     if (!rebuild) return MLIP_OK;
-    MLIP_CUDA_TRY(c, cudaMemsetAsync(c->rebuild_flag, 0, sizeof(int), s));
     c->n_builds += 1;
     std::swap(c->pos4, c->pos4_src);
     std::swap(c->vel, c->vel_src);
     std::swap(c->user_of, c->user_src);
-    return launch_build(c, false, s);
+    return launch_build(c, false, nullptr, nullptr, s);
 }
 
 int mlip_step(mlip_ctx *c, int n_steps, double dt, int rebuild_every, void *stream) {
@@ -564,7 +558,7 @@ int mlip_debug_rebuild(mlip_ctx *c, int spin_limit, int64_t unpublished_tile, vo
     std::swap(c->pos4, c->pos4_src);
     std::swap(c->vel, c->vel_src);
     std::swap(c->user_of, c->user_src);
-    int rc = launch_build(c, false, s);
+    int rc = launch_build(c, false, nullptr, nullptr, s);
     c->lookback_spin_limit = 0;
     c->lookback_unpublished_tile = -1;
     c->n_builds += 1;
@@ -688,12 +682,13 @@ void mlip_destroy(mlip_ctx *c) {
     free_cells(c);
     cudaFree(c->nbr); cudaFree(c->scan_tmp); cudaFree(c->head_w); cudaFree(c->table); cudaFree(c->mass);
     cudaFree(c->head_w_d); cudaFree(c->table_d);
-    cudaFree(c->launch_block); cudaFree(c->status); cudaFree(c->rebuild_flag); cudaFree(c->far_flag); cudaFree(c->nhc); cudaFree(c->tile_ticket);
+    cudaFree(c->launch_block); cudaFree(c->build_word); cudaFree(c->nhc);
     cudaFree(c->species_start); cudaFree(c->stage_pos); cudaFree(c->stage_species); cudaFree(c->stage_force);
     cudaFree(c->stage_out); cudaFree(c->kin_part);
     if (c->status_host) cudaFreeHost(c->status_host);
     if (c->total_host) cudaFreeHost(c->total_host);
     if (c->rebuild_host) cudaFreeHost(c->rebuild_host);
+    if (c->build_host) cudaFreeHost(c->build_host);
     for (int q = 0; q < 2 * mlip_ctx::EV_POOL; ++q) {
         if (c->ev[q]) cudaEventDestroy(c->ev[q]);
         if (c->ev_build[q]) cudaEventDestroy(c->ev_build[q]);

@@ -111,7 +111,7 @@ struct mlip_ctx {
     int32_t *user_src = nullptr;
     // cells
     int32_t *cell_of = nullptr;    // per source atom
-    int32_t *cell_count = nullptr, *cell_start = nullptr, *cell_fill = nullptr;   // [n_cells + 1]
+    int32_t *cell_count = nullptr, *cell_start = nullptr;   // [n_cells + 1]; cell_count is zero between builds
     int32_t *bin_count = nullptr, *bin_start = nullptr;                           // [C * n_cells + 1]
     int32_t *species_start = nullptr;  // dev [C + 1]
     // lists
@@ -122,8 +122,9 @@ struct mlip_ctx {
     int32_t *nbr = nullptr;        // list entries: int32 indices, or uint16 cell-relative codes when list16
     bool list16 = false;           // format of the current lists (mlip_config.list_format = 1 on a grid of >= 3 cells per edge)
     int32_t *cell_id = nullptr;    // [N] build-time cell of each atom as packed coordinates, internal order (allocated for list_format = 1)
-    unsigned long long *tile_state = nullptr;   // [ceil(N / 64) + 1] look-back words of the one-pass rebuild
-    int *tile_ticket = nullptr;
+    unsigned long long *tile_state = nullptr;   // [tile_words(N)] look-back words of the one-pass build
+    int *build_word = nullptr;     // {ticket, private overflow flag, total entries (64 bits)} of the one-pass build, then status, rebuild_flag, far_flag
+    int *build_host = nullptr;     // pinned copy of its first five words
     int64_t nbr_cap = 0, n_entries = 0;
     // scratch
     int64_t *scan_tmp = nullptr;   // block sums for the scans
@@ -178,8 +179,8 @@ inline void timing_begin(cudaEvent_t *pool, int64_t count, cudaStream_t s) { cud
 inline void timing_end(cudaEvent_t *pool, int64_t &count, cudaStream_t s) { cudaEventRecord(pool[2 * (count % mlip_ctx::EV_POOL) + 1], s); count += 1; }
 
 // neighbor.cu
-int launch_pack_source(mlip_ctx *c, const double *pos, const int32_t *species, cudaStream_t s);
-int launch_build(mlip_ctx *c, bool allow_sync_grow, cudaStream_t s);
+int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int32_t *species, cudaStream_t s);
+int64_t tile_words(int64_t n);
 int launch_export(mlip_ctx *c, int64_t *seg_ptr, int32_t *nbr, int64_t capacity, int64_t *n_entries_host, cudaStream_t s);
 int launch_export_noalloc(mlip_ctx *c, int64_t *seg_ptr, int32_t *nbr, int64_t capacity, int64_t *n_entries_host, cudaStream_t s);
 // tables.cu

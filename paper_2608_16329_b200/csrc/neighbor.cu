@@ -3,9 +3,14 @@
 // Section 4.1.4).  Everything runs on the device:
 //   cell id per atom -> counting sort into cell order (ties broken by species, then by the
 //   caller's index, so the internal order is reproducible) -> per-species processing order
-//   -> two passes (count, fill) of a warp-per-atom scan over the 27 surrounding cells.
+//   -> one warp-per-atom traversal of the 27 surrounding cells (two, count and fill, when there is no array yet or it is too small).
+// Small systems are bound by the number of launches and by the longest chain in one thread or warp, large ones by the
+// traversal's instruction issue.
 // The inclusion test is fp64 with separately rounded operations, so the set of pairs is
 // identical to a plain CPU evaluation of the same expression.
+#include <algorithm>
+#include <string.h>
+
 #include "common.cuh"
 #include "scan.cuh"
 
@@ -29,21 +34,33 @@ __device__ __forceinline__ OUT list_entry(int j, int it, int cell_beg) {
     return (OUT)j;
 }
 
-__global__ void k_pack_source(const double *__restrict__ pos, const int32_t *__restrict__ species, int64_t n,
-                              int n_species, double4 *__restrict__ pos4, int32_t *__restrict__ user, int *status) {
+// What a build clears on its way: the look-back words, {ticket, overflow, total} of the one-pass traversal, and the two flags.
+struct BuildClear {
+    unsigned long long *tile_state;
+    int64_t n_words;       // <= number of atoms
+    int *build_word, *far_flag, *rebuild_flag;
+};
+// Cell of every atom and its rank of arrival there (cell_count is zero between builds: k_sort_gather clears it).  PACK: the atoms come
+// from the caller's arrays and are packed into the source set on the way.
+template <bool PACK>
+__global__ void k_cell_id(const double *__restrict__ pos, const int32_t *__restrict__ species, int n_species, double4 *__restrict__ pos4,
+                          int32_t *__restrict__ user, int64_t n, CellGrid g, int32_t *__restrict__ cell_of, int32_t *__restrict__ rank_of,
+                          int32_t *__restrict__ cell_count, int *status, BuildClear clear) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    int s = species[i];
-    if (s < 0 || s >= n_species) { atomicOr(status, FLAG_NONFINITE); s = 0; }
-    pos4[i] = make_double4(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], (double)s);
-    user[i] = (int32_t)i;
-}
-
-__global__ void k_cell_id(const double4 *__restrict__ pos4, int64_t n, CellGrid g, int32_t *__restrict__ cell_of,
-                          int32_t *__restrict__ cell_count, int *status) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double4 p = pos4[i];
+    if (i < clear.n_words) clear.tile_state[i] = 0;
+    if (i == 0) {
+        for (int q = 0; q < 4; ++q) clear.build_word[q] = 0;
+        *clear.far_flag = 0; *clear.rebuild_flag = 0;
+    }
+    double4 p;
+    if (PACK) {
+        int s = species[i];
+        if (s < 0 || s >= n_species) { atomicOr(status, FLAG_NONFINITE); s = 0; }
+        p = make_double4(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], (double)s);
+        pos4[i] = p;
+        user[i] = (int32_t)i;
+    } else p = pos4[i];
     bool ok = (p.x >= 0.0 && p.x < g.box[0]) && (p.y >= 0.0 && p.y < g.box[1]) && (p.z >= 0.0 && p.z < g.box[2]);
     if (!ok) atomicOr(status, FLAG_NONFINITE);
     int cx = ok ? cell_coord(p.x, g.inv_edge[0], g.n[0]) : 0;
@@ -51,84 +68,109 @@ __global__ void k_cell_id(const double4 *__restrict__ pos4, int64_t n, CellGrid 
     int cz = ok ? cell_coord(p.z, g.inv_edge[2], g.n[2]) : 0;
     int c = (cx * g.n[1] + cy) * g.n[2] + cz;
     cell_of[i] = c;
-    atomicAdd(&cell_count[c], 1);
+    rank_of[i] = atomicAdd(&cell_count[c], 1);
 }
 
 __global__ void k_place(const int32_t *__restrict__ cell_of, int64_t n, const int32_t *__restrict__ cell_start,
-                        int32_t *__restrict__ cell_fill, int32_t *__restrict__ slot_src) {
+                        const int32_t *__restrict__ rank_of, int32_t *__restrict__ slot_src) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    int c = cell_of[i];
-    slot_src[cell_start[c] + atomicAdd(&cell_fill[c], 1)] = (int32_t)i;
+    slot_src[cell_start[cell_of[i]] + rank_of[i]] = (int32_t)i;
 }
 
-// One thread per cell: order the cell's atoms by (species, caller index) and count them per species.
+// One warp per cell: order the cell's atoms by (species, caller index) -- an atom's place is the number of smaller keys, counted in
+// shared memory -- move them there from the source set (with their fp32 position relative to the cell's lower corner when `rel` is
+// given: |x_rel| < cell edge, so the rounding is ~5e-7 Angstrom whatever the box size), and count the cell's central atoms per
+// species (caller indices below n_owned; the others are ghosts).  One thread per cell with an insertion sort in global memory
+// took 60 to 80 us at any size below 100,000 atoms, and the moves were a pass of their own.
 // A cell holding more than MAX_CELL_ATOMS atoms (a collapsed or diverged configuration: thousands of atoms in a cube of
-// one list radius) is not sorted -- the insertion sort is quadratic in one thread -- and raises FLAG_NONFINITE, which
-// makes the list kernels and the fused kernels that follow return at once.
+// one list radius) is not sorted and raises FLAG_NONFINITE, which makes the list kernels and the fused kernels that follow
+// return at once.
 constexpr int MAX_CELL_ATOMS = 1024;
-__global__ void k_sort_cells(int n_cells, int n_species, const int32_t *__restrict__ cell_start,
-                             int32_t *__restrict__ slot_src, const double4 *__restrict__ pos4_src,
-                             const int32_t *__restrict__ user_src, int32_t *__restrict__ bin_count, int *status, int32_t n_owned) {
-    // (bin_count counts the atoms that will be central atoms: caller indices below n_owned; the others are ghosts)
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n_cells) return;
-    int beg = cell_start[c], end = cell_start[c + 1];
-    int cnt[MAX_SPECIES] = {0};
-    if (end - beg > MAX_CELL_ATOMS) {
-        atomicOr(status, FLAG_NONFINITE);
-        for (int a = beg; a < end; ++a) { const int src = slot_src[a]; cnt[(int)pos4_src[src].w] += user_src[src] < n_owned; }
-        for (int s = 0; s < n_species; ++s) bin_count[(int64_t)s * n_cells + c] = cnt[s];
-        return;
+constexpr int SORT_WARPS = 4;
+__global__ void __launch_bounds__(SORT_WARPS * 32) k_sort_gather(CellGrid g, int n_species, const int32_t *__restrict__ cell_start,
+                                                                 const int32_t *__restrict__ slot_src, const double4 *__restrict__ pos4_src,
+                                                                 const double *__restrict__ vel_src, const int32_t *__restrict__ user_src,
+                                                                 int32_t n_owned, double4 *__restrict__ pos4, double *__restrict__ vel,
+                                                                 int32_t *__restrict__ user_of, float *__restrict__ disp, float4 *__restrict__ rel,
+                                                                 int32_t *__restrict__ cell_id, int32_t *__restrict__ cell_count,
+                                                                 int32_t *__restrict__ bin_count, int *status) {
+    __shared__ __align__(16) int32_t s_keys[SORT_WARPS][MAX_CELL_ATOMS];
+    const int lane = threadIdx.x & 31, c = blockIdx.x * SORT_WARPS + (threadIdx.x >> 5);
+    if (c >= g.n_cells) return;
+    int32_t *keys = s_keys[threadIdx.x >> 5];
+    const int beg = cell_start[c], m = cell_start[c + 1] - beg;
+    const bool sorted = m <= MAX_CELL_ATOMS;
+    if (lane == 0) {
+        cell_count[c] = 0;
+        if (!sorted) atomicOr(status, FLAG_NONFINITE);
     }
-    for (int a = beg; a < end; ++a) {
-        int src = slot_src[a];
-        int sa = (int)pos4_src[src].w;
-        long long key = ((long long)sa << 32) | (unsigned)user_src[src];
-        cnt[sa] += user_src[src] < n_owned;
-        int b = a - 1;
-        while (b >= beg) {
-            int sb_src = slot_src[b];
-            long long kb = ((long long)(int)pos4_src[sb_src].w << 32) | (unsigned)user_src[sb_src];
-            if (kb <= key) break;
-            slot_src[b + 1] = sb_src;
-            --b;
+    const int cz = c % g.n[2], cy = (c / g.n[2]) % g.n[1], cx = c / (g.n[2] * g.n[1]);
+    const double corner[3] = {(double)cx * (g.box[0] / g.n[0]), (double)cy * (g.box[1] / g.n[1]), (double)cz * (g.box[2] / g.n[2])};
+    const int packed = pack_cell(g, c);
+    if (sorted) {
+        for (int a = lane; a < ((m + 3) & ~3); a += 32) {
+            int key = 0x7fffffff;
+            if (a < m) { const int src = slot_src[beg + a]; key = ((int)pos4_src[src].w << 28) | user_src[src]; }
+            keys[a] = key;
         }
-        slot_src[b + 1] = src;
+        __syncwarp();
     }
-    for (int s = 0; s < n_species; ++s) bin_count[(int64_t)s * n_cells + c] = cnt[s];
+    int owned = 0;   // lane s: central atoms of species s
+    for (int base = 0; base < m; base += 32) {
+        const int a = base + lane;
+        int sa = -1;
+        if (a < m) {
+            const int src = slot_src[beg + a];
+            const double4 p = pos4_src[src];
+            const int user = user_src[src];
+            int dst = beg + a;
+            if (sorted) {
+                const int key = ((int)p.w << 28) | user;
+                int rank = 0;
+                for (int q = 0; q < m; q += 4) {
+                    const int4 o = *reinterpret_cast<const int4 *>(keys + q);
+                    rank += (o.x < key) + (o.y < key) + (o.z < key) + (o.w < key);
+                }
+                dst = beg + rank;
+            }
+            pos4[dst] = p;
+            user_of[dst] = user;
+            if (cell_id) cell_id[dst] = packed;   // build-time cell in the internal order (compact lists)
+            if (rel) rel[dst] = make_float4((float)(p.x - corner[0]), (float)(p.y - corner[1]), (float)(p.z - corner[2]), 0.f);
+            for (int q = 0; q < 3; ++q) {
+                vel[3 * (int64_t)dst + q] = vel_src ? vel_src[3 * (int64_t)src + q] : 0.0;
+                disp[3 * (int64_t)dst + q] = 0.f;
+            }
+            if (user < n_owned) sa = (int)p.w;
+        }
+        for (int s = 0; s < n_species; ++s) {
+            const int v = __popc(__ballot_sync(0xffffffffu, sa == s));
+            if (lane == s) owned += v;
+        }
+    }
+    if (lane < n_species) bin_count[(int64_t)lane * g.n_cells + c] = owned;
 }
 
-__global__ void k_gather(int64_t n, const int32_t *__restrict__ slot_src, const double4 *__restrict__ pos4_src,
-                         const double *__restrict__ vel_src, const int32_t *__restrict__ user_src,
-                         double4 *__restrict__ pos4, double *__restrict__ vel, int32_t *__restrict__ user_of,
-                         float *__restrict__ disp, const int32_t *__restrict__ cell_of, int32_t *__restrict__ cell_id, CellGrid g) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int src = slot_src[i];
-    if (cell_id) cell_id[i] = pack_cell(g, cell_of[src]);   // build-time cell of the atom in the internal order (compact lists)
-    pos4[i] = pos4_src[src];
-    user_of[i] = user_src[src];
-    for (int a = 0; a < 3; ++a) {
-        vel[3 * i + a] = vel_src ? vel_src[3 * (int64_t)src + a] : 0.0;
-        disp[3 * i + a] = 0.f;
-    }
-}
-
-// One thread per cell: the cell's atoms (already species-ordered) go to their (species, cell) bins.
-__global__ void k_center_order(int n_cells, int n_species, const int32_t *__restrict__ cell_start,
-                               const double4 *__restrict__ pos4, const int32_t *__restrict__ bin_start,
-                               int32_t *__restrict__ center_order, int32_t *__restrict__ species_start,
-                               const int32_t *__restrict__ user_of, int32_t n_owned) {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c <= n_species) species_start[c] = c < n_species ? bin_start[(int64_t)c * n_cells] : bin_start[(int64_t)n_species * n_cells];
+// One warp per cell: the cell's atoms, already species-ordered, go to their (species, cell) bins; ghosts, which come last within
+// a species, are never central atoms.
+__global__ void __launch_bounds__(128) k_center_order(int n_cells, int n_species, const int32_t *__restrict__ cell_start,
+                                                      const double4 *__restrict__ pos4, const int32_t *__restrict__ bin_start,
+                                                      int32_t *__restrict__ center_order, int32_t *__restrict__ species_start,
+                                                      const int32_t *__restrict__ user_of, int32_t n_owned) {
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x, c = tid >> 5, lane = tid & 31;
+    if (tid <= n_species) species_start[tid] = bin_start[(int64_t)tid * n_cells];
     if (c >= n_cells) return;
-    int beg = cell_start[c], end = cell_start[c + 1];
-    int prev = -1, r = 0;
-    for (int a = beg; a < end; ++a) {
-        int s = (int)pos4[a].w;
-        if (s != prev) { prev = s; r = 0; }
-        if (user_of[a] < n_owned) center_order[bin_start[(int64_t)s * n_cells + c] + r++] = a;   // ghosts are never central atoms
+    const int beg = cell_start[c], end = cell_start[c + 1];
+    int last = -1, run = 0;   // species of the atom before this chunk and the length of its run so far
+    for (int base = beg; base < end; base += 32) {
+        const int a = base + lane;
+        const int s = a < end ? (int)pos4[a].w : MAX_SPECIES;
+        const unsigned same = __match_any_sync(0xffffffffu, s);
+        const int r = __popc(same & ((1u << lane) - 1u)) + (s == last ? run : 0);
+        if (a < end && user_of[a] < n_owned) center_order[bin_start[(int64_t)s * n_cells + c] + r] = a;
+        last = __shfl_sync(0xffffffffu, s, 31);
+        run = __shfl_sync(0xffffffffu, r, 31) + 1;
     }
 }
 
@@ -230,25 +272,9 @@ __global__ void __launch_bounds__(256) k_neighbors(int64_t n, CellGrid g, double
     if (!FILL && lane == 0) { nbr_count[i] = cnt; nbr_near[i] = cn; }
 }
 
-// Positions relative to the lower corner of the atom's own cell, in fp32 (|x_rel| < cell edge, so the rounding is ~5e-7
-// Angstrom whatever the box size).  Lives in the force array, which is idle during a build.
-__global__ void k_rel_pos(int64_t n, CellGrid g, const double4 *__restrict__ pos4, float4 *__restrict__ rel) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double4 p = pos4[i];
-    const double x[3] = {p.x, p.y, p.z};
-    float r[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int c = cell_coord(x[a], g.inv_edge[a], g.n[a]);
-        r[a] = (float)(x[a] - (double)c * (g.box[a] / g.n[a]));
-    }
-    rel[i] = make_float4(r[0], r[1], r[2], 0.f);
-}
-
 // The same traversal for grids with at least three cells per dimension, on the cell-relative fp32 positions: the
 // separation is x_rel(j) - x_rel(i) + (cell offset) * edge -- the cell offset already names the periodic image, so no
-// minimum-image step and no fp64 arithmetic per candidate.  Candidates within 1e-5 of the list radius (the fp32 distance is
+// minimum-image step and no fp64 arithmetic per candidate (the positions live in the force array, idle during a build).  Candidates within 1e-5 of the list radius (the fp32 distance is
 // good to ~1e-6) are decided by the exact fp64 predicate on the full positions, so the lists are the same bit for bit.
 template <bool FILL, typename OUT>
 __global__ void __launch_bounds__(256) k_neighbors_rel(int64_t n, CellGrid g, double rl2, const double4 *__restrict__ pos4,
@@ -336,17 +362,16 @@ __global__ void __launch_bounds__(256) k_neighbors_rel(int64_t n, CellGrid g, do
     if (!FILL && lane == 0) { nbr_count[i] = cnt; nbr_near[i] = cn; }
 }
 
-// ---- one-pass variant for in-step rebuilds ----
-// Count and fill in a single traversal: a CTA takes a tile of 64 consecutive atoms (8 per warp), collects each atom's hits
+// ---- one-pass variant ----
+// Count and fill in a single traversal: a CTA takes a tile of 64 consecutive atoms (8 per warp; 8 atoms, one per warp, in small
+// systems, where eight traversals one after the other are the kernel's time), collects each atom's hits
 // in shared memory while it counts, obtains the tile's list offset from a decoupled look-back scan over the tiles before
 // it (tile aggregate / inclusive prefix published in one 64-bit word, tiles handed out by a ticket so that every
 // predecessor belongs to a CTA that is already running), and then copies the lists out in full rows.  Offsets are the same exclusive prefix sums the two-pass build produces, so the lists are identical.
 // Every wait is bounded: after `spin_limit` polls (OP_SPIN in production) the tile raises FLAG_NEIGHBOR_OVERFLOW, publishes
 // what it has and goes on.  Offsets are clamped to the capacity and a list that crosses it is cut short, so whatever the
 // outcome every [nbr_off[i], nbr_off[i+1]) lies inside the array and holds atom indices.
-constexpr int OP_PER_WARP = 8;
-constexpr int OP_TILE = 8 * OP_PER_WARP;
-static_assert(OP_TILE == 64, "the in-tile scan handles two counts per lane of one warp");
+constexpr int OP_TILE = 64;   // largest tile: the in-tile scan handles two counts per lane of one warp
 constexpr int OP_SPIN = 1 << 18;
 
 __device__ __forceinline__ bool rel_hit(const float4 &rj, float sx, float sy, float sz, float rl2_lo, float rl2_hi, double rl2,
@@ -362,7 +387,21 @@ __device__ __forceinline__ bool rel_hit(const float4 &rj, float sx, float sy, fl
     return __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez)) < rl2;
 }
 
-// atom ranges of the 27 cells around position p, one cell per lane (lanes 27.. get an empty range)
+// The same decision on the full positions: fp32 screen after the minimum image, exact predicate near the list radius.
+__device__ __forceinline__ bool full_hit(const double4 &pj, const double4 &pi, float rl2_lo, float rl2_hi, double rl2, const CellGrid &g, float &d2f) {
+    const double ex = min_image(__dsub_rn(pj.x, pi.x), g.box[0], g.half[0]);
+    const double ey = min_image(__dsub_rn(pj.y, pi.y), g.box[1], g.half[1]);
+    const double ez = min_image(__dsub_rn(pj.z, pi.z), g.box[2], g.half[2]);
+    const float fx = (float)ex, fy = (float)ey, fz = (float)ez;
+    d2f = fx * fx + fy * fy + fz * fz;
+    if (d2f < rl2_lo) return true;
+    if (d2f > rl2_hi) return false;
+    return __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez)) < rl2;
+}
+
+// atom ranges of the 27 cells around position p, one cell per lane (lanes 27.. get an empty range); !REL: a dimension with fewer
+// than three cells lists each of them once
+template <bool REL>
 __device__ __forceinline__ void cell_ranges(const double4 &p4, const CellGrid &g, const int32_t *__restrict__ cell_start, int lane,
                                             int &cb, int &ce) {
     cb = 0; ce = 0;
@@ -370,12 +409,15 @@ __device__ __forceinline__ void cell_ranges(const double4 &p4, const CellGrid &g
         const int o[3] = {lane / 9, (lane / 3) % 3, lane % 3};
         const double p[3] = {p4.x, p4.y, p4.z};
         int cc[3];
+        bool ok = true;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const int na = g.n[a];
             int c = cell_coord(p[a], g.inv_edge[a], na) + o[a] - 1;
             cc[a] = c < 0 ? c + na : (c >= na ? c - na : c);
+            if (!REL && na < 3) { cc[a] = o[a]; ok = ok && o[a] < na; }
         }
+        if (!ok) return;
         const int c = (cc[0] * g.n[1] + cc[1]) * g.n[2] + cc[2];
         cb = cell_start[c]; ce = cell_start[c + 1];
     }
@@ -385,17 +427,43 @@ __device__ __forceinline__ void cell_ranges(const double4 &p4, const CellGrid &g
 // out[top - 1], ...; only positions below `limit` are written.  Shared-memory pass: top = capacity - 1 (if the list is
 // longer than the buffer the two ends collide and the list is traversed again); global pass: top = list length - 1.
 // Returns the number of hits, and the number of near hits in `n_near`.
-template <typename OUT, typename ENTRY>
+// REL = false: grids with fewer than three cells in a dimension, on the full positions with the minimum image (as k_neighbors).
+template <bool REL, typename OUT, typename ENTRY>
 __device__ __forceinline__ int onepass_traverse(int64_t i, const CellGrid &g, double rl2, const float (&edge)[3], float rl2_lo, float rl2_hi,
                                                 const double4 *__restrict__ pos4, const float4 *__restrict__ rel,
                                                 const int32_t *__restrict__ cell_start, int lane, OUT *out, int top, int limit,
                                                 float near2, int &n_near) {
     // OUT = type of the buffer written here (int32 in shared memory), ENTRY = format of the list (int32 or uint16)
     const double4 pi = pos4[i];
-    const float4 ri = rel[i];
+    float4 ri = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (REL) ri = rel[i];
     int cb, ce;
-    cell_ranges(pi, g, cell_start, lane, cb, ce);
+    cell_ranges<REL>(pi, g, cell_start, lane, cb, ce);
     int cnt = 0, cn = 0;
+    auto take = [&](bool hit, float d2f, int j, int it, int cell_beg) {
+        const bool near = hit && d2f < near2;
+        const unsigned m = __ballot_sync(0xffffffffu, hit), mn = __ballot_sync(0xffffffffu, near), below = (1u << lane) - 1u;
+        const int slot = near ? cn + __popc(mn & below) : top - (cnt - cn + __popc(m & ~mn & below));
+        if (hit && slot >= 0 && slot < limit) out[slot] = (OUT)list_entry<ENTRY>(j, it, cell_beg);
+        cnt += __popc(m);
+        cn += __popc(mn);
+    };
+    if (!REL) {
+        const unsigned cells = __ballot_sync(0xffffffffu, ce > cb);
+        for (unsigned left = cells; left; left &= left - 1) {   // (up to 27 cells, each once)
+            const int it = __ffs(left) - 1;
+            const int beg = __shfl_sync(0xffffffffu, cb, it), end = __shfl_sync(0xffffffffu, ce, it);
+#pragma unroll 4
+            for (int base = beg; base < end; base += 32) {
+                const int j = base + lane;
+                float d2f = 0.f;
+                const bool hit = j < end && j != i && full_hit(pos4[j < end ? j : beg], pi, rl2_lo, rl2_hi, rl2, g, d2f);
+                take(hit, d2f, j, it, beg);
+            }
+        }
+        n_near = cn;
+        return cnt;
+    }
     int beg = __shfl_sync(0xffffffffu, cb, 0), end = __shfl_sync(0xffffffffu, ce, 0);
     float4 rj_next = make_float4(0.f, 0.f, 0.f, 0.f);
     if (beg + lane < end) rj_next = rel[beg + lane];
@@ -416,25 +484,21 @@ __device__ __forceinline__ int onepass_traverse(int64_t i, const CellGrid &g, do
             if (base != cur_beg && j < cur_end) rj = rel[j];
             float d2f = 0.f;
             const bool hit = j < cur_end && j != i && rel_hit(rj, sx, sy, sz, rl2_lo, rl2_hi, rl2, pi, pos4, j, g, d2f);
-            const bool near = hit && d2f < near2;
-            const unsigned m = __ballot_sync(0xffffffffu, hit), mn = __ballot_sync(0xffffffffu, near), below = (1u << lane) - 1u;
-            const int slot = near ? cn + __popc(mn & below) : top - (cnt - cn + __popc(m & ~mn & below));
-            if (hit && slot >= 0 && slot < limit) out[slot] = (OUT)list_entry<ENTRY>(j, it, cur_beg);
-            cnt += __popc(m);
-            cn += __popc(mn);
+            take(hit, d2f, j, it, cur_beg);
         }
     }
     n_near = cn;
     return cnt;
 }
 
+constexpr int64_t ONEPASS_SMALL = 50000;   // see onepass_per_warp
 constexpr int OP_BUF = 160;   // hits kept per atom in shared memory; a longer list is traversed again straight into global memory
 
-template <typename ENTRY>
+template <bool REL, int PER_WARP, typename ENTRY>
 __global__ void __launch_bounds__(256) k_neighbors_onepass(int64_t n, CellGrid g, double rl2, const double4 *__restrict__ pos4,
                                                            const float4 *__restrict__ rel, const int32_t *__restrict__ cell_start,
                                                            int64_t *__restrict__ nbr_off, ENTRY *__restrict__ nbr, int64_t nbr_cap,
-                                                           int *status, unsigned long long *tile_state, int *ticket,
+                                                           int *status, unsigned long long *tile_state, int *build_word,
                                                            const int *global_status, int spin_limit, long long unpublished_tile,
                                                            float near2, int32_t *__restrict__ nbr_near,
                                                            const int32_t *__restrict__ user_of, int32_t n_owned) {
@@ -443,32 +507,33 @@ __global__ void __launch_bounds__(256) k_neighbors_onepass(int64_t n, CellGrid g
     if (*global_status & FLAG_NONFINITE) return;   // a broken configuration is not traversed (see k_sort_cells)
     // look-back word: flag in the top two bits (0 empty, 1 tile aggregate, 2 inclusive prefix), value below
     constexpr unsigned long long OP_AGG = 1ull << 62, OP_INC = 2ull << 62, OP_VAL = (1ull << 62) - 1;
-    extern __shared__ int32_t s_hits[];   // [OP_TILE][OP_BUF]
+    constexpr int TILE_ATOMS = 8 * PER_WARP;
+    extern __shared__ int32_t s_hits[];   // [TILE_ATOMS][OP_BUF]
     __shared__ int s_cnt[OP_TILE], s_near[OP_TILE];
     __shared__ long long s_off[OP_TILE];
     __shared__ long long s_prefix, s_total;
     __shared__ int s_tile;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1);
+    if (threadIdx.x == 0) s_tile = atomicAdd(build_word, 1);
     __syncthreads();
-    const int64_t tile = s_tile, first = tile * OP_TILE;
+    const int64_t tile = s_tile, first = tile * TILE_ATOMS;
     const float edge[3] = {(float)(g.box[0] / g.n[0]), (float)(g.box[1] / g.n[1]), (float)(g.box[2] / g.n[2])};
     const float rl2_lo = (float)(rl2 * (1.0 - 1e-5)), rl2_hi = (float)(rl2 * (1.0 + 1e-5));
 
     // ---- traversal: count, keep the hits ----
-    for (int a = 0; a < OP_PER_WARP; ++a) {
-        const int slot = warp * OP_PER_WARP + a;
+    for (int a = 0; a < PER_WARP; ++a) {
+        const int slot = warp * PER_WARP + a;
         const int64_t i = first + slot;
         int cnt = 0, cn = 0;
         if (i < n && user_of[i] < n_owned)   // (a ghost has no list of its own)
-            cnt = onepass_traverse<int32_t, ENTRY>(i, g, rl2, edge, rl2_lo, rl2_hi, pos4, rel, cell_start, lane, s_hits + slot * OP_BUF, OP_BUF - 1, OP_BUF, near2, cn);
+            cnt = onepass_traverse<REL, int32_t, ENTRY>(i, g, rl2, edge, rl2_lo, rl2_hi, pos4, rel, cell_start, lane, s_hits + slot * OP_BUF, OP_BUF - 1, OP_BUF, near2, cn);
         if (lane == 0) { s_cnt[slot] = cnt; s_near[slot] = cn; }
     }
     __syncthreads();
 
     // ---- offsets: scan inside the tile, look back over the tiles before it ----
     if (warp == 0) {
-        const int c0 = s_cnt[2 * lane], c1 = s_cnt[2 * lane + 1];
+        const int c0 = 2 * lane < TILE_ATOMS ? s_cnt[2 * lane] : 0, c1 = 2 * lane < TILE_ATOMS ? s_cnt[2 * lane + 1] : 0;
         long long incl = c0 + c1;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -513,11 +578,14 @@ __global__ void __launch_bounds__(256) k_neighbors_onepass(int64_t n, CellGrid g
     }
     __syncthreads();
     const long long tile_off = s_prefix;
-    if (first + OP_TILE >= n && threadIdx.x == 0) nbr_off[n] = s_total < nbr_cap ? s_total : nbr_cap;   // the last tile closes the offsets
+    if (first + TILE_ATOMS >= n && threadIdx.x == 0) {   // the last tile closes the offsets
+        nbr_off[n] = s_total < nbr_cap ? s_total : nbr_cap;
+        *reinterpret_cast<long long *>(build_word + 2) = s_total;   // for the host: {ticket, overflow, total}
+    }
 
     // ---- write the lists: full rows from shared memory ----
-    for (int a = 0; a < OP_PER_WARP; ++a) {
-        const int slot = warp * OP_PER_WARP + a;
+    for (int a = 0; a < PER_WARP; ++a) {
+        const int slot = warp * PER_WARP + a;
         const int64_t i = first + slot;
         if (i >= n) break;
         const long long off = tile_off + s_off[slot];
@@ -535,7 +603,7 @@ __global__ void __launch_bounds__(256) k_neighbors_onepass(int64_t n, CellGrid g
             for (int e = lane; e < fit; e += 32) nbr[off + e] = (ENTRY)src[e < near ? e : e + (OP_BUF - cnt)];
         } else {
             int cn;
-            onepass_traverse<ENTRY, ENTRY>(i, g, rl2, edge, rl2_lo, rl2_hi, pos4, rel, cell_start, lane, nbr + off, cnt - 1, fit, near2, cn);
+            onepass_traverse<REL, ENTRY, ENTRY>(i, g, rl2, edge, rl2_lo, rl2_hi, pos4, rel, cell_start, lane, nbr + off, cnt - 1, fit, near2, cn);
         }
     }
 }
@@ -635,13 +703,6 @@ static ListView list_view(const mlip_ctx *c) {
     return lv;
 }
 
-int launch_pack_source(mlip_ctx *c, const double *pos, const int32_t *species, cudaStream_t s) {
-    k_pack_source<<<blocks_for(c->n, 256), 256, 0, s>>>(pos, species, c->n, c->cfg.n_species, c->pos4_src, c->user_src, c->status);
-    c->launches += 1;
-    MLIP_CUDA_TRY(c, cudaGetLastError());
-    return MLIP_OK;
-}
-
 // A synchronising build that met a non-finite or out-of-box position, a species out of range or an over-full cell: the
 // list kernels have not run, so there is nothing to size a list from.  Reports it now and clears the flag.
 static int refuse_broken_input(mlip_ctx *c, cudaStream_t s) {
@@ -651,8 +712,30 @@ static int refuse_broken_input(mlip_ctx *c, cudaStream_t s) {
     return MLIP_ERR_NONFINITE;
 }
 
-// Sort (pos4_src, vel_src, user_src) into cell order and build the lists.
-int launch_build(mlip_ctx *c, bool allow_sync_grow, cudaStream_t s) {
+int64_t tile_words(int64_t n) { return std::max(n / OP_TILE, std::min(n, ONEPASS_SMALL) / 8) + 2; }
+
+// Atoms per warp of the one-pass traversal (tiles of eight warps): one in small systems, where eight traversals one after the other
+// are the kernel's time, eight once such tiles fill the SMs two waves deep (five CTAs each) and fewer tiles are the better choice.  Whole
+// build on the device in us with 1 / 8, 6 species: 864 atoms 65 / 126, 6,912 88 / 136, 16,384 132 / 148, 32,000 202 / 198, 55,296 299 /
+// 337, 87,808 453 / 477, 131,072 643 / 621, 1,048,576 4842 / 4030; one species: 4,394 66 / 116, 65,536 301 / 272.
+static int onepass_per_warp(const mlip_ctx *c) {
+    if (c->lookback_unpublished_tile >= 0 || c->lookback_spin_limit > 0) return 8;   // (diagnostics name 64-atom tiles)
+    return c->n < ONEPASS_SMALL ? 1 : 8;
+}
+
+template <bool REL, int PER_WARP, typename ENTRY>
+static void launch_onepass(mlip_ctx *c, ENTRY *nbr, int *flag, double rl, float near2, cudaStream_t s) {
+    const int spin = c->lookback_spin_limit > 0 ? c->lookback_spin_limit : OP_SPIN;
+    const int64_t n_tiles = (c->n + 8 * PER_WARP - 1) / (8 * PER_WARP);
+    k_neighbors_onepass<REL, PER_WARP, ENTRY><<<(unsigned)n_tiles, 256, sizeof(int32_t) * 8 * PER_WARP * OP_BUF, s>>>(
+        c->n, c->grid, rl * rl, c->pos4, c->force, c->cell_start, c->nbr_off, nbr, c->nbr_cap, flag, c->tile_state, c->build_word, c->status, spin,
+        c->lookback_unpublished_tile, near2, c->nbr_near, c->user_of, (int32_t)c->n_owned);
+    c->launches += 1;
+}
+
+// Sort the source set into cell order and build the lists.  The source is (pos4_src, vel_src, user_src), filled from the caller's
+// arrays first when `pos` is given (velocities then start at zero).
+int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int32_t *species, cudaStream_t s) {
     timing_begin(c->ev_build, c->build_count, s);
     const int64_t n = c->n;
     const CellGrid &g = c->grid;
@@ -662,22 +745,24 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, cudaStream_t s) {
     // before some atom has moved skin / 4, and the fused kernels skip them until then (far_flag, raised by the integrator)
     const double rn = c->cfg.r_cut + 0.5 * c->cfg.skin;
     const float near2 = c->cfg.skin > 0.0 ? (float)(rn * rn * (1.0 + 1e-5)) : 3.0e38f;
-    MLIP_CUDA_TRY(c, cudaMemsetAsync(c->far_flag, 0, sizeof(int), s));
-    MLIP_CUDA_TRY(c, cudaMemsetAsync(c->cell_count, 0, sizeof(int32_t) * (g.n_cells + 1), s));
-    MLIP_CUDA_TRY(c, cudaMemsetAsync(c->cell_fill, 0, sizeof(int32_t) * (g.n_cells + 1), s));
-    k_cell_id<<<blocks_for(n, 256), 256, 0, s>>>(c->pos4_src, n, g, c->cell_of, c->cell_count, c->status);
-    exclusive_scan<int32_t, int32_t>(c->cell_count, c->cell_start, g.n_cells, c->scan_tmp, s);
-    // nbr_count doubles as the slot -> source map until the lists are counted
-    int32_t *slot_src = c->nbr_count;
-    k_place<<<blocks_for(n, 256), 256, 0, s>>>(c->cell_of, n, c->cell_start, c->cell_fill, slot_src);
-    k_sort_cells<<<blocks_for(g.n_cells, 128), 128, 0, s>>>(g.n_cells, C, c->cell_start, slot_src, c->pos4_src, c->user_src, c->bin_count, c->status, (int32_t)c->n_owned);
-    k_gather<<<blocks_for(n, 256), 256, 0, s>>>(n, slot_src, c->pos4_src, c->vel_src, c->user_src, c->pos4, c->vel, c->user_of, c->disp, c->cell_of, c->cell_id, g);
-    exclusive_scan<int32_t, int32_t>(c->bin_count, c->bin_start, (int64_t)C * g.n_cells, c->scan_tmp, s);
-    int nthreads_co = g.n_cells > C + 1 ? g.n_cells : C + 1;
-    k_center_order<<<blocks_for(nthreads_co, 128), 128, 0, s>>>(g.n_cells, C, c->cell_start, c->pos4, c->bin_start, c->center_order, c->species_start, c->user_of, (int32_t)c->n_owned);
     // grids of at least 3 x 3 x 3 cells take the fp32 cell-relative traversal (positions staged in the idle force array)
     const bool rel = g.n[0] >= 3 && g.n[1] >= 3 && g.n[2] >= 3;
     float4 *relpos = c->force;
+    const int per_warp = onepass_per_warp(c);
+    const BuildClear clear{c->tile_state, (n + 8 * per_warp - 1) / (8 * per_warp), c->build_word, c->far_flag, c->rebuild_flag};
+    // scratch: overwritten further down whatever the outcome (nbr_near must not hold scratch: it bounds reads of a list that a
+    // broken configuration leaves as it was)
+    int32_t *rank_of = c->center_order, *slot_src = c->nbr_count;
+    if (pos) k_cell_id<true><<<blocks_for(n, 256), 256, 0, s>>>(pos, species, C, c->pos4_src, c->user_src, n, g, c->cell_of, rank_of, c->cell_count, c->status, clear);
+    else k_cell_id<false><<<blocks_for(n, 256), 256, 0, s>>>(nullptr, nullptr, C, c->pos4_src, c->user_src, n, g, c->cell_of, rank_of, c->cell_count, c->status, clear);
+    int n_launches = exclusive_scan<int32_t, int32_t>(c->cell_count, c->cell_start, g.n_cells, c->scan_tmp, s);
+    k_place<<<blocks_for(n, 256), 256, 0, s>>>(c->cell_of, n, c->cell_start, rank_of, slot_src);
+    k_sort_gather<<<blocks_for(g.n_cells, SORT_WARPS), SORT_WARPS * 32, 0, s>>>(g, C, c->cell_start, slot_src, c->pos4_src, pos ? nullptr : c->vel_src, c->user_src,
+                                                                               (int32_t)c->n_owned, c->pos4, c->vel, c->user_of, c->disp, rel ? relpos : nullptr,
+                                                                               c->cell_id, c->cell_count, c->bin_count, c->status);
+    n_launches += exclusive_scan<int32_t, int32_t>(c->bin_count, c->bin_start, (int64_t)C * g.n_cells, c->scan_tmp, s);
+    k_center_order<<<blocks_for((int64_t)g.n_cells * 32, 128), 128, 0, s>>>(g.n_cells, C, c->cell_start, c->pos4, c->bin_start, c->center_order, c->species_start, c->user_of, (int32_t)c->n_owned);
+    c->launches += n_launches + 4;
     // entry format of this build: 16-bit cell-relative codes if asked for and the grid has 27 distinct cells around every
     // cell, else plain indices.  A change of format gives up the old array (its capacity is counted in entries).
     const bool list16 = c->cfg.list_format == 1 && rel && std::max(g.n[0], std::max(g.n[1], g.n[2])) <= CELL_PACK_MAX;
@@ -691,35 +776,22 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, cudaStream_t s) {
     uint16_t *nbr16 = reinterpret_cast<uint16_t *>(c->nbr);
     // Single traversal whenever a list array exists: always for in-step rebuilds (capacity as it stands, overflow -> status
     // bit), and for a synchronising build as a first try whose overflow flag is private and sends it to the two-pass path.
-    bool rel_ready = false;
-    if (rel && c->tile_state && c->nbr_cap > 0) {
-        const int64_t n_tiles = (n + OP_TILE - 1) / OP_TILE;
-        MLIP_CUDA_TRY(c, cudaMemsetAsync(c->tile_state, 0, sizeof(unsigned long long) * (n_tiles + 1), s));
-        MLIP_CUDA_TRY(c, cudaMemsetAsync(c->tile_ticket, 0, 2 * sizeof(int), s));
-        k_rel_pos<<<blocks_for(n, 256), 256, 0, s>>>(n, g, c->pos4, relpos);
-        rel_ready = true;
-        int *flag = allow_sync_grow ? c->tile_ticket + 1 : c->status;
-        const int spin = c->lookback_spin_limit > 0 ? c->lookback_spin_limit : OP_SPIN;
-        if (list16)
-            k_neighbors_onepass<uint16_t><<<(unsigned)n_tiles, 256, sizeof(int32_t) * OP_TILE * OP_BUF, s>>>(
-                n, g, rl * rl, c->pos4, relpos, c->cell_start, c->nbr_off, nbr16, c->nbr_cap, flag, c->tile_state, c->tile_ticket, c->status, spin,
-                c->lookback_unpublished_tile, near2, c->nbr_near, c->user_of, (int32_t)c->n_owned);
-        else
-            k_neighbors_onepass<int32_t><<<(unsigned)n_tiles, 256, sizeof(int32_t) * OP_TILE * OP_BUF, s>>>(
-                n, g, rl * rl, c->pos4, relpos, c->cell_start, c->nbr_off, c->nbr, c->nbr_cap, flag, c->tile_state, c->tile_ticket, c->status, spin,
-                c->lookback_unpublished_tile, near2, c->nbr_near, c->user_of, (int32_t)c->n_owned);
-        c->launches += 5 + 2 * 3 + 2;   // cell id, place, sort, gather, centre order; two scans; relative positions, lists
+    if (c->nbr_cap > 0) {
+        int *flag = allow_sync_grow ? c->build_word + 1 : c->status;
+        if (list16) per_warp == 1 ? launch_onepass<true, 1, uint16_t>(c, nbr16, flag, rl, near2, s) : launch_onepass<true, 8, uint16_t>(c, nbr16, flag, rl, near2, s);
+        else if (rel) per_warp == 1 ? launch_onepass<true, 1, int32_t>(c, c->nbr, flag, rl, near2, s) : launch_onepass<true, 8, int32_t>(c, c->nbr, flag, rl, near2, s);
+        else per_warp == 1 ? launch_onepass<false, 1, int32_t>(c, c->nbr, flag, rl, near2, s) : launch_onepass<false, 8, int32_t>(c, c->nbr, flag, rl, near2, s);
         MLIP_CUDA_TRY(c, cudaGetLastError());
         bool done = true;
         if (allow_sync_grow) {
-            int overflow = 0;
-            MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->total_host, c->nbr_off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-            MLIP_CUDA_TRY(c, cudaMemcpyAsync(&overflow, c->tile_ticket + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
-            MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->status_host, c->status, sizeof(int), cudaMemcpyDeviceToHost, s));
+            // {ticket, overflow, total, status} are neighbors in memory: one copy
+            MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->build_host, c->build_word, sizeof(int) * 5, cudaMemcpyDeviceToHost, s));
             MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
-            if (*c->status_host & FLAG_NONFINITE) return refuse_broken_input(c, s);
-            done = overflow == 0 && *c->total_host < c->nbr_cap;   // the kernel clamps the total to the capacity
-            if (done) c->n_entries = *c->total_host;
+            if (c->build_host[4] & FLAG_NONFINITE) return refuse_broken_input(c, s);
+            int64_t total;
+            memcpy(&total, c->build_host + 2, sizeof total);
+            done = c->build_host[1] == 0 && total <= c->nbr_cap;
+            if (done) c->n_entries = total;
         }
         if (done) {
             timing_end(c->ev_build, c->build_count, s);
@@ -727,13 +799,10 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, cudaStream_t s) {
         }
     }
     if (rel) {
-        if (!rel_ready) k_rel_pos<<<blocks_for(n, 256), 256, 0, s>>>(n, g, c->pos4, relpos);
         k_neighbors_rel<false, int32_t><<<blocks_for(n * 32, 256), 256, 0, s>>>(n, g, rl * rl, c->pos4, relpos, c->cell_start, c->nbr_count, nullptr, nullptr, 0, c->status, near2, c->nbr_near, c->user_of, (int32_t)c->n_owned);
-        c->launches += 1;
     } else
         k_neighbors<false><<<blocks_for(n * 32, 256), 256, 0, s>>>(n, g, rl * rl, c->pos4, c->cell_start, c->nbr_count, nullptr, nullptr, 0, c->status, near2, c->nbr_near, c->user_of, (int32_t)c->n_owned);
-    exclusive_scan<int32_t, int64_t>(c->nbr_count, c->nbr_off, n, c->scan_tmp, s);
-    c->launches += 5 + 1 + 3 * 3;   // cell id, place, sort, gather, centre order; count; three scans
+    c->launches += 1 + exclusive_scan<int32_t, int64_t>(c->nbr_count, c->nbr_off, n, c->scan_tmp, s);
     MLIP_CUDA_TRY(c, cudaGetLastError());
     if (allow_sync_grow) {
         MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->total_host, c->nbr_off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
@@ -778,10 +847,9 @@ static int export_lists(mlip_ctx *c, int64_t *seg_ptr, int32_t *nbr, int64_t cap
     const int C = c->cfg.n_species;
     k_export_keys<<<blocks_for(n, 256), 256, 0, s>>>(n, c->pos4, c->user_of, c->cell_of);
     k_export_count<<<blocks_for(n * 32, 256), 256, 0, s>>>(n, C, c->nbr_off, list_view(c), c->cell_of, seg_count);
-    exclusive_scan<int32_t, int64_t>(seg_count, seg_ptr, n * C, tmp, s);
+    c->launches += 2 + exclusive_scan<int32_t, int64_t>(seg_count, seg_ptr, n * C, tmp, s);
     MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->total_host, seg_ptr + n * C, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
-    c->launches += 5;
     if (n_entries_host) *n_entries_host = *c->total_host;
     if (*c->total_host > capacity || !nbr) {
         c->err = "neighbor export: capacity too small";
