@@ -323,9 +323,9 @@ class Potential:
         """Per-atom outputs are float32, or float64 on a context created with precision=1."""
         t = self.torch
         real = t.float64 if self.precision == 1 else t.float32
-        out = {"energy": t.zeros(1, dtype=t.float64, device=self.device),
+        out = {"energy": t.empty(1, dtype=t.float64, device=self.device),
                "forces": t.empty((self.n, 3), dtype=real, device=self.device),
-               "virial": t.zeros(9, dtype=t.float64, device=self.device),
+               "virial": t.empty(9, dtype=t.float64, device=self.device),
                "e_atom": t.empty(self.n, dtype=real, device=self.device) if want_e_atom else None}
         call = mlip_compute_f64 if self.precision == 1 else mlip_compute
         call(self.ctx, out["energy"], out["forces"], out["virial"], out["e_atom"])
@@ -371,7 +371,7 @@ class Potential:
 
     def energies(self):
         t = self.torch
-        e = t.zeros(2, dtype=t.float64, device=self.device)
+        e = t.empty(2, dtype=t.float64, device=self.device)
         mlip_get_energies(self.ctx, e[0:1], e[1:2])
         return e
 

@@ -1,5 +1,6 @@
 // C ABI (include/mlip.h): context life cycle, buffer management and the host-side
 // sequencing of the kernels.  No torch types, no exceptions across the boundary.
+#include <algorithm>
 #include <math.h>
 #include <new>
 #include <string.h>
@@ -75,7 +76,11 @@ static int ensure_capacity(mlip_ctx *c, int64_t n, int64_t n_cells) {
         TRY_ALLOC(c->center_order, m); TRY_ALLOC(c->cell_of, m);
         TRY_ALLOC(c->nbr_count, m); TRY_ALLOC(c->nbr_near, m); TRY_ALLOC(c->nbr_off, m + 1);
         if (c->cfg.precision == 1) { TRY_ALLOC(c->force_d, 3 * m); TRY_ALLOC(c->e_atom_d, m); }
-        if (c->cfg.force_mode == 1) TRY_ALLOC(c->force_fx, 3 * m);
+        if (c->cfg.force_mode == 1) {
+            TRY_ALLOC(c->force_fx, 3 * m);
+            MLIP_CUDA_TRY(c, cudaMemset(c->force_fx, 0, sizeof(long long) * 3 * m));   // zero between evaluations from here on
+            MLIP_CUDA_TRY(c, cudaStreamSynchronize(nullptr));
+        }
         TRY_ALLOC(c->tile_state, (size_t)tile_words(n));
         if (c->cfg.list_format == 1) TRY_ALLOC(c->cell_id, m);
         c->cap_atoms = n;
@@ -252,7 +257,7 @@ int mlip_create(mlip_ctx **out, const mlip_config *cfg, const double *enc_w, siz
         if ((rc = dev_alloc(c, &c->nhc, 8)) != MLIP_OK) break;
         if ((rc = dev_alloc(c, &c->species_start, (size_t)MAX_SPECIES + 1)) != MLIP_OK) break;
         if ((rc = dev_alloc(c, &c->stage_out, 10)) != MLIP_OK) break;
-        if ((rc = dev_alloc(c, &c->kin_part, 1184)) != MLIP_OK) break;
+        if ((rc = dev_alloc(c, &c->kin_part, 1185)) != MLIP_OK) break;
         if (cudaMallocHost((void **)&c->status_host, sizeof(int)) != cudaSuccess ||
             cudaMallocHost((void **)&c->total_host, sizeof(int64_t)) != cudaSuccess ||
             cudaMallocHost((void **)&c->rebuild_host, sizeof(int)) != cudaSuccess ||
@@ -260,13 +265,11 @@ int mlip_create(mlip_ctx **out, const mlip_config *cfg, const double *enc_w, siz
             rc = MLIP_ERR_CUDA; c->err = "pinned host allocation failed"; break;
         }
         bool ev_ok = true;
-        for (int q = 0; q < 2 * mlip_ctx::EV_POOL; ++q)
-            ev_ok = ev_ok && cudaEventCreate(&c->ev[q]) == cudaSuccess && cudaEventCreate(&c->ev_build[q]) == cudaSuccess &&
-                    cudaEventCreate(&c->ev_integrate[q]) == cudaSuccess;
+        for (int q = 0; q < mlip_ctx::MARKS; ++q) ev_ok = ev_ok && cudaEventCreate(&c->mark_ev[q]) == cudaSuccess;
         if (!ev_ok) { rc = MLIP_ERR_CUDA; c->err = "event creation failed"; break; }
         if (cudaMemcpy(c->mass, mass, sizeof(double) * cfg->n_species, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemset(c->build_word, 0, sizeof(int) * 8) != cudaSuccess ||
-            cudaMemset(c->nhc, 0, sizeof(double) * 8) != cudaSuccess || cudaMemset(c->launch_block, 0, sizeof(double) * LB_COUNT) != cudaSuccess) {
+            cudaMemset(c->nhc, 0, sizeof(double) * 8) != cudaSuccess || cudaMemset(c->kin_part, 0, sizeof(double) * 1185) != cudaSuccess || cudaMemset(c->launch_block, 0, sizeof(double) * LB_COUNT) != cudaSuccess) {
             rc = MLIP_ERR_CUDA; c->err = "initial upload failed"; break;
         }
         rc = build_tables(c, enc_w, n_enc);
@@ -308,6 +311,7 @@ int mlip_build_neighbors_ghost(mlip_ctx *c, int64_t n_owned, int64_t n_ghost, co
     if (n > (1LL << 28)) return fail(c, MLIP_ERR_UNSUPPORTED, "more than 2^28 atoms per context (the pair queue packs index and species in 32 bits)");
     cudaStream_t s = (cudaStream_t)stream;
     c->last_stream = s;
+    c->mark_open = false;
     cudaSetDevice(c->cfg.device);
     double edges[3];
     int rc = box_edges(c, box, edges);
@@ -368,12 +372,11 @@ int mlip_compute_f64(mlip_ctx *c, double *energy, double *forces, double *virial
     if (!c->built) return fail(c, MLIP_ERR_NOT_BUILT, "no neighbor lists yet");
     cudaStream_t s = (cudaStream_t)stream;
     c->last_stream = s;
+    c->mark_open = false;
     int rc = launch_megakernel_f64(c, s);
     if (rc != MLIP_OK) return rc;
     c->forces_current = true;
-    if (energy) MLIP_CUDA_TRY(c, cudaMemcpyAsync(energy, c->acc + ACC_ENERGY, sizeof(double), cudaMemcpyDeviceToDevice, s));
-    if (virial) MLIP_CUDA_TRY(c, cudaMemcpyAsync(virial, c->acc + ACC_VIRIAL, sizeof(double) * 9, cudaMemcpyDeviceToDevice, s));
-    if (forces || e_atom) rc = launch_scatter_forces_f64(c, forces, e_atom, s);
+    if (energy || virial || forces || e_atom) rc = launch_outputs_f64(c, forces, e_atom, energy, virial, s);
     return rc;
 }
 
@@ -382,12 +385,11 @@ int mlip_compute(mlip_ctx *c, double *energy, float *forces, double *virial, flo
     if (!c->built) return fail(c, MLIP_ERR_NOT_BUILT, "no neighbor lists yet");
     cudaStream_t s = (cudaStream_t)stream;
     c->last_stream = s;
+    c->mark_open = false;
     int rc = evaluate(c, s);
     if (rc != MLIP_OK) return rc;
     c->forces_current = true;
-    if (energy) MLIP_CUDA_TRY(c, cudaMemcpyAsync(energy, c->acc + ACC_ENERGY, sizeof(double), cudaMemcpyDeviceToDevice, s));
-    if (virial) MLIP_CUDA_TRY(c, cudaMemcpyAsync(virial, c->acc + ACC_VIRIAL, sizeof(double) * 9, cudaMemcpyDeviceToDevice, s));
-    if (forces || e_atom) rc = launch_scatter_forces(c, forces, e_atom, s);
+    if (energy || virial || forces || e_atom) rc = launch_outputs(c, forces, e_atom, energy, virial, s);
     return rc;
 }
 
@@ -430,6 +432,7 @@ static int rebuild_if_due(mlip_ctx *c, int rebuild_every, cudaStream_t s) {
     if (rebuild_every < 0 && c->step % -rebuild_every == 0) {   // displacement-triggered: ask the device
         MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->rebuild_host, c->rebuild_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
         MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
+        c->mark_open = false;
         rebuild = *c->rebuild_host != 0;
     }
     if (!rebuild) return MLIP_OK;
@@ -446,19 +449,20 @@ int mlip_step(mlip_ctx *c, int n_steps, double dt, int rebuild_every, void *stre
     if (c->n_owned != c->n) return fail(c, MLIP_ERR_UNSUPPORTED, "a context with ghost atoms evaluates only: the owner of the ghosts integrates them");
     cudaStream_t s = (cudaStream_t)stream;
     c->last_stream = s;
+    c->mark_open = false;
     int rc;
     if (!c->forces_current) {
         if ((rc = evaluate(c, s)) != MLIP_OK) return rc;
         c->forces_current = true;
     }
+    // per step the drift kernel and the evaluation: the half kick that closes a step runs with the next step's drift
     for (int it = 0; it < n_steps; ++it) {
-        if ((rc = launch_kick_drift(c, dt, s)) != MLIP_OK) return rc;
+        if ((rc = launch_kick_drift(c, dt, it > 0, s)) != MLIP_OK) return rc;
         c->step += 1;
         if ((rc = rebuild_if_due(c, rebuild_every, s)) != MLIP_OK) return rc;
         if ((rc = evaluate(c, s)) != MLIP_OK) return rc;
-        if ((rc = launch_kick(c, dt, s)) != MLIP_OK) return rc;
     }
-    return MLIP_OK;
+    return n_steps > 0 ? launch_kick(c, dt, s) : MLIP_OK;
 }
 
 int mlip_step_nvt(mlip_ctx *c, int n_steps, double dt, int rebuild_every, double t_target, double t_damp, void *stream) {
@@ -468,6 +472,7 @@ int mlip_step_nvt(mlip_ctx *c, int n_steps, double dt, int rebuild_every, double
     if (c->n_owned != c->n) return fail(c, MLIP_ERR_UNSUPPORTED, "a context with ghost atoms evaluates only: the owner of the ghosts integrates them");
     cudaStream_t s = (cudaStream_t)stream;
     c->last_stream = s;
+    c->mark_open = false;
     const double kB = 8.617333262e-5;   // eV/K
     c->nhc_nf = 3.0 * (double)c->n - 3.0;
     c->nhc_kT = kB * t_target;
@@ -478,20 +483,18 @@ int mlip_step_nvt(mlip_ctx *c, int n_steps, double dt, int rebuild_every, double
         if ((rc = evaluate(c, s)) != MLIP_OK) return rc;
         c->forces_current = true;
     }
+    // Each thermostat half step takes the kinetic energy of the velocities as they stand (not the previous half step's rescaled
+    // value, so that a run does not depend on how it is split into calls).  The first one's velocity factor is applied inside the
+    // kick-drift kernel, the second one's with the next step's kinetic energy.
     for (int it = 0; it < n_steps; ++it) {
-        // kinetic energy of the velocities as they stand (not the previous half step's rescaled value, so that a run does
-        // not depend on how it is split into calls), then the thermostat half step; its velocity factor is applied
-        // inside the kick-drift kernel
-        if ((rc = launch_kinetic(c, s)) != MLIP_OK) return rc;
-        if ((rc = launch_nhc_half(c, c->nhc_nf, c->nhc_kT, c->nhc_q1, c->nhc_qk, dt, s)) != MLIP_OK) return rc;
-        if ((rc = launch_kick_drift(c, dt, s, c->nhc + 6)) != MLIP_OK) return rc;
+        if (it == 0 && (rc = launch_kinetic(c, 0, true, dt, s)) != MLIP_OK) return rc;
+        if ((rc = launch_kick_drift(c, dt, false, s, c->nhc + 6)) != MLIP_OK) return rc;
         c->step += 1;
         if ((rc = rebuild_if_due(c, rebuild_every, s)) != MLIP_OK) return rc;
         if ((rc = evaluate(c, s)) != MLIP_OK) return rc;
-        if ((rc = launch_kick(c, dt, s)) != MLIP_OK) return rc;
-        if ((rc = launch_kinetic(c, s)) != MLIP_OK) return rc;
-        if ((rc = launch_nhc_half(c, c->nhc_nf, c->nhc_kT, c->nhc_q1, c->nhc_qk, dt, s)) != MLIP_OK) return rc;
-        if ((rc = launch_scale_velocities(c, s)) != MLIP_OK) return rc;
+        if ((rc = launch_kinetic(c, 1, true, dt, s)) != MLIP_OK) return rc;
+        rc = it + 1 < n_steps ? launch_kinetic(c, 2, true, dt, s) : launch_scale_velocities(c, s);
+        if (rc != MLIP_OK) return rc;
     }
     return MLIP_OK;
 }
@@ -530,6 +533,7 @@ int mlip_set_state(mlip_ctx *c, const double *pos, const double *vel, int64_t st
     if (!c->built) return fail(c, MLIP_ERR_NOT_BUILT, "no atoms yet: build the lists from the saved positions first");
     cudaStream_t s = (cudaStream_t)stream;
     c->last_stream = s;
+    c->mark_open = false;
     int rc;
     if (pos) {
         c->forces_current = false;
@@ -553,6 +557,7 @@ int mlip_debug_rebuild(mlip_ctx *c, int spin_limit, int64_t unpublished_tile, vo
     if (!c->built) return fail(c, MLIP_ERR_NOT_BUILT, "no neighbor lists yet");
     cudaStream_t s = (cudaStream_t)stream;
     c->last_stream = s;
+    c->mark_open = false;
     c->lookback_spin_limit = spin_limit;
     c->lookback_unpublished_tile = unpublished_tile;
     std::swap(c->pos4, c->pos4_src);
@@ -577,9 +582,10 @@ int mlip_get_energies(mlip_ctx *c, double *e_pot, double *e_kin, void *stream) {
     if (!c->built) return fail(c, MLIP_ERR_NOT_BUILT, "no atoms yet");
     cudaStream_t s = (cudaStream_t)stream;
     c->last_stream = s;
+    c->mark_open = false;
     if (e_pot) MLIP_CUDA_TRY(c, cudaMemcpyAsync(e_pot, c->acc + ACC_ENERGY, sizeof(double), cudaMemcpyDeviceToDevice, s));
     if (e_kin) {
-        int rc = launch_kinetic(c, s);
+        int rc = launch_kinetic(c, 0, false, 0.0, s);
         if (rc != MLIP_OK) return rc;
         MLIP_CUDA_TRY(c, cudaMemcpyAsync(e_kin, c->acc + ACC_KINETIC, sizeof(double), cudaMemcpyDeviceToDevice, s));
     }
@@ -617,35 +623,32 @@ int mlip_get_counters(mlip_ctx *c, int64_t *n_list_entries, int64_t *n_pairs, in
     return MLIP_OK;
 }
 
-int mlip_kernel_time(mlip_ctx *c, int64_t *n_launches, double *total_ms, int reset) {
-    if (!c) return MLIP_ERR_INVALID_ARG;
-    const int64_t kept = c->ev_count < mlip_ctx::EV_POOL ? c->ev_count : mlip_ctx::EV_POOL;
+// Number and total duration (ms) of the last EV_POOL parts of a kind since its reset.
+static int marks_total(mlip_ctx *c, unsigned char kind, int64_t *count, double *total_ms) {
+    constexpr int R = mlip_ctx::MARKS;
+    const int64_t oldest = std::max<int64_t>(0, c->marks - R);   // marks still in the ring
+    int64_t kept = 0;
     double total = 0.0;
-    for (int64_t q = 0; q < kept; ++q) {
-        const int slot = (int)((c->ev_count - 1 - q) % mlip_ctx::EV_POOL);
+    for (int64_t m = c->marks - 1; m > oldest && m >= c->mark_reset[kind] && kept < mlip_ctx::EV_POOL; --m) {
+        if (c->mark_kind[m % R] != kind) continue;
         float ms = 0.f;
-        MLIP_CUDA_TRY(c, cudaEventSynchronize(c->ev[2 * slot + 1]));
-        MLIP_CUDA_TRY(c, cudaEventElapsedTime(&ms, c->ev[2 * slot], c->ev[2 * slot + 1]));
+        MLIP_CUDA_TRY(c, cudaEventSynchronize(c->mark_ev[m % R]));
+        MLIP_CUDA_TRY(c, cudaEventElapsedTime(&ms, c->mark_ev[(m - 1) % R], c->mark_ev[m % R]));
         total += ms;
+        kept += 1;
     }
-    if (n_launches) *n_launches = kept;
-    if (total_ms) *total_ms = total;
-    if (reset) c->ev_count = 0;
+    if (count) *count = kept;
+    *total_ms = total;
     return MLIP_OK;
 }
 
-// Sum of the last min(count, EV_POOL) event pairs of a pool, in ms.
-static int pool_total(mlip_ctx *c, cudaEvent_t *pool, int64_t count, double *total_ms) {
-    const int64_t kept = count < mlip_ctx::EV_POOL ? count : mlip_ctx::EV_POOL;
+int mlip_kernel_time(mlip_ctx *c, int64_t *n_launches, double *total_ms, int reset) {
+    if (!c) return MLIP_ERR_INVALID_ARG;
     double total = 0.0;
-    for (int64_t q = 0; q < kept; ++q) {
-        const int slot = (int)((count - 1 - q) % mlip_ctx::EV_POOL);
-        float ms = 0.f;
-        MLIP_CUDA_TRY(c, cudaEventSynchronize(pool[2 * slot + 1]));
-        MLIP_CUDA_TRY(c, cudaEventElapsedTime(&ms, pool[2 * slot], pool[2 * slot + 1]));
-        total += ms;
-    }
-    *total_ms = total;
+    const int rc = marks_total(c, MARK_KERNEL, n_launches, &total);
+    if (rc != MLIP_OK) return rc;
+    if (total_ms) *total_ms = total;
+    if (reset) c->mark_reset[MARK_KERNEL] = c->marks;
     return MLIP_OK;
 }
 
@@ -653,13 +656,13 @@ int mlip_get_timings(mlip_ctx *c, double *ms_build, double *ms_kernel, double *m
     if (!c) return MLIP_ERR_INVALID_ARG;
     double b = 0.0, k = 0.0, i = 0.0;
     int rc;
-    if ((rc = pool_total(c, c->ev_build, c->build_count, &b)) != MLIP_OK) return rc;
-    if ((rc = pool_total(c, c->ev, c->ev_count, &k)) != MLIP_OK) return rc;
-    if ((rc = pool_total(c, c->ev_integrate, c->integrate_count, &i)) != MLIP_OK) return rc;
+    if ((rc = marks_total(c, MARK_BUILD, nullptr, &b)) != MLIP_OK) return rc;
+    if ((rc = marks_total(c, MARK_KERNEL, nullptr, &k)) != MLIP_OK) return rc;
+    if ((rc = marks_total(c, MARK_INTEGRATE, nullptr, &i)) != MLIP_OK) return rc;
     if (ms_build) *ms_build = b;
     if (ms_kernel) *ms_kernel = k;
     if (ms_integrate) *ms_integrate = i;
-    if (reset) { c->build_count = 0; c->ev_count = 0; c->integrate_count = 0; }
+    if (reset) for (int64_t &r : c->mark_reset) r = c->marks;
     return MLIP_OK;
 }
 
@@ -689,11 +692,8 @@ void mlip_destroy(mlip_ctx *c) {
     if (c->total_host) cudaFreeHost(c->total_host);
     if (c->rebuild_host) cudaFreeHost(c->rebuild_host);
     if (c->build_host) cudaFreeHost(c->build_host);
-    for (int q = 0; q < 2 * mlip_ctx::EV_POOL; ++q) {
-        if (c->ev[q]) cudaEventDestroy(c->ev[q]);
-        if (c->ev_build[q]) cudaEventDestroy(c->ev_build[q]);
-        if (c->ev_integrate[q]) cudaEventDestroy(c->ev_integrate[q]);
-    }
+    for (cudaEvent_t e : c->mark_ev)
+        if (e) cudaEventDestroy(e);
     delete c;
 }
 

@@ -130,9 +130,9 @@ struct mlip_ctx {
     int64_t *scan_tmp = nullptr;   // block sums for the scans
     int64_t scan_tmp_cap = 0;
     double *launch_block = nullptr;   // one allocation: tile_counter, pair_counter, acc_fx, acc back to back, so that a launch
-                                      // clears its counters and accumulators with a single memset (LAUNCH_CLEAR_BYTES)
+                                      // clears its counters and accumulators in one go (LAUNCH_CLEAR_BYTES)
     double *acc = nullptr;         // [ACC_COUNT] (inside launch_block)
-    double *kin_part = nullptr;    // [1184] per-block kinetic-energy sums (integrate.cu)
+    double *kin_part = nullptr;    // [1184] per-block kinetic-energy sums, then the ticket of the last block (integrate.cu)
     unsigned long long *pair_counter = nullptr;
     int *status = nullptr;         // device status word
     int *rebuild_flag = nullptr;   // set when an atom has moved beyond the rebuild trigger; pinned copy in rebuild_host
@@ -155,12 +155,16 @@ struct mlip_ctx {
     int64_t launches = 0;
     size_t resident = 0;
     cudaStream_t last_stream = nullptr;
-    static constexpr int EV_POOL = 256;
-    cudaEvent_t ev[2 * EV_POOL] = {nullptr};
-    int64_t ev_count = 0;          // launches timed since the last reset
-    // event pairs around list builds and around the integrator's kernels (mlip_get_timings)
-    cudaEvent_t ev_build[2 * EV_POOL] = {nullptr}, ev_integrate[2 * EV_POOL] = {nullptr};
-    int64_t build_count = 0, integrate_count = 0;
+    bool force_cleared = false, block_cleared = false;   // the forces / the counters and totals were cleared for the next evaluation by a kernel before it
+    // Timing marks: a ring of events, each the end of a timed part that began at the mark before it (consecutive parts share
+    // a mark), or the beginning of one.
+    static constexpr int EV_POOL = 256, MARKS = 4 * EV_POOL;
+    cudaEvent_t mark_ev[MARKS] = {nullptr};
+    unsigned char mark_kind[MARKS] = {0};
+    int64_t marks = 0;             // recorded so far
+    int64_t mark_reset[4] = {0};   // per kind: parts that ended before this mark have been reset
+    bool mark_open = false;        // nothing untimed has been enqueued since the last mark
+    cudaStream_t mark_stream = nullptr;
 };
 
 namespace mlip {
@@ -174,9 +178,22 @@ namespace mlip {
         }                                                                                 \
     } while (0)
 
-// Record the start / stop event of the next slot of a timing pool on stream s.
-inline void timing_begin(cudaEvent_t *pool, int64_t count, cudaStream_t s) { cudaEventRecord(pool[2 * (count % mlip_ctx::EV_POOL)], s); }
-inline void timing_end(cudaEvent_t *pool, int64_t &count, cudaStream_t s) { cudaEventRecord(pool[2 * (count % mlip_ctx::EV_POOL) + 1], s); count += 1; }
+// Timed parts of the path (mlip_get_timings).  Between mark_begin and mark_end only the part itself is enqueued.
+enum : unsigned char { MARK_BEGIN = 0, MARK_BUILD = 1, MARK_KERNEL = 2, MARK_INTEGRATE = 3 };
+inline void mark_record(mlip_ctx *c, unsigned char kind, cudaStream_t s) {
+    const int slot = (int)(c->marks % mlip_ctx::MARKS);
+    cudaEventRecord(c->mark_ev[slot], s);
+    c->mark_kind[slot] = kind;
+    c->marks += 1;
+}
+inline void mark_begin(mlip_ctx *c, cudaStream_t s) {
+    if (!c->mark_open || c->mark_stream != s) mark_record(c, MARK_BEGIN, s);
+}
+inline void mark_end(mlip_ctx *c, unsigned char kind, cudaStream_t s) {
+    mark_record(c, kind, s);
+    c->mark_open = true;
+    c->mark_stream = s;
+}
 
 // neighbor.cu
 int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int32_t *species, cudaStream_t s);
@@ -193,13 +210,12 @@ int upload_head_f64(mlip_ctx *c, const double *head_w_host);
 int launch_megakernel_f64(mlip_ctx *c, cudaStream_t s);
 bool f64_shape_supported(int k, int l_max, int basis);
 // integrate.cu
-int launch_kick_drift(mlip_ctx *c, double dt, cudaStream_t s, const double *vscale = nullptr);
-int launch_nhc_half(mlip_ctx *c, double n_f, double kT, double q1, double qk, double dt, cudaStream_t s);
+int launch_kick_drift(mlip_ctx *c, double dt, bool close_step, cudaStream_t s, const double *vscale = nullptr);
 int launch_scale_velocities(mlip_ctx *c, cudaStream_t s);
 int launch_kick(mlip_ctx *c, double dt, cudaStream_t s);
-int launch_kinetic(mlip_ctx *c, cudaStream_t s);
-int launch_scatter_forces(mlip_ctx *c, float *forces, float *e_atom, cudaStream_t s);
-int launch_scatter_forces_f64(mlip_ctx *c, double *forces, double *e_atom, cudaStream_t s);
+int launch_kinetic(mlip_ctx *c, int change, bool thermostat, double dt, cudaStream_t s);
+int launch_outputs(mlip_ctx *c, float *forces, float *e_atom, double *energy, double *virial, cudaStream_t s);
+int launch_outputs_f64(mlip_ctx *c, double *forces, double *e_atom, double *energy, double *virial, cudaStream_t s);
 int launch_set_positions(mlip_ctx *c, const double *pos, cudaStream_t s);
 int launch_set_velocities(mlip_ctx *c, const double *vel, cudaStream_t s);
 int launch_get_state(mlip_ctx *c, double *pos, double *vel, cudaStream_t s);

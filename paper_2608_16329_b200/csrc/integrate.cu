@@ -13,24 +13,45 @@ __device__ __forceinline__ double3 load_force(const float4 *__restrict__ force, 
     return make_double3(f.x, f.y, f.z);
 }
 
-// v += dt/2 a;  x += dt v;  wrap into [0, L);  track the displacement since the last list build.
+// What the evaluation that follows a move accumulates into: forces, and the counters and totals at the head of launch_block.  The kernels
+// that move atoms clear them on the way (a separate clear is a launch, and for the forces a pass, of its own).
+struct EvalClear {
+    float4 *force;       // nullptr: not accumulated into (deterministic mode, fp64 contexts)
+    double *force_d;     // fp64 contexts
+    double *launch_block;
+};
+__device__ __forceinline__ void clear_for_eval(const EvalClear &c, int64_t i) {
+    if (c.force) c.force[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (c.force_d) { c.force_d[3 * i] = 0.0; c.force_d[3 * i + 1] = 0.0; c.force_d[3 * i + 2] = 0.0; }
+    if (i == 0 && c.launch_block)
+        for (int q = 0; q < (int)(LAUNCH_CLEAR_BYTES / sizeof(double)); ++q) c.launch_block[q] = 0.0;
+}
+
+// v += dt/2 a  (CLOSE: twice, the second half kick of one step and the first of the next, which see the same forces);
+// x += dt v;  wrap into [0, L);  track the displacement since the last list build.  Every operation is rounded in a fixed way, so
+// a trajectory does not depend on how it is cut into calls.
+template <bool CLOSE>
 __global__ void k_kick_drift(int64_t n, double dt, CellGrid g, const double *__restrict__ mass, float skin_half2,
-                             double4 *__restrict__ pos4, double *__restrict__ vel, const float4 *__restrict__ force,
-                             const double *__restrict__ force_d, float *__restrict__ disp, int *status, float trigger2,
-                             int *rebuild_flag, const double *__restrict__ vscale, float far2, int *far_flag) {
+                             double4 *__restrict__ pos4, double *__restrict__ vel, const float4 *force,
+                             const double *force_d, float *__restrict__ disp, int *status, float trigger2,
+                             int *rebuild_flag, const double *__restrict__ vscale, float far2, int *far_flag, EvalClear clear) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     double4 p = pos4[i];
-    const double3 f = load_force(force, force_d, i);
+    const double3 f3 = load_force(force, force_d, i);
+    const double f[3] = {f3.x, f3.y, f3.z}, px[3] = {p.x, p.y, p.z};
     const double k = 0.5 * dt * ACC_UNIT / mass[(int)p.w];
     const double sc = vscale ? *vscale : 1.0;   // thermostat factor applied ahead of the kick (NVT)
-    double v[3] = {vel[3 * i] * sc + k * f.x, vel[3 * i + 1] * sc + k * f.y, vel[3 * i + 2] * sc + k * f.z};
-    double x[3] = {p.x + dt * v[0], p.y + dt * v[1], p.z + dt * v[2]};
+    double x[3];
     float d2 = 0.f;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        vel[3 * i + a] = v[a];
-        float d = disp[3 * i + a] + (float)(dt * v[a]);
+        double v = vel[3 * i + a];
+        if (CLOSE) v = fma(k, f[a], v);
+        v = fma(k, f[a], v * sc);
+        vel[3 * i + a] = v;
+        x[a] = fma(dt, v, px[a]);
+        float d = disp[3 * i + a] + (float)(dt * v);
         disp[3 * i + a] = d;
         d2 += d * d;
         const double L = g.box[a];
@@ -42,6 +63,7 @@ __global__ void k_kick_drift(int64_t n, double dt, CellGrid g, const double *__r
     if (d2 > trigger2) *rebuild_flag = 1;   // same value from every writer
     if (!(d2 <= far2)) *far_flag = 1;       // from now on the lists' far entries may come inside r_cut
     pos4[i] = make_double4(x[0], x[1], x[2], p.w);
+    clear_for_eval(clear, i);
 }
 
 // v += dt/2 a
@@ -51,22 +73,23 @@ __global__ void k_kick(int64_t n, double dt, const double *__restrict__ mass, co
     if (i >= n) return;
     const double3 f = load_force(force, force_d, i);
     const double k = 0.5 * dt * ACC_UNIT / mass[(int)pos4[i].w];
-    vel[3 * i] += k * f.x; vel[3 * i + 1] += k * f.y; vel[3 * i + 2] += k * f.z;
+    vel[3 * i] = fma(k, f.x, vel[3 * i]); vel[3 * i + 1] = fma(k, f.y, vel[3 * i + 1]); vel[3 * i + 2] = fma(k, f.z, vel[3 * i + 2]);
 }
 
 // Half-step (dt/2) of a Nose-Hoover chain of three thermostats coupled to the kinetic energy in acc[ACC_KINETIC]
-// (Martyna-Tuckerman-Tobias-Klein factorisation, one Suzuki-Yoshida term).  One thread.  state = {v_eta[3], eta[3], scale}:
+// (Martyna-Tuckerman-Tobias-Klein factorisation, one Suzuki-Yoshida term).  One thread calls it.  state = {v_eta[3], eta[3], scale}:
 //   dv_eta_k/dt = G_k - v_eta_{k+1} v_eta_k,  G_1 = (2 KE - N_f kT) / Q_1,  G_k = (Q_{k-1} v_eta_{k-1}^2 - kT) / Q_k,
 //   particle velocities scale by exp(-v_eta_1 dt/2); the stored kinetic energy is scaled with them.
-__global__ void k_nhc_half(double *state, double *acc, double n_f, double kT, double q1, double qk, double dt) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+struct NhcHalf { double n_f, kT, q1, qk, dt; double *state; };   // state = nullptr: no thermostat
+__device__ void nhc_half(const NhcHalf &h, double *acc) {
     constexpr int M = 3;
+    double *state = h.state;
     double v[M] = {state[0], state[1], state[2]};
-    const double q[M] = {q1, qk, qk}, d = 0.5 * dt;
+    const double q[M] = {h.q1, h.qk, h.qk}, d = 0.5 * h.dt;
     double ke2 = 2.0 * acc[ACC_KINETIC];
     double G[M];
-    G[0] = (ke2 - n_f * kT) / q[0];
-    for (int c = 1; c < M; ++c) G[c] = (q[c - 1] * v[c - 1] * v[c - 1] - kT) / q[c];
+    G[0] = (ke2 - h.n_f * h.kT) / q[0];
+    for (int c = 1; c < M; ++c) G[c] = (q[c - 1] * v[c - 1] * v[c - 1] - h.kT) / q[c];
     v[M - 1] += 0.5 * d * G[M - 1];
     for (int c = M - 2; c >= 0; --c) {
         const double a = exp(-0.25 * d * v[c + 1]);
@@ -75,11 +98,11 @@ __global__ void k_nhc_half(double *state, double *acc, double n_f, double kT, do
     const double scale = exp(-d * v[0]);
     ke2 *= scale * scale;
     for (int c = 0; c < M; ++c) state[3 + c] += d * v[c];
-    G[0] = (ke2 - n_f * kT) / q[0];
+    G[0] = (ke2 - h.n_f * h.kT) / q[0];
     for (int c = 0; c < M - 1; ++c) {
         const double a = exp(-0.25 * d * v[c + 1]);
         v[c] = (v[c] * a + 0.5 * d * G[c]) * a;
-        G[c + 1] = (q[c] * v[c] * v[c] - kT) / q[c + 1];
+        G[c + 1] = (q[c] * v[c] * v[c] - h.kT) / q[c + 1];
     }
     v[M - 1] += 0.5 * d * G[M - 1];
     for (int c = 0; c < M; ++c) state[c] = v[c];
@@ -92,57 +115,87 @@ __global__ void k_scale_velocities(int64_t n3, double *__restrict__ vel, const d
     if (i < n3) vel[i] *= *scale;
 }
 
-// Kinetic energy in two steps with a fixed summation order (grid-stride partial sums per block, then one warp adds the
-// block sums in index order), so that the thermostat -- and with it an NVT trajectory -- is bit-reproducible.
+// Kinetic energy with a fixed summation order (grid-stride partial sums per block, then one warp of the block that finishes last
+// adds the block sums in index order), so that the thermostat -- and with it an NVT trajectory -- is bit-reproducible.  What changes the
+// velocities just before rides along: CHANGE = 1 the half kick that closes a step, 2 the thermostat's factor; and the thermostat half
+// step that needs the energy follows in the last block.  (As kernels of their own these were eight of a step's ten launches:
+// 4,394 atoms 152 us per step, of which the evaluation was 65.)
 constexpr int KIN_BLOCKS = 1184;
-__global__ void k_kinetic(int64_t n, const double *__restrict__ mass, const double4 *__restrict__ pos4,
-                          const double *__restrict__ vel, double *__restrict__ block_sum) {
-    __shared__ double part[32];
+template <int CHANGE>
+__global__ void __launch_bounds__(256) k_kinetic(int64_t n, double dt, const double *__restrict__ mass, const double4 *__restrict__ pos4, double *vel,
+                                                 const float4 *__restrict__ force, const double *__restrict__ force_d, const double *scale,
+                                                 double *block_sum, unsigned int *ticket, double *acc, NhcHalf nhc) {
+    __shared__ double part[8];
+    __shared__ bool last;
     double e = 0.0;
+    const double sc = CHANGE == 2 ? *scale : 1.0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        double vx = vel[3 * i], vy = vel[3 * i + 1], vz = vel[3 * i + 2];
-        e += 0.5 * mass[(int)pos4[i].w] * (vx * vx + vy * vy + vz * vz);
+        double v[3] = {vel[3 * i], vel[3 * i + 1], vel[3 * i + 2]};
+        const double m = mass[(int)pos4[i].w];
+        if (CHANGE == 1) {
+            const double3 f = load_force(force, force_d, i);
+            const double k = 0.5 * dt * ACC_UNIT / m;
+            v[0] = fma(k, f.x, v[0]); v[1] = fma(k, f.y, v[1]); v[2] = fma(k, f.z, v[2]);
+        }
+        if (CHANGE == 2) { v[0] *= sc; v[1] *= sc; v[2] *= sc; }
+        if (CHANGE != 0) { vel[3 * i] = v[0]; vel[3 * i + 1] = v[1]; vel[3 * i + 2] = v[2]; }
+        e = fma(0.5 * m, fma(v[2], v[2], fma(v[1], v[1], __dmul_rn(v[0], v[0]))), e);
     }
     for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = e;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        e = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.0;
-        for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-        if (threadIdx.x == 0) block_sum[blockIdx.x] = e;
+    if (threadIdx.x >= 32) return;
+    e = threadIdx.x < 8 ? part[threadIdx.x] : 0.0;
+    for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (threadIdx.x == 0) {
+        block_sum[blockIdx.x] = e;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncwarp();
+    if (!last) return;
+    __threadfence();
+    e = 0.0;
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += 32) e += *(volatile double *)(block_sum + b);
+    for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (threadIdx.x == 0) {
+        *ticket = 0;
+        acc[ACC_KINETIC] = e / ACC_UNIT;
+        if (nhc.state) nhc_half(nhc, acc);
     }
 }
-__global__ void k_kinetic_finish(int n_blocks, const double *__restrict__ block_sum, double *acc) {
-    double e = 0.0;
-    for (int b = threadIdx.x; b < n_blocks; b += 32) e += block_sum[b];
-    for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-    if (threadIdx.x == 0) acc[ACC_KINETIC] = e / ACC_UNIT;
-}
 
-__global__ void k_scatter_forces(int64_t n, const int32_t *__restrict__ user_of, const float4 *__restrict__ force,
-                                 const float *__restrict__ e_in, float *__restrict__ forces_out, float *__restrict__ e_atom) {
+// Per-atom outputs in the caller's order, and the totals: one launch.  FIN: float4, or double for three per atom.
+template <typename FIN, typename EIN, typename FOUT>
+__global__ void k_outputs(int64_t n, const int32_t *__restrict__ user_of, const FIN *__restrict__ force, const EIN *__restrict__ e_in,
+                          FOUT *__restrict__ forces_out, FOUT *__restrict__ e_atom, const double *__restrict__ acc, double *__restrict__ energy,
+                          double *__restrict__ virial) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float4 f = force[i];
+    if (i == 0) {
+        if (energy) *energy = acc[ACC_ENERGY];
+        if (virial)
+            for (int q = 0; q < 9; ++q) virial[q] = acc[ACC_VIRIAL + q];
+    }
+    if (i >= n || !(forces_out || e_atom)) return;
     const int64_t u = user_of[i];
-    if (forces_out) { forces_out[3 * u] = f.x; forces_out[3 * u + 1] = f.y; forces_out[3 * u + 2] = f.z; }
-    if (e_atom) e_atom[u] = e_in[i];
-}
-
-__global__ void k_scatter_forces_f64(int64_t n, const int32_t *__restrict__ user_of, const double *__restrict__ force,
-                                     const double *__restrict__ e_in, double *__restrict__ forces_out, double *__restrict__ e_atom) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int64_t u = user_of[i];
-    if (forces_out) { forces_out[3 * u] = force[3 * i]; forces_out[3 * u + 1] = force[3 * i + 1]; forces_out[3 * u + 2] = force[3 * i + 2]; }
-    if (e_atom) e_atom[u] = e_in[i];
+    if (forces_out) {
+        if constexpr (sizeof(FIN) == sizeof(float4)) {
+            const float4 f = force[i];
+            forces_out[3 * u] = (FOUT)f.x; forces_out[3 * u + 1] = (FOUT)f.y; forces_out[3 * u + 2] = (FOUT)f.z;
+        } else {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) forces_out[3 * u + q] = (FOUT)force[3 * i + q];
+        }
+    }
+    if (e_atom) e_atom[u] = (FOUT)e_in[i];
 }
 
 __global__ void k_set_positions(int64_t n, const int32_t *__restrict__ user_of, const double *__restrict__ pos,
                                 CellGrid g, float skin_half2, double4 *__restrict__ pos4, float *__restrict__ disp, int *status,
-                                float far2, int *far_flag) {
+                                float far2, int *far_flag, EvalClear clear) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
+    clear_for_eval(clear, i);
     const int64_t u = user_of[i];
     double4 p = pos4[i];
     const double x[3] = {pos[3 * u], pos[3 * u + 1], pos[3 * u + 2]};
@@ -185,62 +238,72 @@ static inline float skin_half2(const mlip_ctx *c) { float h = 0.5f * (float)c->c
 // stay outside r_cut while every atom has moved less than skin / 4 (0.245: room for the fp32 bookkeeping).
 static inline float far_trigger2(const mlip_ctx *c) { float h = 0.245f * (float)c->cfg.skin; return h * h; }
 
-int launch_kick_drift(mlip_ctx *c, double dt, cudaStream_t s, const double *vscale) {
-    timing_begin(c->ev_integrate, c->integrate_count, s);
-    k_kick_drift<<<nb(c->n), 256, 0, s>>>(c->n, dt, c->grid, c->mass, skin_half2(c), c->pos4, c->vel, c->force, c->force_d, c->disp, c->status,
-                                               0.64f * skin_half2(c), c->rebuild_flag, vscale, far_trigger2(c), c->far_flag);
-    timing_end(c->ev_integrate, c->integrate_count, s);
+// The buffers of the next evaluation, to be cleared by the kernel that takes this, which must be the last before it on the stream.
+// `totals`: the evaluation follows in the same call, so nobody reads the last one's energy and counters in between.
+static EvalClear eval_clear(mlip_ctx *c, bool totals) {
+    c->force_cleared = true;
+    if (totals) c->block_cleared = true;
+    const bool f64 = c->cfg.precision == 1;
+    return EvalClear{f64 || c->cfg.force_mode == 1 ? nullptr : c->force, f64 ? c->force_d : nullptr, totals ? c->launch_block : nullptr};
+}
+int launch_kick_drift(mlip_ctx *c, double dt, bool close_step, cudaStream_t s, const double *vscale) {
+    mark_begin(c, s);
+    const EvalClear clear = eval_clear(c, true);
+    auto *kernel = close_step ? k_kick_drift<true> : k_kick_drift<false>;
+    kernel<<<nb(c->n), 256, 0, s>>>(c->n, dt, c->grid, c->mass, skin_half2(c), c->pos4, c->vel, c->force, c->force_d, c->disp, c->status,
+                                    0.64f * skin_half2(c), c->rebuild_flag, vscale, far_trigger2(c), c->far_flag, clear);
+    mark_end(c, MARK_INTEGRATE, s);
     c->launches += 1;
     MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
 int launch_kick(mlip_ctx *c, double dt, cudaStream_t s) {
-    timing_begin(c->ev_integrate, c->integrate_count, s);
+    mark_begin(c, s);
     k_kick<<<nb(c->n), 256, 0, s>>>(c->n, dt, c->mass, c->pos4, c->vel, c->force, c->force_d);
-    timing_end(c->ev_integrate, c->integrate_count, s);
-    c->launches += 1;
-    MLIP_CUDA_TRY(c, cudaGetLastError());
-    return MLIP_OK;
-}
-int launch_nhc_half(mlip_ctx *c, double n_f, double kT, double q1, double qk, double dt, cudaStream_t s) {
-    timing_begin(c->ev_integrate, c->integrate_count, s);
-    k_nhc_half<<<1, 32, 0, s>>>(c->nhc, c->acc, n_f, kT, q1, qk, dt);
-    timing_end(c->ev_integrate, c->integrate_count, s);
+    mark_end(c, MARK_INTEGRATE, s);
     c->launches += 1;
     MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
 int launch_scale_velocities(mlip_ctx *c, cudaStream_t s) {
-    timing_begin(c->ev_integrate, c->integrate_count, s);
+    mark_begin(c, s);
     k_scale_velocities<<<nb(3 * c->n), 256, 0, s>>>(3 * c->n, c->vel, c->nhc + 6);
-    timing_end(c->ev_integrate, c->integrate_count, s);
+    mark_end(c, MARK_INTEGRATE, s);
     c->launches += 1;
     MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
-int launch_kinetic(mlip_ctx *c, cudaStream_t s) {
+int launch_kinetic(mlip_ctx *c, int change, bool thermostat, double dt, cudaStream_t s) {
     int64_t blocks = nb(c->n);
     if (blocks > KIN_BLOCKS) blocks = KIN_BLOCKS;
-    k_kinetic<<<(unsigned)blocks, 256, 0, s>>>(c->n, c->mass, c->pos4, c->vel, c->kin_part);
-    k_kinetic_finish<<<1, 32, 0, s>>>((int)blocks, c->kin_part, c->acc);
-    c->launches += 2;
-    MLIP_CUDA_TRY(c, cudaGetLastError());
-    return MLIP_OK;
-}
-int launch_scatter_forces(mlip_ctx *c, float *forces, float *e_atom, cudaStream_t s) {
-    k_scatter_forces<<<nb(c->n), 256, 0, s>>>(c->n, c->user_of, c->force, c->e_atom, forces, e_atom);
+    const NhcHalf nhc{c->nhc_nf, c->nhc_kT, c->nhc_q1, c->nhc_qk, dt, thermostat ? c->nhc : nullptr};
+    auto *kernel = change == 1 ? k_kinetic<1> : change == 2 ? k_kinetic<2> : k_kinetic<0>;
+    if (thermostat) mark_begin(c, s);
+    kernel<<<(unsigned)blocks, 256, 0, s>>>(c->n, dt, c->mass, c->pos4, c->vel, c->force, c->force_d, c->nhc + 6, c->kin_part,
+                                            reinterpret_cast<unsigned int *>(c->kin_part + KIN_BLOCKS), c->acc, nhc);
+    if (thermostat) mark_end(c, MARK_INTEGRATE, s);
     c->launches += 1;
     MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
-int launch_scatter_forces_f64(mlip_ctx *c, double *forces, double *e_atom, cudaStream_t s) {
-    k_scatter_forces_f64<<<nb(c->n), 256, 0, s>>>(c->n, c->user_of, c->force_d, c->e_atom_d, forces, e_atom);
+int launch_outputs(mlip_ctx *c, float *forces, float *e_atom, double *energy, double *virial, cudaStream_t s) {
+    const unsigned blocks = forces || e_atom ? nb(c->n) : 1;
+    if (c->cfg.precision == 1) k_outputs<double, double, float><<<blocks, 256, 0, s>>>(c->n, c->user_of, c->force_d, c->e_atom_d, forces, e_atom, c->acc, energy, virial);
+    else k_outputs<float4, float, float><<<blocks, 256, 0, s>>>(c->n, c->user_of, c->force, c->e_atom, forces, e_atom, c->acc, energy, virial);
+    c->launches += 1;
+    MLIP_CUDA_TRY(c, cudaGetLastError());
+    return MLIP_OK;
+}
+int launch_outputs_f64(mlip_ctx *c, double *forces, double *e_atom, double *energy, double *virial, cudaStream_t s) {
+    const unsigned blocks = forces || e_atom ? nb(c->n) : 1;
+    k_outputs<double, double, double><<<blocks, 256, 0, s>>>(c->n, c->user_of, c->force_d, c->e_atom_d, forces, e_atom, c->acc, energy, virial);
     c->launches += 1;
     MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
 int launch_set_positions(mlip_ctx *c, const double *pos, cudaStream_t s) {
-    k_set_positions<<<nb(c->n), 256, 0, s>>>(c->n, c->user_of, pos, c->grid, skin_half2(c), c->pos4, c->disp, c->status, far_trigger2(c), c->far_flag);
+    const EvalClear clear = eval_clear(c, false);
+    k_set_positions<<<nb(c->n), 256, 0, s>>>(c->n, c->user_of, pos, c->grid, skin_half2(c), c->pos4, c->disp, c->status, far_trigger2(c), c->far_flag, clear);
     c->launches += 1;
     MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;

@@ -1272,14 +1272,15 @@ int upload_head(mlip_ctx *c, const double *w) {
     return MLIP_OK;
 }
 
-// Deterministic mode: integer sums -> the float / double outputs the rest of the library reads.
-__global__ void k_fixed_finish(int64_t n, const long long *__restrict__ force_fx, const long long *__restrict__ acc_fx,
+// Deterministic mode: integer sums -> the float / double outputs the rest of the library reads; the sums start the next evaluation at zero.
+__global__ void k_fixed_finish(int64_t n, long long *__restrict__ force_fx, const long long *__restrict__ acc_fx,
                                float4 *__restrict__ force, double *__restrict__ acc) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) {
         const double inv = 1.0 / (double)FORCE_FX;
         force[i] = make_float4((float)((double)force_fx[3 * i] * inv), (float)((double)force_fx[3 * i + 1] * inv),
                                (float)((double)force_fx[3 * i + 2] * inv), 0.f);
+        force_fx[3 * i] = force_fx[3 * i + 1] = force_fx[3 * i + 2] = 0;
     }
     if (i == 0) {
         acc[ACC_ENERGY] = (double)acc_fx[0] / ENERGY_FX;
@@ -1290,9 +1291,12 @@ __global__ void k_fixed_finish(int64_t n, const long long *__restrict__ force_fx
 int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     const int64_t n = c->n;
     const bool det = c->cfg.force_mode == 1;
-    if (det) MLIP_CUDA_TRY(c, cudaMemsetAsync(c->force_fx, 0, sizeof(long long) * 3 * n, s));
-    MLIP_CUDA_TRY(c, cudaMemsetAsync(c->force, 0, sizeof(float4) * n, s));
-    MLIP_CUDA_TRY(c, cudaMemsetAsync(c->launch_block, 0, LAUNCH_CLEAR_BYTES, s));   // tile and pair counters, integer and fp64 accumulators
+    if (!(c->force_cleared || det) || !c->block_cleared) {
+        c->mark_open = false;
+        if (!c->force_cleared && !det) MLIP_CUDA_TRY(c, cudaMemsetAsync(c->force, 0, sizeof(float4) * n, s));   // (k_fixed_finish keeps the integer sums clear)
+        if (!c->block_cleared) MLIP_CUDA_TRY(c, cudaMemsetAsync(c->launch_block, 0, LAUNCH_CLEAR_BYTES, s));   // tile and pair counters, integer and fp64 accumulators
+    }
+    c->force_cleared = c->block_cleared = false;
     const bool in_smem = tables_fit_smem(c);
     const int tab_words = in_smem ? table_smem_words(c) : 0;
     // instantiations: {one, two atoms per warp with staggered species, two without, two with tables in global memory}
@@ -1321,15 +1325,13 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     k.nbr_cap = c->nbr_cap; k.head_pack = c->head_w; k.force = c->force; k.e_atom = c->e_atom;
     k.force_fx = c->force_fx; k.acc_fx = c->acc_fx;
     k.acc = c->acc; k.pair_counter = c->pair_counter; k.status = c->status; k.tile_counter = c->tile_counter;
-    const int slot = (int)(c->ev_count % mlip_ctx::EV_POOL);
-    MLIP_CUDA_TRY(c, cudaEventRecord(c->ev[2 * slot], s));
+    mark_begin(c, s);
     kernels[shape][(det ? 2 : 0) + (c->list16 ? 1 : 0)]<<<blocks, NW * 32, smem_bytes, s>>>(k, tab_words);
     if (det) {
         k_fixed_finish<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, c->force_fx, c->acc_fx, c->force, c->acc);
         c->launches += 1;
     }
-    MLIP_CUDA_TRY(c, cudaEventRecord(c->ev[2 * slot + 1], s));
-    c->ev_count += 1;
+    mark_end(c, MARK_KERNEL, s);
     c->launches += 1;
     MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;

@@ -589,15 +589,6 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
     }
 }
 
-// fp64 forces and energies -> the fp32 arrays the fp32 getters read
-__global__ void k_force_to_float(int64_t n, const double *__restrict__ fd, const double *__restrict__ ed, float4 *__restrict__ force,
-                                 float *__restrict__ e_atom) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    force[i] = make_float4((float)fd[3 * i], (float)fd[3 * i + 1], (float)fd[3 * i + 2], 0.f);
-    e_atom[i] = (float)ed[i];
-}
-
 int upload_head_f64(mlip_ctx *c, const double *w) {
     const int C = c->cfg.n_species, n_inv = (c->cfg.l_max + 1) * c->cfg.k;
     const Head64 H(n_inv);
@@ -630,7 +621,7 @@ int upload_head_f64(mlip_ctx *c, const double *w) {
 }
 
 template <int K, int LMAX, int BASIS>
-static cudaError_t launch_shape(mlip_ctx *c, const F64Args &k, cudaStream_t s, cudaEvent_t start, cudaEvent_t stop) {
+static cudaError_t launch_shape(mlip_ctx *c, const F64Args &k, cudaStream_t s) {
     const size_t smem_bytes = sizeof(TileSmem<K, LMAX, BASIS>);
     if (!c->kernel_ready) {
         cudaError_t e = cudaFuncSetAttribute(k_mega_f64<K, LMAX, BASIS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
@@ -646,9 +637,9 @@ static cudaError_t launch_shape(mlip_ctx *c, const F64Args &k, cudaStream_t s, c
     const int per_sm = f64_ctas_per_sm<K, LMAX, BASIS>();
     const int64_t tiles_max = (k.n + F64_TILE - 1) / F64_TILE + k.n_species;
     const int blocks = (int)std::min<int64_t>(tiles_max, (int64_t)per_sm * c->n_sm);
-    cudaEventRecord(start, s);
+    mark_begin(c, s);
     k_mega_f64<K, LMAX, BASIS><<<blocks, F64_TILE * 32, smem_bytes, s>>>(k);
-    cudaEventRecord(stop, s);
+    mark_end(c, MARK_KERNEL, s);
     return cudaGetLastError();
 }
 
@@ -661,8 +652,12 @@ bool f64_shape_supported(int k, int l_max, int basis) {
 
 int launch_megakernel_f64(mlip_ctx *c, cudaStream_t s) {
     const int64_t n = c->n;
-    MLIP_CUDA_TRY(c, cudaMemsetAsync(c->force_d, 0, sizeof(double) * 3 * n, s));
-    MLIP_CUDA_TRY(c, cudaMemsetAsync(c->launch_block, 0, LAUNCH_CLEAR_BYTES, s));   // pair counter and accumulators
+    if (!c->force_cleared || !c->block_cleared) {
+        c->mark_open = false;
+        if (!c->force_cleared) MLIP_CUDA_TRY(c, cudaMemsetAsync(c->force_d, 0, sizeof(double) * 3 * n, s));
+        if (!c->block_cleared) MLIP_CUDA_TRY(c, cudaMemsetAsync(c->launch_block, 0, LAUNCH_CLEAR_BYTES, s));   // pair counter and accumulators
+    }
+    c->force_cleared = c->block_cleared = false;
     F64Args k;
     k.n = n; k.n_species = c->cfg.n_species; k.grid = c->grid; k.rc2 = c->cfg.r_cut * c->cfg.r_cut;
     k.coef = c->table_d; k.knots = c->cfg.table_knots; k.r_min = c->cfg.table_r_min;
@@ -672,11 +667,9 @@ int launch_megakernel_f64(mlip_ctx *c, cudaStream_t s) {
     k.nbr_cap = c->nbr_cap;
     k.head = c->head_w_d; k.force = c->force_d; k.e_atom = c->e_atom_d; k.acc = c->acc;
     k.pair_counter = c->pair_counter; k.status = c->status;
-    const int slot = (int)(c->ev_count % mlip_ctx::EV_POOL);
-    cudaEvent_t e0 = c->ev[2 * slot], e1 = c->ev[2 * slot + 1];
     cudaError_t e = cudaErrorInvalidValue;
     switch (c->cfg.basis * 1000 + c->cfg.k * 10 + c->cfg.l_max) {
-#define MLIP_F64_CASE(K, L, B) case B * 1000 + K * 10 + L: e = launch_shape<K, L, B>(c, k, s, e0, e1); break;
+#define MLIP_F64_CASE(K, L, B) case B * 1000 + K * 10 + L: e = launch_shape<K, L, B>(c, k, s); break;
         MLIP_F64_CASE(16, 1, 0) MLIP_F64_CASE(16, 2, 0) MLIP_F64_CASE(16, 3, 0)
         MLIP_F64_CASE(32, 1, 0) MLIP_F64_CASE(32, 2, 0) MLIP_F64_CASE(32, 3, 0)
         MLIP_F64_CASE(64, 1, 0) MLIP_F64_CASE(64, 2, 0) MLIP_F64_CASE(64, 3, 0)
@@ -686,9 +679,7 @@ int launch_megakernel_f64(mlip_ctx *c, cudaStream_t s) {
 #undef MLIP_F64_CASE
     }
     MLIP_CUDA_TRY(c, e);
-    c->ev_count += 1;
-    k_force_to_float<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, c->force_d, c->e_atom_d, c->force, c->e_atom);
-    c->launches += 2;
+    c->launches += 1;
     MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }

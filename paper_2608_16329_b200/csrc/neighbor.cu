@@ -706,7 +706,7 @@ static ListView list_view(const mlip_ctx *c) {
 // A synchronising build that met a non-finite or out-of-box position, a species out of range or an over-full cell: the
 // list kernels have not run, so there is nothing to size a list from.  Reports it now and clears the flag.
 static int refuse_broken_input(mlip_ctx *c, cudaStream_t s) {
-    timing_end(c->ev_build, c->build_count, s);
+    mark_end(c, MARK_BUILD, s);
     MLIP_CUDA_TRY(c, cudaMemsetAsync(c->status, 0, sizeof(int), s));
     c->err = "non-finite or out-of-box position, species out of range, or more than 1024 atoms in one cell";
     return MLIP_ERR_NONFINITE;
@@ -736,7 +736,8 @@ static void launch_onepass(mlip_ctx *c, ENTRY *nbr, int *flag, double rl, float 
 // Sort the source set into cell order and build the lists.  The source is (pos4_src, vel_src, user_src), filled from the caller's
 // arrays first when `pos` is given (velocities then start at zero).
 int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int32_t *species, cudaStream_t s) {
-    timing_begin(c->ev_build, c->build_count, s);
+    mark_begin(c, s);
+    if (c->cfg.precision == 0) c->force_cleared = false;   // (the force array is used below)
     const int64_t n = c->n;
     const CellGrid &g = c->grid;
     const int C = c->cfg.n_species;
@@ -794,7 +795,7 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
             if (done) c->n_entries = total;
         }
         if (done) {
-            timing_end(c->ev_build, c->build_count, s);
+            mark_end(c, MARK_BUILD, s);
             return MLIP_OK;
         }
     }
@@ -826,7 +827,7 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
     else
         k_neighbors<true><<<blocks_for(n * 32, 256), 256, 0, s>>>(n, g, rl * rl, c->pos4, c->cell_start, c->nbr_count, c->nbr_off, c->nbr, c->nbr_cap, c->status, near2, c->nbr_near, c->user_of, (int32_t)c->n_owned);
     c->launches += 1;
-    timing_end(c->ev_build, c->build_count, s);
+    mark_end(c, MARK_BUILD, s);
     MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
