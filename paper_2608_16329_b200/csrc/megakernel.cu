@@ -910,6 +910,7 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
     group_sync(group);
 }
 
+constexpr int TOTALS = 9 + 16 + 1;   // per warp at the end: virial, E_i sums of up to 16 lanes, pairs
 template <int APW, bool TAB_SMEM, bool DET, bool L16, bool STAGGER>
 __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words) {
     extern __shared__ __align__(128) float smem[];
@@ -1135,23 +1136,41 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
     }
     pc.flush(k.acc, lane);
 
-    // per-warp totals -> global accumulators
-    if (DET) {
-        if (lane < 9) atomicAdd(reinterpret_cast<unsigned long long *>(k.acc_fx + 1 + lane), (unsigned long long)(long long)vir_fx);
-        if (wg == 7 && lane < NA) atomicAdd(reinterpret_cast<unsigned long long *>(k.acc_fx), (unsigned long long)(long long)e_sum);
-    } else {
+    // totals: per warp into shared memory, per CTA to the global accumulators (from every warp they were 27,000 atomics to one
+    // sector of one L2 slice, some 10 us at the end of every launch)
+    __syncthreads();   // everybody is done with shared memory
+    double *sums = reinterpret_cast<double *>(smem) + warp * TOTALS;   // virial [9], E_i sums of the atoms' lanes, pairs
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            float x = vir[q];
+    for (int q = 0; q < 9; ++q) {
+        double x = vir_fx;
+        if (!DET) {
+            float v = vir[q];
 #pragma unroll
-            for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            if (lane == 0) atomicAdd(&k.acc[ACC_VIRIAL + q], (double)x);
+            for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            x = v;
         }
-        if (wg == 7 && lane < NA) atomicAdd(&k.acc[ACC_ENERGY], e_sum);
+        if (lane == (DET ? q : 0)) sums[q] = x;
     }
-    if (lane == 0) atomicAdd(k.pair_counter, n_pairs);
+    if (lane < 16) sums[9 + lane] = wg == 7 && lane < NA ? e_sum : 0.0;
+    if (lane == 0) reinterpret_cast<unsigned long long *>(sums)[25] = n_pairs;
     tmem_fence_before_sync();
     __syncthreads();
+    if (threadIdx.x < TOTALS) {
+        const double *col = reinterpret_cast<const double *>(smem) + threadIdx.x;
+        if (threadIdx.x == 25) {
+            unsigned long long n = 0;
+            for (int w = 0; w < NW; ++w) n += reinterpret_cast<const unsigned long long *>(col)[w * TOTALS];
+            atomicAdd(k.pair_counter, n);
+        } else if (DET) {
+            long long x = 0;
+            for (int w = 0; w < NW; ++w) x += (long long)col[w * TOTALS];
+            atomicAdd(reinterpret_cast<unsigned long long *>(k.acc_fx + (threadIdx.x < 9 ? 1 + threadIdx.x : 0)), (unsigned long long)x);
+        } else {
+            double x = 0.0;
+            for (int w = 0; w < NW; ++w) x += col[w * TOTALS];
+            if (x != 0.0) atomicAdd(&k.acc[threadIdx.x < 9 ? ACC_VIRIAL + threadIdx.x : ACC_ENERGY], x);
+        }
+    }
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm_base), "r"(TM_COLS) : "memory");
 }
 

@@ -576,16 +576,25 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
     }
     pc.flush(k.acc, lane);
 
+    // totals: per warp into shared memory, per CTA to the global accumulators (the tile loop ended with a barrier)
+    double *sums = reinterpret_cast<double *>(smem_raw) + wid * 11;
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
         double x = vir[q];
 #pragma unroll
         for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == 0) atomicAdd(&k.acc[ACC_VIRIAL + q], x);
+        if (lane == 0) sums[q] = x;
     }
     if (lane == 0) {
-        atomicAdd(&k.acc[ACC_ENERGY], e_sum);
-        atomicAdd(k.pair_counter, n_pairs);
+        sums[9] = e_sum;
+        sums[10] = (double)n_pairs;
+    }
+    __syncthreads();
+    if (threadIdx.x < 11) {
+        double x = 0.0;
+        for (int w = 0; w < F64_TILE; ++w) x += reinterpret_cast<const double *>(smem_raw)[w * 11 + threadIdx.x];
+        if (threadIdx.x == 10) atomicAdd(k.pair_counter, (unsigned long long)x);
+        else atomicAdd(&k.acc[threadIdx.x < 9 ? ACC_VIRIAL + threadIdx.x : ACC_ENERGY], x);
     }
 }
 
