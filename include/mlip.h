@@ -272,14 +272,15 @@ int mlip_sync_status(mlip_ctx *ctx);
 /* Counters for reports: list entries, pairs inside r_cut at the last evaluation (syncs), kernels launched. */
 int mlip_get_counters(mlip_ctx *ctx, int64_t *n_list_entries, int64_t *n_pairs_in_cutoff, int64_t *n_launches);
 /*
- * CUDA-event time of the fused-kernel launches since the last reset: number of launches timed
- * and their summed duration in ms (each launch is bracketed by its own event pair on the
- * launching stream; the most recent 256 launches are kept).  Synchronises on the last event.
+ * Device time of the fused-kernel launches since the last reset: number of launches timed
+ * and their summed duration in ms (each launch lies between two CUDA events on the launching stream; below
+ * 100,000 atoms, where events would cost a tenth of a step, the kernels record the device's timer at their begin and
+ * end instead; the most recent 256 launches are kept).  Synchronises with the last of them.
  */
 int mlip_kernel_time(mlip_ctx *ctx, int64_t *n_launches, double *total_ms, int reset);
 
 /*
- * Device time (CUDA events on the launching streams, ms) of the three parts of the path since the last reset:
+ * Device time (taken as for mlip_kernel_time, ms) of the three parts of the path since the last reset:
  * list builds (binning + count + fill), fused-kernel launches, integrator kernels (kicks, drift, thermostat).
  * Each part keeps its last 256 records.  Waits for the recorded events; reset != 0 clears all three (and the
  * record of mlip_kernel_time).  Any pointer may be NULL.

@@ -247,11 +247,9 @@ int mlip_create(mlip_ctx **out, const mlip_config *cfg, const double *enc_w, siz
     c->n_sm = prop.multiProcessorCount;
     do {
         if ((rc = dev_alloc(c, &c->mass, (size_t)cfg->n_species)) != MLIP_OK) break;
-        if ((rc = dev_alloc(c, &c->launch_block, (size_t)LB_COUNT)) != MLIP_OK) break;
-        c->tile_counter = reinterpret_cast<int *>(c->launch_block);
-        c->pair_counter = reinterpret_cast<unsigned long long *>(c->launch_block + LB_PAIR);
-        c->acc_fx = reinterpret_cast<long long *>(c->launch_block + LB_ACC_FX);
-        c->acc = c->launch_block + LB_ACC;
+        if ((rc = dev_alloc(c, &c->launch_base, (size_t)2 * LB_COUNT)) != MLIP_OK) break;
+        next_eval_block(c);
+        if ((rc = dev_alloc(c, &c->stamp, (size_t)2 * mlip_ctx::STAMPS)) != MLIP_OK) break;
         if ((rc = dev_alloc(c, &c->build_word, 8)) != MLIP_OK) break;
         c->status = c->build_word + 4; c->rebuild_flag = c->build_word + 5; c->far_flag = c->build_word + 6;
         if ((rc = dev_alloc(c, &c->nhc, 8)) != MLIP_OK) break;
@@ -269,7 +267,7 @@ int mlip_create(mlip_ctx **out, const mlip_config *cfg, const double *enc_w, siz
         if (!ev_ok) { rc = MLIP_ERR_CUDA; c->err = "event creation failed"; break; }
         if (cudaMemcpy(c->mass, mass, sizeof(double) * cfg->n_species, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemset(c->build_word, 0, sizeof(int) * 8) != cudaSuccess ||
-            cudaMemset(c->nhc, 0, sizeof(double) * 8) != cudaSuccess || cudaMemset(c->kin_part, 0, sizeof(double) * 1185) != cudaSuccess || cudaMemset(c->launch_block, 0, sizeof(double) * LB_COUNT) != cudaSuccess) {
+            cudaMemset(c->nhc, 0, sizeof(double) * 8) != cudaSuccess || cudaMemset(c->kin_part, 0, sizeof(double) * 1185) != cudaSuccess || cudaMemset(c->launch_base, 0, sizeof(double) * 2 * LB_COUNT) != cudaSuccess) {
             rc = MLIP_ERR_CUDA; c->err = "initial upload failed"; break;
         }
         rc = build_tables(c, enc_w, n_enc);
@@ -637,6 +635,18 @@ static int marks_total(mlip_ctx *c, unsigned char kind, int64_t *count, double *
         total += ms;
         kept += 1;
     }
+    if (c->stamps > c->stamp_reset[kind]) {   // parts timed by the kernels themselves
+        constexpr int S = mlip_ctx::STAMPS, H = S / 2;
+        std::vector<unsigned long long> t(2 * S);
+        MLIP_CUDA_TRY(c, cudaStreamSynchronize(c->mark_stream));
+        MLIP_CUDA_TRY(c, cudaMemcpy(t.data(), c->stamp, sizeof(unsigned long long) * 2 * S, cudaMemcpyDeviceToHost));
+        const int64_t first = std::max<int64_t>(c->stamp_reset[kind], (c->stamps - 1) / H * H - H);   // the half being filled and the one before
+        for (int64_t m = c->stamps - 1; m >= std::max<int64_t>(0, first) && kept < mlip_ctx::EV_POOL; --m) {
+            if (c->stamp_kind[m % S] != kind || t[S + m % S] < t[m % S]) continue;
+            total += 1e-6 * (double)(t[S + m % S] - t[m % S]);
+            kept += 1;
+        }
+    }
     if (count) *count = kept;
     *total_ms = total;
     return MLIP_OK;
@@ -648,7 +658,7 @@ int mlip_kernel_time(mlip_ctx *c, int64_t *n_launches, double *total_ms, int res
     const int rc = marks_total(c, MARK_KERNEL, n_launches, &total);
     if (rc != MLIP_OK) return rc;
     if (total_ms) *total_ms = total;
-    if (reset) c->mark_reset[MARK_KERNEL] = c->marks;
+    if (reset) { c->mark_reset[MARK_KERNEL] = c->marks; c->stamp_reset[MARK_KERNEL] = c->stamps; }
     return MLIP_OK;
 }
 
@@ -662,7 +672,8 @@ int mlip_get_timings(mlip_ctx *c, double *ms_build, double *ms_kernel, double *m
     if (ms_build) *ms_build = b;
     if (ms_kernel) *ms_kernel = k;
     if (ms_integrate) *ms_integrate = i;
-    if (reset) for (int64_t &r : c->mark_reset) r = c->marks;
+    if (reset)
+        for (int q = 0; q < 4; ++q) { c->mark_reset[q] = c->marks; c->stamp_reset[q] = c->stamps; }
     return MLIP_OK;
 }
 
@@ -685,7 +696,7 @@ void mlip_destroy(mlip_ctx *c) {
     free_cells(c);
     cudaFree(c->nbr); cudaFree(c->scan_tmp); cudaFree(c->head_w); cudaFree(c->table); cudaFree(c->mass);
     cudaFree(c->head_w_d); cudaFree(c->table_d);
-    cudaFree(c->launch_block); cudaFree(c->build_word); cudaFree(c->nhc);
+    cudaFree(c->launch_base); cudaFree(c->stamp); cudaFree(c->build_word); cudaFree(c->nhc);
     cudaFree(c->species_start); cudaFree(c->stage_pos); cudaFree(c->stage_species); cudaFree(c->stage_force);
     cudaFree(c->stage_out); cudaFree(c->kin_part);
     if (c->status_host) cudaFreeHost(c->status_host);

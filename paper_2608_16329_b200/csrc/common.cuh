@@ -44,7 +44,8 @@ enum : int {
 // accumulator slots (double)
 enum : int { ACC_ENERGY = 0, ACC_VIRIAL = 1, ACC_KINETIC = 10, ACC_COUNT = 32 };
 // launch_block in doubles: [0, 4) tile_counter (MAX_SPECIES ints), [4] pair_counter, [5, 15) acc_fx, [16, 16 + ACC_COUNT) acc;
-// everything up to the kinetic-energy slot of acc is cleared before every fused-kernel launch
+// everything up to the kinetic-energy slot of acc is zero when a fused kernel starts.  There are two such blocks: an evaluation uses one
+// and clears the other, which holds the totals of the evaluation before it, for the next
 constexpr int LB_PAIR = 4, LB_ACC_FX = 5, LB_ACC = 16, LB_COUNT = LB_ACC + ACC_COUNT;
 constexpr size_t LAUNCH_CLEAR_BYTES = sizeof(double) * (LB_ACC + ACC_KINETIC);
 static_assert(MAX_SPECIES * sizeof(int) <= LB_PAIR * sizeof(double), "tile counters must fit before the pair counter");
@@ -124,14 +125,16 @@ struct mlip_ctx {
     int32_t *cell_id = nullptr;    // [N] build-time cell of each atom as packed coordinates, internal order (allocated for list_format = 1)
     unsigned long long *tile_state = nullptr;   // [tile_words(N)] look-back words of the one-pass build
     int *build_word = nullptr;     // {ticket, private overflow flag, total entries (64 bits)} of the one-pass build, then status, rebuild_flag, far_flag
+    float4 *rel_pos = nullptr;     // cell-relative positions of the build in progress
     int *build_host = nullptr;     // pinned copy of its first five words
     int64_t nbr_cap = 0, n_entries = 0;
     // scratch
     int64_t *scan_tmp = nullptr;   // block sums for the scans
     int64_t scan_tmp_cap = 0;
-    double *launch_block = nullptr;   // one allocation: tile_counter, pair_counter, acc_fx, acc back to back, so that a launch
-                                      // clears its counters and accumulators in one go (LAUNCH_CLEAR_BYTES)
-    double *acc = nullptr;         // [ACC_COUNT] (inside launch_block)
+    double *launch_base = nullptr;    // [2][LB_COUNT]: tile_counter, pair_counter, acc_fx, acc back to back, twice; the pointers are into
+                                      // the block of the last evaluation
+    int eval_block = 0;
+    double *acc = nullptr;         // [ACC_COUNT] (inside launch_base)
     double *kin_part = nullptr;    // [1184] per-block kinetic-energy sums, then the ticket of the last block (integrate.cu)
     unsigned long long *pair_counter = nullptr;
     int *status = nullptr;         // device status word
@@ -155,7 +158,7 @@ struct mlip_ctx {
     int64_t launches = 0;
     size_t resident = 0;
     cudaStream_t last_stream = nullptr;
-    bool force_cleared = false, block_cleared = false;   // the forces / the counters and totals were cleared for the next evaluation by a kernel before it
+    bool force_cleared = false;    // the forces were cleared for the next evaluation by a kernel before it
     // Timing marks: a ring of events, each the end of a timed part that began at the mark before it (consecutive parts share
     // a mark), or the beginning of one.
     static constexpr int EV_POOL = 256, MARKS = 4 * EV_POOL;
@@ -165,6 +168,12 @@ struct mlip_ctx {
     int64_t mark_reset[4] = {0};   // per kind: parts that ended before this mark have been reset
     bool mark_open = false;        // nothing untimed has been enqueued since the last mark
     cudaStream_t mark_stream = nullptr;
+    // Below STAMP_BELOW_ATOMS the kernels of a step write their own begin and end times instead: an event between two kernels costs
+    // some 1.5 us and keeps the second from starting early.  Ring in two halves, each reset (begin all ones, end zero) on entry.
+    static constexpr int STAMPS = 8 * EV_POOL;
+    unsigned long long *stamp = nullptr;   // dev: begin [STAMPS], end [STAMPS], nanoseconds of the device's timer
+    unsigned char stamp_kind[STAMPS] = {0};
+    int64_t stamps = 0, stamp_reset[4] = {0};
 };
 
 namespace mlip {
@@ -194,6 +203,71 @@ inline void mark_end(mlip_ctx *c, unsigned char kind, cudaStream_t s) {
     c->mark_open = true;
     c->mark_stream = s;
 }
+
+// A timed kernel of a step: where it writes its times, or nullptr after recording a mark.  timed_end after its launch.
+constexpr int64_t STAMP_BELOW_ATOMS = 100000;   // (about 0.6 ms a step: what the events cost is below 1 % from there on)
+inline unsigned long long *timed_begin(mlip_ctx *c, unsigned char kind, cudaStream_t s) {
+    if (c->n >= STAMP_BELOW_ATOMS) { mark_begin(c, s); return nullptr; }
+    constexpr int R = mlip_ctx::STAMPS, H = R / 2;
+    const int slot = (int)(c->stamps % R);
+    if (slot % H == 0) {
+        cudaMemsetAsync(c->stamp + slot, 0xff, sizeof(unsigned long long) * H, s);
+        cudaMemsetAsync(c->stamp + R + slot, 0, sizeof(unsigned long long) * H, s);
+    }
+    c->stamp_kind[slot] = kind;
+    c->stamps += 1;
+    c->mark_stream = s;
+    c->mark_open = false;
+    return c->stamp + slot;
+}
+inline void timed_end(mlip_ctx *c, unsigned char kind, cudaStream_t s) { if (c->n >= STAMP_BELOW_ATOMS) mark_end(c, kind, s); }
+__device__ __forceinline__ unsigned long long device_time() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+__device__ __forceinline__ void stamp_begin(unsigned long long *stamp) { if (stamp && threadIdx.x == 0) atomicMin(stamp, device_time()); }
+__device__ __forceinline__ void stamp_end(unsigned long long *stamp) { if (stamp && threadIdx.x == 0) atomicMax(stamp + mlip_ctx::STAMPS, device_time()); }
+
+// Programmatic dependent launch: a kernel launched with launch_after may start while the kernel before it on the stream is running
+// (once that one's blocks have all called allow_next or ended) and calls wait_previous before it touches anything an earlier
+// kernel of the stream writes or reads.  Every kernel launched this way waits in all its threads, so that "the previous kernel is
+// complete" holds back along the chain.  Loads of what such kernels exchange must not be marked read-only (const __restrict__, __ldg): the
+// compiler may move those across the wait.
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t launch_after(void (*kernel)(P...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// The counters and totals of a new evaluation become current; returns the other block, which the evaluation clears.
+inline double *next_eval_block(mlip_ctx *c) {
+    double *clear = c->launch_base + (size_t)c->eval_block * LB_COUNT;
+    c->eval_block ^= 1;
+    double *b = c->launch_base + (size_t)c->eval_block * LB_COUNT;
+    c->tile_counter = reinterpret_cast<int *>(b);
+    c->pair_counter = reinterpret_cast<unsigned long long *>(b + LB_PAIR);
+    c->acc_fx = reinterpret_cast<long long *>(b + LB_ACC_FX);
+    c->acc = b + LB_ACC;
+    return clear;
+}
+
+struct EvalClear {
+    float4 *force;       // nullptr: not accumulated into (deterministic mode, fp64 contexts)
+    double *force_d;     // fp64 contexts
+};
+EvalClear eval_clear(mlip_ctx *c);   // integrate.cu
 
 // neighbor.cu
 int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int32_t *species, cudaStream_t s);

@@ -7,24 +7,17 @@
 namespace mlip {
 
 // Force on atom i: the fp64 array when the context evaluates in fp64, else the fp32 one.
-__device__ __forceinline__ double3 load_force(const float4 *__restrict__ force, const double *__restrict__ force_d, int64_t i) {
+__device__ __forceinline__ double3 load_force(const float4 *force, const double *force_d, int64_t i) {
     if (force_d) return make_double3(force_d[3 * i], force_d[3 * i + 1], force_d[3 * i + 2]);
     const float4 f = force[i];
     return make_double3(f.x, f.y, f.z);
 }
 
-// What the evaluation that follows a move accumulates into: forces, and the counters and totals at the head of launch_block.  The kernels
-// that move atoms clear them on the way (a separate clear is a launch, and for the forces a pass, of its own).
-struct EvalClear {
-    float4 *force;       // nullptr: not accumulated into (deterministic mode, fp64 contexts)
-    double *force_d;     // fp64 contexts
-    double *launch_block;
-};
+// The forces that the evaluation after a move accumulates into: the kernels that move atoms clear them on the way (a separate clear is a
+// launch and a pass of its own).
 __device__ __forceinline__ void clear_for_eval(const EvalClear &c, int64_t i) {
     if (c.force) c.force[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (c.force_d) { c.force_d[3 * i] = 0.0; c.force_d[3 * i + 1] = 0.0; c.force_d[3 * i + 2] = 0.0; }
-    if (i == 0 && c.launch_block)
-        for (int q = 0; q < (int)(LAUNCH_CLEAR_BYTES / sizeof(double)); ++q) c.launch_block[q] = 0.0;
 }
 
 // v += dt/2 a  (CLOSE: twice, the second half kick of one step and the first of the next, which see the same forces);
@@ -32,10 +25,12 @@ __device__ __forceinline__ void clear_for_eval(const EvalClear &c, int64_t i) {
 // a trajectory does not depend on how it is cut into calls.
 template <bool CLOSE>
 __global__ void k_kick_drift(int64_t n, double dt, CellGrid g, const double *__restrict__ mass, float skin_half2,
-                             double4 *__restrict__ pos4, double *__restrict__ vel, const float4 *force,
-                             const double *force_d, float *__restrict__ disp, int *status, float trigger2,
-                             int *rebuild_flag, const double *__restrict__ vscale, float far2, int *far_flag, EvalClear clear) {
+                             double4 *pos4, double *vel, const float4 *force, const double *force_d, float *disp, int *status, float trigger2,
+                             int *rebuild_flag, const double *vscale, float far2, int *far_flag, EvalClear clear, unsigned long long *stamp) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    allow_next();
+    wait_previous();
+    stamp_begin(stamp);
     if (i >= n) return;
     double4 p = pos4[i];
     const double3 f3 = load_force(force, force_d, i);
@@ -64,16 +59,21 @@ __global__ void k_kick_drift(int64_t n, double dt, CellGrid g, const double *__r
     if (!(d2 <= far2)) *far_flag = 1;       // from now on the lists' far entries may come inside r_cut
     pos4[i] = make_double4(x[0], x[1], x[2], p.w);
     clear_for_eval(clear, i);
+    stamp_end(stamp);
 }
 
 // v += dt/2 a
-__global__ void k_kick(int64_t n, double dt, const double *__restrict__ mass, const double4 *__restrict__ pos4,
-                       double *__restrict__ vel, const float4 *__restrict__ force, const double *__restrict__ force_d) {
+__global__ void k_kick(int64_t n, double dt, const double *__restrict__ mass, const double4 *pos4, double *vel, const float4 *force,
+                       const double *force_d, unsigned long long *stamp) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    allow_next();
+    wait_previous();
+    stamp_begin(stamp);
     if (i >= n) return;
     const double3 f = load_force(force, force_d, i);
     const double k = 0.5 * dt * ACC_UNIT / mass[(int)pos4[i].w];
     vel[3 * i] = fma(k, f.x, vel[3 * i]); vel[3 * i + 1] = fma(k, f.y, vel[3 * i + 1]); vel[3 * i + 2] = fma(k, f.z, vel[3 * i + 2]);
+    stamp_end(stamp);
 }
 
 // Half-step (dt/2) of a Nose-Hoover chain of three thermostats coupled to the kinetic energy in acc[ACC_KINETIC]
@@ -110,9 +110,13 @@ __device__ void nhc_half(const NhcHalf &h, double *acc) {
     acc[ACC_KINETIC] = 0.5 * ke2;
 }
 
-__global__ void k_scale_velocities(int64_t n3, double *__restrict__ vel, const double *__restrict__ scale) {
+__global__ void k_scale_velocities(int64_t n3, double *vel, const double *scale, unsigned long long *stamp) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    allow_next();
+    wait_previous();
+    stamp_begin(stamp);
     if (i < n3) vel[i] *= *scale;
+    stamp_end(stamp);
 }
 
 // Kinetic energy with a fixed summation order (grid-stride partial sums per block, then one warp of the block that finishes last
@@ -122,11 +126,14 @@ __global__ void k_scale_velocities(int64_t n3, double *__restrict__ vel, const d
 // 4,394 atoms 152 us per step, of which the evaluation was 65.)
 constexpr int KIN_BLOCKS = 1184;
 template <int CHANGE>
-__global__ void __launch_bounds__(256) k_kinetic(int64_t n, double dt, const double *__restrict__ mass, const double4 *__restrict__ pos4, double *vel,
-                                                 const float4 *__restrict__ force, const double *__restrict__ force_d, const double *scale,
-                                                 double *block_sum, unsigned int *ticket, double *acc, NhcHalf nhc) {
+__global__ void __launch_bounds__(256) k_kinetic(int64_t n, double dt, const double *__restrict__ mass, const double4 *pos4, double *vel, const float4 *force,
+                                                 const double *force_d, const double *scale, double *block_sum, unsigned int *ticket, double *acc,
+                                                 NhcHalf nhc, unsigned long long *stamp) {
     __shared__ double part[8];
     __shared__ bool last;
+    allow_next();
+    wait_previous();
+    stamp_begin(stamp);
     double e = 0.0;
     const double sc = CHANGE == 2 ? *scale : 1.0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -162,15 +169,17 @@ __global__ void __launch_bounds__(256) k_kinetic(int64_t n, double dt, const dou
         *ticket = 0;
         acc[ACC_KINETIC] = e / ACC_UNIT;
         if (nhc.state) nhc_half(nhc, acc);
+        stamp_end(stamp);
     }
 }
 
 // Per-atom outputs in the caller's order, and the totals: one launch.  FIN: float4, or double for three per atom.
 template <typename FIN, typename EIN, typename FOUT>
-__global__ void k_outputs(int64_t n, const int32_t *__restrict__ user_of, const FIN *__restrict__ force, const EIN *__restrict__ e_in,
-                          FOUT *__restrict__ forces_out, FOUT *__restrict__ e_atom, const double *__restrict__ acc, double *__restrict__ energy,
+__global__ void k_outputs(int64_t n, const int32_t *__restrict__ user_of, const FIN *force, const EIN *e_in,
+                          FOUT *__restrict__ forces_out, FOUT *__restrict__ e_atom, const double *acc, double *__restrict__ energy,
                           double *__restrict__ virial) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    wait_previous();
     if (i == 0) {
         if (energy) *energy = acc[ACC_ENERGY];
         if (virial)
@@ -190,10 +199,12 @@ __global__ void k_outputs(int64_t n, const int32_t *__restrict__ user_of, const 
     if (e_atom) e_atom[u] = (FOUT)e_in[i];
 }
 
-__global__ void k_set_positions(int64_t n, const int32_t *__restrict__ user_of, const double *__restrict__ pos,
-                                CellGrid g, float skin_half2, double4 *__restrict__ pos4, float *__restrict__ disp, int *status,
+__global__ void k_set_positions(int64_t n, const int32_t *__restrict__ user_of, const double *pos,
+                                CellGrid g, float skin_half2, double4 *pos4, float *disp, int *status,
                                 float far2, int *far_flag, EvalClear clear) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    allow_next();
+    wait_previous();
     if (i >= n) return;
     clear_for_eval(clear, i);
     const int64_t u = user_of[i];
@@ -238,74 +249,65 @@ static inline float skin_half2(const mlip_ctx *c) { float h = 0.5f * (float)c->c
 // stay outside r_cut while every atom has moved less than skin / 4 (0.245: room for the fp32 bookkeeping).
 static inline float far_trigger2(const mlip_ctx *c) { float h = 0.245f * (float)c->cfg.skin; return h * h; }
 
-// The buffers of the next evaluation, to be cleared by the kernel that takes this, which must be the last before it on the stream.
-// `totals`: the evaluation follows in the same call, so nobody reads the last one's energy and counters in between.
-static EvalClear eval_clear(mlip_ctx *c, bool totals) {
+// The forces of the next evaluation, to be cleared by the kernel that takes this, which must be the last before it that reads them.
+EvalClear eval_clear(mlip_ctx *c) {
     c->force_cleared = true;
-    if (totals) c->block_cleared = true;
     const bool f64 = c->cfg.precision == 1;
-    return EvalClear{f64 || c->cfg.force_mode == 1 ? nullptr : c->force, f64 ? c->force_d : nullptr, totals ? c->launch_block : nullptr};
+    return EvalClear{f64 || c->cfg.force_mode == 1 ? nullptr : c->force, f64 ? c->force_d : nullptr};
 }
 int launch_kick_drift(mlip_ctx *c, double dt, bool close_step, cudaStream_t s, const double *vscale) {
-    mark_begin(c, s);
-    const EvalClear clear = eval_clear(c, true);
-    auto *kernel = close_step ? k_kick_drift<true> : k_kick_drift<false>;
-    kernel<<<nb(c->n), 256, 0, s>>>(c->n, dt, c->grid, c->mass, skin_half2(c), c->pos4, c->vel, c->force, c->force_d, c->disp, c->status,
-                                    0.64f * skin_half2(c), c->rebuild_flag, vscale, far_trigger2(c), c->far_flag, clear);
-    mark_end(c, MARK_INTEGRATE, s);
+    unsigned long long *stamp = timed_begin(c, MARK_INTEGRATE, s);
+    MLIP_CUDA_TRY(c, launch_after(close_step ? k_kick_drift<true> : k_kick_drift<false>, nb(c->n), 256, 0, s, c->n, dt, c->grid, c->mass, skin_half2(c),
+                                  c->pos4, c->vel, c->force, c->force_d, c->disp, c->status, 0.64f * skin_half2(c), c->rebuild_flag, vscale,
+                                  far_trigger2(c), c->far_flag, eval_clear(c), stamp));
+    timed_end(c, MARK_INTEGRATE, s);
     c->launches += 1;
-    MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
 int launch_kick(mlip_ctx *c, double dt, cudaStream_t s) {
-    mark_begin(c, s);
-    k_kick<<<nb(c->n), 256, 0, s>>>(c->n, dt, c->mass, c->pos4, c->vel, c->force, c->force_d);
-    mark_end(c, MARK_INTEGRATE, s);
+    unsigned long long *stamp = timed_begin(c, MARK_INTEGRATE, s);
+    MLIP_CUDA_TRY(c, launch_after(k_kick, nb(c->n), 256, 0, s, c->n, dt, c->mass, c->pos4, c->vel, c->force, c->force_d, stamp));
+    timed_end(c, MARK_INTEGRATE, s);
     c->launches += 1;
-    MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
 int launch_scale_velocities(mlip_ctx *c, cudaStream_t s) {
-    mark_begin(c, s);
-    k_scale_velocities<<<nb(3 * c->n), 256, 0, s>>>(3 * c->n, c->vel, c->nhc + 6);
-    mark_end(c, MARK_INTEGRATE, s);
+    unsigned long long *stamp = timed_begin(c, MARK_INTEGRATE, s);
+    MLIP_CUDA_TRY(c, launch_after(k_scale_velocities, nb(3 * c->n), 256, 0, s, 3 * c->n, c->vel, c->nhc + 6, stamp));
+    timed_end(c, MARK_INTEGRATE, s);
     c->launches += 1;
-    MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
 int launch_kinetic(mlip_ctx *c, int change, bool thermostat, double dt, cudaStream_t s) {
-    int64_t blocks = nb(c->n);
-    if (blocks > KIN_BLOCKS) blocks = KIN_BLOCKS;
+    const int64_t blocks = nb(c->n) > KIN_BLOCKS ? KIN_BLOCKS : nb(c->n);
     const NhcHalf nhc{c->nhc_nf, c->nhc_kT, c->nhc_q1, c->nhc_qk, dt, thermostat ? c->nhc : nullptr};
-    auto *kernel = change == 1 ? k_kinetic<1> : change == 2 ? k_kinetic<2> : k_kinetic<0>;
-    if (thermostat) mark_begin(c, s);
-    kernel<<<(unsigned)blocks, 256, 0, s>>>(c->n, dt, c->mass, c->pos4, c->vel, c->force, c->force_d, c->nhc + 6, c->kin_part,
-                                            reinterpret_cast<unsigned int *>(c->kin_part + KIN_BLOCKS), c->acc, nhc);
-    if (thermostat) mark_end(c, MARK_INTEGRATE, s);
+    unsigned long long *stamp = thermostat ? timed_begin(c, MARK_INTEGRATE, s) : nullptr;
+    MLIP_CUDA_TRY(c, launch_after(change == 1 ? k_kinetic<1> : change == 2 ? k_kinetic<2> : k_kinetic<0>, (unsigned)blocks, 256, 0, s, c->n, dt, c->mass,
+                                  c->pos4, c->vel, c->force, c->force_d, c->nhc + 6, c->kin_part, reinterpret_cast<unsigned int *>(c->kin_part + KIN_BLOCKS),
+                                  c->acc, nhc, stamp));
+    if (thermostat) timed_end(c, MARK_INTEGRATE, s);
     c->launches += 1;
-    MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
 int launch_outputs(mlip_ctx *c, float *forces, float *e_atom, double *energy, double *virial, cudaStream_t s) {
     const unsigned blocks = forces || e_atom ? nb(c->n) : 1;
-    if (c->cfg.precision == 1) k_outputs<double, double, float><<<blocks, 256, 0, s>>>(c->n, c->user_of, c->force_d, c->e_atom_d, forces, e_atom, c->acc, energy, virial);
-    else k_outputs<float4, float, float><<<blocks, 256, 0, s>>>(c->n, c->user_of, c->force, c->e_atom, forces, e_atom, c->acc, energy, virial);
+    if (c->cfg.precision == 1)
+        MLIP_CUDA_TRY(c, launch_after(k_outputs<double, double, float>, blocks, 256, 0, s, c->n, c->user_of, c->force_d, c->e_atom_d, forces, e_atom, c->acc, energy, virial));
+    else
+        MLIP_CUDA_TRY(c, launch_after(k_outputs<float4, float, float>, blocks, 256, 0, s, c->n, c->user_of, c->force, c->e_atom, forces, e_atom, c->acc, energy, virial));
     c->launches += 1;
-    MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
 int launch_outputs_f64(mlip_ctx *c, double *forces, double *e_atom, double *energy, double *virial, cudaStream_t s) {
     const unsigned blocks = forces || e_atom ? nb(c->n) : 1;
-    k_outputs<double, double, double><<<blocks, 256, 0, s>>>(c->n, c->user_of, c->force_d, c->e_atom_d, forces, e_atom, c->acc, energy, virial);
+    MLIP_CUDA_TRY(c, launch_after(k_outputs<double, double, double>, blocks, 256, 0, s, c->n, c->user_of, c->force_d, c->e_atom_d, forces, e_atom, c->acc, energy, virial));
     c->launches += 1;
-    MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
 int launch_set_positions(mlip_ctx *c, const double *pos, cudaStream_t s) {
-    const EvalClear clear = eval_clear(c, false);
-    k_set_positions<<<nb(c->n), 256, 0, s>>>(c->n, c->user_of, pos, c->grid, skin_half2(c), c->pos4, c->disp, c->status, far_trigger2(c), c->far_flag, clear);
+    MLIP_CUDA_TRY(c, launch_after(k_set_positions, nb(c->n), 256, 0, s, c->n, c->user_of, pos, c->grid, skin_half2(c), c->pos4, c->disp, c->status,
+                                  far_trigger2(c), c->far_flag, eval_clear(c)));
     c->launches += 1;
-    MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
 int launch_set_velocities(mlip_ctx *c, const double *vel, cudaStream_t s) {

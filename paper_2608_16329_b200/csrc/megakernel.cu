@@ -226,6 +226,8 @@ struct KernelArgs {
     unsigned long long *pair_counter;
     int *status;
     int *tile_counter;
+    double *clear_block;       // the other evaluation block (next_eval_block)
+    unsigned long long *stamp;
 };
 
 // One 256-bit load per gathered atom (a 32-byte sector) instead of two 128-bit ones: halves the
@@ -931,11 +933,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
     float *hc = scr_all + NW * LY::WARP;
     int *ctl = reinterpret_cast<int *>(hc + HC_WORDS);
     const int rows = k.tab.knots + 3;
-    // lists that an in-step rebuild could not complete (capacity, broken configuration) are not evaluated: the outputs
-    // stay at their cleared values and the status word tells the caller why (nothing in this kernel raises these bits,
-    // so every CTA takes the same decision)
-    if (*k.status & (FLAG_NEIGHBOR_OVERFLOW | FLAG_NONFINITE)) return;
-    const bool use_far = *k.far_flag != 0;   // an atom has moved skin / 4 since the build: every list entry counts
+    allow_next();
 
     // all of tensor memory (this is the only CTA on the SM) for the head's weights
     if (warp == 0) {
@@ -957,24 +955,16 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
     PhaseClock pc;
     pc.start();
 
-    // STAGGER (small systems): the CTAs start on different central species, so that the species are worked on side by
-    // side rather than one after the other by mostly idle SMs (864 atoms: 64 instead of 92 us).  Large systems keep the
-    // plain loop: one front through the cell-ordered atoms, and a loop counter as the species costs 1 % less than a
-    // computed one.  Either way a species whose tiles are all claimed already is passed over: staging its tables would
-    // be the only thing left to do.
-    for (int ss = 0; ss < k.n_species; ++ss) {
-        const int species = STAGGER ? (int)((ss + blockIdx.x) % (unsigned)k.n_species) : ss;
-        const int s_beg = __ldg(k.species_start + species), s_end = __ldg(k.species_start + species + 1);
-        const int n_tiles = (s_end - s_beg + NA - 1) / NA;
-        if (n_tiles == 0) continue;
-        if (threadIdx.x == 0) ctl[6 + (ss & 1)] = *reinterpret_cast<volatile int *>(k.tile_counter + species);
-        __syncthreads();   // both groups are done with the previous species' tables
-        if (ctl[6 + (ss & 1)] >= n_tiles) continue;
+    // the tables and weights of a species
+    auto stage = [&](int species) {
         const float *tab = k.tab.coef + (size_t)species * k.n_species * rows * K_RADIAL;
         if (TAB_SMEM) {
             const float4 *src = reinterpret_cast<const float4 *>(tab);
             const int n4 = k.n_species * rows * (K_RADIAL / 4);
-            for (int idx = threadIdx.x; idx < n4; idx += NW * 32) reinterpret_cast<float4 *>(s_tab)[idx] = __ldg(src + idx);
+#pragma unroll 4
+            for (int idx = threadIdx.x; idx < n4; idx += NW * 32)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(reinterpret_cast<float4 *>(s_tab) + idx)), "l"(src + idx) : "memory");
+            asm volatile("cp.async.commit_group;" ::: "memory");
             tv.base = s_tab; tv.saddr = smem_addr(s_tab);
         } else {
             tv.base = tab; tv.saddr = 0;
@@ -982,9 +972,37 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
         const uint32_t *hp = k.head_pack + (size_t)species * HP_TOTAL;
         for (int idx = threadIdx.x; idx < HC_USED; idx += NW * 32) hc[idx] = __uint_as_float(__ldg(hp + HP_TMEM + idx));
         tmem_fill(tm_quarter, hp, warp, lane);
+        if (TAB_SMEM) asm volatile("cp.async.wait_group 0;" ::: "memory");
         tmem_fence_before_sync();
         __syncthreads();
         tmem_fence_after_sync();
+    };
+    // STAGGER (small systems): the CTAs start on different central species, so that the species are worked on side by
+    // side rather than one after the other by mostly idle SMs (864 atoms: 64 instead of 92 us).  Large systems keep the
+    // plain loop: one front through the cell-ordered atoms, and a loop counter as the species costs 1 % less than a
+    // computed one.  Either way a species whose tiles are all claimed already is passed over: staging its tables would
+    // be the only thing left to do.
+    auto species_at = [&](int ss) { return STAGGER ? (int)((ss + blockIdx.x) % (unsigned)k.n_species) : ss; };
+    // The first species is staged ahead of the wait for the kernel before this one (model data only up to here), in whose shadow it then
+    // lies: staging is some 4 us of a small system's 30.
+    stage(species_at(0));
+    wait_previous();
+    stamp_begin(k.stamp);
+    if (blockIdx.x == 0 && threadIdx.x < (int)(LAUNCH_CLEAR_BYTES / sizeof(double))) k.clear_block[threadIdx.x] = 0.0;
+    // lists that an in-step rebuild could not complete (capacity, broken configuration) are not evaluated: the outputs
+    // stay at their cleared values and the status word tells the caller why (nothing in this kernel raises these bits,
+    // so every CTA takes the same decision)
+    const bool skip = (*k.status & (FLAG_NEIGHBOR_OVERFLOW | FLAG_NONFINITE)) != 0;
+    const bool use_far = *k.far_flag != 0;   // an atom has moved skin / 4 since the build: every list entry counts
+    for (int ss = 0; ss < k.n_species && !skip; ++ss) {
+        const int species = species_at(ss);
+        const int s_beg = __ldg(k.species_start + species), s_end = __ldg(k.species_start + species + 1);
+        const int n_tiles = (s_end - s_beg + NA - 1) / NA;
+        if (n_tiles == 0) continue;
+        if (threadIdx.x == 0) ctl[6 + (ss & 1)] = *reinterpret_cast<volatile int *>(k.tile_counter + species);
+        __syncthreads();   // both groups are done with the previous species' tables
+        if (ctl[6 + (ss & 1)] >= n_tiles) continue;
+        if (ss > 0) stage(species);
 
         bool prefetched = false;   // this warp's atom of the coming tile sits in the prefetch buffer
         int look_ahead = -1;       // (group leader) the tile after the current one
@@ -1171,6 +1189,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
             if (x != 0.0) atomicAdd(&k.acc[threadIdx.x < 9 ? ACC_VIRIAL + threadIdx.x : ACC_ENERGY], x);
         }
     }
+    stamp_end(k.stamp);
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm_base), "r"(TM_COLS) : "memory");
 }
 
@@ -1292,9 +1311,10 @@ int upload_head(mlip_ctx *c, const double *w) {
 }
 
 // Deterministic mode: integer sums -> the float / double outputs the rest of the library reads; the sums start the next evaluation at zero.
-__global__ void k_fixed_finish(int64_t n, long long *__restrict__ force_fx, const long long *__restrict__ acc_fx,
-                               float4 *__restrict__ force, double *__restrict__ acc) {
+__global__ void k_fixed_finish(int64_t n, long long *force_fx, const long long *acc_fx, float4 *force, double *acc, unsigned long long *stamp) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    allow_next();
+    wait_previous();
     if (i < n) {
         const double inv = 1.0 / (double)FORCE_FX;
         force[i] = make_float4((float)((double)force_fx[3 * i] * inv), (float)((double)force_fx[3 * i + 1] * inv),
@@ -1305,17 +1325,18 @@ __global__ void k_fixed_finish(int64_t n, long long *__restrict__ force_fx, cons
         acc[ACC_ENERGY] = (double)acc_fx[0] / ENERGY_FX;
         for (int q = 0; q < 9; ++q) acc[ACC_VIRIAL + q] = (double)acc_fx[1 + q] / VIRIAL_FX;
     }
+    stamp_end(stamp);
 }
 
 int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     const int64_t n = c->n;
     const bool det = c->cfg.force_mode == 1;
-    if (!(c->force_cleared || det) || !c->block_cleared) {
+    if (!c->force_cleared && !det) {   // (k_fixed_finish keeps the integer sums clear)
         c->mark_open = false;
-        if (!c->force_cleared && !det) MLIP_CUDA_TRY(c, cudaMemsetAsync(c->force, 0, sizeof(float4) * n, s));   // (k_fixed_finish keeps the integer sums clear)
-        if (!c->block_cleared) MLIP_CUDA_TRY(c, cudaMemsetAsync(c->launch_block, 0, LAUNCH_CLEAR_BYTES, s));   // tile and pair counters, integer and fp64 accumulators
+        MLIP_CUDA_TRY(c, cudaMemsetAsync(c->force, 0, sizeof(float4) * n, s));
     }
-    c->force_cleared = c->block_cleared = false;
+    c->force_cleared = false;
+    double *clear_block = next_eval_block(c);
     const bool in_smem = tables_fit_smem(c);
     const int tab_words = in_smem ? table_smem_words(c) : 0;
     // instantiations: {one, two atoms per warp with staggered species, two without, two with tables in global memory}
@@ -1344,15 +1365,15 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     k.nbr_cap = c->nbr_cap; k.head_pack = c->head_w; k.force = c->force; k.e_atom = c->e_atom;
     k.force_fx = c->force_fx; k.acc_fx = c->acc_fx;
     k.acc = c->acc; k.pair_counter = c->pair_counter; k.status = c->status; k.tile_counter = c->tile_counter;
-    mark_begin(c, s);
-    kernels[shape][(det ? 2 : 0) + (c->list16 ? 1 : 0)]<<<blocks, NW * 32, smem_bytes, s>>>(k, tab_words);
+    k.clear_block = clear_block;
+    k.stamp = timed_begin(c, MARK_KERNEL, s);
+    MLIP_CUDA_TRY(c, launch_after(kernels[shape][(det ? 2 : 0) + (c->list16 ? 1 : 0)], blocks, NW * 32, smem_bytes, s, k, tab_words));
     if (det) {
-        k_fixed_finish<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, c->force_fx, c->acc_fx, c->force, c->acc);
+        MLIP_CUDA_TRY(c, launch_after(k_fixed_finish, (unsigned)((n + 255) / 256), 256, 0, s, n, c->force_fx, c->acc_fx, c->force, c->acc, k.stamp));
         c->launches += 1;
     }
-    mark_end(c, MARK_KERNEL, s);
+    timed_end(c, MARK_KERNEL, s);
     c->launches += 1;
-    MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
 }
 

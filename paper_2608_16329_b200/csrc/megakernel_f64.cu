@@ -97,6 +97,8 @@ struct F64Args {
     double *acc;
     unsigned long long *pair_counter;
     int *status;
+    double *clear_block;       // the other evaluation block (next_eval_block)
+    unsigned long long *stamp;
 };
 
 __device__ __forceinline__ double silu_d(double x, double &dsilu) {
@@ -153,6 +155,10 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     const int C = k.n_species;
+    allow_next();
+    wait_previous();
+    stamp_begin(k.stamp);
+    if (blockIdx.x == 0 && threadIdx.x < (int)(LAUNCH_CLEAR_BYTES / sizeof(double))) k.clear_block[threadIdx.x] = 0.0;
     // lists that an in-step rebuild could not complete (capacity, broken configuration) are not evaluated: the outputs
     // stay at their cleared values and the status word tells the caller why
     if (*k.status & (FLAG_NEIGHBOR_OVERFLOW | FLAG_NONFINITE)) return;
@@ -596,6 +602,7 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
         if (threadIdx.x == 10) atomicAdd(k.pair_counter, (unsigned long long)x);
         else atomicAdd(&k.acc[threadIdx.x < 9 ? ACC_VIRIAL + threadIdx.x : ACC_ENERGY], x);
     }
+    stamp_end(k.stamp);
 }
 
 int upload_head_f64(mlip_ctx *c, const double *w) {
@@ -630,7 +637,7 @@ int upload_head_f64(mlip_ctx *c, const double *w) {
 }
 
 template <int K, int LMAX, int BASIS>
-static cudaError_t launch_shape(mlip_ctx *c, const F64Args &k, cudaStream_t s) {
+static cudaError_t launch_shape(mlip_ctx *c, F64Args &k, cudaStream_t s) {
     const size_t smem_bytes = sizeof(TileSmem<K, LMAX, BASIS>);
     if (!c->kernel_ready) {
         cudaError_t e = cudaFuncSetAttribute(k_mega_f64<K, LMAX, BASIS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
@@ -646,10 +653,10 @@ static cudaError_t launch_shape(mlip_ctx *c, const F64Args &k, cudaStream_t s) {
     const int per_sm = f64_ctas_per_sm<K, LMAX, BASIS>();
     const int64_t tiles_max = (k.n + F64_TILE - 1) / F64_TILE + k.n_species;
     const int blocks = (int)std::min<int64_t>(tiles_max, (int64_t)per_sm * c->n_sm);
-    mark_begin(c, s);
-    k_mega_f64<K, LMAX, BASIS><<<blocks, F64_TILE * 32, smem_bytes, s>>>(k);
-    mark_end(c, MARK_KERNEL, s);
-    return cudaGetLastError();
+    k.stamp = timed_begin(c, MARK_KERNEL, s);
+    const cudaError_t e = launch_after(k_mega_f64<K, LMAX, BASIS>, (unsigned)blocks, F64_TILE * 32, smem_bytes, s, k);
+    timed_end(c, MARK_KERNEL, s);
+    return e;
 }
 
 bool f64_shape_supported(int k, int l_max, int basis) {
@@ -661,12 +668,12 @@ bool f64_shape_supported(int k, int l_max, int basis) {
 
 int launch_megakernel_f64(mlip_ctx *c, cudaStream_t s) {
     const int64_t n = c->n;
-    if (!c->force_cleared || !c->block_cleared) {
+    if (!c->force_cleared) {
         c->mark_open = false;
-        if (!c->force_cleared) MLIP_CUDA_TRY(c, cudaMemsetAsync(c->force_d, 0, sizeof(double) * 3 * n, s));
-        if (!c->block_cleared) MLIP_CUDA_TRY(c, cudaMemsetAsync(c->launch_block, 0, LAUNCH_CLEAR_BYTES, s));   // pair counter and accumulators
+        MLIP_CUDA_TRY(c, cudaMemsetAsync(c->force_d, 0, sizeof(double) * 3 * n, s));
     }
-    c->force_cleared = c->block_cleared = false;
+    c->force_cleared = false;
+    double *clear_block = next_eval_block(c);
     F64Args k;
     k.n = n; k.n_species = c->cfg.n_species; k.grid = c->grid; k.rc2 = c->cfg.r_cut * c->cfg.r_cut;
     k.coef = c->table_d; k.knots = c->cfg.table_knots; k.r_min = c->cfg.table_r_min;
@@ -675,7 +682,7 @@ int launch_megakernel_f64(mlip_ctx *c, cudaStream_t s) {
     k.nbr_off = c->nbr_off; k.nbr_near = c->nbr_near; k.far_flag = c->far_flag; k.nbr = c->nbr; k.nbr16 = c->list16 ? reinterpret_cast<const uint16_t *>(c->nbr) : nullptr; k.cell_id = c->cell_id; k.cell_start = c->cell_start;
     k.nbr_cap = c->nbr_cap;
     k.head = c->head_w_d; k.force = c->force_d; k.e_atom = c->e_atom_d; k.acc = c->acc;
-    k.pair_counter = c->pair_counter; k.status = c->status;
+    k.pair_counter = c->pair_counter; k.status = c->status; k.clear_block = clear_block;
     cudaError_t e = cudaErrorInvalidValue;
     switch (c->cfg.basis * 1000 + c->cfg.k * 10 + c->cfg.l_max) {
 #define MLIP_F64_CASE(K, L, B) case B * 1000 + K * 10 + L: e = launch_shape<K, L, B>(c, k, s); break;

@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(SORT_WARPS * 32) k_sort_gather(CellGrid g, int
                                                                  int32_t n_owned, double4 *__restrict__ pos4, double *__restrict__ vel,
                                                                  int32_t *__restrict__ user_of, float *__restrict__ disp, float4 *__restrict__ rel,
                                                                  int32_t *__restrict__ cell_id, int32_t *__restrict__ cell_count,
-                                                                 int32_t *__restrict__ bin_count, int *status) {
+                                                                 int32_t *__restrict__ bin_count, int *status, EvalClear clear) {
     __shared__ __align__(16) int32_t s_keys[SORT_WARPS][MAX_CELL_ATOMS];
     const int lane = threadIdx.x & 31, c = blockIdx.x * SORT_WARPS + (threadIdx.x >> 5);
     if (c >= g.n_cells) return;
@@ -142,6 +142,8 @@ __global__ void __launch_bounds__(SORT_WARPS * 32) k_sort_gather(CellGrid g, int
                 vel[3 * (int64_t)dst + q] = vel_src ? vel_src[3 * (int64_t)src + q] : 0.0;
                 disp[3 * (int64_t)dst + q] = 0.f;
             }
+            if (clear.force) clear.force[dst] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (clear.force_d) for (int q = 0; q < 3; ++q) clear.force_d[3 * (int64_t)dst + q] = 0.0;
             if (user < n_owned) sa = (int)p.w;
         }
         for (int s = 0; s < n_species; ++s) {
@@ -274,7 +276,7 @@ __global__ void __launch_bounds__(256) k_neighbors(int64_t n, CellGrid g, double
 
 // The same traversal for grids with at least three cells per dimension, on the cell-relative fp32 positions: the
 // separation is x_rel(j) - x_rel(i) + (cell offset) * edge -- the cell offset already names the periodic image, so no
-// minimum-image step and no fp64 arithmetic per candidate (the positions live in the force array, idle during a build).  Candidates within 1e-5 of the list radius (the fp32 distance is
+// minimum-image step and no fp64 arithmetic per candidate (see launch_build for where the positions live).  Candidates within 1e-5 of the list radius (the fp32 distance is
 // good to ~1e-6) are decided by the exact fp64 predicate on the full positions, so the lists are the same bit for bit.
 template <bool FILL, typename OUT>
 __global__ void __launch_bounds__(256) k_neighbors_rel(int64_t n, CellGrid g, double rl2, const double4 *__restrict__ pos4,
@@ -728,7 +730,7 @@ static void launch_onepass(mlip_ctx *c, ENTRY *nbr, int *flag, double rl, float 
     const int spin = c->lookback_spin_limit > 0 ? c->lookback_spin_limit : OP_SPIN;
     const int64_t n_tiles = (c->n + 8 * PER_WARP - 1) / (8 * PER_WARP);
     k_neighbors_onepass<REL, PER_WARP, ENTRY><<<(unsigned)n_tiles, 256, sizeof(int32_t) * 8 * PER_WARP * OP_BUF, s>>>(
-        c->n, c->grid, rl * rl, c->pos4, c->force, c->cell_start, c->nbr_off, nbr, c->nbr_cap, flag, c->tile_state, c->build_word, c->status, spin,
+        c->n, c->grid, rl * rl, c->pos4, c->rel_pos, c->cell_start, c->nbr_off, nbr, c->nbr_cap, flag, c->tile_state, c->build_word, c->status, spin,
         c->lookback_unpublished_tile, near2, c->nbr_near, c->user_of, (int32_t)c->n_owned);
     c->launches += 1;
 }
@@ -737,7 +739,6 @@ static void launch_onepass(mlip_ctx *c, ENTRY *nbr, int *flag, double rl, float 
 // arrays first when `pos` is given (velocities then start at zero).
 int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int32_t *species, cudaStream_t s) {
     mark_begin(c, s);
-    if (c->cfg.precision == 0) c->force_cleared = false;   // (the force array is used below)
     const int64_t n = c->n;
     const CellGrid &g = c->grid;
     const int C = c->cfg.n_species;
@@ -746,9 +747,14 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
     // before some atom has moved skin / 4, and the fused kernels skip them until then (far_flag, raised by the integrator)
     const double rn = c->cfg.r_cut + 0.5 * c->cfg.skin;
     const float near2 = c->cfg.skin > 0.0 ? (float)(rn * rn * (1.0 + 1e-5)) : 3.0e38f;
-    // grids of at least 3 x 3 x 3 cells take the fp32 cell-relative traversal (positions staged in the idle force array)
+    // grids of at least 3 x 3 x 3 cells take the fp32 cell-relative traversal (positions staged by the sort)
     const bool rel = g.n[0] >= 3 && g.n[1] >= 3 && g.n[2] >= 3;
-    float4 *relpos = c->force;
+    // they live in the velocity source when that is not read (a build from the caller's arrays), else in the force array, idle during
+    // a build.  Where they leave it alone the forces are cleared for the evaluation that follows.
+    float4 *relpos = pos ? reinterpret_cast<float4 *>(c->vel_src) : c->force;
+    EvalClear clear_forces = eval_clear(c);
+    if (rel && clear_forces.force == relpos) { clear_forces.force = nullptr; c->force_cleared = false; }
+    c->rel_pos = relpos;
     const int per_warp = onepass_per_warp(c);
     const BuildClear clear{c->tile_state, (n + 8 * per_warp - 1) / (8 * per_warp), c->build_word, c->far_flag, c->rebuild_flag};
     // scratch: overwritten further down whatever the outcome (nbr_near must not hold scratch: it bounds reads of a list that a
@@ -760,7 +766,7 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
     k_place<<<blocks_for(n, 256), 256, 0, s>>>(c->cell_of, n, c->cell_start, rank_of, slot_src);
     k_sort_gather<<<blocks_for(g.n_cells, SORT_WARPS), SORT_WARPS * 32, 0, s>>>(g, C, c->cell_start, slot_src, c->pos4_src, pos ? nullptr : c->vel_src, c->user_src,
                                                                                (int32_t)c->n_owned, c->pos4, c->vel, c->user_of, c->disp, rel ? relpos : nullptr,
-                                                                               c->cell_id, c->cell_count, c->bin_count, c->status);
+                                                                               c->cell_id, c->cell_count, c->bin_count, c->status, clear_forces);
     n_launches += exclusive_scan<int32_t, int32_t>(c->bin_count, c->bin_start, (int64_t)C * g.n_cells, c->scan_tmp, s);
     k_center_order<<<blocks_for((int64_t)g.n_cells * 32, 128), 128, 0, s>>>(g.n_cells, C, c->cell_start, c->pos4, c->bin_start, c->center_order, c->species_start, c->user_of, (int32_t)c->n_owned);
     c->launches += n_launches + 4;

@@ -1,0 +1,55 @@
+"""What the fused launch sequence of a step must keep: independence of how a run is cut into calls, the totals of the last evaluation,
+the timing records."""
+import numpy as np
+import pytest
+
+from helpers import make_pair
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("ensemble", ["nve", "nvt"])
+@pytest.mark.parametrize("cfg,n_cells,cuts", [(5, 6, (1, 4, 2)), (2, 16, (3, 3, 1)), (5, 15, (6, 1))])
+def test_a_run_does_not_depend_on_how_it_is_cut_into_calls(cfg, n_cells, cuts, ensemble):
+    """Bit for bit in the deterministic mode, with a rebuild on the way: the half kick that closes a step runs with the next step's drift
+    inside a call and by itself at its end."""
+    states = []
+    for parts in ((sum(cuts),), cuts):
+        w, _, pot = make_pair(cfg, n_cells, 1.0, force_mode=1)
+        pot.build_neighbors(w.pos, w.species, w.box)
+        pot.set_velocities(w.vel)
+        for n in parts:
+            pot.step(n, 1.0, 3) if ensemble == "nve" else pot.step_nvt(n, 1.0, 3, 300.0, 50.0)
+        pot.sync_status()
+        pos, vel, step = pot.state()
+        states.append((pos.cpu().numpy().tobytes(), vel.cpu().numpy().tobytes(), pot.energies().cpu().numpy().tobytes(), step))
+    assert states[0] == states[1]
+
+
+def test_the_last_evaluations_totals_stay_until_the_next():
+    import paper_2608_16329_b200 as mlip
+    w, _, pot = make_pair(5, 6, 1.0)
+    pot.build_neighbors(w.pos, w.species, w.box)
+    for _ in range(3):
+        e = float(pot.compute()["energy"].cpu())
+        pairs = mlip.mlip_get_counters(pot.ctx)["pairs_in_cutoff"]
+        pot.set_positions(w.pos)
+        assert float(pot.energies()[0].cpu()) == e and mlip.mlip_get_counters(pot.ctx)["pairs_in_cutoff"] == pairs > 0
+
+
+@pytest.mark.parametrize("n_cells", [6, 30])
+def test_timing_records_keep_the_last_256_launches(n_cells):
+    """Below and above the size where the kernels time themselves instead of events (864 and 108,000 atoms)."""
+    import paper_2608_16329_b200 as mlip
+    w, _, pot = make_pair(5, n_cells, 1.0)
+    pot.build_neighbors(w.pos, w.species, w.box)
+    pot.set_velocities(w.vel)
+    pot.step(1, 0.01, 0)
+    mlip.mlip_get_timings(pot.ctx, reset=True)
+    for n, kept in ((20, 20), (300, 256), (900, 256)):
+        pot.step(n, 0.001, 0)
+        launches, ms = mlip.mlip_kernel_time(pot.ctx)
+        build, kernel, integrate = mlip.mlip_get_timings(pot.ctx, reset=True)
+        assert launches == kept and kernel == ms and build == 0.0
+        assert 0.003 * kept < ms < 10.0 * kept and 0.0005 * kept < integrate < 1.0 * kept
+    assert pot.sync_status() == 0
