@@ -443,8 +443,10 @@ __device__ __forceinline__ int onepass_traverse(int64_t i, const CellGrid &g, do
     cell_ranges<REL>(pi, g, cell_start, lane, cb, ce);
     int cnt = 0, cn = 0;
     auto take = [&](bool hit, float d2f, int j, int it, int cell_beg) {
-        const bool near = hit && d2f < near2;
-        const unsigned m = __ballot_sync(0xffffffffu, hit), mn = __ballot_sync(0xffffffffu, near), below = (1u << lane) - 1u;
+        const unsigned m = __ballot_sync(0xffffffffu, hit);
+        if (!m) return;   // (most chunks of the outer cells)
+        const bool near = d2f < near2;
+        const unsigned mn = __ballot_sync(0xffffffffu, hit && near), below = (1u << lane) - 1u;
         const int slot = near ? cn + __popc(mn & below) : top - (cnt - cn + __popc(m & ~mn & below));
         if (hit && slot >= 0 && slot < limit) out[slot] = (OUT)list_entry<ENTRY>(j, it, cell_beg);
         cnt += __popc(m);
@@ -485,7 +487,7 @@ __device__ __forceinline__ int onepass_traverse(int64_t i, const CellGrid &g, do
             const int j = base + lane;
             if (base != cur_beg && j < cur_end) rj = rel[j];
             float d2f = 0.f;
-            const bool hit = j < cur_end && j != i && rel_hit(rj, sx, sy, sz, rl2_lo, rl2_hi, rl2, pi, pos4, j, g, d2f);
+            const bool hit = j < cur_end && !(it == 13 && j == i) && rel_hit(rj, sx, sy, sz, rl2_lo, rl2_hi, rl2, pi, pos4, j, g, d2f);
             take(hit, d2f, j, it, cur_beg);
         }
     }
@@ -649,11 +651,61 @@ __global__ void __launch_bounds__(256) k_export_count(int64_t n, int n_species, 
     if (lane < n_species) seg_count[row + lane] = (int)((((lane >> 1) == 0 ? cnt[0] : (lane >> 1) == 1 ? cnt[1] : (lane >> 1) == 2 ? cnt[2] : cnt[3]) >> (16 * (lane & 1))) & 0xffffu);
 }
 
-// Warp per atom: an entry's place is the number of smaller keys in the list (keys differ within a list), counted against the keys
-// in shared memory, four per load.  Lists longer than the buffer read them again from global memory.  (Ranking by re-reading
-// list, species and caller index for every pair of entries took 2.0 ms for 108,000 atoms with 134 entries each; this takes
-// a tenth.)
+// Sort of 32 x R keys by a warp, ascending in lane * R + r: a bitonic network whose phases start with a mirrored step, so that every
+// compare-exchange puts the smaller key at the lower index.
+template <int R>
+__device__ __forceinline__ void warp_sort(int32_t (&v)[R], int lane) {
+#pragma unroll
+    for (int k = 2; k <= 32 * R; k <<= 1) {
+        if (k <= R) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if ((r & (k >> 1)) == 0) { const int q = r ^ (k - 1); const int lo = min(v[r], v[q]); v[q] = max(v[r], v[q]); v[r] = lo; }
+        } else {
+            const bool lower = (lane & (k / (2 * R))) == 0;
+            int32_t o[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) o[r] = __shfl_xor_sync(0xffffffffu, v[R - 1 - r], k / R - 1);
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = lower ? min(v[r], o[r]) : max(v[r], o[r]);
+        }
+#pragma unroll
+        for (int j = k >> 2; j > 0; j >>= 1) {
+            if (j >= R) {
+                const bool lower = (lane & (j / R)) == 0;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int32_t o = __shfl_xor_sync(0xffffffffu, v[r], j / R);
+                    v[r] = lower ? min(v[r], o) : max(v[r], o);
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if ((r & j) == 0) { const int lo = min(v[r], v[r ^ j]); v[r ^ j] = max(v[r], v[r ^ j]); v[r] = lo; }
+            }
+        }
+    }
+}
+
+// Warp per atom: the list's keys sorted in registers (four or eight to a lane; they differ within a list), turned to full rows through
+// shared memory and written.  Longer lists: an entry's place is the number of smaller keys, read again from global memory.
+// 108,000 atoms with 134 entries each: 2.0 ms when every pair of entries was compared through list, species and caller index, 375 us
+// when keys were ranked against a copy in shared memory (some 2,000 instructions per list), 110 us sorted (about 600).
 constexpr int EXPORT_BUF = 256;
+template <int R>
+__device__ __forceinline__ void export_sorted(const ListView &lv, const int32_t *__restrict__ key, int64_t i, int64_t beg, int m, int32_t *keys,
+                                              int32_t *__restrict__ out, int lane) {
+    int32_t v[R];
+#pragma unroll
+    for (int c = 0; c < R; ++c) v[c] = 32 * c + lane < m ? key[lv.at(i, beg + 32 * c + lane)] : 0x7fffffff;
+    warp_sort<R>(v, lane);
+#pragma unroll
+    for (int c = 0; c < R; c += 4) *reinterpret_cast<int4 *>(keys + lane * R + c) = make_int4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < R; ++c)
+        if (32 * c + lane < m) out[32 * c + lane] = keys[32 * c + lane] & 0x0fffffff;
+}
 __global__ void __launch_bounds__(256) k_export_fill(int64_t n, int n_species, const int64_t *__restrict__ nbr_off, ListView lv,
                                                      const int32_t *__restrict__ key, const int64_t *__restrict__ seg_ptr, int32_t *__restrict__ out) {
     __shared__ __align__(16) int32_t s_keys[8][EXPORT_BUF];
@@ -664,29 +716,8 @@ __global__ void __launch_bounds__(256) k_export_fill(int64_t n, int n_species, c
     const int64_t beg = nbr_off[i];
     const int m = (int)(nbr_off[i + 1] - beg);
     out += seg_ptr[(int64_t)(key[i] & 0x0fffffff) * n_species];   // the species' segments of an atom follow one another
-    if (m <= EXPORT_BUF) {
-        constexpr int PER_LANE = EXPORT_BUF / 32;
-        int32_t mine[PER_LANE], rank[PER_LANE];
-#pragma unroll
-        for (int c = 0; c < PER_LANE; ++c) {
-            const int e = 32 * c + lane;
-            mine[c] = e < m ? key[lv.at(i, beg + e)] : 0x7fffffff;
-            rank[c] = 0;
-            keys[e] = mine[c];
-        }
-        __syncwarp();
-        const int chunks = (m + 31) >> 5;
-        for (int q = 0; q < m; q += 4) {
-            const int4 other = *reinterpret_cast<const int4 *>(keys + q);
-#pragma unroll
-            for (int c = 0; c < PER_LANE; ++c)
-                if (c < chunks) rank[c] += (other.x < mine[c]) + (other.y < mine[c]) + (other.z < mine[c]) + (other.w < mine[c]);
-        }
-#pragma unroll
-        for (int c = 0; c < PER_LANE; ++c)
-            if (32 * c + lane < m) out[rank[c]] = mine[c] & 0x0fffffff;
-        return;
-    }
+    if (m <= EXPORT_BUF / 2) return export_sorted<4>(lv, key, i, beg, m, keys, out, lane);
+    if (m <= EXPORT_BUF) return export_sorted<8>(lv, key, i, beg, m, keys, out, lane);
     for (int e = lane; e < m; e += 32) {
         const int32_t mine = key[lv.at(i, beg + e)];
         int rank = 0;
