@@ -158,6 +158,7 @@ struct mlip_ctx {
     int64_t launches = 0;
     size_t resident = 0;
     cudaStream_t last_stream = nullptr;
+    bool lists_fresh = true;       // lists were built since the last evaluation was launched
     bool force_cleared = false;    // the forces were cleared for the next evaluation by a kernel before it
     // Timing marks: a ring of events, each the end of a timed part that began at the mark before it (consecutive parts share
     // a mark), or the beginning of one.
@@ -237,7 +238,7 @@ __device__ __forceinline__ void stamp_end(unsigned long long *stamp) { if (stamp
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... P, typename... A>
-inline cudaError_t launch_after(void (*kernel)(P...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t s, A... args) {
+inline cudaError_t launch_after_if(bool early, void (*kernel)(P...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t s, A... args) {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -247,8 +248,12 @@ inline cudaError_t launch_after(void (*kernel)(P...), unsigned blocks, unsigned 
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_after(void (*kernel)(P...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t s, A... args) {
+    return launch_after_if(true, kernel, blocks, threads, smem, s, args...);
 }
 
 // The counters and totals of a new evaluation become current; returns the other block, which the evaluation clears.

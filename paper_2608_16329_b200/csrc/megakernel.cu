@@ -983,9 +983,29 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
     // computed one.  Either way a species whose tiles are all claimed already is passed over: staging its tables would
     // be the only thing left to do.
     auto species_at = [&](int ss) { return STAGGER ? (int)((ss + blockIdx.x) % (unsigned)k.n_species) : ss; };
-    // The first species is staged ahead of the wait for the kernel before this one (model data only up to here), in whose shadow it then
-    // lies: staging is some 4 us of a small system's 30.
-    stage(species_at(0));
+    // Every group's first tile is fixed (the CTAs that start on a species take its first tiles, group 0 of each before group 1 of any, which
+    // spreads a small system over the SMs); the later ones are claimed from the species' counter, which counts from there.
+    auto starters = [&](int species) {   // CTAs that start on it
+        return !STAGGER ? (species == 0 ? (int)gridDim.x : 0) : species < (int)gridDim.x ? ((int)gridDim.x - 1 - species) / k.n_species + 1 : 0;
+    };
+    const int first_species = species_at(0);
+    const int first_tile = (STAGGER ? (int)(blockIdx.x / (unsigned)k.n_species) : (int)blockIdx.x) + group * starters(first_species);
+    // The first species is staged, and the lists of the first tile's atoms fetched, ahead of the wait for the kernel before this one: they
+    // change in list builds only, and the launch after a build does not start early.  864 atoms: 4 us of staging and 3 us of
+    // dependent loads and claims out of 31 us a step lie in that kernel's shadow.
+    stage(first_species);
+    NextAtoms<APW> nx0;
+    int near0 = 0;
+    {
+        const int s_end0 = __ldg(k.species_start + first_species + 1);
+        const int slot0 = __ldg(k.species_start + first_species) + first_tile * NA + wg + GW * lane;
+        nx0.k = &k; nx0.pf = pf; nx0.slot = (lane < APW && slot0 < s_end0) ? slot0 : -1;
+        nx0.i = 0; nx0.beg = 0; nx0.len = 0; nx0.use_far = true; nx0.cid = 0;
+        nx0.stage_a();
+        nx0.template stage_b<L16>();
+        if (nx0.slot >= 0) near0 = __ldg(k.nbr_near + nx0.i);
+        nx0.template stage_c<L16>(lane);
+    }
     wait_previous();
     stamp_begin(k.stamp);
     if (blockIdx.x == 0 && threadIdx.x < (int)(LAUNCH_CLEAR_BYTES / sizeof(double))) k.clear_block[threadIdx.x] = 0.0;
@@ -994,26 +1014,34 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
     // so every CTA takes the same decision)
     const bool skip = (*k.status & (FLAG_NEIGHBOR_OVERFLOW | FLAG_NONFINITE)) != 0;
     const bool use_far = *k.far_flag != 0;   // an atom has moved skin / 4 since the build: every list entry counts
+    if (!use_far && nx0.slot >= 0) pf[lane * PF_WORDS + PF_IDX + 3] = near0;   // (the whole lists were fetched: far entries come last)
+    __syncwarp();
     for (int ss = 0; ss < k.n_species && !skip; ++ss) {
         const int species = species_at(ss);
         const int s_beg = __ldg(k.species_start + species), s_end = __ldg(k.species_start + species + 1);
         const int n_tiles = (s_end - s_beg + NA - 1) / NA;
         if (n_tiles == 0) continue;
-        if (threadIdx.x == 0) ctl[6 + (ss & 1)] = *reinterpret_cast<volatile int *>(k.tile_counter + species);
-        __syncthreads();   // both groups are done with the previous species' tables
-        if (ctl[6 + (ss & 1)] >= n_tiles) continue;
-        if (ss > 0) stage(species);
+        const int n_first = NG * starters(species);   // tiles that are not claimed
+        if (ss > 0) {
+            if (threadIdx.x == 0) ctl[6 + (ss & 1)] = *reinterpret_cast<volatile int *>(k.tile_counter + species);
+            __syncthreads();   // both groups are done with the previous species' tables
+            if (n_first + ctl[6 + (ss & 1)] >= n_tiles) continue;
+            stage(species);
+        }
 
-        bool prefetched = false;   // this warp's atom of the coming tile sits in the prefetch buffer
+        bool prefetched = ss == 0 && __shfl_sync(0xffffffffu, nx0.slot, 0) >= 0;   // this warp's atoms of the coming tile sit in the prefetch buffer
         int look_ahead = -1;       // (group leader) the tile after the current one
         // the group's tiles of this species, claimed one ahead: the first is broadcast here, every later one travels with
         // the barrier between encoding and head
-        group_sync(group);
-        if (wg == 0 && lane == 0) ctl[2 * group] = atomicAdd(k.tile_counter + species, 1);
-        group_sync(group);
-        int tile = ctl[2 * group];
+        int tile = first_tile;
+        if (ss > 0) {
+            group_sync(group);
+            if (wg == 0 && lane == 0) ctl[2 * group] = n_first + atomicAdd(k.tile_counter + species, 1);
+            group_sync(group);
+            tile = ctl[2 * group];
+        }
         while (tile < n_tiles) {
-            if (wg == 0 && lane == 0) look_ahead = atomicAdd(k.tile_counter + species, 1);   // consumed after the encoding
+            if (wg == 0 && lane == 0) look_ahead = n_first + atomicAdd(k.tile_counter + species, 1);   // consumed after the encoding
             pc.mark(11);
             const int first = s_beg + tile * NA;
             const int count = min(NA, s_end - first);
@@ -1156,6 +1184,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
 
     // totals: per warp into shared memory, per CTA to the global accumulators (from every warp they were 27,000 atomics to one
     // sector of one L2 slice, some 10 us at the end of every launch)
+    asm volatile("cp.async.wait_all;" ::: "memory");   // (nothing is left in flight but after a skipped evaluation)
     __syncthreads();   // everybody is done with shared memory
     double *sums = reinterpret_cast<double *>(smem) + warp * TOTALS;   // virial [9], E_i sums of the atoms' lanes, pairs
 #pragma unroll
@@ -1367,7 +1396,9 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     k.acc = c->acc; k.pair_counter = c->pair_counter; k.status = c->status; k.tile_counter = c->tile_counter;
     k.clear_block = clear_block;
     k.stamp = timed_begin(c, MARK_KERNEL, s);
-    MLIP_CUDA_TRY(c, launch_after(kernels[shape][(det ? 2 : 0) + (c->list16 ? 1 : 0)], blocks, NW * 32, smem_bytes, s, k, tab_words));
+    const bool early = !c->lists_fresh;   // (the kernel reads the lists before it waits)
+    c->lists_fresh = false;
+    MLIP_CUDA_TRY(c, launch_after_if(early, kernels[shape][(det ? 2 : 0) + (c->list16 ? 1 : 0)], blocks, NW * 32, smem_bytes, s, k, tab_words));
     if (det) {
         MLIP_CUDA_TRY(c, launch_after(k_fixed_finish, (unsigned)((n + 255) / 256), 256, 0, s, n, c->force_fx, c->acc_fx, c->force, c->acc, k.stamp));
         c->launches += 1;

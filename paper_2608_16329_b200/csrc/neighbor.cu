@@ -770,6 +770,7 @@ static void launch_onepass(mlip_ctx *c, ENTRY *nbr, int *flag, double rl, float 
 // arrays first when `pos` is given (velocities then start at zero).
 int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int32_t *species, cudaStream_t s) {
     mark_begin(c, s);
+    c->lists_fresh = true;
     const int64_t n = c->n;
     const CellGrid &g = c->grid;
     const int C = c->cfg.n_species;
