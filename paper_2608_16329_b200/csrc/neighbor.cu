@@ -176,6 +176,104 @@ __global__ void __launch_bounds__(128) k_center_order(int n_cells, int n_species
     }
 }
 
+// ---- the whole binning of a small system by one block ----
+// Cell ids, counting sort, order within the cells, per-species processing order: what the kernels above do in six launches (some 35 us,
+// of which the work is a third) with the per-cell state in shared memory.  An atom's place in its cell is the number of smaller keys there;
+// among those of its own species it is its place in the (species, cell) bin.  An over-full cell is sorted all the same
+// (the system is small) and raises the flag.  Whole synchronising build in us, six launches / one block: 256 atoms 55 / 39, 864 64 / 50,
+// 2,048 66 / 58; with up to eight atoms per thread 4,000 atoms 69 / 79 and 6,912 87 / 116: one SM's memory rate, hence the limit.
+constexpr int SMALL_THREADS = 1024, SMALL_PER_THREAD = 2, SMALL_ATOMS = 2048, SMALL_CELLS = 4096, SMALL_BINS = 16384;
+static_assert(SMALL_ATOMS <= SMALL_THREADS * SMALL_PER_THREAD, "atoms are kept in registers");
+// exclusive scan of v[0 .. n) in place, v[n] = total
+__device__ __forceinline__ void small_scan(int *v, int n, int64_t *ws) {
+    int carry = 0;
+    for (int base = 0; base < n; base += SMALL_THREADS) {
+        const int i = base + threadIdx.x;
+        const int x = i < n ? v[i] : 0;
+        int64_t total;
+        const int ex = (int)block_exclusive_scan(x, total, ws);   // (ends with a barrier)
+        if (i < n) v[i] = carry + ex;
+        carry += (int)total;
+    }
+    if (threadIdx.x == 0) v[n] = carry;
+    __syncthreads();
+}
+template <bool PACK>
+__global__ void __launch_bounds__(SMALL_THREADS) k_bin_small(const double *__restrict__ pos, const int32_t *__restrict__ species, int n, int n_species,
+                                                             int32_t n_owned, CellGrid g, const double4 *__restrict__ pos4_src, const double *__restrict__ vel_src,
+                                                             const int32_t *__restrict__ user_src, double4 *__restrict__ pos4, double *__restrict__ vel,
+                                                             int32_t *__restrict__ user_of, float *__restrict__ disp, float4 *__restrict__ rel,
+                                                             int32_t *__restrict__ cell_id, int32_t *__restrict__ cell_start, int32_t *__restrict__ center_order,
+                                                             int32_t *__restrict__ species_start, int *status, BuildClear clear, EvalClear clear_force) {
+    extern __shared__ int s_small[];   // cell starts [n_cells + 1], bins [n_species * n_cells + 1], keys [n]
+    __shared__ int64_t ws[33];
+    int *start = s_small, *bins = start + g.n_cells + 1, *keys = bins + n_species * g.n_cells + 1;
+    const int n_bins = n_species * g.n_cells;
+    for (int q = threadIdx.x; q < g.n_cells + 1 + n_bins + 1; q += SMALL_THREADS) s_small[q] = 0;
+    for (int q = threadIdx.x; q < clear.n_words; q += SMALL_THREADS) clear.tile_state[q] = 0;
+    if (threadIdx.x == 0) {
+        for (int q = 0; q < 4; ++q) clear.build_word[q] = 0;
+        *clear.far_flag = 0; *clear.rebuild_flag = 0;
+    }
+    __syncthreads();
+    double4 p[SMALL_PER_THREAD];
+    int cell[SMALL_PER_THREAD], key[SMALL_PER_THREAD], place[SMALL_PER_THREAD];
+#pragma unroll
+    for (int q = 0; q < SMALL_PER_THREAD; ++q) {
+        const int i = threadIdx.x + q * SMALL_THREADS;
+        if (i >= n) continue;
+        if (PACK) {
+            int s = species[i];
+            if (s < 0 || s >= n_species) { atomicOr(status, FLAG_NONFINITE); s = 0; }
+            p[q] = make_double4(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], (double)s);
+        } else p[q] = pos4_src[i];
+        const bool ok = (p[q].x >= 0.0 && p[q].x < g.box[0]) && (p[q].y >= 0.0 && p[q].y < g.box[1]) && (p[q].z >= 0.0 && p[q].z < g.box[2]);
+        if (!ok) atomicOr(status, FLAG_NONFINITE);
+        const int cx = ok ? cell_coord(p[q].x, g.inv_edge[0], g.n[0]) : 0;
+        const int cy = ok ? cell_coord(p[q].y, g.inv_edge[1], g.n[1]) : 0;
+        const int cz = ok ? cell_coord(p[q].z, g.inv_edge[2], g.n[2]) : 0;
+        cell[q] = (cx * g.n[1] + cy) * g.n[2] + cz;
+        key[q] = ((int)p[q].w << 28) | (PACK ? i : user_src[i]);
+        place[q] = atomicAdd(&start[cell[q]], 1);
+        if ((key[q] & 0x0fffffff) < n_owned) atomicAdd(&bins[(int)p[q].w * g.n_cells + cell[q]], 1);
+    }
+    __syncthreads();
+    small_scan(start, g.n_cells, ws);
+    small_scan(bins, n_bins, ws);
+    for (int q = threadIdx.x; q <= g.n_cells; q += SMALL_THREADS) cell_start[q] = start[q];
+    if (threadIdx.x <= n_species) species_start[threadIdx.x] = bins[threadIdx.x * g.n_cells];
+#pragma unroll
+    for (int q = 0; q < SMALL_PER_THREAD; ++q)
+        if (threadIdx.x + q * SMALL_THREADS < n) keys[start[cell[q]] + place[q]] = key[q];
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < SMALL_PER_THREAD; ++q) {
+        const int i = threadIdx.x + q * SMALL_THREADS;
+        if (i >= n) continue;
+        const int beg = start[cell[q]], end = start[cell[q] + 1], own_species = key[q] & ~0x0fffffff;
+        if (end - beg > MAX_CELL_ATOMS) atomicOr(status, FLAG_NONFINITE);
+        int below = 0, same = 0;   // smaller keys in the cell; those of the same species
+        for (int a = beg; a < end; ++a) {
+            const int o = keys[a];
+            below += o < key[q];
+            same += o < key[q] && o >= own_species;
+        }
+        const int dst = beg + below, user = key[q] & 0x0fffffff, cz = cell[q] % g.n[2], cy = (cell[q] / g.n[2]) % g.n[1], cx = cell[q] / (g.n[2] * g.n[1]);
+        if (user < n_owned) center_order[bins[(int)p[q].w * g.n_cells + cell[q]] + same] = dst;
+        pos4[dst] = p[q];
+        user_of[dst] = user;
+        if (cell_id) cell_id[dst] = pack_cell(g, cell[q]);
+        if (rel) rel[dst] = make_float4((float)(p[q].x - (double)cx * (g.box[0] / g.n[0])), (float)(p[q].y - (double)cy * (g.box[1] / g.n[1])),
+                                        (float)(p[q].z - (double)cz * (g.box[2] / g.n[2])), 0.f);
+        for (int a = 0; a < 3; ++a) {
+            vel[3 * dst + a] = vel_src ? vel_src[3 * i + a] : 0.0;
+            disp[3 * dst + a] = 0.f;
+        }
+        if (clear_force.force) clear_force.force[dst] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (clear_force.force_d) for (int a = 0; a < 3; ++a) clear_force.force_d[3 * dst + a] = 0.0;
+    }
+}
+
 // Warp per atom over the surrounding cells.  FILL = false counts, FILL = true writes the list.
 // Lanes 0..26 fetch the atom ranges of the (up to) 27 cells in one round trip; the cells are then visited
 // in a fixed order (x, y, z offsets ascending: the order of the list) with the positions of the next
@@ -789,19 +887,30 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
     c->rel_pos = relpos;
     const int per_warp = onepass_per_warp(c);
     const BuildClear clear{c->tile_state, (n + 8 * per_warp - 1) / (8 * per_warp), c->build_word, c->far_flag, c->rebuild_flag};
-    // scratch: overwritten further down whatever the outcome (nbr_near must not hold scratch: it bounds reads of a list that a
-    // broken configuration leaves as it was)
-    int32_t *rank_of = c->center_order, *slot_src = c->nbr_count;
-    if (pos) k_cell_id<true><<<blocks_for(n, 256), 256, 0, s>>>(pos, species, C, c->pos4_src, c->user_src, n, g, c->cell_of, rank_of, c->cell_count, c->status, clear);
-    else k_cell_id<false><<<blocks_for(n, 256), 256, 0, s>>>(nullptr, nullptr, C, c->pos4_src, c->user_src, n, g, c->cell_of, rank_of, c->cell_count, c->status, clear);
-    int n_launches = exclusive_scan<int32_t, int32_t>(c->cell_count, c->cell_start, g.n_cells, c->scan_tmp, s);
-    k_place<<<blocks_for(n, 256), 256, 0, s>>>(c->cell_of, n, c->cell_start, rank_of, slot_src);
-    k_sort_gather<<<blocks_for(g.n_cells, SORT_WARPS), SORT_WARPS * 32, 0, s>>>(g, C, c->cell_start, slot_src, c->pos4_src, pos ? nullptr : c->vel_src, c->user_src,
-                                                                               (int32_t)c->n_owned, c->pos4, c->vel, c->user_of, c->disp, rel ? relpos : nullptr,
-                                                                               c->cell_id, c->cell_count, c->bin_count, c->status, clear_forces);
-    n_launches += exclusive_scan<int32_t, int32_t>(c->bin_count, c->bin_start, (int64_t)C * g.n_cells, c->scan_tmp, s);
-    k_center_order<<<blocks_for((int64_t)g.n_cells * 32, 128), 128, 0, s>>>(g.n_cells, C, c->cell_start, c->pos4, c->bin_start, c->center_order, c->species_start, c->user_of, (int32_t)c->n_owned);
-    c->launches += n_launches + 4;
+    const int64_t n_bins = (int64_t)C * g.n_cells;
+    if (n <= SMALL_ATOMS && g.n_cells <= SMALL_CELLS && n_bins <= SMALL_BINS) {
+        const size_t smem = sizeof(int) * (size_t)(g.n_cells + 1 + n_bins + 1 + n);
+        auto *kernel = pos ? k_bin_small<true> : k_bin_small<false>;
+        if (smem > 40000) MLIP_CUDA_TRY(c, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(int) * (SMALL_CELLS + SMALL_BINS + 2 + SMALL_ATOMS))));
+        kernel<<<1, SMALL_THREADS, smem, s>>>(pos, species, (int)n, C, (int32_t)c->n_owned, g, c->pos4_src, pos ? nullptr : c->vel_src, c->user_src, c->pos4, c->vel,
+                                              c->user_of, c->disp, rel ? relpos : nullptr, c->cell_id, c->cell_start, c->center_order, c->species_start,
+                                              c->status, clear, clear_forces);
+        c->launches += 1;
+    } else {
+        // scratch: overwritten further down whatever the outcome (nbr_near must not hold scratch: it bounds reads of a list that a
+        // broken configuration leaves as it was)
+        int32_t *rank_of = c->center_order, *slot_src = c->nbr_count;
+        if (pos) k_cell_id<true><<<blocks_for(n, 256), 256, 0, s>>>(pos, species, C, c->pos4_src, c->user_src, n, g, c->cell_of, rank_of, c->cell_count, c->status, clear);
+        else k_cell_id<false><<<blocks_for(n, 256), 256, 0, s>>>(nullptr, nullptr, C, c->pos4_src, c->user_src, n, g, c->cell_of, rank_of, c->cell_count, c->status, clear);
+        int n_launches = exclusive_scan<int32_t, int32_t>(c->cell_count, c->cell_start, g.n_cells, c->scan_tmp, s);
+        k_place<<<blocks_for(n, 256), 256, 0, s>>>(c->cell_of, n, c->cell_start, rank_of, slot_src);
+        k_sort_gather<<<blocks_for(g.n_cells, SORT_WARPS), SORT_WARPS * 32, 0, s>>>(g, C, c->cell_start, slot_src, c->pos4_src, pos ? nullptr : c->vel_src, c->user_src,
+                                                                                   (int32_t)c->n_owned, c->pos4, c->vel, c->user_of, c->disp, rel ? relpos : nullptr,
+                                                                                   c->cell_id, c->cell_count, c->bin_count, c->status, clear_forces);
+        n_launches += exclusive_scan<int32_t, int32_t>(c->bin_count, c->bin_start, (int64_t)C * g.n_cells, c->scan_tmp, s);
+        k_center_order<<<blocks_for((int64_t)g.n_cells * 32, 128), 128, 0, s>>>(g.n_cells, C, c->cell_start, c->pos4, c->bin_start, c->center_order, c->species_start, c->user_of, (int32_t)c->n_owned);
+        c->launches += n_launches + 4;
+    }
     // entry format of this build: 16-bit cell-relative codes if asked for and the grid has 27 distinct cells around every
     // cell, else plain indices.  A change of format gives up the old array (its capacity is counted in entries).
     const bool list16 = c->cfg.list_format == 1 && rel && std::max(g.n[0], std::max(g.n[1], g.n[2])) <= CELL_PACK_MAX;
