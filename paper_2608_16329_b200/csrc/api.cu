@@ -264,6 +264,7 @@ int mlip_create(mlip_ctx **out, const mlip_config *cfg, const double *enc_w, siz
         }
         bool ev_ok = true;
         for (int q = 0; q < mlip_ctx::MARKS; ++q) ev_ok = ev_ok && cudaEventCreate(&c->mark_ev[q]) == cudaSuccess;
+        ev_ok = ev_ok && cudaEventCreateWithFlags(&c->check_ev, cudaEventDisableTiming) == cudaSuccess;
         if (!ev_ok) { rc = MLIP_ERR_CUDA; c->err = "event creation failed"; break; }
         if (cudaMemcpy(c->mass, mass, sizeof(double) * cfg->n_species, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemset(c->build_word, 0, sizeof(int) * 8) != cudaSuccess ||
@@ -424,21 +425,35 @@ int mlip_compute_host(mlip_ctx *c, int64_t n, const double *pos_host, const int3
     return MLIP_OK;
 }
 
-// After a drift: rebuild the lists if the policy asks for it (fixed interval, or displacement-triggered).
-static int rebuild_if_due(mlip_ctx *c, int rebuild_every, cudaStream_t s) {
-    bool rebuild = rebuild_every > 0 && c->step % rebuild_every == 0;
-    if (rebuild_every < 0 && c->step % -rebuild_every == 0) {   // displacement-triggered: ask the device
-        MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->rebuild_host, c->rebuild_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-        MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
-        c->mark_open = false;
-        rebuild = *c->rebuild_host != 0;
-    }
-    if (!rebuild) return MLIP_OK;
+static int rebuild_lists(mlip_ctx *c, cudaStream_t s) {
     c->n_builds += 1;
     std::swap(c->pos4, c->pos4_src);
     std::swap(c->vel, c->vel_src);
     std::swap(c->user_of, c->user_src);
     return launch_build(c, false, nullptr, nullptr, s);
+}
+
+// After a drift: rebuild the lists if the policy asks for it (fixed interval, or displacement-triggered), then the evaluation.
+// The displacement trigger asks the device.  Below SPECULATE_BELOW_ATOMS the evaluation is launched while the answer is on its way, for
+// the usual case that the lists stay (an idle GPU costs some 23 us there, and the lists are valid up to the hard limit anyway); if they
+// have to be rebuilt it is repeated with the new ones.  Larger systems wait: a repeated evaluation would cost more than ten such waits.
+constexpr int64_t SPECULATE_BELOW_ATOMS = 12000;   // (some 130 us an evaluation)
+static int rebuild_and_evaluate(mlip_ctx *c, int rebuild_every, cudaStream_t s) {
+    bool rebuild = rebuild_every > 0 && c->step % rebuild_every == 0;
+    int rc;
+    if (rebuild_every < 0 && c->step % -rebuild_every == 0) {
+        MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->rebuild_host, c->rebuild_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+        MLIP_CUDA_TRY(c, cudaEventRecord(c->check_ev, s));
+        c->mark_open = false;
+        const bool ahead = c->n < SPECULATE_BELOW_ATOMS;
+        if (ahead && (rc = evaluate(c, s)) != MLIP_OK) return rc;
+        MLIP_CUDA_TRY(c, cudaEventSynchronize(c->check_ev));
+        c->mark_open = false;
+        rebuild = *c->rebuild_host != 0;
+        if (ahead && !rebuild) return MLIP_OK;
+    }
+    if (rebuild && (rc = rebuild_lists(c, s)) != MLIP_OK) return rc;
+    return evaluate(c, s);
 }
 
 int mlip_step(mlip_ctx *c, int n_steps, double dt, int rebuild_every, void *stream) {
@@ -457,8 +472,7 @@ int mlip_step(mlip_ctx *c, int n_steps, double dt, int rebuild_every, void *stre
     for (int it = 0; it < n_steps; ++it) {
         if ((rc = launch_kick_drift(c, dt, it > 0, s)) != MLIP_OK) return rc;
         c->step += 1;
-        if ((rc = rebuild_if_due(c, rebuild_every, s)) != MLIP_OK) return rc;
-        if ((rc = evaluate(c, s)) != MLIP_OK) return rc;
+        if ((rc = rebuild_and_evaluate(c, rebuild_every, s)) != MLIP_OK) return rc;
     }
     return n_steps > 0 ? launch_kick(c, dt, s) : MLIP_OK;
 }
@@ -482,19 +496,19 @@ int mlip_step_nvt(mlip_ctx *c, int n_steps, double dt, int rebuild_every, double
         c->forces_current = true;
     }
     // Each thermostat half step takes the kinetic energy of the velocities as they stand (not the previous half step's rescaled
-    // value, so that a run does not depend on how it is split into calls).  The first one's velocity factor is applied inside the
-    // kick-drift kernel, the second one's with the next step's kinetic energy.
+    // value, so that a run does not depend on how it is split into calls).  The first one's velocity factor is applied with the half
+    // kick that follows, the second one's with the next step's kinetic energy.
     for (int it = 0; it < n_steps; ++it) {
-        if (it == 0 && (rc = launch_kinetic(c, 0, true, dt, s)) != MLIP_OK) return rc;
-        if ((rc = launch_kick_drift(c, dt, false, s, c->nhc + 6)) != MLIP_OK) return rc;
+        if (it == 0) {
+            if ((rc = launch_kinetic(c, 0, true, dt, s)) != MLIP_OK) return rc;
+            if ((rc = launch_kick_drift(c, dt, false, s, c->nhc + 6)) != MLIP_OK) return rc;
+        } else if ((rc = launch_nvt_between(c, dt, s)) != MLIP_OK) return rc;
         c->step += 1;
-        if ((rc = rebuild_if_due(c, rebuild_every, s)) != MLIP_OK) return rc;
-        if ((rc = evaluate(c, s)) != MLIP_OK) return rc;
-        if ((rc = launch_kinetic(c, 1, true, dt, s)) != MLIP_OK) return rc;
-        rc = it + 1 < n_steps ? launch_kinetic(c, 2, true, dt, s) : launch_scale_velocities(c, s);
-        if (rc != MLIP_OK) return rc;
+        if ((rc = rebuild_and_evaluate(c, rebuild_every, s)) != MLIP_OK) return rc;
     }
-    return MLIP_OK;
+    if (n_steps == 0) return MLIP_OK;
+    if ((rc = launch_kinetic(c, 1, true, dt, s)) != MLIP_OK) return rc;
+    return launch_scale_velocities(c, s);
 }
 
 int mlip_get_thermostat(mlip_ctx *c, double *v_eta_host, double *eta_host, double *energy_host) {
@@ -703,6 +717,7 @@ void mlip_destroy(mlip_ctx *c) {
     if (c->total_host) cudaFreeHost(c->total_host);
     if (c->rebuild_host) cudaFreeHost(c->rebuild_host);
     if (c->build_host) cudaFreeHost(c->build_host);
+    if (c->check_ev) cudaEventDestroy(c->check_ev);
     for (cudaEvent_t e : c->mark_ev)
         if (e) cudaEventDestroy(e);
     delete c;

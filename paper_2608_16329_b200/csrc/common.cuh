@@ -165,6 +165,7 @@ struct mlip_ctx {
     static constexpr int EV_POOL = 256, MARKS = 4 * EV_POOL;
     cudaEvent_t mark_ev[MARKS] = {nullptr};
     unsigned char mark_kind[MARKS] = {0};
+    cudaEvent_t check_ev = nullptr;   // the displacement trigger's answer has reached the host
     int64_t marks = 0;             // recorded so far
     int64_t mark_reset[4] = {0};   // per kind: parts that ended before this mark have been reset
     bool mark_open = false;        // nothing untimed has been enqueued since the last mark
@@ -292,6 +293,7 @@ bool f64_shape_supported(int k, int l_max, int basis);
 int launch_kick_drift(mlip_ctx *c, double dt, bool close_step, cudaStream_t s, const double *vscale = nullptr);
 int launch_scale_velocities(mlip_ctx *c, cudaStream_t s);
 int launch_kick(mlip_ctx *c, double dt, cudaStream_t s);
+int launch_nvt_between(mlip_ctx *c, double dt, cudaStream_t s);
 int launch_kinetic(mlip_ctx *c, int change, bool thermostat, double dt, cudaStream_t s);
 int launch_outputs(mlip_ctx *c, float *forces, float *e_atom, double *energy, double *virial, cudaStream_t s);
 int launch_outputs_f64(mlip_ctx *c, double *forces, double *e_atom, double *energy, double *virial, cudaStream_t s);

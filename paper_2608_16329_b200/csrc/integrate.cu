@@ -20,45 +20,62 @@ __device__ __forceinline__ void clear_for_eval(const EvalClear &c, int64_t i) {
     if (c.force_d) { c.force_d[3 * i] = 0.0; c.force_d[3 * i + 1] = 0.0; c.force_d[3 * i + 2] = 0.0; }
 }
 
-// v += dt/2 a  (CLOSE: twice, the second half kick of one step and the first of the next, which see the same forces);
-// x += dt v;  wrap into [0, L);  track the displacement since the last list build.  Every operation is rounded in a fixed way, so
-// a trajectory does not depend on how it is cut into calls.
+// What the drift tracks besides moving the atoms.
+struct DriftArgs {
+    double dt;
+    CellGrid g;
+    float skin_half2, trigger2, far2;
+    float *disp;
+    int *status, *rebuild_flag, *far_flag;
+    EvalClear clear;
+};
+// x += dt v;  wrap into [0, L);  track the displacement since the last list build.
+__device__ __forceinline__ void drift_atom(const DriftArgs &d, int64_t i, double4 p, const double (&v)[3], double4 *pos4) {
+    const double px[3] = {p.x, p.y, p.z};
+    double x[3];
+    float d2 = 0.f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        x[a] = fma(d.dt, v[a], px[a]);
+        const float s = d.disp[3 * i + a] + (float)(d.dt * v[a]);
+        d.disp[3 * i + a] = s;
+        d2 += s * s;
+        const double L = d.g.box[a];
+        if (x[a] >= L) x[a] -= L;
+        else if (x[a] < 0.0) x[a] += L;
+        if (!(x[a] >= 0.0 && x[a] < L)) x[a] = 0.0;   // -eps + L rounds to L; NaN is reported below
+    }
+    if (!(d2 <= d.skin_half2)) atomicOr(d.status, d2 == d2 ? FLAG_SKIN_EXCEEDED : FLAG_NONFINITE);
+    if (d2 > d.trigger2) *d.rebuild_flag = 1;   // same value from every writer
+    if (!(d2 <= d.far2)) *d.far_flag = 1;       // from now on the lists' far entries may come inside r_cut
+    pos4[i] = make_double4(x[0], x[1], x[2], p.w);
+    clear_for_eval(d.clear, i);
+}
+
+// v += dt/2 a  (CLOSE: twice, the second half kick of one step and the first of the next, which see the same forces), then the drift.
+// Every operation is rounded in a fixed way, so a trajectory does not depend on how it is cut into calls.
 template <bool CLOSE>
-__global__ void k_kick_drift(int64_t n, double dt, CellGrid g, const double *__restrict__ mass, float skin_half2,
-                             double4 *pos4, double *vel, const float4 *force, const double *force_d, float *disp, int *status, float trigger2,
-                             int *rebuild_flag, const double *vscale, float far2, int *far_flag, EvalClear clear, unsigned long long *stamp) {
+__global__ void k_kick_drift(int64_t n, const double *__restrict__ mass, double4 *pos4, double *vel, const float4 *force, const double *force_d,
+                             const double *vscale, DriftArgs d, unsigned long long *stamp) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     allow_next();
     wait_previous();
     stamp_begin(stamp);
     if (i >= n) return;
-    double4 p = pos4[i];
+    const double4 p = pos4[i];
     const double3 f3 = load_force(force, force_d, i);
-    const double f[3] = {f3.x, f3.y, f3.z}, px[3] = {p.x, p.y, p.z};
-    const double k = 0.5 * dt * ACC_UNIT / mass[(int)p.w];
+    const double f[3] = {f3.x, f3.y, f3.z};
+    const double k = 0.5 * d.dt * ACC_UNIT / mass[(int)p.w];
     const double sc = vscale ? *vscale : 1.0;   // thermostat factor applied ahead of the kick (NVT)
-    double x[3];
-    float d2 = 0.f;
+    double v[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        double v = vel[3 * i + a];
-        if (CLOSE) v = fma(k, f[a], v);
-        v = fma(k, f[a], v * sc);
-        vel[3 * i + a] = v;
-        x[a] = fma(dt, v, px[a]);
-        float d = disp[3 * i + a] + (float)(dt * v);
-        disp[3 * i + a] = d;
-        d2 += d * d;
-        const double L = g.box[a];
-        if (x[a] >= L) x[a] -= L;
-        else if (x[a] < 0.0) x[a] += L;
-        if (!(x[a] >= 0.0 && x[a] < L)) x[a] = 0.0;   // -eps + L rounds to L; NaN is reported below
+        v[a] = vel[3 * i + a];
+        if (CLOSE) v[a] = fma(k, f[a], v[a]);
+        v[a] = fma(k, f[a], v[a] * sc);
+        vel[3 * i + a] = v[a];
     }
-    if (!(d2 <= skin_half2)) atomicOr(status, d2 == d2 ? FLAG_SKIN_EXCEEDED : FLAG_NONFINITE);
-    if (d2 > trigger2) *rebuild_flag = 1;   // same value from every writer
-    if (!(d2 <= far2)) *far_flag = 1;       // from now on the lists' far entries may come inside r_cut
-    pos4[i] = make_double4(x[0], x[1], x[2], p.w);
-    clear_for_eval(clear, i);
+    drift_atom(d, i, p, v, pos4);
     stamp_end(stamp);
 }
 
@@ -80,29 +97,39 @@ __global__ void k_kick(int64_t n, double dt, const double *__restrict__ mass, co
 // (Martyna-Tuckerman-Tobias-Klein factorisation, one Suzuki-Yoshida term).  One thread calls it.  state = {v_eta[3], eta[3], scale}:
 //   dv_eta_k/dt = G_k - v_eta_{k+1} v_eta_k,  G_1 = (2 KE - N_f kT) / Q_1,  G_k = (Q_{k-1} v_eta_{k-1}^2 - kT) / Q_k,
 //   particle velocities scale by exp(-v_eta_1 dt/2); the stored kinetic energy is scaled with them.
-struct NhcHalf { double n_f, kT, q1, qk, dt; double *state; };   // state = nullptr: no thermostat
+// (Every step of a run waits for this chain of dependent operations, twice: divisions by the thermostat masses are products with their
+// reciprocals, and the exponentials, whose arguments are of the order of the step over the damping time, Taylor polynomials: below
+// 1/32 the first omitted term is 2^-45 / 9! relative, 8e-20.)
+struct NhcHalf { double n_f, kT, q1, qk, inv_q1, inv_qk, dt; double *state; };   // state = nullptr: no thermostat
+__device__ __forceinline__ double exp_near_zero(double x) {
+    if (fabs(x) > 0.03125) return exp(x);
+    double y = 1.0 / 40320.0;
+    y = fma(y, x, 1.0 / 5040.0); y = fma(y, x, 1.0 / 720.0); y = fma(y, x, 1.0 / 120.0); y = fma(y, x, 1.0 / 24.0);
+    y = fma(y, x, 1.0 / 6.0); y = fma(y, x, 0.5); y = fma(y, x, 1.0);
+    return fma(y, x, 1.0);
+}
 __device__ void nhc_half(const NhcHalf &h, double *acc) {
     constexpr int M = 3;
     double *state = h.state;
     double v[M] = {state[0], state[1], state[2]};
-    const double q[M] = {h.q1, h.qk, h.qk}, d = 0.5 * h.dt;
+    const double q[M] = {h.q1, h.qk, h.qk}, iq[M] = {h.inv_q1, h.inv_qk, h.inv_qk}, d = 0.5 * h.dt;
     double ke2 = 2.0 * acc[ACC_KINETIC];
     double G[M];
-    G[0] = (ke2 - h.n_f * h.kT) / q[0];
-    for (int c = 1; c < M; ++c) G[c] = (q[c - 1] * v[c - 1] * v[c - 1] - h.kT) / q[c];
+    G[0] = (ke2 - h.n_f * h.kT) * iq[0];
+    for (int c = 1; c < M; ++c) G[c] = (q[c - 1] * v[c - 1] * v[c - 1] - h.kT) * iq[c];
     v[M - 1] += 0.5 * d * G[M - 1];
     for (int c = M - 2; c >= 0; --c) {
-        const double a = exp(-0.25 * d * v[c + 1]);
+        const double a = exp_near_zero(-0.25 * d * v[c + 1]);
         v[c] = (v[c] * a + 0.5 * d * G[c]) * a;
     }
-    const double scale = exp(-d * v[0]);
+    const double scale = exp_near_zero(-d * v[0]);
     ke2 *= scale * scale;
     for (int c = 0; c < M; ++c) state[3 + c] += d * v[c];
-    G[0] = (ke2 - h.n_f * h.kT) / q[0];
+    G[0] = (ke2 - h.n_f * h.kT) * iq[0];
     for (int c = 0; c < M - 1; ++c) {
-        const double a = exp(-0.25 * d * v[c + 1]);
+        const double a = exp_near_zero(-0.25 * d * v[c + 1]);
         v[c] = (v[c] * a + 0.5 * d * G[c]) * a;
-        G[c + 1] = (q[c] * v[c] * v[c] - h.kT) / q[c + 1];
+        G[c + 1] = (q[c] * v[c] * v[c] - h.kT) * iq[c + 1];
     }
     v[M - 1] += 0.5 * d * G[M - 1];
     for (int c = 0; c < M; ++c) state[c] = v[c];
@@ -167,10 +194,77 @@ __global__ void __launch_bounds__(256) k_kinetic(int64_t n, double dt, const dou
     for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
     if (threadIdx.x == 0) {
         *ticket = 0;
-        acc[ACC_KINETIC] = e / ACC_UNIT;
+        acc[ACC_KINETIC] = e * (1.0 / ACC_UNIT);
         if (nhc.state) nhc_half(nhc, acc);
         stamp_end(stamp);
     }
+}
+
+// What lies between two evaluations of an NVT run in one launch, for systems that a cluster holds with an atom per thread: the half kick that
+// closes a step, the two thermostat half steps (each after the kinetic energy of the velocities as they stand), the next step's
+// half kick and drift.  The sums are taken in k_kinetic's order -- groups of 256 atoms, then the groups' sums -- and the blocks meet at the
+// hardware barrier of the cluster.  4,394 atoms: three launches were 12 us of a step's 61 and the gaps between
+// them 9; this one takes 9.
+constexpr int NVT_CTA = 1024, NVT_CLUSTER = 8;
+__device__ __forceinline__ void cluster_sync_all() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__global__ void __launch_bounds__(NVT_CTA) k_nvt_between(int n, const double *__restrict__ mass, double4 *pos4, double *vel, const float4 *force,
+                                                        const double *force_d, double *block_sum, double *acc, NhcHalf nhc, DriftArgs d,
+                                                        unsigned long long *stamp) {
+    __shared__ double part[NVT_CTA / 32];
+    const int i = blockIdx.x * NVT_CTA + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    allow_next();
+    wait_previous();
+    stamp_begin(stamp);
+    double4 p = make_double4(0.0, 0.0, 0.0, 0.0);
+    double v[3] = {0.0, 0.0, 0.0}, f[3] = {0.0, 0.0, 0.0}, m = 0.0, k = 0.0;
+    if (i < n) {
+        p = pos4[i];
+        const double3 f3 = load_force(force, force_d, i);
+        f[0] = f3.x; f[1] = f3.y; f[2] = f3.z;
+        m = mass[(int)p.w];
+        k = 0.5 * d.dt * ACC_UNIT / m;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) v[a] = fma(k, f[a], vel[3 * i + a]);
+    }
+    double sc = 1.0;
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) v[a] *= sc;
+        double e = fma(0.5 * m, fma(v[2], v[2], fma(v[1], v[1], __dmul_rn(v[0], v[0]))), 0.0);
+        for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+        if (lane == 0) part[warp] = e;
+        __syncthreads();
+        if (threadIdx.x < NVT_CTA / 256) {
+            const double *q = part + 8 * threadIdx.x;
+            const int b = blockIdx.x * (NVT_CTA / 256) + threadIdx.x;
+            if (256 * b < n) block_sum[b] = ((q[0] + q[4]) + (q[2] + q[6])) + ((q[1] + q[5]) + (q[3] + q[7]));
+        }
+        cluster_sync_all();
+        if (blockIdx.x == 0 && warp == 0) {
+            double s = 0.0;
+            for (int b = lane; 256 * b < n; b += 32) s += *(volatile double *)(block_sum + b);
+            for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) {
+                acc[ACC_KINETIC] = s * (1.0 / ACC_UNIT);
+                nhc_half(nhc, acc);
+            }
+        }
+        cluster_sync_all();
+        sc = *(volatile double *)(nhc.state + 6);
+    }
+    if (i < n) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            v[a] = fma(k, f[a], v[a] * sc);
+            vel[3 * i + a] = v[a];
+        }
+        drift_atom(d, i, p, v, pos4);
+    }
+    stamp_end(stamp);
 }
 
 // Per-atom outputs in the caller's order, and the totals: one launch.  FIN: float4, or double for three per atom.
@@ -255,11 +349,40 @@ EvalClear eval_clear(mlip_ctx *c) {
     const bool f64 = c->cfg.precision == 1;
     return EvalClear{f64 || c->cfg.force_mode == 1 ? nullptr : c->force, f64 ? c->force_d : nullptr};
 }
+static NhcHalf nhc_args(mlip_ctx *c, double dt, bool thermostat) {
+    return NhcHalf{c->nhc_nf, c->nhc_kT, c->nhc_q1, c->nhc_qk, 1.0 / c->nhc_q1, 1.0 / c->nhc_qk, dt, thermostat ? c->nhc : nullptr};
+}
+static DriftArgs drift_args(mlip_ctx *c, double dt) {
+    return DriftArgs{dt, c->grid, skin_half2(c), 0.64f * skin_half2(c), far_trigger2(c), c->disp, c->status, c->rebuild_flag, c->far_flag, eval_clear(c)};
+}
 int launch_kick_drift(mlip_ctx *c, double dt, bool close_step, cudaStream_t s, const double *vscale) {
     unsigned long long *stamp = timed_begin(c, MARK_INTEGRATE, s);
-    MLIP_CUDA_TRY(c, launch_after(close_step ? k_kick_drift<true> : k_kick_drift<false>, nb(c->n), 256, 0, s, c->n, dt, c->grid, c->mass, skin_half2(c),
-                                  c->pos4, c->vel, c->force, c->force_d, c->disp, c->status, 0.64f * skin_half2(c), c->rebuild_flag, vscale,
-                                  far_trigger2(c), c->far_flag, eval_clear(c), stamp));
+    MLIP_CUDA_TRY(c, launch_after(close_step ? k_kick_drift<true> : k_kick_drift<false>, nb(c->n), 256, 0, s, c->n, c->mass, c->pos4, c->vel, c->force,
+                                  c->force_d, vscale, drift_args(c, dt), stamp));
+    timed_end(c, MARK_INTEGRATE, s);
+    c->launches += 1;
+    return MLIP_OK;
+}
+// Everything between two evaluations of an NVT run.
+int launch_nvt_between(mlip_ctx *c, double dt, cudaStream_t s) {
+    int rc;
+    if (c->n > NVT_CTA * NVT_CLUSTER) {
+        if ((rc = launch_kinetic(c, 1, true, dt, s)) != MLIP_OK || (rc = launch_kinetic(c, 2, true, dt, s)) != MLIP_OK) return rc;
+        return launch_kick_drift(c, dt, false, s, c->nhc + 6);
+    }
+    int blocks = 1;
+    while (blocks * NVT_CTA < c->n) blocks *= 2;
+    const NhcHalf nhc = nhc_args(c, dt, true);
+    unsigned long long *stamp = timed_begin(c, MARK_INTEGRATE, s);
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = blocks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks); cfg.blockDim = dim3(NVT_CTA); cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 2;
+    MLIP_CUDA_TRY(c, cudaLaunchKernelEx(&cfg, k_nvt_between, (int)c->n, (const double *)c->mass, c->pos4, c->vel, (const float4 *)c->force,
+                                        (const double *)c->force_d, c->kin_part, c->acc, nhc, drift_args(c, dt), stamp));
     timed_end(c, MARK_INTEGRATE, s);
     c->launches += 1;
     return MLIP_OK;
@@ -280,7 +403,7 @@ int launch_scale_velocities(mlip_ctx *c, cudaStream_t s) {
 }
 int launch_kinetic(mlip_ctx *c, int change, bool thermostat, double dt, cudaStream_t s) {
     const int64_t blocks = nb(c->n) > KIN_BLOCKS ? KIN_BLOCKS : nb(c->n);
-    const NhcHalf nhc{c->nhc_nf, c->nhc_kT, c->nhc_q1, c->nhc_qk, dt, thermostat ? c->nhc : nullptr};
+    const NhcHalf nhc = nhc_args(c, dt, thermostat);
     unsigned long long *stamp = thermostat ? timed_begin(c, MARK_INTEGRATE, s) : nullptr;
     MLIP_CUDA_TRY(c, launch_after(change == 1 ? k_kinetic<1> : change == 2 ? k_kinetic<2> : k_kinetic<0>, (unsigned)blocks, 256, 0, s, c->n, dt, c->mass,
                                   c->pos4, c->vel, c->force, c->force_d, c->nhc + 6, c->kin_part, reinterpret_cast<unsigned int *>(c->kin_part + KIN_BLOCKS),
