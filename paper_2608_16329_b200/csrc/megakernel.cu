@@ -230,14 +230,6 @@ struct KernelArgs {
     unsigned long long *stamp;
 };
 
-// One 256-bit load per gathered atom (a 32-byte sector) instead of two 128-bit ones: halves the
-// number of L1 wavefronts of the uncoalesced position gathers.
-__device__ __forceinline__ double4 load_pos4(const double4 *p) {
-    double4 v;
-    asm volatile("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];" : "=d"(v.x), "=d"(v.y), "=d"(v.z), "=d"(v.w) : "l"(p));
-    return v;
-}
-
 // The radial tables of the current central species: in shared memory or, when they do not fit, in global memory (same
 // layout).  Rows are numbered through the neighbor species.
 struct TableView {
@@ -381,7 +373,9 @@ __device__ __forceinline__ int encode_atom(const KernelArgs &k, const TableView 
                 const float4 e = pq[first + lane];
                 const float d2 = e.x * e.x + e.y * e.y + e.z * e.z, rinv = rsqrtf(d2), r = d2 * rinv;
                 harmonics(e.x * rinv, e.y * rinv, e.z * rinv, h);
-                const int iv = spline_basis<false, float>(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, b, nullptr, k.status);
+                float u;
+                const int iv = spline_interval(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, u, k.status);
+                cubic_basis(u, b);
                 row = (__float_as_int(e.w) >> J_BITS) * (k.tab.knots + 3) + iv;
             } else {
 #pragma unroll
@@ -551,7 +545,10 @@ __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView
             if (lane < n) {
                 const float4 ent = pq[first + lane];
                 const float d2 = ent.x * ent.x + ent.y * ent.y + ent.z * ent.z, r = d2 * rsqrtf(d2);
-                const int iv = spline_basis<true, float, true>(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, b, db, k.status);
+                float u;
+                const int iv = spline_interval(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, u, k.status);
+                cubic_basis(u, b);
+                cubic_basis_deriv(u, 1.f, db);
                 row = (__float_as_int(ent.w) >> J_BITS) * (k.tab.knots + 3) + iv;
             }
             const int turn = (lane - row) & 3;

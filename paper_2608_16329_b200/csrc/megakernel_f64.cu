@@ -61,16 +61,26 @@ struct TileSmem {
     static constexpr int D = Shape::D;
     static constexpr int NINV = (LMAX + 1) * K;
     static constexpr int XS = (NINV + 31) / 32 * 32 + 2;
-    double x[F64_TILE][XS];                 // invariants, then dE/dG
-    double y[2][F64_TILE][F64_YS];          // activations of the previous / current layer
-    double sd[HEAD_L][F64_TILE][F64_YS];    // SiLU'(pre-activation) per layer
-    double dp[2][F64_TILE][F64_YS];         // dE/dpre of the layer being propagated
-    union {
+    union PerWarp {
         double dv[16 * (12 + 16 * ((D + 7) / 8))];   // derivation staging of the tensor form: 16 pairs x (b, b', offset | V, T, pad)
         double w[D * K];                    // W_i = dE_i/dP_i (Eq. 7), derivation; P_i on its way from fragments to lane = channel
         double te[(D + 5) * 36];            // encoding hand-over of the tensor form: D rows of h, 4 of b, table offsets, 32 pairs (+ 4 pad) each
-    } pw[F64_TILE];
-    int q[F64_TILE][F64_QCAP];              // neighbor indices of the pairs inside r_cut: kept from the encoding to the derivation
+    };
+    struct Regression {                     // (between encoding and derivation nothing per warp but the queue is alive)
+        double y[2][F64_TILE][F64_YS];          // activations of the previous / current layer
+        double sd[HEAD_L][F64_TILE][F64_YS];    // SiLU'(pre-activation) per layer
+        double dp[2][F64_TILE][F64_YS];         // dE/dpre of the layer being propagated
+    };
+    double x[F64_TILE][XS];                 // invariants, then dE/dG
+    union {
+        PerWarp pw[F64_TILE];
+        Regression r;
+    };
+    // The pairs inside r_cut, kept from the encoding to the derivation: pair vector, 1 / r, position in the spline interval, neighbor index,
+    // table row.  (Gathered and computed again -- a round trip to L2, a square root and two divisions per pair -- they cost 12 of a
+    // warp's 140 thousand cycles per atom.)
+    double qd[F64_TILE][5][F64_QCAP];
+    int qj[F64_TILE][F64_QCAP], qrow[F64_TILE][F64_QCAP];
 };
 
 struct F64Args {
@@ -187,7 +197,7 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
         int64_t beg = 0, end = 0;
         if (have) {
             i = (int)MLIP_CHECK_INDEX(k.center_order[slot], k.n, k.status);
-            pi = k.pos4[i];
+            pi = load_pos4(k.pos4 + i);
             beg = k.nbr_off[i]; end = use_far ? k.nbr_off[i + 1] : beg + k.nbr_near[i];
         }
         // compact lists: lane q < 27 holds the first atom of the q-th cell around the atom's build-time cell
@@ -204,6 +214,11 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
         // (k = pair, columns = channels): lane (g, t) evaluates g of pair t at channels 16 q + 2 g, + 1 (q < K / 16), so the
         // eight lanes of a pair read 128 contiguous bytes of a table row per load and four rows are in flight per step; the
         // accumulators go through shared memory to lane = channel afterwards.
+        auto keep_pair = [&](int slot, int j, double dx, double dy, double dz, double rinv, double u, int row) {
+            sm.qd[wid][0][slot] = dx; sm.qd[wid][1][slot] = dy; sm.qd[wid][2][slot] = dz;
+            sm.qd[wid][3][slot] = rinv; sm.qd[wid][4][slot] = u;
+            sm.qj[wid][slot] = j; sm.qrow[wid][slot] = row;
+        };
         constexpr int MT = (D + 7) / 8, NTK = K / 8, PS = 36;   // PS = 4 mod 16 doubles: the A-fragment reads fall on 32 different banks
         double P[D][CPL];
 #pragma unroll
@@ -225,7 +240,7 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
                 double dx = 0.0, dy = 0.0, dz = 0.0, d2 = 1.0;
                 int sj = 0;
                 if (e < end) {
-                    const double4 pj = k.pos4[j_e];
+                    const double4 pj = load_pos4(k.pos4 + j_e);
                     dx = min_image(pj.x - pi.x, k.grid.box[0], k.grid.half[0]);
                     dy = min_image(pj.y - pi.y, k.grid.box[1], k.grid.half[1]);
                     dz = min_image(pj.z - pi.z, k.grid.box[2], k.grid.half[2]);
@@ -237,17 +252,20 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
                 const int nv = __popc(mask);
                 if (valid) {   // the pairs inside r_cut take consecutive columns of the hand-over rows
                     const int col = __popc(mask & ((1u << lane) - 1u));
-                    if (n_mine + col < F64_QCAP) sm.q[wid][n_mine + col] = j_e;
                     const double r = sqrt(d2), rinv = 1.0 / r;
                     double h[D > D_ANG ? D : D_ANG], b[4];
                     if (CLOSED) harmonics(dx * rinv, dy * rinv, dz * rinv, h);
                     else angular_values<LMAX, BASIS>(dx * rinv, dy * rinv, dz * rinv, h);
-                    const int iv = spline_basis<false, double>(r, k.r_min, k.inv_h, k.knots, b, nullptr, k.status);
+                    double u;
+                    const int iv = spline_interval(r, k.r_min, k.inv_h, k.knots, u, k.status);
+                    cubic_basis(u, b);
+                    const int row = (si * C + sj) * (k.knots + 3) + iv;
+                    if (n_mine + col < F64_QCAP) keep_pair(n_mine + col, j_e, dx, dy, dz, rinv, u, row);
     #pragma unroll
                     for (int a = 0; a < D; ++a) hs[a * PS + col] = h[a];
     #pragma unroll
                     for (int m = 0; m < 4; ++m) bq[m * PS + col] = b[m];
-                    offs[col] = __longlong_as_double(((long long)(si * C + sj) * (k.knots + 3) + iv) * K);
+                    offs[col] = __longlong_as_double((long long)row * K);
                 }
                 n_mine += nv;
                 __syncwarp();
@@ -332,21 +350,21 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
 #pragma unroll 1
                 for (int h0 = 0; h0 < NINV / 16; h0 += HS) head_dot<HS>(c0, c1, wrow + 16 * h0, xb + 16 * h0);
                 y0 = silu_d(c0, d0); y1 = silu_d(c1, d1);
-                sm.y[0][2 * t][n] = y0; sm.y[0][2 * t + 1][n] = y1;
-                sm.sd[0][2 * t][n] = d0; sm.sd[0][2 * t + 1][n] = d1;
+                sm.r.y[0][2 * t][n] = y0; sm.r.y[0][2 * t + 1][n] = y1;
+                sm.r.sd[0][2 * t][n] = d0; sm.r.sd[0][2 * t + 1][n] = d1;
             }
             __syncthreads();
 #pragma unroll 1
             for (int L = 1; L < HEAD_L; ++L) {
                 double c0 = hd[H.bias + L * HEAD_H + n], c1 = c0;
-                head_dot<HEAD_H / 16>(c0, c1, hd + H.wl + (L - 1) * HEAD_H * HEAD_H + n * HEAD_H + 4 * t, &sm.y[(L - 1) & 1][g][4 * t]);
+                head_dot<HEAD_H / 16>(c0, c1, hd + H.wl + (L - 1) * HEAD_H * HEAD_H + n * HEAD_H + 4 * t, &sm.r.y[(L - 1) & 1][g][4 * t]);
                 y0 += silu_d(c0, d0); y1 += silu_d(c1, d1);
-                sm.y[L & 1][2 * t][n] = y0; sm.y[L & 1][2 * t + 1][n] = y1;
-                sm.sd[L][2 * t][n] = d0; sm.sd[L][2 * t + 1][n] = d1;
+                sm.r.y[L & 1][2 * t][n] = y0; sm.r.y[L & 1][2 * t + 1][n] = y1;
+                sm.r.sd[L][2 * t][n] = d0; sm.r.sd[L][2 * t + 1][n] = d1;
                 __syncthreads();
             }
             {   // output layer: warp = atom
-                const double *yf = sm.y[(HEAD_L - 1) & 1][wid];
+                const double *yf = sm.r.y[(HEAD_L - 1) & 1][wid];
                 double e_i = hd[H.wout + lane] * yf[lane] + hd[H.wout + 32 + lane] * yf[lane + 32];
 #pragma unroll
                 for (int o = 16; o; o >>= 1) e_i += __shfl_xor_sync(0xffffffffu, e_i, o);
@@ -356,21 +374,21 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
             // reverse: this lane keeps dE/dy[n] of atoms 2t, 2t + 1; each hidden layer adds W^T (dE/dy . SiLU') through its
             // skip.  The transposed copies make the reverse pass read weight rows exactly as the forward pass does.
             double g0 = hd[H.wout + n], g1 = g0;
-            sm.dp[(HEAD_L - 1) & 1][2 * t][n] = g0 * sm.sd[HEAD_L - 1][2 * t][n];
-            sm.dp[(HEAD_L - 1) & 1][2 * t + 1][n] = g1 * sm.sd[HEAD_L - 1][2 * t + 1][n];
+            sm.r.dp[(HEAD_L - 1) & 1][2 * t][n] = g0 * sm.r.sd[HEAD_L - 1][2 * t][n];
+            sm.r.dp[(HEAD_L - 1) & 1][2 * t + 1][n] = g1 * sm.r.sd[HEAD_L - 1][2 * t + 1][n];
             __syncthreads();
 #pragma unroll 1
             for (int L = HEAD_L - 1; L >= 1; --L) {
-                head_dot<HEAD_H / 16>(g0, g1, hd + H.wlt + (L - 1) * HEAD_H * HEAD_H + n * HEAD_H + 4 * t, &sm.dp[L & 1][g][4 * t]);
-                sm.dp[(L - 1) & 1][2 * t][n] = g0 * sm.sd[L - 1][2 * t][n];
-                sm.dp[(L - 1) & 1][2 * t + 1][n] = g1 * sm.sd[L - 1][2 * t + 1][n];
+                head_dot<HEAD_H / 16>(g0, g1, hd + H.wlt + (L - 1) * HEAD_H * HEAD_H + n * HEAD_H + 4 * t, &sm.r.dp[L & 1][g][4 * t]);
+                sm.r.dp[(L - 1) & 1][2 * t][n] = g0 * sm.r.sd[L - 1][2 * t][n];
+                sm.r.dp[(L - 1) & 1][2 * t + 1][n] = g1 * sm.r.sd[L - 1][2 * t + 1][n];
                 __syncthreads();
             }
             // layer 0: dE/dG [NINV x 8] = W0^T dp, written over the invariants; warp = every 8th block of 8 inputs
 #pragma unroll 1
             for (int m = wid; m < NINV / 8; m += F64_TILE) {
                 double c0 = 0.0, c1 = 0.0;
-                head_dot<HEAD_H / 16>(c0, c1, hd + H.w0t + (size_t)(8 * m + g) * HEAD_H + 4 * t, &sm.dp[0][g][4 * t]);
+                head_dot<HEAD_H / 16>(c0, c1, hd + H.w0t + (size_t)(8 * m + g) * HEAD_H + 4 * t, &sm.r.dp[0][g][4 * t]);
                 sm.x[2 * t][8 * m + g] = c0; sm.x[2 * t + 1][8 * m + g] = c1;
             }
             __syncthreads();
@@ -405,7 +423,6 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
         static_assert(NB * (BS + VTS) * sizeof(double) <= sizeof(sm.pw[0]), "derivation staging must fit the hand-over buffer");
         double fx = 0.0, fy = 0.0, fz = 0.0;
         int nq = 0, qh = 0;                        // ring: nq indices from position qh
-        int *queue = sm.q[wid];
         double Bf[NT][K / 4];
         {
 #pragma unroll
@@ -420,20 +437,19 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
         pc.mark(5);
         auto process = [&](int nb) {
             pc.mark(6);
-            const int j = lane < nb ? queue[(qh + lane) & (F64_QCAP - 1)] : 0;
+            const int slot = (qh + lane) & (F64_QCAP - 1);
+            int j = 0;
             double x = 0.0, y = 0.0, z = 0.0, rinv = 0.0, ux = 0.0, uy = 0.0, uz = 0.0;
             double b[4] = {0.0, 0.0, 0.0, 0.0}, db[4] = {0.0, 0.0, 0.0, 0.0};
             const double *cf = k.coef;
             if (lane < nb) {
-                const double4 pj = k.pos4[j];
-                x = min_image(pj.x - pi.x, k.grid.box[0], k.grid.half[0]);
-                y = min_image(pj.y - pi.y, k.grid.box[1], k.grid.half[1]);
-                z = min_image(pj.z - pi.z, k.grid.box[2], k.grid.half[2]);
-                const double r = sqrt(x * x + y * y + z * z);
-                rinv = 1.0 / r;
+                j = sm.qj[wid][slot];
+                x = sm.qd[wid][0][slot]; y = sm.qd[wid][1][slot]; z = sm.qd[wid][2][slot]; rinv = sm.qd[wid][3][slot];
                 ux = x * rinv; uy = y * rinv; uz = z * rinv;
-                const int iv = spline_basis<true, double>(r, k.r_min, k.inv_h, k.knots, b, db, k.status);
-                cf = k.coef + ((size_t)(si * C + (int)pj.w) * (k.knots + 3) + iv) * K;
+                const double u = sm.qd[wid][4][slot];
+                cubic_basis(u, b);
+                cubic_basis_deriv(u, k.inv_h, db);
+                cf = k.coef + (size_t)sm.qrow[wid][slot] * K;
             }
             double s = 0.0, tx = 0.0, ty = 0.0, tz = 0.0, tu = 0.0;
             {
@@ -548,15 +564,24 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
                 const int64_t e = base + lane;
                 bool valid = false;
                 const int j = entry(e, e < end);
+                double dx = 0.0, dy = 0.0, dz = 0.0, d2 = 1.0;
+                int sj = 0;
                 if (e < end) {
-                    const double4 pj = k.pos4[j];
-                    const double dx = min_image(pj.x - pi.x, k.grid.box[0], k.grid.half[0]);
-                    const double dy = min_image(pj.y - pi.y, k.grid.box[1], k.grid.half[1]);
-                    const double dz = min_image(pj.z - pi.z, k.grid.box[2], k.grid.half[2]);
-                    valid = dx * dx + dy * dy + dz * dz < k.rc2;
+                    const double4 pj = load_pos4(k.pos4 + j);
+                    dx = min_image(pj.x - pi.x, k.grid.box[0], k.grid.half[0]);
+                    dy = min_image(pj.y - pi.y, k.grid.box[1], k.grid.half[1]);
+                    dz = min_image(pj.z - pi.z, k.grid.box[2], k.grid.half[2]);
+                    d2 = dx * dx + dy * dy + dz * dz;
+                    sj = (int)pj.w;
+                    valid = d2 < k.rc2;
                 }
                 const unsigned m = __ballot_sync(0xffffffffu, valid);
-                if (valid) queue[(qh + nq + __popc(m & ((1u << lane) - 1u))) & (F64_QCAP - 1)] = j;
+                if (valid) {
+                    const double r = sqrt(d2), rinv = 1.0 / r;
+                    double u;
+                    const int iv = spline_interval(r, k.r_min, k.inv_h, k.knots, u, k.status);
+                    keep_pair((qh + nq + __popc(m & ((1u << lane) - 1u))) & (F64_QCAP - 1), j, dx, dy, dz, rinv, u, (si * C + sj) * (k.knots + 3) + iv);
+                }
                 nq += __popc(m);
                 base += 32;
                 __syncwarp();

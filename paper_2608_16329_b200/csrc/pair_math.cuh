@@ -6,6 +6,14 @@
 
 namespace mlip {
 
+// One 256-bit load per gathered atom (a 32-byte sector) instead of two 128-bit ones: halves the
+// number of L1 wavefronts of the uncoalesced position gathers.
+__device__ __forceinline__ double4 load_pos4(const double4 *p) {
+    double4 v;
+    asm volatile("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];" : "=d"(v.x), "=d"(v.y), "=d"(v.z), "=d"(v.w) : "l"(p));
+    return v;
+}
+
 // Irreducible harmonic polynomials up to l = 3 of a unit vector (one valid solution of the
 // projection constraints of Section 3.3.1: harmonic, orthonormal under the multinomial metric).
 template <typename T>
@@ -63,29 +71,33 @@ __device__ __forceinline__ void harmonics_project(T x, T y, T z, const T *v, con
     tu = x * gx + y * gy + z * gz;
 }
 
-// Spline interval and cubic B-spline basis (and its r-derivative) at distance r for a table of
-// `knots` intervals of width 1 / inv_h starting at r_min.
-// PER_KNOT: the derivative per knot interval instead of per Angstrom (without the factor inv_h).
-template <bool DERIV, typename T, bool PER_KNOT = false>
-__device__ __forceinline__ int spline_basis(T r, T r_min, T inv_h, int knots, T *b, T *db, int *status) {
+// Spline interval of distance r in a table of `knots` intervals of width 1 / inv_h starting at r_min, and the position u in it (0..1).
+template <typename T>
+__device__ __forceinline__ int spline_interval(T r, T r_min, T inv_h, int knots, T &u, int *status) {
     T xk = (r - r_min) * inv_h;
     if (xk < T(0)) { atomicOr(status, FLAG_TABLE_RANGE); xk = T(0); }
     int i = (int)xk;
     i = i > knots - 1 ? knots - 1 : i;
-    T u = xk - (T)i, u2 = u * u, u3 = u2 * u, w = T(1) - u;
-    const T sixth = T(1) / T(6);
+    u = xk - (T)i;
+    return i;
+}
+// Cubic B-spline basis at position u of an interval.
+template <typename T>
+__device__ __forceinline__ void cubic_basis(T u, T *b) {
+    const T u2 = u * u, u3 = u2 * u, w = T(1) - u, sixth = T(1) / T(6);
     b[0] = w * w * w * sixth;
     b[1] = (T(3) * u3 - T(6) * u2 + T(4)) * sixth;
     b[2] = (T(-3) * u3 + T(3) * u2 + T(3) * u + T(1)) * sixth;
     b[3] = u3 * sixth;
-    if (DERIV) {
-        const T per = PER_KNOT ? T(1) : inv_h;
-        db[0] = T(-0.5) * w * w * per;
-        db[1] = (T(1.5) * u2 - T(2) * u) * per;
-        db[2] = (T(-1.5) * u2 + u + T(0.5)) * per;
-        db[3] = T(0.5) * u2 * per;
-    }
-    return i;
+}
+// Its derivative times `scale`: inv_h for the derivative per Angstrom, 1 for that per knot interval.
+template <typename T>
+__device__ __forceinline__ void cubic_basis_deriv(T u, T scale, T *db) {
+    const T u2 = u * u, w = T(1) - u;
+    db[0] = T(-0.5) * w * w * scale;
+    db[1] = (T(1.5) * u2 - T(2) * u) * scale;
+    db[2] = (T(-1.5) * u2 + u + T(0.5)) * scale;
+    db[3] = T(0.5) * u2 * scale;
 }
 
 }  // namespace mlip
