@@ -76,10 +76,10 @@ struct TileSmem {
         PerWarp pw[F64_TILE];
         Regression r;
     };
-    // The pairs inside r_cut, kept from the encoding to the derivation: pair vector, 1 / r, position in the spline interval, neighbor index,
-    // table row.  (Gathered and computed again -- a round trip to L2, a square root and two divisions per pair -- they cost 12 of a
-    // warp's 140 thousand cycles per atom.)
-    double qd[F64_TILE][5][F64_QCAP];
+    // The pairs inside r_cut, kept from the encoding to the derivation: pair vector, 1 / r, neighbor index, first row of the table.
+    // (Gathered and computed again -- a round trip to L2, a square root and two divisions per pair -- they cost 12 of a warp's 140
+    // thousand cycles per atom.  The spline position is taken from 1 / r again: with it here two CTAs of d = 20 do not fit.)
+    double qd[F64_TILE][4][F64_QCAP];
     int qj[F64_TILE][F64_QCAP], qrow[F64_TILE][F64_QCAP];
 };
 
@@ -214,10 +214,10 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
         // (k = pair, columns = channels): lane (g, t) evaluates g of pair t at channels 16 q + 2 g, + 1 (q < K / 16), so the
         // eight lanes of a pair read 128 contiguous bytes of a table row per load and four rows are in flight per step; the
         // accumulators go through shared memory to lane = channel afterwards.
-        auto keep_pair = [&](int slot, int j, double dx, double dy, double dz, double rinv, double u, int row) {
+        auto keep_pair = [&](int slot, int j, double dx, double dy, double dz, double rinv, int sj) {
             sm.qd[wid][0][slot] = dx; sm.qd[wid][1][slot] = dy; sm.qd[wid][2][slot] = dz;
-            sm.qd[wid][3][slot] = rinv; sm.qd[wid][4][slot] = u;
-            sm.qj[wid][slot] = j; sm.qrow[wid][slot] = row;
+            sm.qd[wid][3][slot] = rinv;
+            sm.qj[wid][slot] = j; sm.qrow[wid][slot] = (si * C + sj) * (k.knots + 3);
         };
         constexpr int MT = (D + 7) / 8, NTK = K / 8, PS = 36;   // PS = 4 mod 16 doubles: the A-fragment reads fall on 32 different banks
         double P[D][CPL];
@@ -259,13 +259,12 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
                     double u;
                     const int iv = spline_interval(r, k.r_min, k.inv_h, k.knots, u, k.status);
                     cubic_basis(u, b);
-                    const int row = (si * C + sj) * (k.knots + 3) + iv;
-                    if (n_mine + col < F64_QCAP) keep_pair(n_mine + col, j_e, dx, dy, dz, rinv, u, row);
+                    if (n_mine + col < F64_QCAP) keep_pair(n_mine + col, j_e, dx, dy, dz, rinv, sj);
     #pragma unroll
                     for (int a = 0; a < D; ++a) hs[a * PS + col] = h[a];
     #pragma unroll
                     for (int m = 0; m < 4; ++m) bq[m * PS + col] = b[m];
-                    offs[col] = __longlong_as_double((long long)row * K);
+                    offs[col] = __longlong_as_double(((long long)(si * C + sj) * (k.knots + 3) + iv) * K);
                 }
                 n_mine += nv;
                 __syncwarp();
@@ -446,10 +445,11 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
                 j = sm.qj[wid][slot];
                 x = sm.qd[wid][0][slot]; y = sm.qd[wid][1][slot]; z = sm.qd[wid][2][slot]; rinv = sm.qd[wid][3][slot];
                 ux = x * rinv; uy = y * rinv; uz = z * rinv;
-                const double u = sm.qd[wid][4][slot];
+                double u;
+                const int iv = spline_interval((x * x + y * y + z * z) * rinv, k.r_min, k.inv_h, k.knots, u, k.status);
                 cubic_basis(u, b);
                 cubic_basis_deriv(u, k.inv_h, db);
-                cf = k.coef + (size_t)sm.qrow[wid][slot] * K;
+                cf = k.coef + (size_t)(sm.qrow[wid][slot] + iv) * K;
             }
             double s = 0.0, tx = 0.0, ty = 0.0, tz = 0.0, tu = 0.0;
             {
@@ -577,10 +577,7 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
                 }
                 const unsigned m = __ballot_sync(0xffffffffu, valid);
                 if (valid) {
-                    const double r = sqrt(d2), rinv = 1.0 / r;
-                    double u;
-                    const int iv = spline_interval(r, k.r_min, k.inv_h, k.knots, u, k.status);
-                    keep_pair((qh + nq + __popc(m & ((1u << lane) - 1u))) & (F64_QCAP - 1), j, dx, dy, dz, rinv, u, (si * C + sj) * (k.knots + 3) + iv);
+                    keep_pair((qh + nq + __popc(m & ((1u << lane) - 1u))) & (F64_QCAP - 1), j, dx, dy, dz, 1.0 / sqrt(d2), sj);
                 }
                 nq += __popc(m);
                 base += 32;
@@ -664,6 +661,7 @@ int upload_head_f64(mlip_ctx *c, const double *w) {
 template <int K, int LMAX, int BASIS>
 static cudaError_t launch_shape(mlip_ctx *c, F64Args &k, cudaStream_t s) {
     const size_t smem_bytes = sizeof(TileSmem<K, LMAX, BASIS>);
+    static_assert((sizeof(TileSmem<K, LMAX, BASIS>) + 2048) * f64_ctas_per_sm<K, LMAX, BASIS>() <= 228 * 1024, "the resident CTAs' shared memory (with a kilobyte of their own) must fit the SM");
     if (!c->kernel_ready) {
         cudaError_t e = cudaFuncSetAttribute(k_mega_f64<K, LMAX, BASIS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
         if (e != cudaSuccess) return e;
