@@ -250,16 +250,15 @@ int mlip_create(mlip_ctx **out, const mlip_config *cfg, const double *enc_w, siz
         if ((rc = dev_alloc(c, &c->launch_base, (size_t)2 * LB_COUNT)) != MLIP_OK) break;
         next_eval_block(c);
         if ((rc = dev_alloc(c, &c->stamp, (size_t)2 * mlip_ctx::STAMPS)) != MLIP_OK) break;
-        if ((rc = dev_alloc(c, &c->build_word, 8)) != MLIP_OK) break;
-        c->status = c->build_word + 4; c->rebuild_flag = c->build_word + 5; c->far_flag = c->build_word + 6;
+        if ((rc = dev_alloc(c, &c->build_word, mlip_ctx::BUILD_WORDS)) != MLIP_OK) break;
+        c->status = c->build_word + 4; c->rebuild_flag = c->build_word + 5; c->far_flag = c->build_word + 6; c->species_start = c->build_word + 8;
         if ((rc = dev_alloc(c, &c->nhc, 8)) != MLIP_OK) break;
-        if ((rc = dev_alloc(c, &c->species_start, (size_t)MAX_SPECIES + 1)) != MLIP_OK) break;
         if ((rc = dev_alloc(c, &c->stage_out, 10)) != MLIP_OK) break;
         if ((rc = dev_alloc(c, &c->kin_part, 1185)) != MLIP_OK) break;
         if (cudaMallocHost((void **)&c->status_host, sizeof(int)) != cudaSuccess ||
             cudaMallocHost((void **)&c->total_host, sizeof(int64_t)) != cudaSuccess ||
             cudaMallocHost((void **)&c->rebuild_host, sizeof(int)) != cudaSuccess ||
-            cudaMallocHost((void **)&c->build_host, sizeof(int) * 8) != cudaSuccess) {
+            cudaMallocHost((void **)&c->build_host, sizeof(int) * mlip_ctx::BUILD_WORDS) != cudaSuccess) {
             rc = MLIP_ERR_CUDA; c->err = "pinned host allocation failed"; break;
         }
         bool ev_ok = true;
@@ -267,7 +266,7 @@ int mlip_create(mlip_ctx **out, const mlip_config *cfg, const double *enc_w, siz
         ev_ok = ev_ok && cudaEventCreateWithFlags(&c->check_ev, cudaEventDisableTiming) == cudaSuccess;
         if (!ev_ok) { rc = MLIP_ERR_CUDA; c->err = "event creation failed"; break; }
         if (cudaMemcpy(c->mass, mass, sizeof(double) * cfg->n_species, cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemset(c->build_word, 0, sizeof(int) * 8) != cudaSuccess ||
+            cudaMemset(c->build_word, 0, sizeof(int) * mlip_ctx::BUILD_WORDS) != cudaSuccess ||
             cudaMemset(c->nhc, 0, sizeof(double) * 8) != cudaSuccess || cudaMemset(c->kin_part, 0, sizeof(double) * 1185) != cudaSuccess || cudaMemset(c->launch_base, 0, sizeof(double) * 2 * LB_COUNT) != cudaSuccess) {
             rc = MLIP_ERR_CUDA; c->err = "initial upload failed"; break;
         }
@@ -711,7 +710,7 @@ void mlip_destroy(mlip_ctx *c) {
     cudaFree(c->nbr); cudaFree(c->scan_tmp); cudaFree(c->head_w); cudaFree(c->table); cudaFree(c->mass);
     cudaFree(c->head_w_d); cudaFree(c->table_d);
     cudaFree(c->launch_base); cudaFree(c->stamp); cudaFree(c->build_word); cudaFree(c->nhc);
-    cudaFree(c->species_start); cudaFree(c->stage_pos); cudaFree(c->stage_species); cudaFree(c->stage_force);
+    cudaFree(c->stage_pos); cudaFree(c->stage_species); cudaFree(c->stage_force);
     cudaFree(c->stage_out); cudaFree(c->kin_part);
     if (c->status_host) cudaFreeHost(c->status_host);
     if (c->total_host) cudaFreeHost(c->total_host);

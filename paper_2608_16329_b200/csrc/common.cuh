@@ -114,7 +114,8 @@ struct mlip_ctx {
     int32_t *cell_of = nullptr;    // per source atom
     int32_t *cell_count = nullptr, *cell_start = nullptr;   // [n_cells + 1]; cell_count is zero between builds
     int32_t *bin_count = nullptr, *bin_start = nullptr;                           // [C * n_cells + 1]
-    int32_t *species_start = nullptr;  // dev [C + 1]
+    int32_t *species_start = nullptr;  // dev [C + 1] (behind build_word)
+    int32_t species_host[mlip::MAX_SPECIES + 1] = {0};   // its copy since the last synchronising build (rebuilds inside steps do not change it)
     // lists
     int32_t *nbr_count = nullptr;  // [N]
     int32_t *nbr_near = nullptr;   // [N] leading entries of each list that were within r_cut + skin / 2 at build time
@@ -124,9 +125,10 @@ struct mlip_ctx {
     bool list16 = false;           // format of the current lists (mlip_config.list_format = 1 on a grid of >= 3 cells per edge)
     int32_t *cell_id = nullptr;    // [N] build-time cell of each atom as packed coordinates, internal order (allocated for list_format = 1)
     unsigned long long *tile_state = nullptr;   // [tile_words(N)] look-back words of the one-pass build
-    int *build_word = nullptr;     // {ticket, private overflow flag, total entries (64 bits)} of the one-pass build, then status, rebuild_flag, far_flag
+    int *build_word = nullptr;     // {ticket, private overflow flag, total entries (64 bits)} of the one-pass build, then status, rebuild_flag, far_flag, -, species_start
     float4 *rel_pos = nullptr;     // cell-relative positions of the build in progress
-    int *build_host = nullptr;     // pinned copy of its first five words
+    int *build_host = nullptr;     // pinned copy
+    static constexpr int BUILD_WORDS = 8 + mlip::MAX_SPECIES + 1;
     int64_t nbr_cap = 0, n_entries = 0;
     // scratch
     int64_t *scan_tmp = nullptr;   // block sums for the scans

@@ -208,7 +208,8 @@ struct KernelArgs {
     TableDesc tab;
     const double4 *pos4;
     const int32_t *center_order;
-    const int32_t *species_start;
+    int species_start[MAX_SPECIES + 1];   // in center_order (a step's own rebuilds do not change it)
+    int first_cta[MAX_SPECIES + 1];       // STAGGER: the first CTA that starts on a species
     const int64_t *nbr_off;
     const int32_t *nbr_near;   // leading entries of each list that can be inside r_cut while far_flag is down
     const int *far_flag;
@@ -911,7 +912,7 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
 
 constexpr int TOTALS = 9 + 16 + 1;   // per warp at the end: virial, E_i sums of up to 16 lanes, pairs
 template <int APW, bool TAB_SMEM, bool DET, bool L16, bool STAGGER>
-__global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words) {
+__global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ KernelArgs k, int tab_words) {
     extern __shared__ __align__(128) float smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     using LY = Layout<APW>;
@@ -974,19 +975,21 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
         __syncthreads();
         tmem_fence_after_sync();
     };
-    // STAGGER (small systems): the CTAs start on different central species, so that the species are worked on side by
-    // side rather than one after the other by mostly idle SMs (864 atoms: 64 instead of 92 us).  Large systems keep the
+    // STAGGER (small systems): the CTAs start on different central species, in proportion to the species' tiles, so that the species are
+    // worked on side by side rather than one after the other by mostly idle SMs.  Large systems keep the
     // plain loop: one front through the cell-ordered atoms, and a loop counter as the species costs 1 % less than a
     // computed one.  Either way a species whose tiles are all claimed already is passed over: staging its tables would
     // be the only thing left to do.
-    auto species_at = [&](int ss) { return STAGGER ? (int)((ss + blockIdx.x) % (unsigned)k.n_species) : ss; };
     // Every group's first tile is fixed (the CTAs that start on a species take its first tiles, group 0 of each before group 1 of any, which
     // spreads a small system over the SMs); the later ones are claimed from the species' counter, which counts from there.
     auto starters = [&](int species) {   // CTAs that start on it
-        return !STAGGER ? (species == 0 ? (int)gridDim.x : 0) : species < (int)gridDim.x ? ((int)gridDim.x - 1 - species) / k.n_species + 1 : 0;
+        return STAGGER ? k.first_cta[species + 1] - k.first_cta[species] : species == 0 ? (int)gridDim.x : 0;
     };
-    const int first_species = species_at(0);
-    const int first_tile = (STAGGER ? (int)(blockIdx.x / (unsigned)k.n_species) : (int)blockIdx.x) + group * starters(first_species);
+    int first_species = 0;
+    if (STAGGER)
+        while (first_species + 1 < k.n_species && k.first_cta[first_species + 1] <= (int)blockIdx.x) ++first_species;
+    auto species_at = [&](int ss) { return !STAGGER ? ss : first_species + ss < k.n_species ? first_species + ss : first_species + ss - k.n_species; };
+    const int first_tile = (int)blockIdx.x - (STAGGER ? k.first_cta[first_species] : 0) + group * starters(first_species);
     // The first species is staged, and the lists of the first tile's atoms fetched, ahead of the wait for the kernel before this one: they
     // change in list builds only, and the launch after a build does not start early.  864 atoms: 4 us of staging and 3 us of
     // dependent loads and claims out of 31 us a step lie in that kernel's shadow.
@@ -994,8 +997,8 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
     NextAtoms<APW> nx0;
     int near0 = 0;
     {
-        const int s_end0 = __ldg(k.species_start + first_species + 1);
-        const int slot0 = __ldg(k.species_start + first_species) + first_tile * NA + wg + GW * lane;
+        const int s_end0 = k.species_start[first_species + 1];
+        const int slot0 = k.species_start[first_species] + first_tile * NA + wg + GW * lane;
         nx0.k = &k; nx0.pf = pf; nx0.slot = (lane < APW && slot0 < s_end0) ? slot0 : -1;
         nx0.i = 0; nx0.beg = 0; nx0.len = 0; nx0.use_far = true; nx0.cid = 0;
         nx0.stage_a();
@@ -1015,7 +1018,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(KernelArgs k, int tab_words
     __syncwarp();
     for (int ss = 0; ss < k.n_species && !skip; ++ss) {
         const int species = species_at(ss);
-        const int s_beg = __ldg(k.species_start + species), s_end = __ldg(k.species_start + species + 1);
+        const int s_beg = k.species_start[species], s_end = k.species_start[species + 1];
         const int n_tiles = (s_end - s_beg + NA - 1) / NA;
         if (n_tiles == 0) continue;
         const int n_first = NG * starters(species);   // tiles that are not claimed
@@ -1374,8 +1377,10 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     const int shape = !in_smem ? 3 : n >= STAGGER_BELOW_ATOMS ? 2 : n >= ONE_PER_WARP_BELOW_ATOMS ? 1 : 0;
     const int apw = shape == 0 ? 1 : 2;
     const size_t smem_bytes = sizeof(float) * (size_t)((apw == 1 ? Layout<1>::FIXED : Layout<2>::FIXED) + tab_words);
-    const int64_t tiles_max = (n + GW * apw - 1) / (GW * apw) + c->cfg.n_species;
-    const int blocks = (int)std::min<int64_t>(tiles_max, (int64_t)c->n_sm);
+    const int C = c->cfg.n_species, tile_atoms = GW * apw;
+    int64_t tiles[MAX_SPECIES], all = 0;
+    for (int q = 0; q < C; ++q) all += tiles[q] = (c->species_host[q + 1] - c->species_host[q] + tile_atoms - 1) / tile_atoms;
+    const int blocks = (int)std::min<int64_t>(all, (int64_t)c->n_sm);
     if (!c->kernel_ready) {
         for (int q = 0; q < 16; ++q) {
             const int most = (q < 4 ? Layout<1>::FIXED : Layout<2>::FIXED) + (q < 12 ? tab_words : 0);
@@ -1386,12 +1391,22 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     }
     KernelArgs k;
     k.n = n; k.n_species = c->cfg.n_species; k.grid = c->grid; k.rc2 = c->cfg.r_cut * c->cfg.r_cut; k.tab = c->tab;
-    k.pos4 = c->pos4; k.center_order = c->center_order; k.species_start = c->species_start;
+    k.pos4 = c->pos4; k.center_order = c->center_order;
     k.nbr_off = c->nbr_off; k.nbr_near = c->nbr_near; k.far_flag = c->far_flag; k.nbr = c->nbr; k.nbr16 = reinterpret_cast<const uint16_t *>(c->nbr); k.cell_id = c->cell_id; k.cell_start = c->cell_start;
     k.nbr_cap = c->nbr_cap; k.head_pack = c->head_w; k.force = c->force; k.e_atom = c->e_atom;
     k.force_fx = c->force_fx; k.acc_fx = c->acc_fx;
     k.acc = c->acc; k.pair_counter = c->pair_counter; k.status = c->status; k.tile_counter = c->tile_counter;
     k.clear_block = clear_block;
+    // CTAs in proportion to the species' tiles, at least one to a species that has any.  (One evaluation in us with the CTAs dealt out to the
+    // species in turn / in proportion: 864 atoms 90:5:5 46 / 23.5, 6,912 atoms 80 / 66, 13,824 atoms 47:12:41 116 / 96; six equal
+    // species, where in turn left some with more tiles than groups, 864 atoms 35.7 / 28.4, 23,328 atoms 221 / 198.)
+    int64_t weight[MAX_SPECIES], total = 0, before = 0;
+    for (int q = 0; q < C; ++q) total += weight[q] = tiles[q] > 0 ? std::max<int64_t>(tiles[q], 2 * all / blocks) : 0;
+    for (int q = 0; q <= MAX_SPECIES; ++q) {
+        k.species_start[q] = c->species_host[std::min(q, C)];
+        k.first_cta[q] = q < C ? (int)(before * blocks / total) : blocks;
+        if (q < C) before += weight[q];
+    }
     k.stamp = timed_begin(c, MARK_KERNEL, s);
     const bool early = !c->lists_fresh;   // (the kernel reads the lists before it waits)
     c->lists_fresh = false;

@@ -932,10 +932,11 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
         MLIP_CUDA_TRY(c, cudaGetLastError());
         bool done = true;
         if (allow_sync_grow) {
-            // {ticket, overflow, total, status} are neighbors in memory: one copy
-            MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->build_host, c->build_word, sizeof(int) * 5, cudaMemcpyDeviceToHost, s));
+            // {ticket, overflow, total, status} and the species' starts are neighbors in memory: one copy
+            MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->build_host, c->build_word, sizeof(int) * mlip_ctx::BUILD_WORDS, cudaMemcpyDeviceToHost, s));
             MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
             if (c->build_host[4] & FLAG_NONFINITE) return refuse_broken_input(c, s);
+            memcpy(c->species_host, c->build_host + 8, sizeof c->species_host);
             int64_t total;
             memcpy(&total, c->build_host + 2, sizeof total);
             done = c->build_host[1] == 0 && total <= c->nbr_cap;
@@ -954,9 +955,10 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
     MLIP_CUDA_TRY(c, cudaGetLastError());
     if (allow_sync_grow) {
         MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->total_host, c->nbr_off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->status_host, c->status, sizeof(int), cudaMemcpyDeviceToHost, s));
+        MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->build_host, c->build_word, sizeof(int) * mlip_ctx::BUILD_WORDS, cudaMemcpyDeviceToHost, s));
         MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
-        if (*c->status_host & FLAG_NONFINITE) return refuse_broken_input(c, s);
+        if (c->build_host[4] & FLAG_NONFINITE) return refuse_broken_input(c, s);
+        memcpy(c->species_host, c->build_host + 8, sizeof c->species_host);
         c->n_entries = *c->total_host;
         if (c->n_entries > c->nbr_cap) {
             int64_t want = c->n_entries + c->n_entries / 8 + 1024;

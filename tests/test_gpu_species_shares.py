@@ -1,0 +1,34 @@
+"""Start of the fused kernel's CTAs on the species in proportion to their tiles: species with no atom, with one atom, with nearly all
+of them; fewer tiles than SMs, and systems of two-atom tiles."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("cells,counts", [(4, (0, 1, 0)), (4, (1, 0, 1)), (4, (8, 9, 0)), (5, (250, 0, 1)), (6, (1, 1, 1, 1, 1, 1, 1)),
+                                          (7, (100, 0, 200, 0, 300, 0, 1)), (15, (1, 17, 12000)), (15, (0, 6000, 1))])
+def test_uneven_species_match_the_oracle(cells, counts):
+    """counts: atoms of the first species; the last one takes the rest.  Tolerances: those of the order-one workloads, forces
+    relative to their RMS where that exceeds 1 eV/Angstrom."""
+    import paper_2608_16329_b200 as mlip
+    rng = np.random.default_rng(cells + len(counts))
+    a, n_species = 3.9, len(counts) + 1
+    box = np.full(3, a * cells)
+    pos = wl.lattice_sites((cells, cells, cells), a, wl._FCC_BASIS) + rng.normal(0.0, 0.03, (4 * cells ** 3, 3))
+    pos -= np.floor(pos / box) * box
+    species = np.full(len(pos), n_species - 1, dtype=np.int32)
+    species[rng.permutation(len(pos))[:sum(counts)]] = np.repeat(np.arange(len(counts)), counts)
+    enc, head = wl.make_weights(n_species, seed=78, enc_out_scale=0.05, head_out_scale=0.3)
+    pot = mlip.Potential(n_species, 6.0, 0.5, enc, head, np.full(n_species, 50.0))
+    pot.build_neighbors(pos, species, box)
+    out = pot.compute(want_e_atom=True)
+    pot.sync_status()
+    ref = oracle.evaluate(oracle.Model(n_species, 6.0, enc, head), pos, species, box)
+    scale = max(1.0, float(np.sqrt((ref["forces"] ** 2).sum(1).mean())))
+    assert abs(float(out["energy"].cpu()) - ref["energy"]) <= 1e-6 * abs(ref["energy"])
+    assert np.abs(out["forces"].cpu().numpy() - ref["forces"]).max() <= 1e-4 * scale
+    assert np.abs(out["e_atom"].cpu().numpy() - ref["e_atom"]).max() <= 2e-5 * max(1.0, np.abs(ref["e_atom"]).max())
