@@ -89,7 +89,6 @@ constexpr int HC_WORDS = (HC_USED + 15) / 16 * 16;
 // (kernel us with 8- / 16-atom tiles, 6 species: 864 atoms 47 / 53, 6,912 96 / 97, 16,384 174 / 166, 55,296 499 / 474, 131,072
 // 1119 / 1046; one species: 4,394 63 / 66, 16,000 140 / 135, 65,536 476 / 441).
 constexpr int64_t ONE_PER_WARP_BELOW_ATOMS = 12000;
-constexpr int64_t STAGGER_BELOW_ATOMS = 200000;                 // systems below this size start their CTAs on different species
 // Shared memory per tile shape.  Two atoms per warp halve the regression's barriers, weight fetches and idle time per atom
 // (each warp owns 16 neurons x 8 atoms of a 16-atom tile instead of half of the warps owning an 8-atom tile); one atom per warp
 // spreads a small system over more SMs.
@@ -209,7 +208,7 @@ struct KernelArgs {
     const double4 *pos4;
     const int32_t *center_order;
     int species_start[MAX_SPECIES + 1];   // in center_order (a step's own rebuilds do not change it)
-    int first_cta[MAX_SPECIES + 1];       // STAGGER: the first CTA that starts on a species
+    int first_cta[MAX_SPECIES + 1];       // the first CTA that starts on a species
     const int64_t *nbr_off;
     const int32_t *nbr_near;   // leading entries of each list that can be inside r_cut while far_flag is down
     const int *far_flag;
@@ -911,7 +910,7 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
 }
 
 constexpr int TOTALS = 9 + 16 + 1;   // per warp at the end: virial, E_i sums of up to 16 lanes, pairs
-template <int APW, bool TAB_SMEM, bool DET, bool L16, bool STAGGER>
+template <int APW, bool TAB_SMEM, bool DET, bool L16>
 __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ KernelArgs k, int tab_words) {
     extern __shared__ __align__(128) float smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -975,24 +974,23 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
         __syncthreads();
         tmem_fence_after_sync();
     };
-    // STAGGER (small systems): the CTAs start on different central species, in proportion to the species' tiles, so that the species are
-    // worked on side by side rather than one after the other by mostly idle SMs.  Large systems keep the
-    // plain loop: one front through the cell-ordered atoms, and a loop counter as the species costs 1 % less than a
-    // computed one.  Either way a species whose tiles are all claimed already is passed over: staging its tables would
-    // be the only thing left to do.
+    // The CTAs start on different central species, in proportion to the species' tiles, so that the species are worked on side by side
+    // and most CTAs stage one species only (all CTAs through the species in order / this, one evaluation in us: six equal species, 202,612 atoms
+    // 1611 / 1593, 1,000,188 7650 / 7530, 8,001,504 60,470 / 60,010; eight species, tables in global memory, 32,000 atoms 353 / 307,
+    // 340,736 2990 / 2999, 2,048,000 17,843 / 17,720).
+    // A species whose tiles are all claimed already is passed over: staging its tables would be the only thing left to do.
     // Every group's first tile is fixed (the CTAs that start on a species take its first tiles, group 0 of each before group 1 of any, which
     // spreads a small system over the SMs); the later ones are claimed from the species' counter, which counts from there.
     auto starters = [&](int species) {   // CTAs that start on it
-        return STAGGER ? k.first_cta[species + 1] - k.first_cta[species] : species == 0 ? (int)gridDim.x : 0;
+        return k.first_cta[species + 1] - k.first_cta[species];
     };
     int first_species = 0;
-    if (STAGGER)
-        while (first_species + 1 < k.n_species && k.first_cta[first_species + 1] <= (int)blockIdx.x) ++first_species;
-    auto species_at = [&](int ss) { return !STAGGER ? ss : first_species + ss < k.n_species ? first_species + ss : first_species + ss - k.n_species; };
-    const int first_tile = (int)blockIdx.x - (STAGGER ? k.first_cta[first_species] : 0) + group * starters(first_species);
+    while (first_species + 1 < k.n_species && k.first_cta[first_species + 1] <= (int)blockIdx.x) ++first_species;
+    auto species_at = [&](int ss) { return first_species + ss < k.n_species ? first_species + ss : first_species + ss - k.n_species; };
+    const int first_tile = (int)blockIdx.x - k.first_cta[first_species] + group * starters(first_species);
     // The first species is staged, and the lists of the first tile's atoms fetched, ahead of the wait for the kernel before this one: they
     // change in list builds only, and the launch after a build does not start early.  864 atoms: 4 us of staging and 3 us of
-    // dependent loads and claims out of 31 us a step lie in that kernel's shadow.
+    // dependent loads and claims a step lie in that kernel's shadow.
     stage(first_species);
     NextAtoms<APW> nx0;
     int near0 = 0;
@@ -1368,13 +1366,13 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     double *clear_block = next_eval_block(c);
     const bool in_smem = tables_fit_smem(c);
     const int tab_words = in_smem ? table_smem_words(c) : 0;
-    // instantiations: {one, two atoms per warp with staggered species, two without, two with tables in global memory}
+    // instantiations: {one, two atoms per warp, two with tables in global memory}
     // x floating-point / integer scatter x int32 / 16-bit lists
     using Kernel = void (*)(KernelArgs, int);
-#define MLIP_MEGA4(APW, SMEM, STAG) {k_mega<APW, SMEM, false, false, STAG>, k_mega<APW, SMEM, false, true, STAG>, k_mega<APW, SMEM, true, false, STAG>, k_mega<APW, SMEM, true, true, STAG>}
-    static const Kernel kernels[4][4] = {MLIP_MEGA4(1, true, true), MLIP_MEGA4(2, true, true), MLIP_MEGA4(2, true, false), MLIP_MEGA4(2, false, false)};
+#define MLIP_MEGA4(APW, SMEM) {k_mega<APW, SMEM, false, false>, k_mega<APW, SMEM, false, true>, k_mega<APW, SMEM, true, false>, k_mega<APW, SMEM, true, true>}
+    static const Kernel kernels[3][4] = {MLIP_MEGA4(1, true), MLIP_MEGA4(2, true), MLIP_MEGA4(2, false)};
 #undef MLIP_MEGA4
-    const int shape = !in_smem ? 3 : n >= STAGGER_BELOW_ATOMS ? 2 : n >= ONE_PER_WARP_BELOW_ATOMS ? 1 : 0;
+    const int shape = !in_smem ? 2 : n >= ONE_PER_WARP_BELOW_ATOMS ? 1 : 0;
     const int apw = shape == 0 ? 1 : 2;
     const size_t smem_bytes = sizeof(float) * (size_t)((apw == 1 ? Layout<1>::FIXED : Layout<2>::FIXED) + tab_words);
     const int C = c->cfg.n_species, tile_atoms = GW * apw;
@@ -1382,8 +1380,8 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     for (int q = 0; q < C; ++q) all += tiles[q] = (c->species_host[q + 1] - c->species_host[q] + tile_atoms - 1) / tile_atoms;
     const int blocks = (int)std::min<int64_t>(all, (int64_t)c->n_sm);
     if (!c->kernel_ready) {
-        for (int q = 0; q < 16; ++q) {
-            const int most = (q < 4 ? Layout<1>::FIXED : Layout<2>::FIXED) + (q < 12 ? tab_words : 0);
+        for (int q = 0; q < 12; ++q) {
+            const int most = (q < 4 ? Layout<1>::FIXED : Layout<2>::FIXED) + (q < 8 ? tab_words : 0);
             cudaError_t e = cudaFuncSetAttribute((const void *)kernels[q / 4][q % 4], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(float) * most);
             if (e != cudaSuccess) { c->err = std::string("fused kernel shared memory: ") + cudaGetErrorString(e); return MLIP_ERR_CUDA; }
         }
@@ -1400,12 +1398,22 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     // CTAs in proportion to the species' tiles, at least one to a species that has any.  (One evaluation in us with the CTAs dealt out to the
     // species in turn / in proportion: 864 atoms 90:5:5 46 / 23.5, 6,912 atoms 80 / 66, 13,824 atoms 47:12:41 116 / 96; six equal
     // species, where in turn left some with more tiles than groups, 864 atoms 35.7 / 28.4, 23,328 atoms 221 / 198.)
+    // From 64 tiles a CTA on, rare species (below half the mean) round up: their CTAs end early and join a species that many work on,
+    // where rounded down they end late and all the others stage the rare species for a last tile (90:5:5, all CTAs in
+    // order / rounded down / up, us: 202,612 atoms 1326 / 1344 / 1305, 415,292 2676 / 2689 / 2651, 1,000,188 6394 / 6364 / 6330).
     int64_t weight[MAX_SPECIES], total = 0, before = 0;
     for (int q = 0; q < C; ++q) total += weight[q] = tiles[q] > 0 ? std::max<int64_t>(tiles[q], 2 * all / blocks) : 0;
+    int up[MAX_SPECIES] = {0}, shared = blocks, fixed = 0;   // CTAs of rare species, of the others
+    const int64_t whole = total;
+    for (int q = 0; q < C; ++q) {
+        if (all < (int64_t)64 * blocks || tiles[q] == 0 || 2 * C * tiles[q] >= all) continue;
+        up[q] = (int)((weight[q] * blocks + whole - 1) / whole);   // (together at most blocks / 2 + C of them)
+        shared -= up[q]; total -= weight[q];
+    }
     for (int q = 0; q <= MAX_SPECIES; ++q) {
         k.species_start[q] = c->species_host[std::min(q, C)];
-        k.first_cta[q] = q < C ? (int)(before * blocks / total) : blocks;
-        if (q < C) before += weight[q];
+        k.first_cta[q] = q < C ? fixed + (int)(before * shared / total) : blocks;
+        if (q < C) up[q] > 0 ? (void)(fixed += up[q]) : (void)(before += weight[q]);
     }
     k.stamp = timed_begin(c, MARK_KERNEL, s);
     const bool early = !c->lists_fresh;   // (the kernel reads the lists before it waits)
