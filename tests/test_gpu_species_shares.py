@@ -57,6 +57,6 @@ def test_rare_species_of_a_large_system_match_the_double_precision_path(counts):
         pot.close()
     one, ref = got
     scale = max(1.0, float(np.sqrt((ref["forces"] ** 2).sum(1).mean())))
-    assert abs(float(one["energy"]) - float(ref["energy"])) <= 1e-6 * abs(float(ref["energy"]))
+    assert abs(one["energy"].item() - ref["energy"].item()) <= 1e-6 * abs(ref["energy"].item())
     assert np.abs(one["forces"] - ref["forces"]).max() <= 1e-4 * scale
     assert np.abs(one["e_atom"] - ref["e_atom"]).max() <= 2e-5 * max(1.0, np.abs(ref["e_atom"]).max())
