@@ -38,8 +38,8 @@
 // TF32 terms) and A_lo B_hi + A_hi B_lo + A_hi B_hi is accumulated in fp32.  fp16 halves the tensor instructions and the fragment
 // registers of TF32.  Its narrow exponent range (full precision over 2^18 below the largest scaled value, an absolute error of 2^-40
 // of it further down) is met by exact powers of two: the radial tables are stored scaled per central species and channel
-// (tables.cu) with the regression's first layer scaled to match and equalised per input (upload_head), and the activations and
-// W_i carry per-atom scales that are taken back in fp32.
+// (tables.cu) with the regression's first layer scaled to match and equalised per input (upload_head), and the activations (per atom
+// and 16 neurons) and W_i (per atom) carry scales taken from their largest value, which fp32 takes back.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -77,13 +77,10 @@ constexpr int PF_CS = 96;                                       // compact lists
 static_assert(PF_IDX / 2 + 1 <= PF_CS && PF_CS + 27 <= PF_IDX, "prefetch buffer layout for compact lists");
 constexpr int PF_WORDS = PF_IDX + 4;                            // + {atom, list start (2 words), list length}
 static_assert(2 * 2 * ZS_WORDS <= GW * SCR_WORDS, "layer activations alias the scratch of the group's warps");
-// Head constants of the current species: biases, w_out, b_out, then the powers of two and bounds of the fp16 scaling:
-//   pre-activation of layer L (input scaled by a per-atom 2^s): acc * (2^-s * HC_WS[L]) + bias
-//   |input of layer L| <= HC_BND[2L-2] * max|G| + HC_BND[2L-1]  (L = 1..3; row-sum norms of the weights)
-//   dE/dpre of layer L is stored times HC_SR[L]; its product with the weights is unscaled by HC_UR[L]
+// Head constants of the current species: biases, w_out, b_out, then the powers of two of the fp16 scaling:
+//   a product with layer L's weights is unscaled by HC_WS[L], besides the scale of the activations
 //   the invariants enter, and dE/dG leaves, times HC_CS[input]: the powers of two that equalise the first layer's columns
-constexpr int HC_WOUT = HEAD_L * HEAD_H, HC_BOUT = HC_WOUT + HEAD_H, HC_WS = HC_BOUT + 1, HC_BND = HC_WS + HEAD_L;
-constexpr int HC_SR = HC_BND + 2 * (HEAD_L - 1), HC_UR = HC_SR + HEAD_L, HC_CS = HC_UR + HEAD_L, HC_USED = HC_CS + N_INV;
+constexpr int HC_WOUT = HEAD_L * HEAD_H, HC_BOUT = HC_WOUT + HEAD_H, HC_WS = HC_BOUT + 1, HC_CS = HC_WS + HEAD_L, HC_USED = HC_CS + N_INV;
 constexpr int HC_WORDS = (HC_USED + 15) / 16 * 16;
 // Systems below this size take tiles of 8 atoms, one per warp: with few tiles per SM the chain through one tile is what counts
 // (kernel us with 8- / 16-atom tiles, 6 species: 864 atoms 47 / 53, 6,912 96 / 97, 16,384 174 / 166, 55,296 499 / 474, 131,072
@@ -98,7 +95,8 @@ struct Layout {
     static constexpr int POOL = APW == 1 ? 160 : 256;           // pair queue of a warp, shared by its atoms, kept from encoding to derivation
     static constexpr int Q_WORDS = 4 * POOL;
     static constexpr int SX = NA * X_STRIDE;                    // dE/dG
-    static constexpr int SC = 2 * HEAD_L * NA;                  // per-atom scales (see split_invariants)
+    static constexpr int US = NA / 2 * (HEAD_H / 16);           // one layer's activation scales (see act_store_scaled)
+    static constexpr int SC = 2 * US + NA;                      // two layers of them, then the invariants' (see split_invariants)
     static constexpr int EP = 4 * NA;                           // E_i partial sums of the four m-tiles
     static constexpr int GROUP = APW * XS_WORDS + SX + SC + EP;
     static constexpr int INFO = 4 * APW;                        // per warp: {atom, queued pairs, queue start, -} of its atoms, from encoding to derivation
@@ -177,6 +175,11 @@ __device__ __forceinline__ float scale_for(float bound) {
     return __uint_as_float((uint32_t)(e > 253 ? 253 : e) << 23);
 }
 __device__ __forceinline__ float inverse_pow2(float s) { return __uint_as_float((254u << 23) - __float_as_uint(s)); }
+// Two such scales at once, as bf16 halves: the inverses for the values whose upper 16 bits (sign clear) are the halves of `most`, and
+// the scales from them.
+__device__ __forceinline__ uint32_t inverse_scales(uint32_t most) { return (__vmaxu2(most, 0x07800780u) & 0x7f807f80u) - 0x07000700u; }
+__device__ __forceinline__ uint32_t inverse_of(uint32_t w) { return 0x7f007f00u - w; }
+__device__ __forceinline__ float2 unpack_bf16(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)); }
 
 // The tensor pipe truncates when it adds into its fp32 accumulator, so the energy path keeps accumulation chains short (a fresh
 // accumulator per k-step, folded into the running sum by a rounded fp32 add): a long chain of same-sign terms otherwise drifts
@@ -692,8 +695,9 @@ __device__ __forceinline__ void group_sync(int group) {
 
 // Head contraction on the tensor pipe: C^T[16 rows of W x 8 atoms] over four 16-wide k-steps.  A = wr (32 columns of tensor
 // memory), B = activations in fragment order from shared memory; every k-step gets its own accumulator (four independent
-// chains of three products), summed in fp32.
-__device__ __forceinline__ void head_gemm(float (&c)[4], const uint32_t (&wr)[32], const uint4 *__restrict__ act) {
+// chains of three products), summed in fp32.  SCALED: `inv` holds the k-steps' scales of the lane's two atoms (act_store_scaled).
+template <bool SCALED>
+__device__ __forceinline__ void head_gemm(float (&c)[4], const uint32_t (&wr)[32], const uint4 *__restrict__ act, const uint32_t *inv = nullptr) {
     float acc[4][4];
     uint4 b[4];
 #pragma unroll
@@ -704,8 +708,20 @@ __device__ __forceinline__ void head_gemm(float (&c)[4], const uint32_t (&wr)[32
     for (int u = 0; u < 4; ++u) mma_f16(acc[u], wr[8 * u], wr[8 * u + 1], wr[8 * u + 2], wr[8 * u + 3], b[u].y, b[u].w);
 #pragma unroll
     for (int u = 0; u < 4; ++u) mma_f16(acc[u], wr[8 * u], wr[8 * u + 1], wr[8 * u + 2], wr[8 * u + 3], b[u].x, b[u].z);
+    if (!SCALED) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) c[e] = (acc[0][e] + acc[1][e]) + (acc[2][e] + acc[3][e]);
+        for (int e = 0; e < 4; ++e) c[e] = (acc[0][e] + acc[1][e]) + (acc[2][e] + acc[3][e]);
+        return;
+    }
+    const uint4 w = *reinterpret_cast<const uint4 *>(inv);
+    const float2 s[4] = {unpack_bf16(w.x), unpack_bf16(w.y), unpack_bf16(w.z), unpack_bf16(w.w)};
+#pragma unroll
+    for (int e = 0; e < 4; e += 2) {
+        float2 sum = make_float2(acc[0][e] * s[0].x, acc[0][e + 1] * s[0].y);
+#pragma unroll
+        for (int u = 1; u < 4; ++u) sum = ffma2(make_float2(acc[u][e], acc[u][e + 1]), s[u], sum);
+        c[e] = sum.x; c[e + 1] = sum.y;
+    }
 }
 
 // Activations in B-fragment order.  k-step s covers neurons (or inputs) 16 s .. 16 s + 15, its k-index 2 j + h standing for
@@ -715,6 +731,27 @@ __device__ __forceinline__ void head_gemm(float (&c)[4], const uint32_t (&wr)[32
 __device__ __forceinline__ int act_row(int a) { return (a & 4) | ((a & 1) << 1) | ((a >> 1) & 1); }
 __device__ __forceinline__ void act_store(float *act, int kstep, int atom, int j, uint32_t hi, uint32_t lo) {
     *reinterpret_cast<uint2 *>(act + kstep * ACT_KSTEP + (act_row(atom) * 4 + (j & 3)) * 4 + 2 * (j >> 2)) = make_uint2(hi, lo);
+}
+
+// One warp's 16 neurons (m-tile mt) of the lane's atoms, values {n0 a, n0 a+1, n1 a, n1 a+1}, as the next contraction's k-step: scaled by the
+// power of two that brings the largest of an atom's 16 values just below 2^15, the inverse (bf16 pairs [atom pair][k-step]) beside them.
+// Measured, not taken from the weights' norms: a product over the layers of row or column sums of large weights lies so far above the
+// values that the lower halves, and with them the forces' digits, were lost (hidden layers x 300 with small pre-activations: 8e-2
+// relative, now 1e-6).  Three shuffles in the chain from layer to layer, a store and a 16-byte load per contraction: an evaluation of 5,544
+// atoms 61.8 -> 63.3 us, 65,536 atoms NVE 4924 -> 5013 us per 10 steps, 8,001,504 atoms 683.8 -> 691.5 ms.
+__device__ __forceinline__ void act_store_scaled(float *act, uint32_t *inv, int mt, int atom, int g, int t, const float (&m)[4]) {
+    const float b0 = fmaxf(fabsf(m[0]), fabsf(m[2])), b1 = fmaxf(fabsf(m[1]), fabsf(m[3]));
+    uint32_t most = __byte_perm(__float_as_uint(b0), __float_as_uint(b1), 0x7632);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) most = __vmaxu2(most, __shfl_xor_sync(0xffffffffu, most, o));
+    const uint32_t w = inverse_scales(most);
+    if (g == 0) inv[(atom >> 1) * (HEAD_H / 16) + mt] = w;
+    const float2 s = unpack_bf16(inverse_of(w));
+    uint32_t hi, lo;
+    split_h2(m[0] * s.x, m[2] * s.x, hi, lo);
+    act_store(act, mt, 2 * t, g, hi, lo);
+    split_h2(m[1] * s.y, m[3] * s.y, hi, lo);
+    act_store(act, mt, 2 * t + 1, g, hi, lo);
 }
 
 // Prefetch of the warp's atoms in the group's NEXT tile, spread over three points of the head so
@@ -776,9 +813,9 @@ struct NextAtoms {
 };
 
 // ---------------- Regression (Eq. 6) forward and reverse for the group's tile ----------------
-// One atom's invariants (warp = atom) -> scaled fp16 pairs in fragment order, and the atom's scales for all layers:
-// sc[2 L][atom] = 2^s of layer L's input, sc[2 L + 1][atom] = the factor that takes layer L's product back.
-__device__ __forceinline__ void split_invariants(const float *xrow, float *xs, float *sc, const float *hc, int atom, int n_atoms, int lane) {
+// One atom's invariants (warp = atom) -> scaled fp16 pairs in fragment order, and sc[atom] = the factor that takes the first layer's
+// product back.
+__device__ __forceinline__ void split_invariants(const float *xrow, float *xs, float *sc, const float *hc, int atom, int lane) {
     xs += (atom >> 3) * XS_WORDS;
     // lane handles the pairs (c, c + 8) number lane and lane + 32 of the 64: k-step p / 8, j = p % 8
     const int j = lane & 7, s0 = lane >> 3, s1 = s0 + 4;
@@ -792,17 +829,13 @@ __device__ __forceinline__ void split_invariants(const float *xrow, float *xs, f
     act_store(xs, s0, atom & 7, j, hi, lo);
     split_h2(b0 * sx, b1 * sx, hi, lo);
     act_store(xs, s1, atom & 7, j, hi, lo);
-    if (lane < HEAD_L) {
-        const float s = lane == 0 ? sx : scale_for(hc[HC_BND + 2 * (lane - 1)] * most + hc[HC_BND + 2 * (lane - 1) + 1]);
-        sc[2 * lane * n_atoms + atom] = s;
-        sc[(2 * lane + 1) * n_atoms + atom] = inverse_pow2(s) * hc[HC_WS + lane];
-    }
+    if (lane == 0) sc[atom] = inverse_pow2(sx) * hc[HC_WS];
 }
 
 // In: xs = split invariants.  Out: sX = dE/dG [atom][128]; per-atom energies written.  wg = warp within the group: it owns
 // m-tile wg % 4 (16 neurons) of the atoms 8 (wg / 4) .. + 7 through all layers (one atom per warp: warps 4..7 own nothing).
 template <int APW, bool DET, bool L16>
-__device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, float *sX, const float *sc, float *ep, float *zs, const float *hc,
+__device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, float *sX, const float *sc, uint32_t *us, float *ep, float *zs, const float *hc,
                                           uint32_t tm, int count, int first, int group, int wg, int lane, double &e_sum, NextAtoms<APW> &nx, PhaseClock &pc) {
     constexpr int NA = GW * APW;
     const int g = lane >> 2, t = lane & 3, mt = wg & 3, nt = wg >> 2;
@@ -810,6 +843,8 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
     const bool owner = APW == 2 || wg < 4;
     const int a0 = (APW == 2 ? 8 * nt : 0) + 2 * t;   // the lane's atoms: a0, a0 + 1
     const int n0 = 16 * mt + g, n1 = n0 + 8;    // and neurons: its values are {n0 a0, n0 a0+1, n1 a0, n1 a0+1}
+    constexpr int US = Layout<APW>::US;
+    const uint32_t *my_us = us + (a0 >> 1) * (HEAD_H / 16);   // the lane's atoms' activation scales, of a layer in buffer 0
     if (APW == 2) { xs += nt * XS_WORDS; zs += nt * 2 * ZS_WORDS; }
     float y[4] = {0.f, 0.f, 0.f, 0.f};          // running activations (the skip path)
     float dz[4];                                // dE/dy in the reverse pass
@@ -823,26 +858,26 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
             float c[4];
             tmem_ld32(tm + (L == 0 ? TM_FWD0 : TM_FWD + 32 * (L - 1)), w);
             tmem_wait_ld();
-            head_gemm(c, w, reinterpret_cast<const uint4 *>(L == 0 ? xs : zin) + frag);
+            float2 u = make_float2(hc[HC_WS + L], hc[HC_WS + L]);
             if (L == 0) {
                 float c2[4];
+                head_gemm<false>(c, w, reinterpret_cast<const uint4 *>(xs) + frag);
                 tmem_ld32(tm + TM_FWD0 + 32, w);
                 tmem_wait_ld();
-                head_gemm(c2, w, reinterpret_cast<const uint4 *>(xs + 4 * ACT_KSTEP) + frag);
+                head_gemm<false>(c2, w, reinterpret_cast<const uint4 *>(xs + 4 * ACT_KSTEP) + frag);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) c[e] += c2[e];
+                u = *reinterpret_cast<const float2 *>(sc + a0);
+            } else {
+                head_gemm<true>(c, w, reinterpret_cast<const uint4 *>(zin) + frag, my_us + ((L + 1) & 1) * US);
             }
             pc.mark(12);
-            const float2 u = *reinterpret_cast<const float2 *>(sc + (2 * L + 1) * NA + a0);
             const float bias0 = hc[L * HEAD_H + n0], bias1 = hc[L * HEAD_H + n1];
             y[0] += silu_f(c[0] * u.x + bias0, sd[L][0]); y[1] += silu_f(c[1] * u.y + bias0, sd[L][1]);
             y[2] += silu_f(c[2] * u.x + bias1, sd[L][2]); y[3] += silu_f(c[3] * u.y + bias1, sd[L][3]);
-            float m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f;   // what goes to the next contraction
-            if (L < HEAD_L - 1) {
-                const float2 s = *reinterpret_cast<const float2 *>(sc + 2 * (L + 1) * NA + a0);
-                m0 = y[0] * s.x; m1 = y[1] * s.y; m2 = y[2] * s.x; m3 = y[3] * s.y;
-            } else {   // output layer and the start of the reverse pass: dE/dy = w_out
-                const float wo0 = hc[HC_WOUT + n0], wo1 = hc[HC_WOUT + n1], s = hc[HC_SR + L];
+            float m[4] = {y[0], y[1], y[2], y[3]};   // what goes to the next contraction
+            if (L == HEAD_L - 1) {   // output layer and the start of the reverse pass: dE/dy = w_out
+                const float wo0 = hc[HC_WOUT + n0], wo1 = hc[HC_WOUT + n1];
                 float e0 = wo0 * y[0] + wo1 * y[2], e1 = wo0 * y[1] + wo1 * y[3];
 #pragma unroll
                 for (int o = 4; o < 32; o <<= 1) {
@@ -851,13 +886,10 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
                 }
                 if (g == 0) *reinterpret_cast<float2 *>(ep + mt * NA + a0) = make_float2(e0, e1);
                 dz[0] = dz[1] = wo0; dz[2] = dz[3] = wo1;
-                m0 = (wo0 * s) * sd[L][0]; m1 = (wo0 * s) * sd[L][1]; m2 = (wo1 * s) * sd[L][2]; m3 = (wo1 * s) * sd[L][3];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) m[e] = dz[e] * sd[L][e];
             }
-            uint32_t hi, lo;
-            split_h2(m0, m2, hi, lo);
-            act_store(zout, mt, 2 * t, g, hi, lo);
-            split_h2(m1, m3, hi, lo);
-            act_store(zout, mt, 2 * t + 1, g, hi, lo);
+            act_store_scaled(zout, us + (L & 1) * US, mt, a0, g, t, m);
         }
         if (L == 0) nx.stage_a();
         if (L == 1) nx.template stage_b<L16>();
@@ -881,16 +913,12 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
             float c[4];
             tmem_ld32(tm + TM_BWD + 32 * (L - 1), w);
             tmem_wait_ld();
-            head_gemm(c, w, reinterpret_cast<const uint4 *>(zin) + frag);
-            const float u = hc[HC_UR + L], s = hc[HC_SR + L - 1];
+            head_gemm<true>(c, w, reinterpret_cast<const uint4 *>(zin) + frag, my_us + (L & 1) * US);
+            const float u = hc[HC_WS + L];
             float m[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) { dz[e] += c[e] * u; m[e] = dz[e] * sd[L - 1][e] * s; }
-            uint32_t hi, lo;
-            split_h2(m[0], m[2], hi, lo);
-            act_store(zout, mt, 2 * t, g, hi, lo);
-            split_h2(m[1], m[3], hi, lo);
-            act_store(zout, mt, 2 * t + 1, g, hi, lo);
+            for (int e = 0; e < 4; ++e) { dz[e] += c[e] * u; m[e] = dz[e] * sd[L - 1][e]; }
+            act_store_scaled(zout, us + ((L + 1) & 1) * US, mt, a0, g, t, m);
         }
         group_sync(group);
     }
@@ -901,8 +929,8 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
         float c[4];
         tmem_ld32(tm + TM_BWD0 + 32 * (m >> 2), w);
         tmem_wait_ld();
-        head_gemm(c, w, reinterpret_cast<const uint4 *>(zs) + frag);   // layer 0's dE/dpre: buffer 0
-        const float u = hc[HC_UR], ua = u * hc[HC_CS + 16 * m + g], ub = u * hc[HC_CS + 16 * m + g + 8];
+        head_gemm<true>(c, w, reinterpret_cast<const uint4 *>(zs) + frag, my_us);   // layer 0's dE/dpre: buffer 0
+        const float u = hc[HC_WS], ua = u * hc[HC_CS + 16 * m + g], ub = u * hc[HC_CS + 16 * m + g + 8];
         float *p = sX + a0 * X_STRIDE + 16 * m + g;
         p[0] = c[0] * ua; p[X_STRIDE] = c[1] * ua; p[8] = c[2] * ub; p[X_STRIDE + 8] = c[3] * ub;
     }
@@ -920,7 +948,8 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
     const int g = lane >> 2, t = lane & 3;
     float *s_tab = smem;                                   // [C][rows][K_RADIAL] when TAB_SMEM
     float *xs = smem + (TAB_SMEM ? tab_words : 0) + group * LY::GROUP;
-    float *sX = xs + APW * XS_WORDS, *sc = sX + LY::SX, *ep = sc + LY::SC;
+    float *sX = xs + APW * XS_WORDS, *sc = sX + LY::SX + 2 * LY::US, *ep = sc + NA;
+    uint32_t *us = reinterpret_cast<uint32_t *>(sX + LY::SX);
     float *scr_all = smem + (TAB_SMEM ? tab_words : 0) + NG * LY::GROUP;
     float *zs = scr_all + group * GW * SCR_WORDS;          // layer activations = the scratch of the group's warps
     float *scr = scr_all + warp * SCR_WORDS;
@@ -1105,7 +1134,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
                     for (int c = lane; c < N_INV; c += 32) xrow[c] = 0.f;
                 }
                 __syncwarp();
-                split_invariants(xrow, xs, sc, hc, wg + GW * u, NA, lane);
+                split_invariants(xrow, xs, sc, hc, wg + GW * u, lane);
                 __syncwarp();   // (the next atom's hand-over rows overwrite the invariants)
             }
             tmem_wait_st();
@@ -1121,7 +1150,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
             const int next_slot = s_beg + tile_next * NA + wg + GW * lane;
             nx.slot = (lane < APW && tile_next < n_tiles && next_slot < s_end) ? next_slot : -1;
             nx.i = 0; nx.beg = 0; nx.len = 0; nx.use_far = use_far; nx.cid = 0;
-            head_tile<APW, DET, L16>(k, xs, sX, sc, ep, zs, hc, tm_quarter, count, first, group, wg, lane, e_sum, nx, pc);
+            head_tile<APW, DET, L16>(k, xs, sX, sc, us, ep, zs, hc, tm_quarter, count, first, group, wg, lane, e_sum, nx, pc);
             prefetched = tile_next < n_tiles && s_beg + tile_next * NA + wg < s_end;
             pc.mark(9);
 
@@ -1278,43 +1307,15 @@ int upload_head(mlip_ctx *c, const double *w) {
         }
         for (int o = 0; o < HEAD_H; ++o)
             for (int q = 0; q < N_INV; ++q) first[(size_t)o * N_INV + q] *= most_of[q];
-        // powers of two: weights of a layer to below 2^14; bounds of the layers' inputs from row sums, of dE/dpre from column sums
-        // (both a little enlarged for the device's fp32 arithmetic)
+        // powers of two: the weights of a layer to below 2^14
         float *wscale = scales.w[s];
-        double row_sum[HEAD_L], bias_max[HEAD_L], col_sum[HEAD_L], wout_max = 0.0;
         for (int L = 0; L < HEAD_L; ++L) {
-            const int in = in_of[L];
-            double most = 0.0, col[N_INV] = {0.0};
-            row_sum[L] = bias_max[L] = col_sum[L] = 0.0;
-            for (int o = 0; o < HEAD_H; ++o) {
-                double r = 0.0;
-                for (int q = 0; q < in; ++q) { const double a = fabs(layer[L][(size_t)o * in + q]); r += a; col[q] += a; most = std::max(most, a); }
-                row_sum[L] = std::max(row_sum[L], r);
-                bias_max[L] = std::max(bias_max[L], fabs(layer[L][(size_t)in * HEAD_H + o]));
-            }
-            for (int q = 0; q < in; ++q) col_sum[L] = std::max(col_sum[L], col[q]);
+            double most = 0.0;
+            for (int q = 0; q < HEAD_H * in_of[L]; ++q) most = std::max(most, fabs(layer[L][q]));
             int e = 0;
             if (most > 0.0) frexp(most, &e);
             wscale[L] = pow2f(std::min(14 - e, 60));
-        }
-        for (int o = 0; o < HEAD_H; ++o) wout_max = std::max(wout_max, fabs(out[o]));
-        // |SiLU(x)| <= |x|, |SiLU'(x)| < 1.1: |y_0| <= A max|G| + B, |y_L| <= (1 + r_L) |y_{L-1}| + b_L
-        double A = row_sum[0], B = bias_max[0];
-        for (int L = 1; L < HEAD_L; ++L) {
-            hc[HC_BND + 2 * (L - 1)] = (float)(1.001 * A);
-            hc[HC_BND + 2 * (L - 1) + 1] = (float)(1.001 * B);
-            A *= 1.0 + row_sum[L];
-            B = B * (1.0 + row_sum[L]) + bias_max[L];
-        }
-        double dz = wout_max;
-        for (int L = HEAD_L - 1; L >= 0; --L) {
-            int e = 0;
-            if (dz > 0.0) frexp(1.101 * dz, &e);
-            const float sr = pow2f(std::min(15 - e, 60));
-            hc[HC_SR + L] = sr;
-            hc[HC_UR + L] = 1.f / (sr * wscale[L]);
             hc[HC_WS + L] = 1.f / wscale[L];
-            dz *= 1.0 + 1.1 * col_sum[L];
         }
         for (int L = 0; L < HEAD_L; ++L)
             for (int o = 0; o < HEAD_H; ++o) hc[L * HEAD_H + o] = (float)layer[L][(size_t)in_of[L] * HEAD_H + o];
