@@ -1381,8 +1381,9 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     for (int q = 0; q < C; ++q) all += tiles[q] = (c->species_host[q + 1] - c->species_host[q] + tile_atoms - 1) / tile_atoms;
     const int blocks = (int)std::min<int64_t>(all, (int64_t)c->n_sm);
     if (!c->kernel_ready) {
+        // A limit of the kernels, shared by every context of the process: the same whatever this one's tables need.
         for (int q = 0; q < 12; ++q) {
-            const int most = (q < 4 ? Layout<1>::FIXED : Layout<2>::FIXED) + (q < 8 ? tab_words : 0);
+            const int most = q < 8 ? SMEM_LIMIT_WORDS : Layout<2>::FIXED;
             cudaError_t e = cudaFuncSetAttribute((const void *)kernels[q / 4][q % 4], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(float) * most);
             if (e != cudaSuccess) { c->err = std::string("fused kernel shared memory: ") + cudaGetErrorString(e); return MLIP_ERR_CUDA; }
         }
