@@ -1050,9 +1050,9 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
         if (n_tiles == 0) continue;
         const int n_first = NG * starters(species);   // tiles that are not claimed
         if (ss > 0) {
-            if (threadIdx.x == 0) ctl[6 + (ss & 1)] = *reinterpret_cast<volatile int *>(k.tile_counter + species);
-            __syncthreads();   // both groups are done with the previous species' tables
-            if (n_first + ctl[6 + (ss & 1)] >= n_tiles) continue;
+            // both groups are done with the previous species' tables; the barrier itself carries the decision (a word of shared memory could
+            // be written for the next species before a warp has read it: not every turn of this loop has a barrier)
+            if (__syncthreads_or(threadIdx.x == 0 && n_first + *reinterpret_cast<volatile int *>(k.tile_counter + species) >= n_tiles)) continue;
             stage(species);
         }
 
