@@ -193,6 +193,9 @@ int mlip_set_velocities(mlip_ctx *ctx, const double *vel, void *stream);
  *   energy dev [1] double (sum of E_i)      forces dev [N][3] float, F = -dE/dr
  *   virial dev [9] double, row-major Xi_ab = -sum_i sum_j (r_ij)_a (dE_i/dr_ij)_b
  *   e_atom dev [N] float
+ * This call, mlip_set_positions and steps without a rebuild may be captured into a CUDA graph after a first evaluation outside
+ * it, and replayed in any order with other calls; the graph holds the addresses of the context's buffers, so it ends with
+ * a build for more atoms or cells, or with longer lists.
  */
 int mlip_compute(mlip_ctx *ctx, double *energy, float *forces, double *virial, float *e_atom, void *stream);
 

@@ -113,6 +113,13 @@ static int box_edges(mlip_ctx *c, const double *cell, double *edges) {
     return MLIP_OK;
 }
 
+// What every entry that enqueues evaluations, moves or builds does first.
+static void enter(mlip_ctx *c, cudaStream_t s) {
+    c->last_stream = s;
+    c->mark_open = false;
+    note_capture(c, s);
+}
+
 static int set_grid(mlip_ctx *c, const double *box) {
     const double rl = c->cfg.r_cut + c->cfg.skin;
     CellGrid g;
@@ -248,7 +255,7 @@ int mlip_create(mlip_ctx **out, const mlip_config *cfg, const double *enc_w, siz
     do {
         if ((rc = dev_alloc(c, &c->mass, (size_t)cfg->n_species)) != MLIP_OK) break;
         if ((rc = dev_alloc(c, &c->launch_base, (size_t)2 * LB_COUNT)) != MLIP_OK) break;
-        next_eval_block(c);
+        set_eval_block(c, c->launch_base);
         if ((rc = dev_alloc(c, &c->stamp, (size_t)2 * mlip_ctx::STAMPS)) != MLIP_OK) break;
         if ((rc = dev_alloc(c, &c->build_word, mlip_ctx::BUILD_WORDS)) != MLIP_OK) break;
         c->status = c->build_word + 4; c->rebuild_flag = c->build_word + 5; c->far_flag = c->build_word + 6; c->species_start = c->build_word + 8;
@@ -308,8 +315,7 @@ int mlip_build_neighbors_ghost(mlip_ctx *c, int64_t n_owned, int64_t n_ghost, co
     if (n_owned < 1 || n_ghost < 0 || !pos || !species || !box) return fail(c, MLIP_ERR_INVALID_ARG, "bad arguments to mlip_build_neighbors");
     if (n > (1LL << 28)) return fail(c, MLIP_ERR_UNSUPPORTED, "more than 2^28 atoms per context (the pair queue packs index and species in 32 bits)");
     cudaStream_t s = (cudaStream_t)stream;
-    c->last_stream = s;
-    c->mark_open = false;
+    enter(c, s);
     cudaSetDevice(c->cfg.device);
     double edges[3];
     int rc = box_edges(c, box, edges);
@@ -347,7 +353,7 @@ int mlip_get_neighbors_noalloc(mlip_ctx *c, int64_t *seg_ptr, int32_t *nbr, int6
 int mlip_set_positions(mlip_ctx *c, const double *pos, void *stream) {
     if (!c || !pos) return MLIP_ERR_INVALID_ARG;
     if (!c->built) return fail(c, MLIP_ERR_NOT_BUILT, "no neighbor lists yet");
-    c->last_stream = (cudaStream_t)stream;
+    enter(c, (cudaStream_t)stream);
     c->forces_current = false;
     return launch_set_positions(c, pos, (cudaStream_t)stream);
 }
@@ -369,9 +375,8 @@ int mlip_compute_f64(mlip_ctx *c, double *energy, double *forces, double *virial
     if (c->cfg.precision != 1) return fail(c, MLIP_ERR_UNSUPPORTED, "mlip_compute_f64 needs a context created with precision = 1");
     if (!c->built) return fail(c, MLIP_ERR_NOT_BUILT, "no neighbor lists yet");
     cudaStream_t s = (cudaStream_t)stream;
-    c->last_stream = s;
-    c->mark_open = false;
-    int rc = launch_megakernel_f64(c, s);
+    enter(c, s);
+    int rc = evaluate(c, s);
     if (rc != MLIP_OK) return rc;
     c->forces_current = true;
     if (energy || virial || forces || e_atom) rc = launch_outputs_f64(c, forces, e_atom, energy, virial, s);
@@ -382,8 +387,7 @@ int mlip_compute(mlip_ctx *c, double *energy, float *forces, double *virial, flo
     if (!c) return MLIP_ERR_INVALID_ARG;
     if (!c->built) return fail(c, MLIP_ERR_NOT_BUILT, "no neighbor lists yet");
     cudaStream_t s = (cudaStream_t)stream;
-    c->last_stream = s;
-    c->mark_open = false;
+    enter(c, s);
     int rc = evaluate(c, s);
     if (rc != MLIP_OK) return rc;
     c->forces_current = true;
@@ -460,8 +464,7 @@ int mlip_step(mlip_ctx *c, int n_steps, double dt, int rebuild_every, void *stre
     if (!c->built) return fail(c, MLIP_ERR_NOT_BUILT, "no neighbor lists yet");
     if (c->n_owned != c->n) return fail(c, MLIP_ERR_UNSUPPORTED, "a context with ghost atoms evaluates only: the owner of the ghosts integrates them");
     cudaStream_t s = (cudaStream_t)stream;
-    c->last_stream = s;
-    c->mark_open = false;
+    enter(c, s);
     int rc;
     if (!c->forces_current) {
         if ((rc = evaluate(c, s)) != MLIP_OK) return rc;
@@ -482,8 +485,7 @@ int mlip_step_nvt(mlip_ctx *c, int n_steps, double dt, int rebuild_every, double
     if (c->n < 2) return fail(c, MLIP_ERR_INVALID_ARG, "the thermostat needs at least two atoms");
     if (c->n_owned != c->n) return fail(c, MLIP_ERR_UNSUPPORTED, "a context with ghost atoms evaluates only: the owner of the ghosts integrates them");
     cudaStream_t s = (cudaStream_t)stream;
-    c->last_stream = s;
-    c->mark_open = false;
+    enter(c, s);
     const double kB = 8.617333262e-5;   // eV/K
     c->nhc_nf = 3.0 * (double)c->n - 3.0;
     c->nhc_kT = kB * t_target;
@@ -543,8 +545,7 @@ int mlip_set_state(mlip_ctx *c, const double *pos, const double *vel, int64_t st
     if (!c || step < 0) return MLIP_ERR_INVALID_ARG;
     if (!c->built) return fail(c, MLIP_ERR_NOT_BUILT, "no atoms yet: build the lists from the saved positions first");
     cudaStream_t s = (cudaStream_t)stream;
-    c->last_stream = s;
-    c->mark_open = false;
+    enter(c, s);
     int rc;
     if (pos) {
         c->forces_current = false;
@@ -567,8 +568,7 @@ int mlip_debug_rebuild(mlip_ctx *c, int spin_limit, int64_t unpublished_tile, vo
     if (!c || spin_limit < 1) return MLIP_ERR_INVALID_ARG;
     if (!c->built) return fail(c, MLIP_ERR_NOT_BUILT, "no neighbor lists yet");
     cudaStream_t s = (cudaStream_t)stream;
-    c->last_stream = s;
-    c->mark_open = false;
+    enter(c, s);
     c->lookback_spin_limit = spin_limit;
     c->lookback_unpublished_tile = unpublished_tile;
     std::swap(c->pos4, c->pos4_src);
@@ -592,8 +592,7 @@ int mlip_get_energies(mlip_ctx *c, double *e_pot, double *e_kin, void *stream) {
     if (!c) return MLIP_ERR_INVALID_ARG;
     if (!c->built) return fail(c, MLIP_ERR_NOT_BUILT, "no atoms yet");
     cudaStream_t s = (cudaStream_t)stream;
-    c->last_stream = s;
-    c->mark_open = false;
+    enter(c, s);
     if (e_pot) MLIP_CUDA_TRY(c, cudaMemcpyAsync(e_pot, c->acc + ACC_ENERGY, sizeof(double), cudaMemcpyDeviceToDevice, s));
     if (e_kin) {
         int rc = launch_kinetic(c, 0, false, 0.0, s);

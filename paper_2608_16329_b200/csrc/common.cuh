@@ -45,7 +45,7 @@ enum : int {
 enum : int { ACC_ENERGY = 0, ACC_VIRIAL = 1, ACC_KINETIC = 10, ACC_COUNT = 32 };
 // launch_block in doubles: [0, 4) tile_counter (MAX_SPECIES ints), [4] pair_counter, [5, 15) acc_fx, [16, 16 + ACC_COUNT) acc;
 // everything up to the kinetic-energy slot of acc is zero when a fused kernel starts.  There are two such blocks: an evaluation uses one
-// and clears the other, which holds the totals of the evaluation before it, for the next
+// and clears the other, which holds the totals of the evaluation before it, for the next (but see note_capture)
 constexpr int LB_PAIR = 4, LB_ACC_FX = 5, LB_ACC = 16, LB_COUNT = LB_ACC + ACC_COUNT;
 constexpr size_t LAUNCH_CLEAR_BYTES = sizeof(double) * (LB_ACC + ACC_KINETIC);
 static_assert(MAX_SPECIES * sizeof(int) <= LB_PAIR * sizeof(double), "tile counters must fit before the pair counter");
@@ -135,7 +135,7 @@ struct mlip_ctx {
     int64_t scan_tmp_cap = 0;
     double *launch_base = nullptr;    // [2][LB_COUNT]: tile_counter, pair_counter, acc_fx, acc back to back, twice; the pointers are into
                                       // the block of the last evaluation
-    int eval_block = 0;
+    bool captured = false;            // calls of this context have been captured into a graph (note_capture)
     double *acc = nullptr;         // [ACC_COUNT] (inside launch_base)
     double *kin_part = nullptr;    // [1184] per-block kinetic-energy sums, then the ticket of the last block (integrate.cu)
     unsigned long long *pair_counter = nullptr;
@@ -259,16 +259,26 @@ inline cudaError_t launch_after(void (*kernel)(P...), unsigned blocks, unsigned 
     return launch_after_if(true, kernel, blocks, threads, smem, s, args...);
 }
 
-// The counters and totals of a new evaluation become current; returns the other block, which the evaluation clears.
-inline double *next_eval_block(mlip_ctx *c) {
-    double *clear = c->launch_base + (size_t)c->eval_block * LB_COUNT;
-    c->eval_block ^= 1;
-    double *b = c->launch_base + (size_t)c->eval_block * LB_COUNT;
+// A captured call may be replayed at any time, in any order with others: what this context remembers on the host of the launches before a
+// call (which of the two blocks is clear, whether the forces are, the species' starts) then says nothing about the device.  From the
+// first captured call on every evaluation keeps to one block and clears it and the forces itself, and reads the species' starts from
+// the device.  Called on entry by what enqueues on a stream.
+inline void note_capture(mlip_ctx *c, cudaStream_t s) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &status) != cudaSuccess) cudaGetLastError();
+    if (status != cudaStreamCaptureStatusNone) c->captured = true;
+}
+// The two blocks of the evaluation about to be launched: its own, and the one that it clears.  set_eval_block once it is launched.
+struct EvalBlocks { double *use, *clear; };
+inline EvalBlocks next_eval_blocks(const mlip_ctx *c) {
+    double *now = c->acc - LB_ACC, *other = now == c->launch_base ? now + LB_COUNT : c->launch_base;
+    return c->captured ? EvalBlocks{now, other} : EvalBlocks{other, now};
+}
+inline void set_eval_block(mlip_ctx *c, double *b) {
     c->tile_counter = reinterpret_cast<int *>(b);
     c->pair_counter = reinterpret_cast<unsigned long long *>(b + LB_PAIR);
     c->acc_fx = reinterpret_cast<long long *>(b + LB_ACC_FX);
     c->acc = b + LB_ACC;
-    return clear;
 }
 
 struct EvalClear {

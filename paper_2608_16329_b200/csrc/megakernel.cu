@@ -82,6 +82,8 @@ static_assert(2 * 2 * ZS_WORDS <= GW * SCR_WORDS, "layer activations alias the s
 //   the invariants enter, and dE/dG leaves, times HC_CS[input]: the powers of two that equalise the first layer's columns
 constexpr int HC_WOUT = HEAD_L * HEAD_H, HC_BOUT = HC_WOUT + HEAD_H, HC_WS = HC_BOUT + 1, HC_CS = HC_WS + HEAD_L, HC_USED = HC_CS + N_INV;
 constexpr int HC_WORDS = (HC_USED + 15) / 16 * 16;
+constexpr int CTL_WORDS = 16;   // per group {tile, tile after it}; tensor-memory base; the species' starts
+static_assert(5 + MAX_SPECIES + 1 <= CTL_WORDS, "control words");
 // Systems below this size take tiles of 8 atoms, one per warp: with few tiles per SM the chain through one tile is what counts
 // (kernel us with 8- / 16-atom tiles, 6 species: 864 atoms 47 / 53, 6,912 96 / 97, 16,384 174 / 166, 55,296 499 / 474, 131,072
 // 1119 / 1046; one species: 4,394 63 / 66, 16,000 140 / 135, 65,536 476 / 441).
@@ -101,7 +103,7 @@ struct Layout {
     static constexpr int GROUP = APW * XS_WORDS + SX + SC + EP;
     static constexpr int INFO = 4 * APW;                        // per warp: {atom, queued pairs, queue start, -} of its atoms, from encoding to derivation
     static constexpr int WARP = Q_WORDS + SCR_WORDS + APW * PF_WORDS + INFO;
-    static constexpr int FIXED = NG * GROUP + NW * WARP + HC_WORDS + 16;
+    static constexpr int FIXED = NG * GROUP + NW * WARP + HC_WORDS + CTL_WORDS;
 };
 constexpr int SMEM_LIMIT_WORDS = 227 * 1024 / 4 - 256;
 
@@ -211,6 +213,7 @@ struct KernelArgs {
     const double4 *pos4;
     const int32_t *center_order;
     int species_start[MAX_SPECIES + 1];   // in center_order (a step's own rebuilds do not change it)
+    const int *species_dev;               // the same on the device, read instead in launches that may be replayed; else nullptr
     int first_cta[MAX_SPECIES + 1];       // the first CTA that starts on a species
     const int64_t *nbr_off;
     const int32_t *nbr_near;   // leading entries of each list that can be inside r_cut while far_flag is down
@@ -1008,6 +1011,8 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
     // 1611 / 1593, 1,000,188 7650 / 7530, 8,001,504 60,470 / 60,010; eight species, tables in global memory, 32,000 atoms 353 / 307,
     // 340,736 2990 / 2999, 2,048,000 17,843 / 17,720).
     // A species whose tiles are all claimed already is passed over: staging its tables would be the only thing left to do.
+    volatile int *species_start = ctl + 5;   // [n_species + 1], complete after the staging's barrier
+    if ((int)threadIdx.x <= k.n_species) species_start[threadIdx.x] = k.species_dev ? k.species_dev[threadIdx.x] : k.species_start[threadIdx.x];
     // Every group's first tile is fixed (the CTAs that start on a species take its first tiles, group 0 of each before group 1 of any, which
     // spreads a small system over the SMs); the later ones are claimed from the species' counter, which counts from there.
     auto starters = [&](int species) {   // CTAs that start on it
@@ -1024,8 +1029,8 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
     NextAtoms<APW> nx0;
     int near0 = 0;
     {
-        const int s_end0 = k.species_start[first_species + 1];
-        const int slot0 = k.species_start[first_species] + first_tile * NA + wg + GW * lane;
+        const int s_end0 = species_start[first_species + 1];
+        const int slot0 = species_start[first_species] + first_tile * NA + wg + GW * lane;
         nx0.k = &k; nx0.pf = pf; nx0.slot = (lane < APW && slot0 < s_end0) ? slot0 : -1;
         nx0.i = 0; nx0.beg = 0; nx0.len = 0; nx0.use_far = true; nx0.cid = 0;
         nx0.stage_a();
@@ -1045,32 +1050,30 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
     __syncwarp();
     for (int ss = 0; ss < k.n_species && !skip; ++ss) {
         const int species = species_at(ss);
-        const int s_beg = k.species_start[species], s_end = k.species_start[species + 1];
-        const int n_tiles = (s_end - s_beg + NA - 1) / NA;
-        if (n_tiles == 0) continue;
-        const int n_first = NG * starters(species);   // tiles that are not claimed
+        const int s_end = species_start[species + 1];
+        if (species_start[species] == s_end) continue;
+        auto claimed = [&](int count) { return species_start[species] + (NG * starters(species) + count) * NA; };   // first atom of a claimed tile
         if (ss > 0) {
             // both groups are done with the previous species' tables; the barrier itself carries the decision (a word of shared memory could
             // be written for the next species before a warp has read it: not every turn of this loop has a barrier)
-            if (__syncthreads_or(threadIdx.x == 0 && n_first + *reinterpret_cast<volatile int *>(k.tile_counter + species) >= n_tiles)) continue;
+            if (__syncthreads_or(threadIdx.x == 0 && claimed(*reinterpret_cast<volatile int *>(k.tile_counter + species)) >= s_end)) continue;
             stage(species);
         }
 
         bool prefetched = ss == 0 && __shfl_sync(0xffffffffu, nx0.slot, 0) >= 0;   // this warp's atoms of the coming tile sit in the prefetch buffer
         int look_ahead = -1;       // (group leader) the tile after the current one
-        // the group's tiles of this species, claimed one ahead: the first is broadcast here, every later one travels with
-        // the barrier between encoding and head
-        int tile = first_tile;
+        // the group's tiles of this species, each by its first place in the processing order, claimed one ahead: the first is broadcast
+        // here, every later one travels with the barrier between encoding and head
+        int first = species_start[species] + first_tile * NA;
         if (ss > 0) {
             group_sync(group);
-            if (wg == 0 && lane == 0) ctl[2 * group] = n_first + atomicAdd(k.tile_counter + species, 1);
+            if (wg == 0 && lane == 0) ctl[2 * group] = claimed(atomicAdd(k.tile_counter + species, 1));
             group_sync(group);
-            tile = ctl[2 * group];
+            first = ctl[2 * group];
         }
-        while (tile < n_tiles) {
-            if (wg == 0 && lane == 0) look_ahead = n_first + atomicAdd(k.tile_counter + species, 1);   // consumed after the encoding
+        while (first < s_end) {
+            if (wg == 0 && lane == 0) look_ahead = claimed(atomicAdd(k.tile_counter + species, 1));   // consumed after the encoding
             pc.mark(11);
-            const int first = s_beg + tile * NA;
             const int count = min(NA, s_end - first);
 
             // ---------------- Encoding + invariants: the warp's atoms wg, wg + 8 one after the other ----------------
@@ -1142,16 +1145,16 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
             pc.mark(7);
             group_sync(group);
             pc.mark(8);
-            const int tile_next = ctl[2 * group + 1];
+            const int first_next = ctl[2 * group + 1];
 
             // ---------------- Regression (and the prefetch for the next tile) ----------------
             NextAtoms<APW> nx;
             nx.k = &k; nx.pf = pf;
-            const int next_slot = s_beg + tile_next * NA + wg + GW * lane;
-            nx.slot = (lane < APW && tile_next < n_tiles && next_slot < s_end) ? next_slot : -1;
+            const int next_slot = first_next + wg + GW * lane;
+            nx.slot = lane < APW && next_slot < s_end ? next_slot : -1;
             nx.i = 0; nx.beg = 0; nx.len = 0; nx.use_far = use_far; nx.cid = 0;
             head_tile<APW, DET, L16>(k, xs, sX, sc, us, ep, zs, hc, tm_quarter, count, first, group, wg, lane, e_sum, nx, pc);
-            prefetched = tile_next < n_tiles && s_beg + tile_next * NA + wg < s_end;
+            prefetched = first_next + wg < s_end;
             pc.mark(9);
 
             // ---------------- Derivation: the second atom first (a rescan of the first one's list would overwrite its queue) ----
@@ -1204,7 +1207,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
                 }
             }
             pc.mark(10);
-            tile = tile_next;
+            first = first_next;
         }
     }
     pc.flush(k.acc, lane);
@@ -1359,12 +1362,12 @@ __global__ void k_fixed_finish(int64_t n, long long *force_fx, const long long *
 int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     const int64_t n = c->n;
     const bool det = c->cfg.force_mode == 1;
-    if (!c->force_cleared && !det) {   // (k_fixed_finish keeps the integer sums clear)
+    const EvalBlocks blk = next_eval_blocks(c);
+    if ((!c->force_cleared || c->captured) && !det) {   // (k_fixed_finish keeps the integer sums clear)
         c->mark_open = false;
         MLIP_CUDA_TRY(c, cudaMemsetAsync(c->force, 0, sizeof(float4) * n, s));
     }
-    c->force_cleared = false;
-    double *clear_block = next_eval_block(c);
+    if (c->captured) MLIP_CUDA_TRY(c, cudaMemsetAsync(blk.use, 0, LAUNCH_CLEAR_BYTES, s));
     const bool in_smem = tables_fit_smem(c);
     const int tab_words = in_smem ? table_smem_words(c) : 0;
     // instantiations: {one, two atoms per warp, two with tables in global memory}
@@ -1394,9 +1397,10 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     k.pos4 = c->pos4; k.center_order = c->center_order;
     k.nbr_off = c->nbr_off; k.nbr_near = c->nbr_near; k.far_flag = c->far_flag; k.nbr = c->nbr; k.nbr16 = reinterpret_cast<const uint16_t *>(c->nbr); k.cell_id = c->cell_id; k.cell_start = c->cell_start;
     k.nbr_cap = c->nbr_cap; k.head_pack = c->head_w; k.force = c->force; k.e_atom = c->e_atom;
-    k.force_fx = c->force_fx; k.acc_fx = c->acc_fx;
-    k.acc = c->acc; k.pair_counter = c->pair_counter; k.status = c->status; k.tile_counter = c->tile_counter;
-    k.clear_block = clear_block;
+    k.force_fx = c->force_fx; k.acc_fx = reinterpret_cast<long long *>(blk.use + LB_ACC_FX);
+    k.acc = blk.use + LB_ACC; k.pair_counter = reinterpret_cast<unsigned long long *>(blk.use + LB_PAIR);
+    k.status = c->status; k.tile_counter = reinterpret_cast<int *>(blk.use);
+    k.clear_block = blk.clear; k.species_dev = c->captured ? c->species_start : nullptr;
     // CTAs in proportion to the species' tiles, at least one to a species that has any.  (One evaluation in us with the CTAs dealt out to the
     // species in turn / in proportion: 864 atoms 90:5:5 46 / 23.5, 6,912 atoms 80 / 66, 13,824 atoms 47:12:41 116 / 96; six equal
     // species, where in turn left some with more tiles than groups, 864 atoms 35.7 / 28.4, 23,328 atoms 221 / 198.)
@@ -1419,8 +1423,9 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     }
     k.stamp = timed_begin(c, MARK_KERNEL, s);
     const bool early = !c->lists_fresh;   // (the kernel reads the lists before it waits)
-    c->lists_fresh = false;
     MLIP_CUDA_TRY(c, launch_after_if(early, kernels[shape][(det ? 2 : 0) + (c->list16 ? 1 : 0)], blocks, NW * 32, smem_bytes, s, k, tab_words));
+    c->lists_fresh = c->force_cleared = false;
+    set_eval_block(c, blk.use);
     if (det) {
         MLIP_CUDA_TRY(c, launch_after(k_fixed_finish, (unsigned)((n + 255) / 256), 256, 0, s, n, c->force_fx, c->acc_fx, c->force, c->acc, k.stamp));
         c->launches += 1;

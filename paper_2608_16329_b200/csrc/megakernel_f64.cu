@@ -691,12 +691,12 @@ bool f64_shape_supported(int k, int l_max, int basis) {
 
 int launch_megakernel_f64(mlip_ctx *c, cudaStream_t s) {
     const int64_t n = c->n;
-    if (!c->force_cleared) {
+    const EvalBlocks blk = next_eval_blocks(c);
+    if (!c->force_cleared || c->captured) {
         c->mark_open = false;
         MLIP_CUDA_TRY(c, cudaMemsetAsync(c->force_d, 0, sizeof(double) * 3 * n, s));
     }
-    c->force_cleared = false;
-    double *clear_block = next_eval_block(c);
+    if (c->captured) MLIP_CUDA_TRY(c, cudaMemsetAsync(blk.use, 0, LAUNCH_CLEAR_BYTES, s));
     F64Args k;
     k.n = n; k.n_species = c->cfg.n_species; k.grid = c->grid; k.rc2 = c->cfg.r_cut * c->cfg.r_cut;
     k.coef = c->table_d; k.knots = c->cfg.table_knots; k.r_min = c->cfg.table_r_min;
@@ -704,8 +704,8 @@ int launch_megakernel_f64(mlip_ctx *c, cudaStream_t s) {
     k.pos4 = c->pos4; k.center_order = c->center_order; k.species_start = c->species_start;
     k.nbr_off = c->nbr_off; k.nbr_near = c->nbr_near; k.far_flag = c->far_flag; k.nbr = c->nbr; k.nbr16 = c->list16 ? reinterpret_cast<const uint16_t *>(c->nbr) : nullptr; k.cell_id = c->cell_id; k.cell_start = c->cell_start;
     k.nbr_cap = c->nbr_cap;
-    k.head = c->head_w_d; k.force = c->force_d; k.e_atom = c->e_atom_d; k.acc = c->acc;
-    k.pair_counter = c->pair_counter; k.status = c->status; k.clear_block = clear_block;
+    k.head = c->head_w_d; k.force = c->force_d; k.e_atom = c->e_atom_d; k.acc = blk.use + LB_ACC;
+    k.pair_counter = reinterpret_cast<unsigned long long *>(blk.use + LB_PAIR); k.status = c->status; k.clear_block = blk.clear;
     cudaError_t e = cudaErrorInvalidValue;
     switch (c->cfg.basis * 1000 + c->cfg.k * 10 + c->cfg.l_max) {
 #define MLIP_F64_CASE(K, L, B) case B * 1000 + K * 10 + L: e = launch_shape<K, L, B>(c, k, s); break;
@@ -718,6 +718,8 @@ int launch_megakernel_f64(mlip_ctx *c, cudaStream_t s) {
 #undef MLIP_F64_CASE
     }
     MLIP_CUDA_TRY(c, e);
+    c->force_cleared = false;
+    set_eval_block(c, blk.use);
     c->launches += 1;
     MLIP_CUDA_TRY(c, cudaGetLastError());
     return MLIP_OK;
