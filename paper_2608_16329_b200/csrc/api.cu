@@ -367,7 +367,10 @@ int mlip_set_velocities(mlip_ctx *c, const double *vel, void *stream) {
 
 // The fused evaluation in the context's precision.
 static int evaluate(mlip_ctx *c, cudaStream_t s) {
-    return c->cfg.precision == 1 ? launch_megakernel_f64(c, s) : launch_megakernel(c, s);
+    c->forces_current = false;
+    const int rc = c->cfg.precision == 1 ? launch_megakernel_f64(c, s) : launch_megakernel(c, s);
+    c->forces_current = rc == MLIP_OK;
+    return rc;
 }
 
 int mlip_compute_f64(mlip_ctx *c, double *energy, double *forces, double *virial, double *e_atom, void *stream) {
@@ -378,7 +381,6 @@ int mlip_compute_f64(mlip_ctx *c, double *energy, double *forces, double *virial
     enter(c, s);
     int rc = evaluate(c, s);
     if (rc != MLIP_OK) return rc;
-    c->forces_current = true;
     if (energy || virial || forces || e_atom) rc = launch_outputs_f64(c, forces, e_atom, energy, virial, s);
     return rc;
 }
@@ -390,7 +392,6 @@ int mlip_compute(mlip_ctx *c, double *energy, float *forces, double *virial, flo
     enter(c, s);
     int rc = evaluate(c, s);
     if (rc != MLIP_OK) return rc;
-    c->forces_current = true;
     if (energy || virial || forces || e_atom) rc = launch_outputs(c, forces, e_atom, energy, virial, s);
     return rc;
 }
@@ -444,6 +445,7 @@ constexpr int64_t SPECULATE_BELOW_ATOMS = 12000;   // (some 130 us an evaluation
 static int rebuild_and_evaluate(mlip_ctx *c, int rebuild_every, cudaStream_t s) {
     bool rebuild = rebuild_every > 0 && c->step % rebuild_every == 0;
     int rc;
+    c->forces_current = false;   // (the drift cleared them)
     if (rebuild_every < 0 && c->step % -rebuild_every == 0) {
         MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->rebuild_host, c->rebuild_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
         MLIP_CUDA_TRY(c, cudaEventRecord(c->check_ev, s));
@@ -466,10 +468,7 @@ int mlip_step(mlip_ctx *c, int n_steps, double dt, int rebuild_every, void *stre
     cudaStream_t s = (cudaStream_t)stream;
     enter(c, s);
     int rc;
-    if (!c->forces_current) {
-        if ((rc = evaluate(c, s)) != MLIP_OK) return rc;
-        c->forces_current = true;
-    }
+    if (!c->forces_current && (rc = evaluate(c, s)) != MLIP_OK) return rc;
     // per step the drift kernel and the evaluation: the half kick that closes a step runs with the next step's drift
     for (int it = 0; it < n_steps; ++it) {
         if ((rc = launch_kick_drift(c, dt, it > 0, s)) != MLIP_OK) return rc;
@@ -492,10 +491,7 @@ int mlip_step_nvt(mlip_ctx *c, int n_steps, double dt, int rebuild_every, double
     c->nhc_qk = c->nhc_kT * t_damp * t_damp;
     c->nhc_q1 = c->nhc_nf * c->nhc_qk;
     int rc;
-    if (!c->forces_current) {
-        if ((rc = evaluate(c, s)) != MLIP_OK) return rc;
-        c->forces_current = true;
-    }
+    if (!c->forces_current && (rc = evaluate(c, s)) != MLIP_OK) return rc;
     // Each thermostat half step takes the kinetic energy of the velocities as they stand (not the previous half step's rescaled
     // value, so that a run does not depend on how it is split into calls).  The first one's velocity factor is applied with the half
     // kick that follows, the second one's with the next step's kinetic energy.

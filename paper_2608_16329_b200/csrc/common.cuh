@@ -187,6 +187,7 @@ namespace mlip {
         cudaError_t e_ = (call);                                                          \
         if (e_ != cudaSuccess) {                                                          \
             (ctx)->err = std::string(#call) + ": " + cudaGetErrorString(e_);              \
+            cudaGetLastError();   /* a later call's check must not meet this error again */ \
             return e_ == cudaErrorMemoryAllocation ? MLIP_ERR_OOM : MLIP_ERR_CUDA;        \
         }                                                                                 \
     } while (0)

@@ -1,4 +1,4 @@
-"""Calls captured into a CUDA graph and replayed, alone and in turn with ordinary calls."""
+"""Calls captured into a CUDA graph and replayed, alone and in turn with ordinary calls, and calls that fail inside a capture."""
 import numpy as np
 import pytest
 import torch
@@ -89,3 +89,28 @@ def test_captured_steps_replay(ensemble):
         assert pot.sync_status() == 0
         states.append(b"".join(t.cpu().numpy().tobytes() for t in (*pot.state()[:2], pot.energies())))
     assert states[0] == states[1]
+
+
+def test_a_call_that_fails_leaves_the_next_ones_alone():
+    """A list build waits for the device, which a capture does not allow: the call is refused, and neither its error nor what it had
+    noted for the next evaluation stays behind."""
+    import paper_2608_16329_b200 as mlip
+    from cuda.bindings import runtime
+    w, _, pot = make_pair(5, 6, 1.0)
+    _, _, other = make_pair(2, 6, 1.0)
+    pot.build_neighbors(w.pos, w.species, w.box)
+    want = pot.compute()
+    pos, species = torch.as_tensor(w.pos, device="cuda"), torch.as_tensor(w.species, device="cuda")
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    assert runtime.cudaStreamBeginCapture(stream.cuda_stream, runtime.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed)[0] == 0
+    with pytest.raises(mlip.MlipError):
+        mlip.mlip_build_neighbors(pot.ctx, pos, species, w.box, stream.cuda_stream)
+    runtime.cudaStreamEndCapture(stream.cuda_stream)
+    runtime.cudaGetLastError()
+    wo, _, _ = make_pair(2, 6, 1.0)
+    other.build_neighbors(wo.pos, wo.species, wo.box)
+    other.compute()
+    pot.build_neighbors(w.pos, w.species, w.box)
+    _same(pot.compute(), want, False, torch.float32)
+    assert pot.sync_status() == 0 and other.sync_status() == 0
