@@ -7,10 +7,11 @@
 namespace mlip {
 
 // One 256-bit load per gathered atom (a 32-byte sector) instead of two 128-bit ones: halves the
-// number of L1 wavefronts of the uncoalesced position gathers.
+// number of L1 wavefronts of the uncoalesced position gathers.  An ordinary load, not one through the read-only path: the fused kernels
+// are resident before the kernel that moves the atoms has ended (wait_previous), so positions change during their lifetime.
 __device__ __forceinline__ double4 load_pos4(const double4 *p) {
     double4 v;
-    asm volatile("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];" : "=d"(v.x), "=d"(v.y), "=d"(v.z), "=d"(v.w) : "l"(p));
+    asm volatile("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];" : "=d"(v.x), "=d"(v.y), "=d"(v.z), "=d"(v.w) : "l"(p));
     return v;
 }
 

@@ -53,3 +53,30 @@ def test_timing_records_keep_the_last_256_launches(n_cells):
         assert launches == kept and kernel == ms and build == 0.0
         assert 0.003 * kept < ms < 10.0 * kept and 0.0005 * kept < integrate < 1.0 * kept
     assert pot.sync_status() == 0
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("cfg,n_cells", [(5, 6), (5, 15)])
+def test_every_evaluation_sees_the_positions_set_just_before_it(cfg, n_cells, precision):
+    """Sixty times two configurations in turn without a wait between them: the fused kernel is resident while the positions are still
+    being written.  Sums in another order: 1e-6 of the forces' size (1e-12 in double)."""
+    import torch
+    w, _, pot = make_pair(cfg, n_cells, 1.0, precision=precision)
+    pot.build_neighbors(w.pos, w.species, w.box)
+    moved = w.pos + np.random.default_rng(1).uniform(-0.1, 0.1, w.pos.shape)
+    moved -= np.floor(moved / w.box) * w.box
+    both = [torch.as_tensor(np.where(x >= w.box, 0.0, x), device="cuda") for x in (w.pos, moved)]
+    want = []
+    for x in both:
+        pot.set_positions(x)
+        torch.cuda.synchronize()
+        want.append(pot.compute()["forces"].clone())
+        torch.cuda.synchronize()
+    got = []
+    for turn in range(60):
+        pot.set_positions(both[turn % 2])
+        got.append(pot.compute()["forces"])
+    tol = (1e-6, 1e-12)[precision]
+    for turn, f in enumerate(got):
+        assert (f - want[turn % 2]).abs().max() <= tol * want[turn % 2].abs().max(), turn
+    assert pot.sync_status() == 0
