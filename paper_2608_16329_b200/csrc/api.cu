@@ -645,9 +645,10 @@ static int marks_total(mlip_ctx *c, unsigned char kind, int64_t *count, double *
     }
     if (c->stamps > c->stamp_reset[kind]) {   // parts timed by the kernels themselves
         constexpr int S = mlip_ctx::STAMPS, H = S / 2;
-        std::vector<unsigned long long> t(2 * S);
-        MLIP_CUDA_TRY(c, cudaStreamSynchronize(c->mark_stream));
-        MLIP_CUDA_TRY(c, cudaMemcpy(t.data(), c->stamp, sizeof(unsigned long long) * 2 * S, cudaMemcpyDeviceToHost));
+        unsigned long long t[2 * S];   // (32 KB)
+        cudaSetDevice(c->cfg.device);
+        MLIP_CUDA_TRY(c, cudaDeviceSynchronize());   // (the streams that the kernels ran on need not exist any more)
+        MLIP_CUDA_TRY(c, cudaMemcpy(t, c->stamp, sizeof t, cudaMemcpyDeviceToHost));
         const int64_t first = std::max<int64_t>(c->stamp_reset[kind], (c->stamps - 1) / H * H - H);   // the half being filled and the one before
         for (int64_t m = c->stamps - 1; m >= std::max<int64_t>(0, first) && kept < mlip_ctx::EV_POOL; --m) {
             if (c->stamp_kind[m % S] != kind || t[S + m % S] < t[m % S]) continue;

@@ -80,3 +80,23 @@ def test_every_evaluation_sees_the_positions_set_just_before_it(cfg, n_cells, pr
     for turn, f in enumerate(got):
         assert (f - want[turn % 2]).abs().max() <= tol * want[turn % 2].abs().max(), turn
     assert pot.sync_status() == 0
+
+
+def test_timing_records_outlive_the_streams_they_were_taken_on():
+    import paper_2608_16329_b200 as mlip
+    import torch
+    from cuda.bindings import runtime
+    w, _, pot = make_pair(5, 6, 1.0)
+    pot.build_neighbors(w.pos, w.species, w.box)
+    pot.compute()
+    torch.cuda.synchronize()
+    mlip.mlip_kernel_time(pot.ctx, reset=True)
+    for _ in range(3):
+        err, stream = runtime.cudaStreamCreate()
+        assert err == 0
+        mlip.mlip_compute(pot.ctx, stream=int(stream))
+        assert runtime.cudaStreamSynchronize(stream)[0] == 0 and runtime.cudaStreamDestroy(stream)[0] == 0
+    launches, ms = mlip.mlip_kernel_time(pot.ctx)
+    assert launches == 3 and 0.003 < ms < 30.0
+    pot.compute()
+    assert pot.sync_status() == 0
