@@ -278,7 +278,9 @@ int mlip_get_counters(mlip_ctx *ctx, int64_t *n_list_entries, int64_t *n_pairs_i
  * Device time of the fused-kernel launches since the last reset: number of launches timed
  * and their summed duration in ms (each launch lies between two CUDA events on the launching stream; below
  * 100,000 atoms, where events would cost a tenth of a step, the kernels record the device's timer at their begin and
- * end instead; the most recent 256 launches are kept).  Synchronises with the last of them.
+ * end instead; the most recent 256 launches are kept).  Waits for the device.  A kernel that starts while the one ahead
+ * of it still runs counts from that one's end: what it does before then -- a fused launch that does not follow a list build stages
+ * its first tables, weights and lists, about 3 us -- is hidden in the other's time and counted there.
  */
 int mlip_kernel_time(mlip_ctx *ctx, int64_t *n_launches, double *total_ms, int reset);
 

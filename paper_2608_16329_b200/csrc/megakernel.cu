@@ -234,6 +234,7 @@ struct KernelArgs {
     int *tile_counter;
     double *clear_block;       // the other evaluation block (next_eval_block)
     unsigned long long *stamp;
+    bool early;                // launched to start before the kernel ahead of it has ended
 };
 
 // The radial tables of the current central species: in shared memory or, when they do not fit, in global memory (same
@@ -963,6 +964,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
     int *ctl = reinterpret_cast<int *>(hc + HC_WORDS);
     const int rows = k.tab.knots + 3;
     allow_next();
+    if (!k.early) stamp_begin(k.stamp);   // (else from the end of the kernel ahead, whose time hides the staging)
 
     // all of tensor memory (this is the only CTA on the SM) for the head's weights
     if (warp == 0) {
@@ -1422,8 +1424,8 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
         if (q < C) up[q] > 0 ? (void)(fixed += up[q]) : (void)(before += weight[q]);
     }
     k.stamp = timed_begin(c, MARK_KERNEL, s);
-    const bool early = !c->lists_fresh;   // (the kernel reads the lists before it waits)
-    MLIP_CUDA_TRY(c, launch_after_if(early, kernels[shape][(det ? 2 : 0) + (c->list16 ? 1 : 0)], blocks, NW * 32, smem_bytes, s, k, tab_words));
+    k.early = !c->lists_fresh;   // (the kernel reads the lists before it waits)
+    MLIP_CUDA_TRY(c, launch_after_if(k.early, kernels[shape][(det ? 2 : 0) + (c->list16 ? 1 : 0)], blocks, NW * 32, smem_bytes, s, k, tab_words));
     c->lists_fresh = c->force_cleared = false;
     set_eval_block(c, blk.use);
     if (det) {

@@ -100,3 +100,25 @@ def test_timing_records_outlive_the_streams_they_were_taken_on():
     assert launches == 3 and 0.003 < ms < 30.0
     pot.compute()
     assert pot.sync_status() == 0
+
+
+def test_a_launch_that_overlaps_no_other_is_timed_from_its_begin():
+    """The fused launch behind a list build stages its tables (215 KB per CTA, some 3 us) by itself; in a sequence of evaluations the kernel
+    ahead hides that.  864 atoms, mean of 100 launches each."""
+    import paper_2608_16329_b200 as mlip
+    import torch
+    w, _, pot = make_pair(5, 6, 1.0)
+    mean = []
+    for builds in (False, True):
+        pot.build_neighbors(w.pos, w.species, w.box)
+        pot.compute()
+        torch.cuda.synchronize()
+        mlip.mlip_kernel_time(pot.ctx, reset=True)
+        for _ in range(100):
+            if builds:
+                pot.build_neighbors(w.pos, w.species, w.box)
+            pot.compute()
+        n, ms = mlip.mlip_kernel_time(pot.ctx)
+        mean.append(1e3 * ms / n)
+    print(f"fused kernel, 864 atoms: {mean[0]:.1f} us in a sequence, {mean[1]:.1f} us behind a build")
+    assert mean[1] > mean[0] + 1.5   # (2.9 us here; the staging left out: 0.2)
