@@ -299,7 +299,7 @@ constexpr int SECOND_ROOM = NARROW_CHUNKS * 32;
 // Compact lists: lane q < 27 holds the first atom of the q-th cell around atom i's build-time cell; an entry's index is
 // that base (one shuffle) plus the position coded in its low bits.
 __device__ __forceinline__ int cell_base_of_lane(const KernelArgs &k, int i, int lane) {
-    return lane < 27 ? __ldg(k.cell_start + neighbor_cell(k.grid, __ldg(k.cell_id + i), lane)) : 0;
+    return lane < 27 ? __ldg(k.cell_start + MLIP_CHECK_INDEX(neighbor_cell(k.grid, __ldg(k.cell_id + i), lane), k.grid.n_cells, k.status)) : 0;
 }
 template <int SCAN_CHUNKS, bool L16>
 __device__ __forceinline__ int collect_pairs_n(const KernelArgs &k, const double4 &pi, int64_t beg, int64_t &cur, int64_t end, float4 *pq, int cap, int lane,
@@ -772,7 +772,7 @@ struct NextAtoms {
     int64_t beg;
     int len;
     int cid;          // compact lists: the atom's build-time cell
-    __device__ __forceinline__ void stage_a() { if (slot >= 0) i = __ldg(k->center_order + slot); }
+    __device__ __forceinline__ void stage_a() { if (slot >= 0) i = (int)MLIP_CHECK_INDEX(__ldg(k->center_order + MLIP_CHECK_INDEX(slot, k->n, k->status)), k->n, k->status); }
     template <bool L16>
     __device__ __forceinline__ void stage_b() {
         if (slot >= 0) {
@@ -796,15 +796,19 @@ struct NextAtoms {
 #pragma unroll
                 for (int c = 0; c < (PF_IDX / 2 + 1 + 31) / 32; ++c) {
                     const int e = 32 * c + lane;
-                    if (e < words) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(sidx + e)), "l"(src + e) : "memory");
+                    if (e < words) {
+                        const int at = MLIP_CHECK_INDEX(b - odd + 2 * e, k->nbr_cap, k->status) == b - odd + 2 * e ? e : 0;
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(sidx + e)), "l"(src + at) : "memory");
+                    }
                 }
                 if (lane < 27)
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(sidx + PF_CS + lane)), "l"(k->cell_start + neighbor_cell(k->grid, cell, lane)) : "memory");
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(sidx + PF_CS + lane)),
+                                 "l"(k->cell_start + MLIP_CHECK_INDEX(neighbor_cell(k->grid, cell, lane), k->grid.n_cells, k->status)) : "memory");
             } else {
 #pragma unroll
                 for (int c = 0; c < PF_IDX / 32; ++c) {
                     const int e = 32 * c + lane;
-                    if (e < n) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(sidx + e)), "l"(k->nbr + b + e) : "memory");
+                    if (e < n) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(sidx + e)), "l"(k->nbr + MLIP_CHECK_INDEX(b + e, k->nbr_cap, k->status)) : "memory");
                 }
             }
         }
@@ -904,7 +908,7 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
     }
     if (wg == 7 && lane < count) {
         const float e_i = ((ep[lane] + ep[NA + lane]) + (ep[2 * NA + lane] + ep[3 * NA + lane])) + hc[HC_BOUT];
-        k.e_atom[__ldg(k.center_order + first + lane)] = e_i;
+        k.e_atom[MLIP_CHECK_INDEX(__ldg(k.center_order + first + lane), k.n, k.status)] = e_i;
         e_sum += DET ? rint((double)e_i * ENERGY_FX) : (double)e_i;   // DET: exact integer sums
     }
 

@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
             beg = k.nbr_off[i]; end = use_far ? k.nbr_off[i + 1] : beg + k.nbr_near[i];
         }
         // compact lists: lane q < 27 holds the first atom of the q-th cell around the atom's build-time cell
-        const int cs = (k.nbr16 && have && lane < 27) ? k.cell_start[neighbor_cell(k.grid, k.cell_id[i], lane)] : 0;
+        const int cs = (k.nbr16 && have && lane < 27) ? k.cell_start[MLIP_CHECK_INDEX(neighbor_cell(k.grid, k.cell_id[i], lane), k.grid.n_cells, k.status)] : 0;
         auto entry = [&](int64_t e, bool live) {   // index of list entry e (every lane of the warp calls this together)
             if (!k.nbr16) return live ? (int)MLIP_CHECK_INDEX(k.nbr[MLIP_CHECK_INDEX(e, k.nbr_cap, k.status)], k.n, k.status) : 0;
             const int code = live ? k.nbr16[MLIP_CHECK_INDEX(e, k.nbr_cap, k.status)] : 0;

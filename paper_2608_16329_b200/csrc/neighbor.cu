@@ -717,10 +717,14 @@ struct ListView {
     const uint16_t *nbr16;
     const int32_t *cell_id, *cell_start;
     CellGrid grid;
+    int64_t n, nbr_cap;   // atoms, room for entries (range-checked builds)
+    int *status;
     __device__ __forceinline__ int at(int64_t i, int64_t e) const {
-        if (!nbr16) return nbr[e];
+        e = MLIP_CHECK_INDEX(e, nbr_cap, status);
+        if (!nbr16) return (int)MLIP_CHECK_INDEX(nbr[e], n, status);
         const int code = nbr16[e];
-        return cell_start[neighbor_cell(grid, cell_id[i], code >> L16_SHIFT)] + (code & L16_MASK);
+        const int j = cell_start[MLIP_CHECK_INDEX(neighbor_cell(grid, cell_id[i], code >> L16_SHIFT), grid.n_cells, status)] + (code & L16_MASK);
+        return (int)MLIP_CHECK_INDEX(j, n, status);
     }
 };
 
@@ -743,7 +747,7 @@ __global__ void __launch_bounds__(256) k_export_count(int64_t n, int n_species, 
 #pragma unroll
         for (int w = 0; w < 4; ++w) cnt[w] += (s >> 1) == w ? 1u << (16 * (s & 1)) : 0u;
     }
-    const int64_t row = (int64_t)(key[i] & 0x0fffffff) * n_species;
+    const int64_t row = (int64_t)MLIP_CHECK_INDEX(key[i] & 0x0fffffff, n, lv.status) * n_species;
 #pragma unroll
     for (int w = 0; w < 4; ++w) cnt[w] = __reduce_add_sync(0xffffffffu, cnt[w]);
     if (lane < n_species) seg_count[row + lane] = (int)((((lane >> 1) == 0 ? cnt[0] : (lane >> 1) == 1 ? cnt[1] : (lane >> 1) == 2 ? cnt[2] : cnt[3]) >> (16 * (lane & 1))) & 0xffffu);
@@ -813,7 +817,7 @@ __global__ void __launch_bounds__(256) k_export_fill(int64_t n, int n_species, c
     int32_t *keys = s_keys[threadIdx.x >> 5];
     const int64_t beg = nbr_off[i];
     const int m = (int)(nbr_off[i + 1] - beg);
-    out += seg_ptr[(int64_t)(key[i] & 0x0fffffff) * n_species];   // the species' segments of an atom follow one another
+    out += seg_ptr[(int64_t)MLIP_CHECK_INDEX(key[i] & 0x0fffffff, n, lv.status) * n_species];   // the species' segments of an atom follow one another
     if (m <= EXPORT_BUF / 2) return export_sorted<4>(lv, key, i, beg, m, keys, out, lane);
     if (m <= EXPORT_BUF) return export_sorted<8>(lv, key, i, beg, m, keys, out, lane);
     for (int e = lane; e < m; e += 32) {
@@ -831,6 +835,7 @@ static ListView list_view(const mlip_ctx *c) {
     lv.nbr = c->nbr;
     lv.nbr16 = c->list16 ? reinterpret_cast<const uint16_t *>(c->nbr) : nullptr;
     lv.cell_id = c->cell_id; lv.cell_start = c->cell_start; lv.grid = c->grid;
+    lv.n = c->n; lv.nbr_cap = c->nbr_cap; lv.status = c->status;
     return lv;
 }
 
