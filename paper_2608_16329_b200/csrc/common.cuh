@@ -43,7 +43,7 @@ enum : int {
 
 // accumulator slots (double)
 enum : int { ACC_ENERGY = 0, ACC_VIRIAL = 1, ACC_KINETIC = 10, ACC_COUNT = 32 };
-// launch_block in doubles: [0, 4) tile_counter (MAX_SPECIES ints), [4] pair_counter, [5, 15) acc_fx, [16, 16 + ACC_COUNT) acc;
+// launch_base, one block in doubles: [0, 4) tile_counter (MAX_SPECIES ints), [4] pair_counter, [5, 15) acc_fx, [16, 16 + ACC_COUNT) acc;
 // everything up to the kinetic-energy slot of acc is zero when a fused kernel starts.  There are two such blocks: an evaluation uses one
 // and clears the other, which holds the totals of the evaluation before it, for the next (but see note_capture)
 constexpr int LB_PAIR = 4, LB_ACC_FX = 5, LB_ACC = 16, LB_COUNT = LB_ACC + ACC_COUNT;

@@ -85,8 +85,11 @@ constexpr int HC_WORDS = (HC_USED + 15) / 16 * 16;
 constexpr int CTL_WORDS = 16;   // per group {tile, tile after it}; tensor-memory base; the species' starts
 static_assert(5 + MAX_SPECIES + 1 <= CTL_WORDS, "control words");
 // Systems below this size take tiles of 8 atoms, one per warp: with few tiles per SM the chain through one tile is what counts
-// (kernel us with 8- / 16-atom tiles, 6 species: 864 atoms 47 / 53, 6,912 96 / 97, 16,384 174 / 166, 55,296 499 / 474, 131,072
-// 1119 / 1046; one species: 4,394 63 / 66, 16,000 140 / 135, 65,536 476 / 441).
+// (one evaluation in us with 8- / 16-atom tiles, 6 species: 256 atoms 26 / 35, 864 29 / 36, 4,000 55 / 53, 6,912 85 / 90, 10,976 115 / 125,
+// 16,384 166 / 162, 32,000 292 / 271, 131,072 1125 / 1063; one species: 686 atoms 26 / 28, 4,394 45 / 43, 8,192 78 / 73, 11,664 95 / 103,
+// 16,000 128 / 133, 31,250 241 / 224, 65,536 472 / 433; three: 10,976 97 / 106, 16,384 140 / 137.  In between it depends on how full the
+// last round of tiles is).  Tables in global memory (seven species or more, or many knots): compiled with 16-atom tiles only; 8-atom ones
+// would be faster below the same size (8 species: 864 atoms 27 / 40, 10,976 122 / 140, 16,384 183 / 181, 131,072 1215 / 1212).
 constexpr int64_t ONE_PER_WARP_BELOW_ATOMS = 12000;
 // Shared memory per tile shape.  Two atoms per warp halve the regression's barriers, weight fetches and idle time per atom
 // (each warp owns 16 neurons x 8 atoms of a 16-atom tile instead of half of the warps owning an 8-atom tile); one atom per warp
@@ -569,11 +572,7 @@ __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView
         __syncwarp();
         pc.mark(4);
         const int nmt = (n + 15) >> 4;
-#ifndef MLIP_MTILE_UNROLL
-#define MLIP_MTILE_UNROLL 1
-#endif
-        constexpr int mtile_unroll = MLIP_MTILE_UNROLL;
-#pragma unroll mtile_unroll
+#pragma unroll 1
         for (int mt = 0; mt < nmt; ++mt) {
             // A = [G; G'] (16 pairs x 32 channels): rows pairs g, g + 8; this lane evaluates channels 8t .. 8t+7
             // (one accumulator per output here: the truncating accumulation costs ~1e-6 relative on a

@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(256) k_neighbors(int64_t n, CellGrid g, double
                                                    const int32_t *__restrict__ user_of, int32_t n_owned) {
     const int lane = threadIdx.x & 31;
     int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (i >= n || (*status & FLAG_NONFINITE)) return;   // a broken configuration is not traversed (see k_sort_cells)
+    if (i >= n || (*status & FLAG_NONFINITE)) return;   // a broken configuration is not traversed (see k_sort_gather)
     if (user_of[i] >= n_owned) {   // a ghost is listed by others but has no list of its own
         if (!FILL && lane == 0) { nbr_count[i] = 0; nbr_near[i] = 0; }
         return;
@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(256) k_neighbors_onepass(int64_t n, CellGrid g
                                                            const int32_t *__restrict__ user_of, int32_t n_owned) {
     // `unpublished_tile` >= 0 (diagnostic builds of the lists only) names a tile that never publishes its look-back word,
     // so that its successor's bounded wait can be seen to run out; -1 in production.
-    if (*global_status & FLAG_NONFINITE) return;   // a broken configuration is not traversed (see k_sort_cells)
+    if (*global_status & FLAG_NONFINITE) return;   // a broken configuration is not traversed (see k_sort_gather)
     // look-back word: flag in the top two bits (0 empty, 1 tile aggregate, 2 inclusive prefix), value below
     constexpr unsigned long long OP_AGG = 1ull << 62, OP_INC = 2ull << 62, OP_VAL = (1ull << 62) - 1;
     constexpr int TILE_ATOMS = 8 * PER_WARP;
