@@ -10,6 +10,7 @@
 // identical to a plain CPU evaluation of the same expression.
 #include <algorithm>
 #include <string.h>
+#include <type_traits>
 
 #include "common.cuh"
 #include "scan.cuh"
@@ -474,6 +475,57 @@ __global__ void __launch_bounds__(256) k_neighbors_rel(int64_t n, CellGrid g, do
 constexpr int OP_TILE = 64;   // largest tile: the in-tile scan handles two counts per lane of one warp
 constexpr int OP_SPIN = 1 << 18;
 
+// Offsets of a tile's lists, by one warp: exclusive sums of the counts inside the tile to `off`, the entries of all tiles before it to
+// *prefix and with its own to *total.
+template <int TILE_ATOMS>
+__device__ __forceinline__ void tile_offsets(int64_t tile, const int *cnt, long long *off, long long *prefix_out, long long *total_out, int *status,
+                                             unsigned long long *tile_state, int spin_limit, long long unpublished_tile, int lane) {
+    // look-back word: flag in the top two bits (0 empty, 1 tile aggregate, 2 inclusive prefix), value below
+    constexpr unsigned long long OP_AGG = 1ull << 62, OP_INC = 2ull << 62, OP_VAL = (1ull << 62) - 1;
+    static_assert(TILE_ATOMS <= 64, "two counts per lane");
+    const int c0 = 2 * lane < TILE_ATOMS ? cnt[2 * lane] : 0, c1 = 2 * lane < TILE_ATOMS ? cnt[2 * lane + 1] : 0;
+    long long incl = c0 + c1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (2 * lane < TILE_ATOMS) { off[2 * lane] = incl - c0 - c1; off[2 * lane + 1] = incl - c1; }
+    const long long aggregate = __shfl_sync(0xffffffffu, incl, 31);
+    volatile unsigned long long *state = tile_state;
+    long long prefix = 0;
+    if (tile > 0) {
+        if (lane == 0 && tile != unpublished_tile) state[tile] = OP_AGG | (unsigned long long)aggregate;
+        int64_t hi = tile - 1;
+        int spins = 0;
+        for (;;) {   // windows of 32 predecessors, nearest first
+            const int64_t p = hi - lane;
+            unsigned long long v = OP_INC;
+            if (p >= 0) v = state[p];
+            const unsigned flag = (unsigned)(v >> 62);
+            const unsigned inc = __ballot_sync(0xffffffffu, flag == 2), empty = __ballot_sync(0xffffffffu, flag == 0);
+            const int first_inc = inc ? __ffs(inc) - 1 : 32;
+            const unsigned need = first_inc >= 31 ? 0xffffffffu : ((2u << first_inc) - 1u);
+            if (empty & need) {   // a tile in the window has not published yet
+                if (++spins > spin_limit) { if (lane == 0) atomicOr(status, FLAG_NEIGHBOR_OVERFLOW); break; }
+                __nanosleep(200);
+                continue;
+            }
+            long long val = (lane <= first_inc && p >= 0) ? (long long)(v & OP_VAL) : 0;
+#pragma unroll
+            for (int o = 16; o; o >>= 1) val += __shfl_xor_sync(0xffffffffu, val, o);
+            prefix += val;
+            if (first_inc < 32) break;
+            hi -= 32;
+        }
+    }
+    if (lane == 0) {
+        if (tile != unpublished_tile) state[tile] = OP_INC | (unsigned long long)(prefix + aggregate);
+        *prefix_out = prefix;
+        *total_out = prefix + aggregate;
+    }
+}
+
 __device__ __forceinline__ bool rel_hit(const float4 &rj, float sx, float sy, float sz, float rl2_lo, float rl2_hi, double rl2,
                                         const double4 &pi, const double4 *__restrict__ pos4, int j, const CellGrid &g, float &d2f) {
     const float dx = rj.x + sx, dy = rj.y + sy, dz = rj.z + sz;
@@ -593,7 +645,7 @@ __device__ __forceinline__ int onepass_traverse(int64_t i, const CellGrid &g, do
     return cnt;
 }
 
-constexpr int64_t ONEPASS_SMALL = 50000;   // see onepass_per_warp
+constexpr int64_t ONEPASS_SMALL = 18000;   // see onepass_per_warp
 constexpr int OP_BUF = 160;   // hits kept per atom in shared memory; a longer list is traversed again straight into global memory
 
 template <bool REL, int PER_WARP, typename ENTRY>
@@ -607,8 +659,6 @@ __global__ void __launch_bounds__(256) k_neighbors_onepass(int64_t n, CellGrid g
     // `unpublished_tile` >= 0 (diagnostic builds of the lists only) names a tile that never publishes its look-back word,
     // so that its successor's bounded wait can be seen to run out; -1 in production.
     if (*global_status & FLAG_NONFINITE) return;   // a broken configuration is not traversed (see k_sort_gather)
-    // look-back word: flag in the top two bits (0 empty, 1 tile aggregate, 2 inclusive prefix), value below
-    constexpr unsigned long long OP_AGG = 1ull << 62, OP_INC = 2ull << 62, OP_VAL = (1ull << 62) - 1;
     constexpr int TILE_ATOMS = 8 * PER_WARP;
     extern __shared__ int32_t s_hits[];   // [TILE_ATOMS][OP_BUF]
     __shared__ int s_cnt[OP_TILE], s_near[OP_TILE];
@@ -634,50 +684,7 @@ __global__ void __launch_bounds__(256) k_neighbors_onepass(int64_t n, CellGrid g
     __syncthreads();
 
     // ---- offsets: scan inside the tile, look back over the tiles before it ----
-    if (warp == 0) {
-        const int c0 = 2 * lane < TILE_ATOMS ? s_cnt[2 * lane] : 0, c1 = 2 * lane < TILE_ATOMS ? s_cnt[2 * lane + 1] : 0;
-        long long incl = c0 + c1;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        s_off[2 * lane] = incl - c0 - c1;
-        s_off[2 * lane + 1] = incl - c1;
-        const long long aggregate = __shfl_sync(0xffffffffu, incl, 31);
-        volatile unsigned long long *state = tile_state;
-        long long prefix = 0;
-        if (tile > 0) {
-            if (lane == 0 && tile != unpublished_tile) state[tile] = OP_AGG | (unsigned long long)aggregate;
-            int64_t hi = tile - 1;
-            int spins = 0;
-            for (;;) {   // windows of 32 predecessors, nearest first
-                const int64_t p = hi - lane;
-                unsigned long long v = OP_INC;
-                if (p >= 0) v = state[p];
-                const unsigned flag = (unsigned)(v >> 62);
-                const unsigned inc = __ballot_sync(0xffffffffu, flag == 2), empty = __ballot_sync(0xffffffffu, flag == 0);
-                const int first_inc = inc ? __ffs(inc) - 1 : 32;
-                const unsigned need = first_inc >= 31 ? 0xffffffffu : ((2u << first_inc) - 1u);
-                if (empty & need) {   // a tile in the window has not published yet
-                    if (++spins > spin_limit) { if (lane == 0) atomicOr(status, FLAG_NEIGHBOR_OVERFLOW); break; }
-                    __nanosleep(200);
-                    continue;
-                }
-                long long val = (lane <= first_inc && p >= 0) ? (long long)(v & OP_VAL) : 0;
-#pragma unroll
-                for (int o = 16; o; o >>= 1) val += __shfl_xor_sync(0xffffffffu, val, o);
-                prefix += val;
-                if (first_inc < 32) break;
-                hi -= 32;
-            }
-        }
-        if (lane == 0) {
-            if (tile != unpublished_tile) state[tile] = OP_INC | (unsigned long long)(prefix + aggregate);
-            s_prefix = prefix;
-            s_total = prefix + aggregate;
-        }
-    }
+    if (warp == 0) tile_offsets<TILE_ATOMS>(tile, s_cnt, s_off, &s_prefix, &s_total, status, tile_state, spin_limit, unpublished_tile, lane);
     __syncthreads();
     const long long tile_off = s_prefix;
     if (first + TILE_ATOMS >= n && threadIdx.x == 0) {   // the last tile closes the offsets
@@ -706,6 +713,244 @@ __global__ void __launch_bounds__(256) k_neighbors_onepass(int64_t n, CellGrid g
         } else {
             int cn;
             onepass_traverse<REL, ENTRY, ENTRY>(i, g, rl2, edge, rl2_lo, rl2_hi, pos4, rel, cell_start, lane, nbr + off, cnt - 1, fit, near2, cn);
+        }
+    }
+}
+
+// ---- lane = central atom ----
+// The same lists from the same tiles of 64 atoms, two warps to a tile, for systems that fill the chip that way: each lane owns one of 32
+// consecutive atoms, the candidates of the cells around them pass through shared memory 32 at a time and every lane tests every
+// one (a broadcast read, packed fp32 arithmetic, no ballots and no ranks: a lane appends to its own row).  Consecutive atoms lie in cells that
+// follow one another along z, so the cells around them are nine columns of (cells spanned + 2) layers; a lane takes part in the
+// three layers around its own cell only.  Each lane meets the candidates in the order of the warp-per-atom traversal, with the same
+// arithmetic, so the lists agree entry by entry.
+// Rows hold 16-bit codes (near hits from the front, far hits from the back); `buf` entries, a multiple of four, from the mean density.
+constexpr int LN_WARPS = OP_TILE / 32, LN_THREADS = 32 * LN_WARPS;
+constexpr int LN_SPAN = 4;                          // cells along z that a group of lanes may span: 9 x 6 cells, two to a lane
+constexpr int LN_STAGE = 2 * 3 * 32;                // two chunks of candidates, x, y, z
+static_assert(9 * (LN_SPAN + 2) <= 64, "cell ranges, two per lane");
+__host__ __device__ constexpr int ln_row(int buf) { return buf + 2; }   // in entries: an odd number of words
+inline size_t ln_smem(int buf) { return sizeof(float) * LN_STAGE * LN_WARPS + sizeof(uint16_t) * OP_TILE * ln_row(buf); }
+
+__device__ __forceinline__ float2 pack_add(float2 a, float b) {
+    unsigned long long ra, rb, rd;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(ra) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(rb) : "f"(b));
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(rd));
+    return d;
+}
+__device__ __forceinline__ float2 pack_norm2(float2 x, float2 y, float2 z) {   // x x + y y + z z, rounded as fma(z, z, fma(y, y, x x))
+    unsigned long long rx, ry, rz, rd;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(rx) : "f"(x.x), "f"(x.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(ry) : "f"(y.x), "f"(y.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(rz) : "f"(z.x), "f"(z.y));
+    asm("mul.rn.f32x2 %0, %1, %1;" : "=l"(rd) : "l"(rx));
+    asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(rd) : "l"(ry));
+    asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(rd) : "l"(rz));
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(rd));
+    return d;
+}
+
+template <typename ENTRY>
+__global__ void __launch_bounds__(LN_THREADS) k_neighbors_lanes(int64_t n, CellGrid g, double rl2, const double4 *__restrict__ pos4,
+                                                                const float4 *__restrict__ rel, const int32_t *__restrict__ cell_start,
+                                                                int64_t *__restrict__ nbr_off, ENTRY *__restrict__ nbr, int64_t nbr_cap,
+                                                                int *status, unsigned long long *tile_state, int *build_word,
+                                                                const int *global_status, int spin_limit, long long unpublished_tile,
+                                                                float near2, int32_t *__restrict__ nbr_near,
+                                                                const int32_t *__restrict__ user_of, int32_t n_owned, int buf) {
+    if (*global_status & FLAG_NONFINITE) return;   // a broken configuration is not traversed (see k_sort_gather)
+    extern __shared__ __align__(16) float s_lanes[];
+    __shared__ int s_cnt[OP_TILE];
+    __shared__ long long s_off[OP_TILE];
+    __shared__ long long s_prefix, s_total;
+    __shared__ int s_tile;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) s_tile = atomicAdd(build_word, 1);
+    __syncthreads();
+    const int64_t tile = s_tile, first = tile * OP_TILE + 32 * warp, i = first + lane;
+    float *stage = s_lanes + warp * LN_STAGE;
+    uint16_t *rows = reinterpret_cast<uint16_t *>(s_lanes + LN_WARPS * LN_STAGE) + 32 * warp * ln_row(buf), *row = rows + lane * ln_row(buf);
+    const float edge[3] = {(float)(g.box[0] / g.n[0]), (float)(g.box[1] / g.n[1]), (float)(g.box[2] / g.n[2])};
+    const float rl2_lo = (float)(rl2 * (1.0 - 1e-5)), rl2_hi = (float)(rl2 * (1.0 + 1e-5));
+    constexpr float FAR_AWAY = 1e18f;   // no hit, and no overflow in the squared distance
+
+    // ---- traversal ----
+    const bool live = i < n && user_of[i] < n_owned;   // (a ghost has no list of its own)
+    float4 ri = make_float4(0.f, 0.f, 0.f, 0.f);
+    int cx = 0, cy = 0, cz = 0;
+    if (live) {
+        const double4 p = pos4[i];
+        ri = rel[i];
+        cx = cell_coord(p.x, g.inv_edge[0], g.n[0]); cy = cell_coord(p.y, g.inv_edge[1], g.n[1]); cz = cell_coord(p.z, g.inv_edge[2], g.n[2]);
+    }
+    const float rl2_mid = (float)rl2, band = (float)(rl2 * 1.1e-5);
+    // shared-memory addresses of the places for the next near and the next far hit; once they have crossed nothing is stored, only counted
+    const int row_at = (int)__cvta_generic_to_shared(row), row_end = row_at + 2 * (buf - 1);
+    int near_at = row_at, far_at = row_end;
+    for (unsigned left = __ballot_sync(0xffffffffu, live); left;) {   // groups of lanes with cells along one column
+        const int lead = __ffs(left) - 1;
+        const int X = __shfl_sync(0xffffffffu, cx, lead), Y = __shfl_sync(0xffffffffu, cy, lead), Z = __shfl_sync(0xffffffffu, cz, lead);
+        const bool mine = (left >> lane & 1u) && cx == X && cy == Y && cz - Z < LN_SPAN;   // (atoms come in cell order: cz >= Z)
+        const unsigned group = __ballot_sync(0xffffffffu, mine);
+        left &= ~group;
+        const int layers = __shfl_sync(0xffffffffu, cz, 31 - __clz(group)) - Z + 3, per_column = 65536 / layers + 1;
+        // atom range of the q-th cell of the walk (columns in x, y order, layers Z - 1 .. upwards)
+        auto range = [&](int q, int &b, int &e) {
+            b = e = 0;
+            if (q >= 9 * layers) return;
+            const int col = q * per_column >> 16;
+            int x = X + col / 3 - 1, y = Y + col % 3 - 1, z = Z + (q - col * layers) - 1;
+            x = x < 0 ? x + g.n[0] : (x >= g.n[0] ? x - g.n[0] : x);
+            y = y < 0 ? y + g.n[1] : (y >= g.n[1] ? y - g.n[1] : y);
+            z = z < 0 ? z + g.n[2] : (z >= g.n[2] ? z - g.n[2] : z);
+            const int c = (x * g.n[1] + y) * g.n[2] + z;
+            b = cell_start[c]; e = cell_start[c + 1];
+        };
+        int beg0, end0, beg1, end1;
+        range(lane, beg0, end0);
+        range(lane + 32, beg1, end1);
+        unsigned long long cells = __ballot_sync(0xffffffffu, end0 > beg0) | (unsigned long long)__ballot_sync(0xffffffffu, end1 > beg1) << 32;
+        int q = 0, cell_beg = 0, base = 0, end = 0;   // the chunk being fetched: atoms base .. of cell q
+        auto advance = [&]() {
+            base += 32;
+            if (base < end) return true;
+            if (!cells) return false;
+            q = __ffsll(cells) - 1;
+            cells &= cells - 1;
+            cell_beg = base = __shfl_sync(0xffffffffu, q < 32 ? beg0 : beg1, q & 31);
+            end = __shfl_sync(0xffffffffu, q < 32 ? end0 : end1, q & 31);
+            return true;
+        };
+        const float4 nobody = make_float4(FAR_AWAY, FAR_AWAY, FAR_AWAY, 0.f);
+        bool more = advance();
+        float4 r = more && base + lane < end ? rel[base + lane] : nobody;
+        for (int parity = 0; more; parity ^= 1) {
+            const int col = q * per_column >> 16, dz = Z + (q - col * layers) - 1 - cz, chunk = base, pos = base - cell_beg, m = min(32, end - base);
+            float *st = stage + parity * (LN_STAGE / 2);
+            st[lane] = r.x; st[32 + lane] = r.y; st[64 + lane] = r.z;
+            more = advance();
+            if (more) r = base + lane < end ? rel[base + lane] : nobody;
+            // separation = x_rel(j) + shift, shift = (cell offset) * edge - x_rel(i)
+            const bool in = mine && dz >= -1 && dz <= 1;
+            const float sx = in ? (float)(col / 3 - 1) * edge[0] - ri.x : FAR_AWAY;
+            const float sy = (float)(col % 3 - 1) * edge[1] - ri.y;
+            const float sz = (float)dz * edge[2] - ri.z;
+            const int code = ((3 * col + dz + 1) << L16_SHIFT) + pos;
+            const int self = dz == 0 ? code + (int)(i - chunk) : -1;   // (the central column) the lane's own atom
+            __syncwarp();   // (the buffer before last was read before the last one's barrier)
+            // the hit's code (%5) to the near (%0) or far (%1) place, which moves on; predicate h: hit
+#define MLIP_APPEND " setp.lt.and.f32 nr, %2, %4, h; setp.ge.and.f32 fr, %2, %4, h; selp.u32 at, %0, %1, nr;" \
+                    " @h st.shared.u16 [at], %5; @nr add.s32 %0, %0, 2; @fr sub.s32 %1, %1, 2;}"
+            auto test = [&](auto own_column) {
+                constexpr bool OWN = decltype(own_column)::value;
+                for (int c0 = 0; c0 < m; c0 += 8) {   // (a chunk's places behind its last candidate are out of reach)
+                    float2 d2[4];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float4 x = *reinterpret_cast<const float4 *>(st + c0 + 4 * h), y = *reinterpret_cast<const float4 *>(st + 32 + c0 + 4 * h),
+                                     z = *reinterpret_cast<const float4 *>(st + 64 + c0 + 4 * h);
+                        d2[2 * h] = pack_norm2(pack_add(make_float2(x.x, x.y), sx), pack_add(make_float2(y.x, y.y), sy), pack_add(make_float2(z.x, z.y), sz));
+                        d2[2 * h + 1] = pack_norm2(pack_add(make_float2(x.z, x.w), sx), pack_add(make_float2(y.z, y.w), sy), pack_add(make_float2(z.z, z.w), sz));
+                    }
+                    float closest = 3.0e38f;   // to the list radius
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 off = pack_add(d2[e], -rl2_mid);
+                        closest = fminf(closest, fminf(fabsf(off.x), fabsf(off.y)));
+                    }
+                    if (__any_sync(0xffffffffu, closest <= band || far_at - near_at < 2 * 7)) {
+                        // a candidate within 1e-5 of the list radius, where the exact predicate on the full positions decides, or a row
+                        // that may end among the eight
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const float v = e & 1 ? d2[e >> 1].y : d2[e >> 1].x;
+                            bool hit = v <= rl2_hi && !(OWN && code + c0 + e == self);
+                            if (hit && v >= rl2_lo) {
+                                const double4 pi = pos4[i], pj = pos4[chunk + c0 + e];
+                                const double ex = min_image(__dsub_rn(pj.x, pi.x), g.box[0], g.half[0]);
+                                const double ey = min_image(__dsub_rn(pj.y, pi.y), g.box[1], g.half[1]);
+                                const double ez = min_image(__dsub_rn(pj.z, pi.z), g.box[2], g.half[2]);
+                                hit = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez)) < rl2;
+                            }
+                            if (hit) {
+                                const bool near = v < near2;
+                                if (near_at <= far_at) asm volatile("st.shared.u16 [%0], %1;" ::"r"(near ? near_at : far_at), "r"(code + c0 + e));
+                                if (near) near_at += 2; else far_at -= 2;
+                            }
+                        }
+                    } else {   // no branches: few lanes have a hit, and a divergent branch costs more than the instructions it skips
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const float v = e & 1 ? d2[e >> 1].y : d2[e >> 1].x;
+                            if (OWN) asm volatile("{.reg .pred h, nr, fr; .reg .u32 at; setp.ne.s32 h, %5, %6; setp.le.and.f32 h, %2, %3, h;" MLIP_APPEND
+                                                  : "+r"(near_at), "+r"(far_at) : "f"(v), "f"(rl2_hi), "f"(near2), "r"(code + c0 + e), "r"(self));
+                            else asm volatile("{.reg .pred h, nr, fr; .reg .u32 at; setp.le.f32 h, %2, %3;" MLIP_APPEND
+                                              : "+r"(near_at), "+r"(far_at) : "f"(v), "f"(rl2_hi), "f"(near2), "r"(code + c0 + e));
+                        }
+                    }
+                }
+            };
+#undef MLIP_APPEND
+            if (col == 4) test(std::true_type{});
+            else test(std::false_type{});
+        }
+        __syncwarp();   // (the next group's first chunk may go where a lane still reads)
+    }
+    const int cn = (near_at - row_at) >> 1, cnt = cn + ((row_end - far_at) >> 1);   // near hits, hits
+    s_cnt[32 * warp + lane] = cnt;
+    __syncthreads();
+    if (warp == 0) tile_offsets<OP_TILE>(tile, s_cnt, s_off, &s_prefix, &s_total, status, tile_state, spin_limit, unpublished_tile, lane);
+    __syncthreads();
+    if (tile * OP_TILE + OP_TILE >= n && threadIdx.x == 0) {   // the last tile closes the offsets
+        nbr_off[n] = s_total < nbr_cap ? s_total : nbr_cap;
+        *reinterpret_cast<long long *>(build_word + 2) = s_total;   // for the host: {ticket, overflow, total}
+    }
+
+    // ---- write the lists: full rows from shared memory ----
+    const long long off = s_prefix + s_off[32 * warp + lane];
+    int fit = cnt;   // entries of this list that the array still holds
+    if (i < n) {
+        if (off + cnt > nbr_cap) {
+            atomicOr(status, FLAG_NEIGHBOR_OVERFLOW);
+            fit = off < nbr_cap ? (int)(nbr_cap - off) : 0;
+        }
+        nbr_off[i] = off < nbr_cap ? off : nbr_cap;
+        nbr_near[i] = cn < fit ? cn : fit;
+    }
+    int cell_of_bases = -1, bases = 0;   // lane q < 27: first atom of the q-th cell around that cell
+    for (int a = 0; a < 32; ++a) {
+        const int m = __shfl_sync(0xffffffffu, fit, a), all = __shfl_sync(0xffffffffu, cnt, a), near = __shfl_sync(0xffffffffu, cn, a);
+        if (m == 0) continue;   // (atoms beyond the last and ghosts have none either)
+        const long long to = __shfl_sync(0xffffffffu, off, a);
+        if (all > buf) {
+            int ignored;
+            onepass_traverse<true, ENTRY, ENTRY>(first + a, g, rl2, edge, rl2_lo, rl2_hi, pos4, rel, cell_start, lane, nbr + to, all - 1, m, near2, ignored);
+            continue;
+        }
+        if (sizeof(ENTRY) == 4) {
+            const int X = __shfl_sync(0xffffffffu, cx, a), Y = __shfl_sync(0xffffffffu, cy, a), Z = __shfl_sync(0xffffffffu, cz, a);
+            const int cell = (X * g.n[1] + Y) * g.n[2] + Z;
+            if (cell != cell_of_bases) {
+                cell_of_bases = cell;
+                if (lane < 27) {
+                    int x = X + lane / 9 - 1, y = Y + (lane / 3) % 3 - 1, z = Z + lane % 3 - 1;
+                    x = x < 0 ? x + g.n[0] : (x >= g.n[0] ? x - g.n[0] : x);
+                    y = y < 0 ? y + g.n[1] : (y >= g.n[1] ? y - g.n[1] : y);
+                    z = z < 0 ? z + g.n[2] : (z >= g.n[2] ? z - g.n[2] : z);
+                    bases = cell_start[(x * g.n[1] + y) * g.n[2] + z];
+                }
+            }
+        }
+        const uint16_t *src = rows + a * ln_row(buf);
+        for (int e0 = 0; e0 < m; e0 += 32) {
+            const int e = e0 + lane, code = e < m ? src[e < near ? e : e + (buf - all)] : 0;
+            int entry = code;
+            if (sizeof(ENTRY) == 4) entry = __shfl_sync(0xffffffffu, bases, code >> L16_SHIFT) + (code & L16_MASK);
+            if (e < m) nbr[to + e] = (ENTRY)entry;
         }
     }
 }
@@ -851,9 +1096,11 @@ static int refuse_broken_input(mlip_ctx *c, cudaStream_t s) {
 int64_t tile_words(int64_t n) { return std::max(n / OP_TILE, std::min(n, ONEPASS_SMALL) / 8) + 2; }
 
 // Atoms per warp of the one-pass traversal (tiles of eight warps): one in small systems, where eight traversals one after the other
-// are the kernel's time, eight once such tiles fill the SMs two waves deep (five CTAs each) and fewer tiles are the better choice.  Whole
-// build on the device in us with 1 / 8, 6 species: 864 atoms 65 / 126, 6,912 88 / 136, 16,384 132 / 148, 32,000 202 / 198, 55,296 299 /
-// 337, 87,808 453 / 477, 131,072 643 / 621, 1,048,576 4842 / 4030; one species: 4,394 66 / 116, 65,536 301 / 272.
+// are the kernel's time; from there on tiles of 64 atoms, eight to a warp or (grids of three cells per dimension and more, k_neighbors_lanes) one to
+// a lane.  Whole build on the device in us, one atom to a warp / to a lane: 6 species 6,912 atoms 80 / 126, 10,976 101 / 129, 16,384 125 / 128, 32,000
+// 186 / 140; one species 8,192 81 / 113, 16,000 115 / 114, 31,250 164 / 125; three 32,768 176 / 118.  Eight atoms to a warp / one to a lane:
+// 6 species 55,296 atoms 317 / 162, 108,000 468 / 271, 1,000,188 2801 / 1379, 8,001,504 21,470 / 9874; three 1,953,125 5406 / 1911; one 65,536
+// 252 / 140.
 static int onepass_per_warp(const mlip_ctx *c) {
     if (c->lookback_unpublished_tile >= 0 || c->lookback_spin_limit > 0) return 8;   // (diagnostics name 64-atom tiles)
     return c->n < ONEPASS_SMALL ? 1 : 8;
@@ -867,6 +1114,24 @@ static void launch_onepass(mlip_ctx *c, ENTRY *nbr, int *flag, double rl, float 
         c->n, c->grid, rl * rl, c->pos4, c->rel_pos, c->cell_start, c->nbr_off, nbr, c->nbr_cap, flag, c->tile_state, c->build_word, c->status, spin,
         c->lookback_unpublished_tile, near2, c->nbr_near, c->user_of, (int32_t)c->n_owned);
     c->launches += 1;
+}
+
+// Row of a lane: the mean list at the system's density and 30 percent (lattice shells, composition), in entries.  Longer lists are traversed again.
+static int lanes_row(const mlip_ctx *c, double rl) {
+    const double volume = c->grid.box[0] * c->grid.box[1] * c->grid.box[2], mean = (double)c->n / volume * (4.0 / 3.0 * 3.14159265358979 * rl * rl * rl);
+    return std::min(std::max((int)(1.3 * mean) + 16, 64), 640) / 4 * 4;
+}
+
+template <typename ENTRY>
+static int launch_lanes(mlip_ctx *c, ENTRY *nbr, int *flag, double rl, float near2, cudaStream_t s) {
+    const int spin = c->lookback_spin_limit > 0 ? c->lookback_spin_limit : OP_SPIN, buf = lanes_row(c, rl);
+    const size_t smem = ln_smem(buf);
+    if (smem > 40000) MLIP_CUDA_TRY(c, cudaFuncSetAttribute(k_neighbors_lanes<ENTRY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ln_smem(640)));
+    k_neighbors_lanes<ENTRY><<<(unsigned)((c->n + OP_TILE - 1) / OP_TILE), LN_THREADS, smem, s>>>(
+        c->n, c->grid, rl * rl, c->pos4, c->rel_pos, c->cell_start, c->nbr_off, nbr, c->nbr_cap, flag, c->tile_state, c->build_word, c->status, spin,
+        c->lookback_unpublished_tile, near2, c->nbr_near, c->user_of, (int32_t)c->n_owned, buf);
+    c->launches += 1;
+    return MLIP_OK;
 }
 
 // Sort the source set into cell order and build the lists.  The source is (pos4_src, vel_src, user_src), filled from the caller's
@@ -931,9 +1196,12 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
     // bit), and for a synchronising build as a first try whose overflow flag is private and sends it to the two-pass path.
     if (c->nbr_cap > 0) {
         int *flag = allow_sync_grow ? c->build_word + 1 : c->status;
-        if (list16) per_warp == 1 ? launch_onepass<true, 1, uint16_t>(c, nbr16, flag, rl, near2, s) : launch_onepass<true, 8, uint16_t>(c, nbr16, flag, rl, near2, s);
-        else if (rel) per_warp == 1 ? launch_onepass<true, 1, int32_t>(c, c->nbr, flag, rl, near2, s) : launch_onepass<true, 8, int32_t>(c, c->nbr, flag, rl, near2, s);
+        int rc = MLIP_OK;
+        if (rel && per_warp == 8) rc = list16 ? launch_lanes(c, nbr16, flag, rl, near2, s) : launch_lanes(c, c->nbr, flag, rl, near2, s);
+        else if (list16) launch_onepass<true, 1, uint16_t>(c, nbr16, flag, rl, near2, s);
+        else if (rel) launch_onepass<true, 1, int32_t>(c, c->nbr, flag, rl, near2, s);
         else per_warp == 1 ? launch_onepass<false, 1, int32_t>(c, c->nbr, flag, rl, near2, s) : launch_onepass<false, 8, int32_t>(c, c->nbr, flag, rl, near2, s);
+        if (rc != MLIP_OK) return rc;
         MLIP_CUDA_TRY(c, cudaGetLastError());
         bool done = true;
         if (allow_sync_grow) {
