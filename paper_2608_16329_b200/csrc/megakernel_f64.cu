@@ -211,8 +211,7 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
 
         // ---------------- Encoding: P = H^T G (Eq. 4) ----------------
         // Four pairs per m8n8k4 step on the fp64 tensor pipe.  A = H^T (rows = angular components, k = pair), B = G
-        // (k = pair, columns = channels): lane (g, t) evaluates g of pair t at channels 16 q + 2 g, + 1 (q < K / 16), so the
-        // eight lanes of a pair read 128 contiguous bytes of a table row per load and four rows are in flight per step; the
+        // (k = pair, columns = channels): column g of n-tile nt is channel 16 (nt / 2) + 2 g + nt % 2; the
         // accumulators go through shared memory to lane = channel afterwards.
         auto keep_pair = [&](int slot, int j, double dx, double dy, double dz, double rinv, int sj) {
             sm.qd[wid][0][slot] = dx; sm.qd[wid][1][slot] = dy; sm.qd[wid][2][slot] = dz;
@@ -269,23 +268,32 @@ __global__ void __launch_bounds__(F64_TILE * 32, f64_ctas_per_sm<K, LMAX, BASIS>
                 n_mine += nv;
                 __syncwarp();
                 pc.mark(0);
+                // lane 8 q + c evaluates g of the step's pair q at channels 16 v + 2 c, + 1: a load goes through L1 eight lanes at a time, and
+                // those eight then read one 128-byte line.  (Evaluated where the B operand wants them -- lanes 4 c + q -- the eight lanes touch
+                // four lines for a quarter of each: 32 wavefronts per pair instead of 8 + 2 for the shuffles, the kernel's busiest unit.  55,296
+                // atoms 1573 -> 1357 us, k = 64 at 6,912 384 -> 316, k = 16 1000 -> 911.)
+                const int pair_of = lane >> 3, chunk = lane & 7;
+#pragma unroll 1
                 for (int p0 = 0; p0 < nv; p0 += 4) {
-                    const int p = p0 + t;
-                    const bool live = p < nv;   // a step past the last pair contracts zeros against the table's first rows
-                    const double *cf = k.coef + (live ? __double_as_longlong(offs[p]) : 0ll) + 2 * g;
+                    const int ps = p0 + pair_of, p = p0 + t;   // a step past the last pair contracts zeros against the table's first rows
+                    const bool live_s = ps < nv, live = p < nv;
+                    const double *cf = k.coef + (live_s ? __double_as_longlong(offs[ps]) : 0ll) + 2 * chunk;
                     double gq[NTK];
 #pragma unroll
                     for (int nt = 0; nt < NTK; ++nt) gq[nt] = 0.0;
 #pragma unroll
                     for (int m = 0; m < 4; ++m) {
-                        const double bm = live ? bq[m * PS + p] : 0.0;
+                        const double bm = live_s ? bq[m * PS + ps] : 0.0;
                         double cc[NTK];
 #pragma unroll
-                        for (int v = 0; v < NTK; v += 2)   // 16 bytes per lane: the eight lanes of a pair read 128 contiguous bytes
+                        for (int v = 0; v < NTK; v += 2)   // 16 bytes per lane: eight lanes, a phase of the load, read 128 contiguous bytes
                             asm volatile("ld.global.nc.v2.f64 {%0,%1}, [%2];" : "=d"(cc[v]), "=d"(cc[v + 1]) : "l"(cf + m * K + 8 * v));
 #pragma unroll
                         for (int nt = 0; nt < NTK; ++nt) gq[nt] = fma(bm, cc[nt], gq[nt]);
                     }
+                    // to the B operand: lane (g, t) takes chunk g of pair t
+#pragma unroll
+                    for (int nt = 0; nt < NTK; ++nt) gq[nt] = __shfl_sync(0xffffffffu, gq[nt], 8 * t + g);
 #pragma unroll
                     for (int mt = 0; mt < MT; ++mt) {
                         const double av = (live && 8 * mt + g < D) ? hs[(8 * mt + g) * PS + p] : 0.0;
