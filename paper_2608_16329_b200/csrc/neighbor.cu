@@ -973,29 +973,38 @@ struct ListView {
     }
 };
 
-// An atom's place in every canonical list: species, then caller index, in one word (8 species, 2^28 atoms).
-__global__ void k_export_keys(int64_t n, const double4 *__restrict__ pos4, const int32_t *__restrict__ user_of, int32_t *__restrict__ key) {
+// An atom's place in every canonical list: species, then caller index, in one word (8 species, 2^28 atoms); the lengths of the
+// lists in the caller's order.
+__global__ void k_export_keys(int64_t n, const double4 *__restrict__ pos4, const int32_t *__restrict__ user_of, const int64_t *__restrict__ nbr_off,
+                              int32_t *__restrict__ key, int32_t *__restrict__ len) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) key[i] = ((int)pos4[i].w << 28) | user_of[i];
+    if (i >= n) return;
+    const int user = user_of[i];
+    key[i] = ((int)pos4[i].w << 28) | user;
+    len[user] = (int)(nbr_off[i + 1] - nbr_off[i]);
 }
 
-// Warp per atom: entries per species.  Each lane counts in 16-bit fields (a list holds at most 27 x MAX_CELL_ATOMS entries).
-__global__ void __launch_bounds__(256) k_export_count(int64_t n, int n_species, const int64_t *__restrict__ nbr_off, ListView lv,
-                                                      const int32_t *__restrict__ key, int32_t *__restrict__ seg_count) {
+// Warp per atom: entries per species, one count to a lane.  Each lane counts in 16-bit fields (a list holds at most 27 x MAX_CELL_ATOMS entries).
+__device__ __forceinline__ int species_counts(const ListView &lv, const int32_t *__restrict__ key, int64_t i, int64_t beg, int64_t end, int lane) {
     static_assert(27 * MAX_CELL_ATOMS < 65536 && MAX_SPECIES == 8, "16-bit fields, two to a word");
-    const int lane = threadIdx.x & 31;
-    int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (i >= n) return;
     unsigned cnt[4] = {0, 0, 0, 0};
-    for (int64_t e = nbr_off[i] + lane; e < nbr_off[i + 1]; e += 32) {
+    for (int64_t e = beg + lane; e < end; e += 32) {
         const int s = (int)((unsigned)key[lv.at(i, e)] >> 28);
 #pragma unroll
         for (int w = 0; w < 4; ++w) cnt[w] += (s >> 1) == w ? 1u << (16 * (s & 1)) : 0u;
     }
-    const int64_t row = (int64_t)MLIP_CHECK_INDEX(key[i] & 0x0fffffff, n, lv.status) * n_species;
 #pragma unroll
     for (int w = 0; w < 4; ++w) cnt[w] = __reduce_add_sync(0xffffffffu, cnt[w]);
-    if (lane < n_species) seg_count[row + lane] = (int)((((lane >> 1) == 0 ? cnt[0] : (lane >> 1) == 1 ? cnt[1] : (lane >> 1) == 2 ? cnt[2] : cnt[3]) >> (16 * (lane & 1))) & 0xffffu);
+    return (int)((((lane >> 1) == 0 ? cnt[0] : (lane >> 1) == 1 ? cnt[1] : (lane >> 1) == 2 ? cnt[2] : cnt[3]) >> (16 * (lane & 1))) & 0xffffu);
+}
+// Segment lengths without the lists (a call whose array is too small reports those): the fill kernel finds the segments itself.
+__global__ void __launch_bounds__(256) k_export_count(int64_t n, int n_species, const int64_t *__restrict__ nbr_off, ListView lv,
+                                                      const int32_t *__restrict__ key, int32_t *__restrict__ seg_count) {
+    const int lane = threadIdx.x & 31;
+    int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= n) return;
+    const int count = species_counts(lv, key, i, nbr_off[i], nbr_off[i + 1], lane);
+    if (lane < n_species) seg_count[(int64_t)MLIP_CHECK_INDEX(key[i] & 0x0fffffff, n, lv.status) * n_species + lane] = count;
 }
 
 // Sort of 32 x R keys by a warp, ascending in lane * R + r: a bitonic network whose phases start with a mirrored step, so that every
@@ -1038,10 +1047,13 @@ __device__ __forceinline__ void warp_sort(int32_t (&v)[R], int lane) {
 // shared memory and written.  Longer lists: an entry's place is the number of smaller keys, read again from global memory.
 // 108,000 atoms with 134 entries each: 2.0 ms when every pair of entries was compared through list, species and caller index, 375 us
 // when keys were ranked against a copy in shared memory (some 2,000 instructions per list), 110 us sorted (about 600).
+// The first segment of an atom starts at seg_ptr[its caller index * n_species], which the scan of the list lengths has written; the
+// others start where the species changes in the sorted keys.  (Counted by a pass of
+// their own, with a scan over all n_species times as many segments: 108,000 atoms 500 instead of 463 us for build and export.)
 constexpr int EXPORT_BUF = 256;
 template <int R>
-__device__ __forceinline__ void export_sorted(const ListView &lv, const int32_t *__restrict__ key, int64_t i, int64_t beg, int m, int32_t *keys,
-                                              int32_t *__restrict__ out, int lane) {
+__device__ __forceinline__ void export_sorted(const ListView &lv, const int32_t *__restrict__ key, int64_t i, int64_t beg, int m, int32_t *keys, int n_species,
+                                              int64_t off, int64_t *__restrict__ seg, int32_t *__restrict__ out, int lane) {
     int32_t v[R];
 #pragma unroll
     for (int c = 0; c < R; ++c) v[c] = 32 * c + lane < m ? key[lv.at(i, beg + 32 * c + lane)] : 0x7fffffff;
@@ -1050,11 +1062,21 @@ __device__ __forceinline__ void export_sorted(const ListView &lv, const int32_t 
     for (int c = 0; c < R; c += 4) *reinterpret_cast<int4 *>(keys + lane * R + c) = make_int4(v[c], v[c + 1], v[c + 2], v[c + 3]);
     __syncwarp();
 #pragma unroll
-    for (int c = 0; c < R; ++c)
-        if (32 * c + lane < m) out[32 * c + lane] = keys[32 * c + lane] & 0x0fffffff;
+    for (int c = 0; c < R; ++c) {
+        const int e = 32 * c + lane;
+        if (e < m) out[e] = keys[e] & 0x0fffffff;
+    }
+    if (lane > 0 && lane < n_species) {   // lane q: the entries of species below q
+        int below = 0;
+#pragma unroll
+        for (int step = 16 * R; step; step >>= 1)
+            if (keys[below + step - 1] < lane << 28) below += step;
+        if (keys[below] < lane << 28) ++below;
+        seg[lane] = off + below;
+    }
 }
 __global__ void __launch_bounds__(256) k_export_fill(int64_t n, int n_species, const int64_t *__restrict__ nbr_off, ListView lv,
-                                                     const int32_t *__restrict__ key, const int64_t *__restrict__ seg_ptr, int32_t *__restrict__ out) {
+                                                     const int32_t *__restrict__ key, int64_t *__restrict__ seg_ptr, int32_t *__restrict__ out) {
     __shared__ __align__(16) int32_t s_keys[8][EXPORT_BUF];
     const int lane = threadIdx.x & 31;
     int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1062,9 +1084,15 @@ __global__ void __launch_bounds__(256) k_export_fill(int64_t n, int n_species, c
     int32_t *keys = s_keys[threadIdx.x >> 5];
     const int64_t beg = nbr_off[i];
     const int m = (int)(nbr_off[i + 1] - beg);
-    out += seg_ptr[(int64_t)MLIP_CHECK_INDEX(key[i] & 0x0fffffff, n, lv.status) * n_species];   // the species' segments of an atom follow one another
-    if (m <= EXPORT_BUF / 2) return export_sorted<4>(lv, key, i, beg, m, keys, out, lane);
-    if (m <= EXPORT_BUF) return export_sorted<8>(lv, key, i, beg, m, keys, out, lane);
+    int64_t *seg = seg_ptr + (int64_t)MLIP_CHECK_INDEX(key[i] & 0x0fffffff, n, lv.status) * n_species;   // the species' segments of an atom follow one another
+    const int64_t off = *seg;
+    out += off;
+    if (m <= EXPORT_BUF / 2) return export_sorted<4>(lv, key, i, beg, m, keys, n_species, off, seg, out, lane);
+    if (m <= EXPORT_BUF) return export_sorted<8>(lv, key, i, beg, m, keys, n_species, off, seg, out, lane);
+    const int count = species_counts(lv, key, i, beg, beg + m, lane);
+    int before = 0;   // lane q: entries of the species below q
+    for (int q = 0; q + 1 < n_species; ++q) { const int c = __shfl_sync(0xffffffffu, count, q); before += lane > q ? c : 0; }
+    if (lane > 0 && lane < n_species) seg[lane] = off + before;
     for (int e = lane; e < m; e += 32) {
         const int32_t mine = key[lv.at(i, beg + e)];
         int rank = 0;
@@ -1254,34 +1282,39 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
     return MLIP_OK;
 }
 
-// The lists cannot be exported while the status word says that the last in-step rebuild did not complete them.
+// The lists cannot be exported while the status word says that the last in-step rebuild did not complete them.  Leaves the number of
+// entries in total_host.
 static int lists_whole(mlip_ctx *c, cudaStream_t s) {
     MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->status_host, c->status, sizeof(int), cudaMemcpyDeviceToHost, s));
+    MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->total_host, c->nbr_off + c->n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
     if (*c->status_host & FLAG_NONFINITE) { c->err = "neighbor export: the configuration is broken (see mlip_sync_status)"; return MLIP_ERR_NONFINITE; }
     if (*c->status_host & FLAG_NEIGHBOR_OVERFLOW) { c->err = "neighbor export: the last rebuild overflowed the list (see mlip_sync_status)"; return MLIP_ERR_NEIGHBOR_OVERFLOW; }
     return MLIP_OK;
 }
 
-// Keys, counts, scan; then, if the caller's array holds them, the lists.  `seg_count` [n * C] and `tmp` (scan_tmp_items(n * C)) are scratch;
+// Keys, scan of the list lengths, lists; if the caller's array cannot hold them, the segments only.  `counts` [n * C] and `tmp` (scan_tmp_items(n * C)) are scratch;
 // the keys go to cell_of, which is read during list builds only.
-static int export_lists(mlip_ctx *c, int64_t *seg_ptr, int32_t *nbr, int64_t capacity, int64_t *n_entries_host, int32_t *seg_count, int64_t *tmp, cudaStream_t s) {
+static int export_lists(mlip_ctx *c, int64_t *seg_ptr, int32_t *nbr, int64_t capacity, int64_t *n_entries_host, int32_t *counts, int64_t *tmp, cudaStream_t s) {
     const int64_t n = c->n;
     const int C = c->cfg.n_species;
-    k_export_keys<<<blocks_for(n, 256), 256, 0, s>>>(n, c->pos4, c->user_of, c->cell_of);
-    k_export_count<<<blocks_for(n * 32, 256), 256, 0, s>>>(n, C, c->nbr_off, list_view(c), c->cell_of, seg_count);
-    c->launches += 2 + exclusive_scan<int32_t, int64_t>(seg_count, seg_ptr, n * C, tmp, s);
-    MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->total_host, seg_ptr + n * C, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
     if (n_entries_host) *n_entries_host = *c->total_host;
-    if (*c->total_host > capacity || !nbr) {
+    const bool room = nbr && *c->total_host <= capacity;
+    k_export_keys<<<blocks_for(n, 256), 256, 0, s>>>(n, c->pos4, c->user_of, c->nbr_off, c->cell_of, counts);
+    c->launches += 2;
+    if (room) {
+        c->launches += exclusive_scan<int32_t, int64_t>(counts, seg_ptr, n, tmp, s, C);
+        k_export_fill<<<blocks_for(n * 32, 256), 256, 0, s>>>(n, C, c->nbr_off, list_view(c), c->cell_of, seg_ptr, nbr);
+    } else {
+        k_export_count<<<blocks_for(n * 32, 256), 256, 0, s>>>(n, C, c->nbr_off, list_view(c), c->cell_of, counts);
+        c->launches += exclusive_scan<int32_t, int64_t>(counts, seg_ptr, n * C, tmp, s);
+    }
+    MLIP_CUDA_TRY(c, cudaGetLastError());
+    MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
+    if (!room) {
         c->err = "neighbor export: capacity too small";
         return MLIP_ERR_NEIGHBOR_OVERFLOW;
     }
-    k_export_fill<<<blocks_for(n * 32, 256), 256, 0, s>>>(n, C, c->nbr_off, list_view(c), c->cell_of, seg_ptr, nbr);
-    c->launches += 1;
-    MLIP_CUDA_TRY(c, cudaGetLastError());
-    MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
     return MLIP_OK;
 }
 

@@ -1,5 +1,5 @@
 // Exclusive prefix sums over device arrays (three small kernels: tile sums,
-// scan of the tile sums, rescan with offsets; one block in one kernel for a few tiles).  out has n + 1 entries.
+// scan of the tile sums, rescan with offsets; one block in one kernel for a few tiles).  out has n + 1 entries (n * stride + 1).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -67,7 +67,7 @@ static __global__ void __launch_bounds__(SCAN_THREADS) scan_of_sums(int64_t *sum
 
 template <typename TIn, typename TOut>
 __global__ void __launch_bounds__(SCAN_THREADS) scan_apply(const TIn *__restrict__ in, TOut *__restrict__ out, int64_t n,
-                                                           const int64_t *__restrict__ sums, int64_t nb) {
+                                                           const int64_t *__restrict__ sums, int64_t nb, int stride) {
     __shared__ int64_t ws[33];
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
     int64_t item[SCAN_ITEMS], v = 0;
@@ -80,16 +80,16 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_apply(const TIn *__restrict
     int64_t run = sums[blockIdx.x] + block_exclusive_scan(v, total, ws);
 #pragma unroll
     for (int i = 0; i < SCAN_ITEMS; ++i) {
-        if (base + i < n) out[base + i] = (TOut)run;
+        if (base + i < n) out[(base + i) * stride] = (TOut)run;
         run += item[i];
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = (TOut)sums[nb];
+    if (blockIdx.x == 0 && threadIdx.x == 0) out[n * stride] = (TOut)sums[nb];
 }
 
 // A few tiles by one block: about 2 us each, against three launches.
 constexpr int64_t SCAN_ONE_BLOCK = 4 * SCAN_TILE;
 template <typename TIn, typename TOut>
-__global__ void __launch_bounds__(SCAN_THREADS) scan_one_block(const TIn *__restrict__ in, TOut *__restrict__ out, int64_t n) {
+__global__ void __launch_bounds__(SCAN_THREADS) scan_one_block(const TIn *__restrict__ in, TOut *__restrict__ out, int64_t n, int stride) {
     __shared__ int64_t ws[33];
     int64_t carry = 0;
     for (int64_t tile = 0; tile < n; tile += SCAN_TILE) {
@@ -100,25 +100,25 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_one_block(const TIn *__rest
         int64_t run = carry + block_exclusive_scan(v, total, ws);
 #pragma unroll
         for (int i = 0; i < SCAN_ITEMS; ++i) {
-            if (base + i < n) out[base + i] = (TOut)run;
+            if (base + i < n) out[(base + i) * stride] = (TOut)run;
             run += item[i];
         }
         carry += total;
     }
-    if (threadIdx.x == 0) out[n] = (TOut)carry;
+    if (threadIdx.x == 0) out[n * stride] = (TOut)carry;
 }
 
-// Enqueue an exclusive scan; `tmp` must hold n / SCAN_TILE + 2 int64 values.  Returns the number of kernels launched.
+// Enqueue an exclusive scan (to every stride-th place of `out`); `tmp` must hold n / SCAN_TILE + 2 int64 values.  Returns the number of kernels launched.
 template <typename TIn, typename TOut>
-inline int exclusive_scan(const TIn *in, TOut *out, int64_t n, int64_t *tmp, cudaStream_t s) {
+inline int exclusive_scan(const TIn *in, TOut *out, int64_t n, int64_t *tmp, cudaStream_t s, int stride = 1) {
     if (n <= SCAN_ONE_BLOCK) {
-        scan_one_block<TIn, TOut><<<1, SCAN_THREADS, 0, s>>>(in, out, n);
+        scan_one_block<TIn, TOut><<<1, SCAN_THREADS, 0, s>>>(in, out, n, stride);
         return 1;
     }
     const int64_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
     scan_tile_sums<TIn><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, n, tmp);
     scan_of_sums<<<1, SCAN_THREADS, 0, s>>>(tmp, nb);
-    scan_apply<TIn, TOut><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, out, n, tmp, nb);
+    scan_apply<TIn, TOut><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, out, n, tmp, nb, stride);
     return 3;
 }
 
