@@ -7,7 +7,7 @@
 //   walks through the central species in order; for each it stages that species' radial tables
 //   (one per neighbor species) and head constants in shared memory, then each group takes tiles of
 //   16 (small systems: 8) central atoms of that species from a global counter (each warp encodes and
-//   derives two of them, one after the other) and runs them on its own,
+//   derives two of them, side by side in its pair loops) and runs them on its own,
 //   synchronising only inside the group (named barriers), so that one group's latency-bound head
 //   overlaps the other group's pair loops.
 //   Encoding    The warp scans the atom's list (lane = entry), queues the pairs inside r_cut in
@@ -66,7 +66,7 @@ constexpr int X_STRIDE = 132; // dE/dG per atom
 // collide: 6 instead of 4 wavefronts per pair in the derivation, and a shuffle per value in the encoding.
 static_assert(K_RADIAL == 32, "a table row is eight 16-byte chunks");
 constexpr int SCR_WORDS = 32 * ST_STRIDE + 32 * 4;              // scratch of a warp: hand-over rows, table row addresses
-static_assert(32 * BS_STRIDE <= SCR_WORDS && N_INV <= 32 * ST_STRIDE, "the derivation's hand-over and the invariants must fit the encoding's");
+static_assert(32 * BS_STRIDE <= SCR_WORDS && N_INV <= X_STRIDE, "the derivation's hand-over must fit the encoding's, the invariants the row of dE/dG");
 // Regression buffers of a group.  Activations are kept as B fragments: per 16-input k-step, atom row and quad lane one
 // 16-byte vector {b0 hi, b0 lo, b1 hi, b1 lo} of fp16 pairs (see act_store).
 constexpr int ACT_KSTEP = 32 * 4;                               // words per k-step
@@ -253,35 +253,37 @@ __device__ __forceinline__ float4 table_load(const TableView &tv, uint32_t off) 
     else v = __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(tv.base) + off));
     return v;
 }
+static_assert(table_swizzle(2) == (table_swizzle(0) ^ 4) && table_swizzle(3) == (table_swizzle(1) ^ 4) && table_swizzle(0) == (table_swizzle(2) ^ 4), "see RowOffsets");
 template <bool TAB_SMEM> constexpr int OFF_WORDS = TAB_SMEM ? 2 : 4;
 // Byte addresses of a pair's four rows in the order they are taken, handed from the lane that owns the pair to the lanes that
 // evaluate it: 16-bit shared-memory addresses (the tables come first in shared memory and end below 64 KB) or 32-bit offsets.
 template <bool TAB_SMEM> struct RowOffsets;
 template <> struct RowOffsets<true> {
     uint2 o;
-    // rows first + ((turn + s) & 3), s = 0..3
+    // rows first + ((turn + s) & 3), s = 0..3.  A chunk's position two steps on differs in one bit (table_swizzle(r + 2) is table_swizzle(r) ^ 4):
+    // that bit travels with the addresses, so that a lane keeps the positions of two steps.
     __device__ __forceinline__ void make(const TableView &tv, int first, int turn) {
         const uint32_t order = __funnelshift_r(0x03020100u, 0x03020100u, 8 * turn);   // bytes turn, turn + 1, .. mod 4
         const uint32_t both = (tv.saddr + 128u * first) * 0x10001u;
         o.x = __byte_perm(order, 0, 0x4140) * 128u + both;
-        o.y = __byte_perm(order, 0, 0x4342) * 128u + both;
+        o.y = __byte_perm(order, 0, 0x4342) * 128u + (both ^ 0x400040u);
     }
     __device__ __forceinline__ void store(float *p) const { *reinterpret_cast<uint2 *>(p) = o; }
     __device__ __forceinline__ void load(const float *p) { o = *reinterpret_cast<const uint2 *>(p); }
-    // address of step s's row with the chunk position (a multiple of 16 below 128) put into its free low bits
-    __device__ __forceinline__ uint32_t at(int s, uint32_t chunk) const {
+    // address of step s's row with the chunk position of step s & 1 (a multiple of 16 below 128) in its low bits
+    __device__ __forceinline__ uint32_t at(int s, const uint32_t (&chunk)[2]) const {
         const uint32_t w = s < 2 ? o.x : o.y;
-        return s & 1 ? (w >> 16) | chunk : (w & 0xffffu) | chunk;
+        return (s & 1 ? w >> 16 : w & 0xffffu) ^ chunk[s & 1];
     }
 };
 template <> struct RowOffsets<false> {
     uint4 o;
     __device__ __forceinline__ void make(const TableView &, int first, int turn) {
-        o = make_uint4(128u * (first + (turn & 3)), 128u * (first + ((turn + 1) & 3)), 128u * (first + ((turn + 2) & 3)), 128u * (first + ((turn + 3) & 3)));
+        o = make_uint4(128u * (first + (turn & 3)), 128u * (first + ((turn + 1) & 3)), 128u * (first + ((turn + 2) & 3)) ^ 64u, 128u * (first + ((turn + 3) & 3)) ^ 64u);
     }
     __device__ __forceinline__ void store(float *p) const { *reinterpret_cast<uint4 *>(p) = o; }
     __device__ __forceinline__ void load(const float *p) { o = *reinterpret_cast<const uint4 *>(p); }
-    __device__ __forceinline__ uint32_t at(int s, uint32_t chunk) const { return (s == 0 ? o.x : s == 1 ? o.y : s == 2 ? o.z : o.w) | chunk; }
+    __device__ __forceinline__ uint32_t at(int s, const uint32_t (&chunk)[2]) const { return (s == 0 ? o.x : s == 1 ? o.y : s == 2 ? o.z : o.w) ^ chunk[s & 1]; }
 };
 // b[0..3] -> b[turn], b[turn + 1], .. (mod 4): spline weights in the order the rows are taken
 __device__ __forceinline__ float4 rotate4(const float (&b)[4], int turn) {
@@ -354,116 +356,198 @@ __device__ __forceinline__ int collect_pairs(const KernelArgs &k, const double4 
     return collect_pairs_n<WIDE_CHUNKS, L16>(k, pi, beg, cur, end, pq, cap, lane, sidx, n_pref, cs);
 }
 
-// ---------------- Encoding of one atom: returns the moment as accumulator fragments ----------------
-// `queued` returns the number of pairs left in the queue when the whole list fitted in one round
-// (the derivation then reuses them), or -1.
-template <bool TAB_SMEM, bool L16>
-__device__ __forceinline__ int encode_atom(const KernelArgs &k, const TableView &tv, const double4 &pi, int64_t beg, int64_t end,
-                                           float4 *pq, int cap, float *stage, int lane, float (&Pf)[4][4], int &queued, const int *sidx, int n_pref,
-                                           int cs, PhaseClock &pc) {
-    const int g = lane >> 2, t = lane & 3;
-    float *offs = stage + 32 * ST_STRIDE;
-    // k-step fragments: lane (g, t) evaluates chunk g (channels 4g ..) of pairs 2t, 2t + 1, 2t + 8, 2t + 9 of the k-step.  A pair
-    // in slot p takes its rows in the residue order p / 2, p / 2 + 1, .. (mod 4): the eight lanes of a load phase, two chunks of
-    // four pairs, then fall into eight bank groups.
-    uint32_t chunk[4];
+// The pairs of a warp's two atoms, the second one's from the next multiple of sixteen on: the batches of 32 pairs in which the loops work
+// then run over both (78 + 78 pairs are five of them, not three and three), and the gathers of both atoms are in flight together.  Lists of up
+// to 96 entries each whose indices were prefetched (NextAtoms).  One evaluation in us, one atom after the other / side by side: 1,000,188 atoms
+// of six species 7661 / 7466, 2,000,000 of the ionic solid (42 pairs) 11,367 / 10,726; 58 and 54 pairs, where no batch is saved, 432 / 434 and 1683 / 1687.
+template <bool L16>
+__device__ __forceinline__ void collect_two(const KernelArgs &k, const int *pf, int n_atoms, float4 *pq, int lane, int &n0, int &n1) {
+    constexpr int CH = NARROW_CHUNKS;
+    int jj[2][CH], len[2];
+    double4 pi[2];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) chunk[q] = 16u * (g ^ table_swizzle((t + q) & 3));
-    const uint32_t a_addr = smem_addr(stage) + ((lane & 7) + ((lane >> 4) << 3)) * (ST_STRIDE * 4) + ((lane >> 3) & 1) * 16;
+    for (int u = 0; u < 2; ++u) {
+        const int *sidx = pf + u * PF_WORDS;
+        len[u] = u < n_atoms ? sidx[PF_IDX + 3] : 0;
+        const int odd = sidx[PF_IDX + 1] & 1;   // of the list's start (see stage_c)
+        pi[u] = load_pos4(k.pos4 + (u < n_atoms ? sidx[PF_IDX] : 0));
+        const int cs = L16 && lane < 27 ? sidx[PF_CS + lane] : 0;
+#pragma unroll
+        for (int c = 0; c < CH; ++c) {
+            const int e = 32 * c + lane;
+            if (L16) {
+                const int code = e < len[u] ? reinterpret_cast<const uint16_t *>(sidx)[e + odd] : 0;
+                const int base = __shfl_sync(0xffffffffu, cs, code >> L16_SHIFT);
+                jj[u][c] = e < len[u] ? base + (code & L16_MASK) : -1;
+            } else {
+                jj[u][c] = e < len[u] ? sidx[e] : -1;
+            }
+            if (jj[u][c] >= 0) jj[u][c] = (int)MLIP_CHECK_INDEX(jj[u][c], k.n, k.status);
+        }
+    }
+    double4 pp[2][CH];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int c = 0; c < CH; ++c) pp[u][c] = load_pos4(k.pos4 + (jj[u][c] < 0 ? 0 : jj[u][c]));
+    int at = 0;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int first = at;
+#pragma unroll
+        for (int c = 0; c < CH; ++c) {
+            if (32 * c >= len[u]) continue;   // warp-uniform: nothing in this chunk
+            const double dx = min_image(pp[u][c].x - pi[u].x, k.grid.box[0], k.grid.half[0]);
+            const double dy = min_image(pp[u][c].y - pi[u].y, k.grid.box[1], k.grid.half[1]);
+            const double dz = min_image(pp[u][c].z - pi[u].z, k.grid.box[2], k.grid.half[2]);
+            const double d2 = dx * dx + dy * dy + dz * dz;
+            const bool valid = jj[u][c] >= 0 && d2 < k.rc2;
+            const unsigned m = __ballot_sync(0xffffffffu, valid);
+            if (valid)
+                pq[at + __popc(m & ((1u << lane) - 1u))] =
+                    make_float4((float)dx, (float)dy, (float)dz, __int_as_float(jj[u][c] | ((int)pp[u][c].w << J_BITS)));
+            at += __popc(m);
+        }
+        if (u == 0) { n0 = at; at = (at + 15) & ~15; }
+        else n1 = at - first;
+    }
+    __syncwarp();
+}
+static_assert(2 * NARROW_CHUNKS * 32 <= Layout<2>::POOL, "two short lists fit the queue");
+
+// ---------------- Encoding ----------------
+// A lane's place in the encoding's k-steps: lane (g, t) evaluates chunk g (channels 4g ..) of pairs 2t, 2t + 1, 2t + 8, 2t + 9 of the
+// k-step.  A pair in slot p takes its rows in the residue order p / 2, p / 2 + 1, .. (mod 4): the eight lanes of a load phase, two
+// chunks of four pairs, then fall into eight bank groups.
+struct EncodeLane {
+    uint32_t chunk[2], a_addr;
+    __device__ __forceinline__ EncodeLane(const float *stage, int lane) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) chunk[q] = 16u * ((lane >> 2) ^ table_swizzle(((lane & 3) + q) & 3));
+        a_addr = smem_addr(stage) + ((lane & 7) + ((lane >> 4) << 3)) * (ST_STRIDE * 4) + ((lane >> 3) & 1) * 16;
+    }
+};
+// Lane = pair: harmonics (Eq. 3) and spline basis of queue entry `slot` into the hand-over rows; zeros where there is no pair.
+template <bool TAB_SMEM>
+__device__ __forceinline__ void encode_rows(const KernelArgs &k, const TableView &tv, const float4 *pq, int slot, bool live, float *stage, int lane) {
+    float h[D_ANG], b[4];
+    int row = 0;
+    if (live) {
+        const float4 e = pq[slot];
+        const float d2 = e.x * e.x + e.y * e.y + e.z * e.z, rinv = rsqrtf(d2), r = d2 * rinv;
+        harmonics(e.x * rinv, e.y * rinv, e.z * rinv, h);
+        float u;
+        const int iv = spline_interval(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, u, k.status);
+        cubic_basis(u, b);
+        row = (__float_as_int(e.w) >> J_BITS) * (k.tab.knots + 3) + iv;
+    } else {
+#pragma unroll
+        for (int a = 0; a < D_ANG; ++a) h[a] = 0.f;
+        b[0] = b[1] = b[2] = b[3] = 0.f;
+    }
+    uint32_t hi[8], lo[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) split_h2(h[2 * q], h[2 * q + 1], hi[q], lo[q]);
+    uint4 *dst = reinterpret_cast<uint4 *>(stage + lane * ST_STRIDE);
+    dst[0] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    dst[1] = make_uint4(hi[4], hi[5], hi[6], hi[7]);
+    dst[2] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    dst[3] = make_uint4(lo[4], lo[5], lo[6], lo[7]);
+    const int turn = ((lane >> 1) - row) & 3;
+    *reinterpret_cast<float4 *>(dst + 4) = rotate4(b, turn);
+    RowOffsets<TAB_SMEM> ro;
+    ro.make(tv, row, turn);
+    ro.store(stage + 32 * ST_STRIDE + lane * OFF_WORDS<TAB_SMEM>);
+}
+// Eq. 4 for the sixteen pairs of hand-over rows 16 ks .. (HALF: none behind the eighth, whose radial functions are not evaluated; with the
+// derivation's half tiles and the sums over lanes by halves: 256,000 atoms of 54 pairs 1687 -> 1627 us an evaluation, the ionic solid 10,726 -> 10,362,
+// six species 7466 -> 7458.  With one atom per warp the second form of the code cost 864 atoms 27 -> 29 us: not there.)
+template <bool TAB_SMEM, bool HALF>
+__device__ __forceinline__ void encode_kstep(const TableView &tv, const float *stage, const EncodeLane &el, int ks, int t, float (&Pf)[4][4]) {
+    const float *offs = stage + 32 * ST_STRIDE;
+    // A = H^T (16 x 16 pairs), stored pair by pair: transposed on the way in
+    uint32_t ah[4], al[4];
+    ldmatrix_x4_trans(ah, el.a_addr + ks * (16 * ST_STRIDE * 4));
+    ldmatrix_x4_trans(al, el.a_addr + ks * (16 * ST_STRIDE * 4) + 32);
+    // B = G (16 pairs x 8 channels per n-tile; column g of n-tile c is channel 4 g + c): g = sum_m b_m c_m (Eq. 2)
+    uint32_t bh[4][2], bl[4][2];
+    if (HALF) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) bh[c][1] = bl[c][1] = 0u;
+    }
+#pragma unroll
+    for (int half = 0; half < (HALF ? 1 : 2); ++half) {
+        float gv[2][4];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int slot = 16 * ks + 8 * half + 2 * t + u;
+            const float4 b = *reinterpret_cast<const float4 *>(stage + slot * ST_STRIDE + 16);
+            RowOffsets<TAB_SMEM> ro;
+            ro.load(offs + slot * OFF_WORDS<TAB_SMEM>);
+            const float bw[4] = {b.x, b.y, b.z, b.w};
+            float2 lo = make_float2(0.f, 0.f), hi = lo;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const float4 c = table_load<TAB_SMEM>(tv, ro.at(m, el.chunk));
+                lo = ffma2(make_float2(bw[m], bw[m]), make_float2(c.x, c.y), lo);
+                hi = ffma2(make_float2(bw[m], bw[m]), make_float2(c.z, c.w), hi);
+            }
+            gv[u][0] = lo.x; gv[u][1] = lo.y; gv[u][2] = hi.x; gv[u][3] = hi.y;
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) split_h2(gv[0][c], gv[1][c], bh[c][half], bl[c][half]);
+    }
+    // the three terms of each n-tile are issued interleaved over the n-tiles
+    float c[4][4];
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) mma_f16_z(c[nt], al[0], al[1], al[2], al[3], bh[nt][0], bh[nt][1]);
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) mma_f16(c[nt], ah[0], ah[1], ah[2], ah[3], bl[nt][0], bl[nt][1]);
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) mma_f16(c[nt], ah[0], ah[1], ah[2], ah[3], bh[nt][0], bh[nt][1]);
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) {
+        const float2 s01 = add2(make_float2(Pf[nt][0], Pf[nt][1]), make_float2(c[nt][0], c[nt][1]));
+        const float2 s23 = add2(make_float2(Pf[nt][2], Pf[nt][3]), make_float2(c[nt][2], c[nt][3]));
+        Pf[nt][0] = s01.x; Pf[nt][1] = s01.y; Pf[nt][2] = s23.x; Pf[nt][3] = s23.y;
+    }
+}
+__device__ __forceinline__ void clear_fragments(float (&Pf)[4][4]) {
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) Pf[a][b] = 0.f;
+}
 
-    auto batch = [&](int first, int n) {
-        {   // lane = pair: harmonics (Eq. 3) and spline basis
-            float h[D_ANG], b[4];
-            int row = 0;
-            if (lane < n) {
-                const float4 e = pq[first + lane];
-                const float d2 = e.x * e.x + e.y * e.y + e.z * e.z, rinv = rsqrtf(d2), r = d2 * rinv;
-                harmonics(e.x * rinv, e.y * rinv, e.z * rinv, h);
-                float u;
-                const int iv = spline_interval(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, u, k.status);
-                cubic_basis(u, b);
-                row = (__float_as_int(e.w) >> J_BITS) * (k.tab.knots + 3) + iv;
-            } else {
-#pragma unroll
-                for (int a = 0; a < D_ANG; ++a) h[a] = 0.f;
-                b[0] = b[1] = b[2] = b[3] = 0.f;
-            }
-            uint32_t hi[8], lo[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) split_h2(h[2 * q], h[2 * q + 1], hi[q], lo[q]);
-            uint4 *dst = reinterpret_cast<uint4 *>(stage + lane * ST_STRIDE);
-            dst[0] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-            dst[1] = make_uint4(hi[4], hi[5], hi[6], hi[7]);
-            dst[2] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-            dst[3] = make_uint4(lo[4], lo[5], lo[6], lo[7]);
-            const int turn = ((lane >> 1) - row) & 3;
-            *reinterpret_cast<float4 *>(dst + 4) = rotate4(b, turn);
-            RowOffsets<TAB_SMEM> ro;
-            ro.make(tv, row, turn);
-            ro.store(offs + lane * OFF_WORDS<TAB_SMEM>);
-        }
-        __syncwarp();
-        pc.mark(1);
-        const int nks = (n + 15) >> 4;
-#pragma unroll
-        for (int ks = 0; ks < 2; ++ks) {
-            if (ks >= nks) break;
-            // A = H^T (16 x 16 pairs), stored pair by pair: transposed on the way in
-            uint32_t ah[4], al[4];
-            ldmatrix_x4_trans(ah, a_addr + ks * (16 * ST_STRIDE * 4));
-            ldmatrix_x4_trans(al, a_addr + ks * (16 * ST_STRIDE * 4) + 32);
-            // B = G (16 pairs x 8 channels per n-tile; column g of n-tile c is channel 4 g + c): g = sum_m b_m c_m (Eq. 2)
-            uint32_t bh[4][2], bl[4][2];
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                float gv[2][4];
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int slot = 16 * ks + 8 * half + 2 * t + u;
-                    const float4 b = *reinterpret_cast<const float4 *>(stage + slot * ST_STRIDE + 16);
-                    RowOffsets<TAB_SMEM> ro;
-                    ro.load(offs + slot * OFF_WORDS<TAB_SMEM>);
-                    const float bw[4] = {b.x, b.y, b.z, b.w};
-                    float2 lo = make_float2(0.f, 0.f), hi = lo;
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) {
-                        const float4 c = table_load<TAB_SMEM>(tv, ro.at(m, chunk[m]));
-                        lo = ffma2(make_float2(bw[m], bw[m]), make_float2(c.x, c.y), lo);
-                        hi = ffma2(make_float2(bw[m], bw[m]), make_float2(c.z, c.w), hi);
-                    }
-                    gv[u][0] = lo.x; gv[u][1] = lo.y; gv[u][2] = hi.x; gv[u][3] = hi.y;
-                }
-#pragma unroll
-                for (int c = 0; c < 4; ++c) split_h2(gv[0][c], gv[1][c], bh[c][half], bl[c][half]);
-            }
-            // Eq. 4 for sixteen pairs; the three terms of each n-tile are issued interleaved over the n-tiles
-            float c[4][4];
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) mma_f16_z(c[nt], al[0], al[1], al[2], al[3], bh[nt][0], bh[nt][1]);
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) mma_f16(c[nt], ah[0], ah[1], ah[2], ah[3], bl[nt][0], bl[nt][1]);
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) mma_f16(c[nt], ah[0], ah[1], ah[2], ah[3], bh[nt][0], bh[nt][1]);
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                const float2 s01 = add2(make_float2(Pf[nt][0], Pf[nt][1]), make_float2(c[nt][0], c[nt][1]));
-                const float2 s23 = add2(make_float2(Pf[nt][2], Pf[nt][3]), make_float2(c[nt][2], c[nt][3]));
-                Pf[nt][0] = s01.x; Pf[nt][1] = s01.y; Pf[nt][2] = s23.x; Pf[nt][3] = s23.y;
-            }
-        }
-        __syncwarp();
-        pc.mark(2);
-    };
+// One atom on its own: returns the number of pairs and the moment as accumulator fragments.
+// `queued` returns the number of pairs left in the queue when the whole list fitted in one round
+// (the derivation then reuses them), or -1.
+// (UNROLL = 2, tiles of one atom per warp: two k-steps side by side and no half ones, the chain through a tile being their time)
+template <bool TAB_SMEM, bool L16, int UNROLL>
+__device__ __forceinline__ int encode_atom(const KernelArgs &k, const TableView &tv, const double4 &pi, int64_t beg, int64_t end,
+                                           float4 *pq, int cap, float *stage, int lane, float (&Pf)[4][4], int &queued, const int *sidx, int n_pref,
+                                           int cs, PhaseClock &pc) {
+    const EncodeLane el(stage, lane);
+    clear_fragments(Pf);
     int total = 0, rounds = 0, n = 0;
     int64_t cur = beg;
     do {
         n = collect_pairs<L16>(k, pi, beg, cur, end, pq, cap, lane, sidx, n_pref, cs);
         pc.mark(0);
-        for (int q0 = 0; q0 < n; q0 += 32) batch(q0, min(32, n - q0));
+        for (int q0 = 0; q0 < n; q0 += 32) {
+            encode_rows<TAB_SMEM>(k, tv, pq, q0 + lane, q0 + lane < n, stage, lane);
+            __syncwarp();
+            pc.mark(1);
+#pragma unroll UNROLL
+            for (int ks = 0; ks < 2; ++ks) {
+                const int left = n - q0 - 16 * ks;
+                if (left <= 0) break;
+                if (UNROLL == 2 || left > 8) encode_kstep<TAB_SMEM, false>(tv, stage, el, ks, lane & 3, Pf);
+                else encode_kstep<TAB_SMEM, true>(tv, stage, el, ks, lane & 3, Pf);
+            }
+            __syncwarp();
+            pc.mark(2);
+        }
         total += n;
         ++rounds;
     } while (cur < end);
@@ -533,134 +617,174 @@ __device__ __forceinline__ void tmem_fill(uint32_t quarter_base, const uint32_t 
     tmem_wait_st();
 }
 
-// ---------------- Derivation of one atom (Eq. 8-10) ----------------
-template <bool TAB_SMEM, bool DET, bool L16>
-__device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView &tv, int i,
-                                            float4 *pq, int cap, float *scr, int queued, int lane, const uint32_t (&Wh)[2][2][2],
-                                            const uint32_t (&Wl)[2][2][2], float w_scale_inv, float (&vir)[9], uint32_t tm_vt, PhaseClock &pc) {
-    // Wh, Wl [k-step][n-tile][b0, b1]: B fragments of W_i^T times 1 / w_scale_inv; k-step q holds channels 8t + 4q .. + 3 of lane (g, t)
-    const int g = lane >> 2, t = lane & 3;
-    float *bs = scr;
-    // tile fragments: lane (g, t) evaluates chunks 2t, 2t + 1 of pairs g, g + 8.  A pair in slot p takes its rows in the residue
-    // order p, p + 1, .. (mod 4): of the two pairs in a load phase one reads the even, the other the odd chunk positions.
-    uint32_t chunk[4];
+// ---------------- Derivation (Eq. 8-10) ----------------
+// Lane = pair: spline basis and its derivative of queue entry `slot` into the hand-over rows; zeros where there is no pair.
+template <bool TAB_SMEM>
+__device__ __forceinline__ void derive_rows(const KernelArgs &k, const TableView &tv, const float4 *pq, int slot, bool live, float *bs, int lane) {
+    float b[4] = {0.f, 0.f, 0.f, 0.f}, db[4] = {0.f, 0.f, 0.f, 0.f};
+    int row = 0;
+    if (live) {
+        const float4 ent = pq[slot];
+        const float d2 = ent.x * ent.x + ent.y * ent.y + ent.z * ent.z, r = d2 * rsqrtf(d2);
+        float u;
+        const int iv = spline_interval(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, u, k.status);
+        cubic_basis(u, b);
+        cubic_basis_deriv(u, 1.f, db);
+        row = (__float_as_int(ent.w) >> J_BITS) * (k.tab.knots + 3) + iv;
+    }
+    const int turn = (lane - row) & 3;
+    float *dst = bs + lane * BS_STRIDE;
+    *reinterpret_cast<float4 *>(dst) = rotate4(b, turn);
+    *reinterpret_cast<float4 *>(dst + 4) = rotate4(db, turn);
+    RowOffsets<TAB_SMEM> ro;
+    ro.make(tv, row, turn);
+    ro.store(dst + 8);
+}
+// W_i = dE_i/dP_i as B fragments of W_i^T times 1 / inv; k-step q holds channels 8t + 4q .. + 3 of lane (g, t).
+struct WFragments {
+    uint32_t hi[2][2][2], lo[2][2][2];   // [k-step][n-tile][b0, b1]
+};
+// V and T of the sixteen pairs of hand-over rows 16 mt .. to tensor memory.  Tile fragments: lane (g, t) evaluates chunks 2t, 2t + 1 of pairs
+// g, g + 8.  A pair in slot p takes its rows in the residue order p, p + 1, .. (mod 4): of the two pairs in a load phase one reads the
+// even, the other the odd chunk positions.  HALF: no pair behind the eighth.
+template <bool TAB_SMEM, bool HALF>
+__device__ __forceinline__ void derive_tile(const TableView &tv, const float *bs, int mt, int g, const uint32_t (&chunk)[2], const WFragments &W, uint32_t tm_vt) {
+    // A = [G; G'] (16 pairs x 32 channels): rows pairs g, g + 8; this lane evaluates channels 8t .. 8t+7
+    // (one accumulator per output here: the truncating accumulation costs ~1e-6 relative on a
+    // short chain, irrelevant for forces, and the registers are needed elsewhere).  G' is the derivative per knot interval.
+    float V[2][4], T[2][4];
+    uint32_t ah[2][4], al[2][4], dh[2][4], dl[2][4];   // [k-step][fragment register]
+    if (HALF) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) chunk[q] = 16u * ((2 * t) ^ table_swizzle((g + q) & 3));
-    float fx = 0.f, fy = 0.f, fz = 0.f;
+        for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+            for (int r = 1; r < 4; r += 2) ah[ks][r] = al[ks][r] = dh[ks][r] = dl[ks][r] = 0u;
+    }
+#pragma unroll
+    for (int q = 0; q < (HALF ? 1 : 2); ++q) {
+        const float *rp = bs + (16 * mt + g + 8 * q) * BS_STRIDE;
+        const float4 b = *reinterpret_cast<const float4 *>(rp), db = *reinterpret_cast<const float4 *>(rp + 4);
+        RowOffsets<TAB_SMEM> ro;
+        ro.load(rp + 8);
+        const float bw[4] = {b.x, b.y, b.z, b.w}, dbw[4] = {db.x, db.y, db.z, db.w};
+        float2 G2[4], dG2[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) { G2[c] = make_float2(0.f, 0.f); dG2[c] = make_float2(0.f, 0.f); }
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const uint32_t at = ro.at(m, chunk);
+            const float4 c0 = table_load<TAB_SMEM>(tv, at), c1 = table_load<TAB_SMEM>(tv, at ^ 16u);
+            const float2 cv[4] = {make_float2(c0.x, c0.y), make_float2(c0.z, c0.w), make_float2(c1.x, c1.y), make_float2(c1.z, c1.w)};
+            const float2 b2 = make_float2(bw[m], bw[m]), db2 = make_float2(dbw[m], dbw[m]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) { G2[c] = ffma2(b2, cv[c], G2[c]); dG2[c] = ffma2(db2, cv[c], dG2[c]); }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {   // channel pair c: k-step c / 2, fragment register q + 2 (c % 2)
+            split_h2(G2[c].x, G2[c].y, ah[c >> 1][q + 2 * (c & 1)], al[c >> 1][q + 2 * (c & 1)]);
+            split_h2(dG2[c].x, dG2[c].y, dh[c >> 1][q + 2 * (c & 1)], dl[c >> 1][q + 2 * (c & 1)]);
+        }
+    }
+    // Eq. 9 (rows of V: a = 0..7 and 8..15) and W g' (Eq. 8 re-associated); cross terms first, the four
+    // independent accumulators interleaved
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks) {
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+            if (ks == 0) {
+                mma_f16_z(V[nt], al[ks][0], al[ks][1], al[ks][2], al[ks][3], W.hi[ks][nt][0], W.hi[ks][nt][1]);
+                mma_f16_z(T[nt], dl[ks][0], dl[ks][1], dl[ks][2], dl[ks][3], W.hi[ks][nt][0], W.hi[ks][nt][1]);
+            } else {
+                mma_f16(V[nt], al[ks][0], al[ks][1], al[ks][2], al[ks][3], W.hi[ks][nt][0], W.hi[ks][nt][1]);
+                mma_f16(T[nt], dl[ks][0], dl[ks][1], dl[ks][2], dl[ks][3], W.hi[ks][nt][0], W.hi[ks][nt][1]);
+            }
+        }
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+            mma_f16(V[nt], ah[ks][0], ah[ks][1], ah[ks][2], ah[ks][3], W.lo[ks][nt][0], W.lo[ks][nt][1]);
+            mma_f16(T[nt], dh[ks][0], dh[ks][1], dh[ks][2], dh[ks][3], W.lo[ks][nt][0], W.lo[ks][nt][1]);
+        }
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+            mma_f16(V[nt], ah[ks][0], ah[ks][1], ah[ks][2], ah[ks][3], W.hi[ks][nt][0], W.hi[ks][nt][1]);
+            mma_f16(T[nt], dh[ks][0], dh[ks][1], dh[ks][2], dh[ks][3], W.hi[ks][nt][0], W.hi[ks][nt][1]);
+        }
+    }
+    // The accumulator fragments of the 16 pairs go to tensor memory as 16 lanes (pair) x 32 columns (V, T); read back
+    // with lane = pair.  (Through shared memory the same exchange was 188 of the kernel's 1,958 L1 wavefronts per atom.)
+    tmem_st_vt(tm_vt + ((uint32_t)(16 * mt) << 16), V, T);
+}
+// Lane = pair: projection onto the pair vector (Eq. 10), scatter of the reaction; returns the force on the central atom.
+template <bool DET>
+__device__ __forceinline__ float3 project_pair(const KernelArgs &k, const float4 &ent, const uint32_t (&vt)[32], float w_scale_inv, float (&vir)[9]) {
+    float v[D_ANG], tt[D_ANG];
+#pragma unroll
+    for (int q = 0; q < D_ANG; ++q) { v[q] = __uint_as_float(vt[q]); tt[q] = __uint_as_float(vt[16 + q]); }
+    const float x = ent.x, y = ent.y, z = ent.z;
+    const float rinv = rsqrtf(x * x + y * y + z * z);
+    const int j = __float_as_int(ent.w) & ((1 << J_BITS) - 1);
+    const float ux = x * rinv, uy = y * rinv, uz = z * rinv;
+    float s, tx, ty, tz, tu;
+    harmonics_project(ux, uy, uz, v, tt, s, tx, ty, tz, tu);
+    // f_ij = (g' . u_ij) r^ + J_ang^T v_ij,  J_ang = (grad_u h)(I - u u^T) / r, the scales taken back
+    const float sr = s * (w_scale_inv * k.tab.inv_h), vr = rinv * w_scale_inv;
+    const float qx = sr * ux + (tx - tu * ux) * vr;
+    const float qy = sr * uy + (ty - tu * uy) * vr;
+    const float qz = sr * uz + (tz - tu * uz) * vr;
+    if (DET) fixed_add3(k.force_fx + 3 * (size_t)j, -qx, -qy, -qz);
+    else atomicAdd(&k.force[j], make_float4(-qx, -qy, -qz, 0.f));   // one 128-bit reduction per pair
+    vir[0] -= x * qx; vir[1] -= x * qy; vir[2] -= x * qz;
+    vir[3] -= y * qx; vir[4] -= y * qy; vir[5] -= y * qz;
+    vir[6] -= z * qx; vir[7] -= z * qy; vir[8] -= z * qz;
+    return make_float3(qx, qy, qz);
+}
+// The sum over the lanes, each step sending what the lane does not keep: six shuffles (they use the shared-memory pipe) instead of fifteen.
+template <bool DET>
+__device__ __forceinline__ void add_own_force(const KernelArgs &k, int i, float3 f, int lane) {
+    const bool upper = lane & 16, odd = lane & 8;
+    float p = upper ? f.z : f.x, q = upper ? 0.f : f.y;
+    p += __shfl_xor_sync(0xffffffffu, upper ? f.x : f.z, 16);
+    q += __shfl_xor_sync(0xffffffffu, upper ? f.y : 0.f, 16);
+    float v = (odd ? q : p) + __shfl_xor_sync(0xffffffffu, odd ? p : q, 8);
+#pragma unroll
+    for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((lane & 7) == 0 && lane < 24) {   // lanes 0, 8, 16: x, y, z
+        if (DET) atomicAdd(reinterpret_cast<unsigned long long *>(k.force_fx + 3 * (size_t)i + (lane >> 3)), (unsigned long long)__float2ll_rn(v * FORCE_FX));
+        else atomicAdd(&k.force[i].x + (lane >> 3), v);
+    }
+}
+__device__ __forceinline__ void derive_chunks(uint32_t (&chunk)[2], int lane) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) chunk[q] = 16u * ((2 * (lane & 3)) ^ table_swizzle(((lane >> 2) + q) & 3));
+}
+
+// One atom on its own.
+template <int APW, bool TAB_SMEM, bool DET, bool L16>
+__device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView &tv, int i,
+                                            float4 *pq, int cap, float *scr, int queued, int lane, const WFragments &W, float w_scale_inv,
+                                            float (&vir)[9], uint32_t tm_vt, PhaseClock &pc) {
+    uint32_t chunk[2];
+    derive_chunks(chunk, lane);
+    float3 f = make_float3(0.f, 0.f, 0.f);
 
     auto batch = [&](int first, int n) {
-        {   // lane = pair: spline basis and its derivative
-            float b[4] = {0.f, 0.f, 0.f, 0.f}, db[4] = {0.f, 0.f, 0.f, 0.f};
-            int row = 0;
-            if (lane < n) {
-                const float4 ent = pq[first + lane];
-                const float d2 = ent.x * ent.x + ent.y * ent.y + ent.z * ent.z, r = d2 * rsqrtf(d2);
-                float u;
-                const int iv = spline_interval(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, u, k.status);
-                cubic_basis(u, b);
-                cubic_basis_deriv(u, 1.f, db);
-                row = (__float_as_int(ent.w) >> J_BITS) * (k.tab.knots + 3) + iv;
-            }
-            const int turn = (lane - row) & 3;
-            float *dst = bs + lane * BS_STRIDE;
-            *reinterpret_cast<float4 *>(dst) = rotate4(b, turn);
-            *reinterpret_cast<float4 *>(dst + 4) = rotate4(db, turn);
-            RowOffsets<TAB_SMEM> ro;
-            ro.make(tv, row, turn);
-            ro.store(dst + 8);
-        }
+        derive_rows<TAB_SMEM>(k, tv, pq, first + lane, lane < n, scr, lane);
         __syncwarp();
         pc.mark(4);
         const int nmt = (n + 15) >> 4;
 #pragma unroll 1
         for (int mt = 0; mt < nmt; ++mt) {
-            // A = [G; G'] (16 pairs x 32 channels): rows pairs g, g + 8; this lane evaluates channels 8t .. 8t+7
-            // (one accumulator per output here: the truncating accumulation costs ~1e-6 relative on a
-            // short chain, irrelevant for forces, and the registers are needed elsewhere).  G' is the derivative per knot interval.
-            float V[2][4], T[2][4];
-            uint32_t ah[2][4], al[2][4], dh[2][4], dl[2][4];   // [k-step][fragment register]
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const float *rp = bs + (16 * mt + g + 8 * q) * BS_STRIDE;
-                const float4 b = *reinterpret_cast<const float4 *>(rp), db = *reinterpret_cast<const float4 *>(rp + 4);
-                RowOffsets<TAB_SMEM> ro;
-                ro.load(rp + 8);
-                const float bw[4] = {b.x, b.y, b.z, b.w}, dbw[4] = {db.x, db.y, db.z, db.w};
-                float2 G2[4], dG2[4];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) { G2[c] = make_float2(0.f, 0.f); dG2[c] = make_float2(0.f, 0.f); }
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    const uint32_t at = ro.at(m, chunk[m]);
-                    const float4 c0 = table_load<TAB_SMEM>(tv, at), c1 = table_load<TAB_SMEM>(tv, at ^ 16u);
-                    const float2 cv[4] = {make_float2(c0.x, c0.y), make_float2(c0.z, c0.w), make_float2(c1.x, c1.y), make_float2(c1.z, c1.w)};
-                    const float2 b2 = make_float2(bw[m], bw[m]), db2 = make_float2(dbw[m], dbw[m]);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) { G2[c] = ffma2(b2, cv[c], G2[c]); dG2[c] = ffma2(db2, cv[c], dG2[c]); }
-                }
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {   // channel pair c: k-step c / 2, fragment register q + 2 (c % 2)
-                    split_h2(G2[c].x, G2[c].y, ah[c >> 1][q + 2 * (c & 1)], al[c >> 1][q + 2 * (c & 1)]);
-                    split_h2(dG2[c].x, dG2[c].y, dh[c >> 1][q + 2 * (c & 1)], dl[c >> 1][q + 2 * (c & 1)]);
-                }
-            }
-            // Eq. 9 (rows of V: a = 0..7 and 8..15) and W g' (Eq. 8 re-associated); cross terms first, the four
-            // independent accumulators interleaved
-#pragma unroll
-            for (int ks = 0; ks < 2; ++ks) {
-#pragma unroll
-                for (int nt = 0; nt < 2; ++nt) {
-                    if (ks == 0) {
-                        mma_f16_z(V[nt], al[ks][0], al[ks][1], al[ks][2], al[ks][3], Wh[ks][nt][0], Wh[ks][nt][1]);
-                        mma_f16_z(T[nt], dl[ks][0], dl[ks][1], dl[ks][2], dl[ks][3], Wh[ks][nt][0], Wh[ks][nt][1]);
-                    } else {
-                        mma_f16(V[nt], al[ks][0], al[ks][1], al[ks][2], al[ks][3], Wh[ks][nt][0], Wh[ks][nt][1]);
-                        mma_f16(T[nt], dl[ks][0], dl[ks][1], dl[ks][2], dl[ks][3], Wh[ks][nt][0], Wh[ks][nt][1]);
-                    }
-                }
-#pragma unroll
-                for (int nt = 0; nt < 2; ++nt) {
-                    mma_f16(V[nt], ah[ks][0], ah[ks][1], ah[ks][2], ah[ks][3], Wl[ks][nt][0], Wl[ks][nt][1]);
-                    mma_f16(T[nt], dh[ks][0], dh[ks][1], dh[ks][2], dh[ks][3], Wl[ks][nt][0], Wl[ks][nt][1]);
-                }
-#pragma unroll
-                for (int nt = 0; nt < 2; ++nt) {
-                    mma_f16(V[nt], ah[ks][0], ah[ks][1], ah[ks][2], ah[ks][3], Wh[ks][nt][0], Wh[ks][nt][1]);
-                    mma_f16(T[nt], dh[ks][0], dh[ks][1], dh[ks][2], dh[ks][3], Wh[ks][nt][0], Wh[ks][nt][1]);
-                }
-            }
-            // The accumulator fragments of the 16 pairs go to tensor memory as 16 lanes (pair) x 32 columns (V, T); read back
-            // below with lane = pair.  (Through shared memory the same exchange was 188 of the kernel's 1,958 L1 wavefronts per
-            // atom.)
-            tmem_st_vt(tm_vt + ((uint32_t)(16 * mt) << 16), V, T);
+            if (APW == 1 || n - 16 * mt > 8) derive_tile<TAB_SMEM, false>(tv, scr, mt, lane >> 2, chunk, W, tm_vt);
+            else derive_tile<TAB_SMEM, true>(tv, scr, mt, lane >> 2, chunk, W, tm_vt);
         }
         tmem_wait_st();
         pc.mark(5);
         uint32_t vt[32];
         tmem_ld32(tm_vt, vt);
         tmem_wait_ld();
-        if (lane < n) {   // lane = pair: projection onto the pair vector (Eq. 10) and scatter
-            float v[D_ANG], tt[D_ANG];
-#pragma unroll
-            for (int q = 0; q < D_ANG; ++q) { v[q] = __uint_as_float(vt[q]); tt[q] = __uint_as_float(vt[16 + q]); }
-            const float4 ent = pq[first + lane];
-            const float x = ent.x, y = ent.y, z = ent.z;
-            const float rinv = rsqrtf(x * x + y * y + z * z);
-            const int j = __float_as_int(ent.w) & ((1 << J_BITS) - 1);
-            const float ux = x * rinv, uy = y * rinv, uz = z * rinv;
-            float s, tx, ty, tz, tu;
-            harmonics_project(ux, uy, uz, v, tt, s, tx, ty, tz, tu);
-            // f_ij = (g' . u_ij) r^ + J_ang^T v_ij,  J_ang = (grad_u h)(I - u u^T) / r, the scales taken back
-            const float sr = s * (w_scale_inv * k.tab.inv_h), vr = rinv * w_scale_inv;
-            const float qx = sr * ux + (tx - tu * ux) * vr;
-            const float qy = sr * uy + (ty - tu * uy) * vr;
-            const float qz = sr * uz + (tz - tu * uz) * vr;
-            fx += qx; fy += qy; fz += qz;
-            if (DET) fixed_add3(k.force_fx + 3 * (size_t)j, -qx, -qy, -qz);
-            else atomicAdd(&k.force[j], make_float4(-qx, -qy, -qz, 0.f));   // one 128-bit reduction per pair
-            vir[0] -= x * qx; vir[1] -= x * qy; vir[2] -= x * qz;
-            vir[3] -= y * qx; vir[4] -= y * qy; vir[5] -= y * qz;
-            vir[6] -= z * qx; vir[7] -= z * qy; vir[8] -= z * qz;
+        if (lane < n) {
+            const float3 q = project_pair<DET>(k, pq[first + lane], vt, w_scale_inv, vir);
+            f.x += q.x; f.y += q.y; f.z += q.z;
         }
         __syncwarp();
         pc.mark(6);
@@ -679,16 +803,7 @@ __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView
             for (int q0 = 0; q0 < n; q0 += 32) batch(q0, min(32, n - q0));
         } while (cur < end);
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        fx += __shfl_xor_sync(0xffffffffu, fx, o);
-        fy += __shfl_xor_sync(0xffffffffu, fy, o);
-        fz += __shfl_xor_sync(0xffffffffu, fz, o);
-    }
-    if (lane == 0) {
-        if (DET) fixed_add3(k.force_fx + 3 * (size_t)i, fx, fy, fz);
-        else atomicAdd(&k.force[i], make_float4(fx, fy, fz, 0.f));
-    }
+    add_own_force<DET>(k, i, f, lane);
 }
 
 // Barrier among the 256 threads of one group (hardware barrier 1 + group).
@@ -1086,64 +1201,144 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
                 asm volatile("cp.async.wait_group 0;" ::: "memory");
                 __syncwarp();
             }
-            int q_used = 0;   // pairs of the queue that are kept for the derivation
-#pragma unroll 1
-            for (int u = 0; u < APW; ++u) {
-                float *xrow = scr;                        // the atom's invariants (the encoding is done with the scratch)
-                if (wg + GW * u < count) {
-                    int i, n_pref = 0, cs = 0, queued = -1;
-                    int64_t beg, end;
-                    const int *nidx = pf + u * PF_WORDS;
-                    if (prefetched) {
-                        i = nidx[PF_IDX];
-                        beg = ((int64_t)nidx[PF_IDX + 2] << 32) | (unsigned)nidx[PF_IDX + 1];
-                        end = beg + nidx[PF_IDX + 3];
-                        n_pref = min(PF_IDX, nidx[PF_IDX + 3]);
-                        if (L16) cs = lane < 27 ? nidx[PF_CS + lane] : 0;
-                    } else {
-                        i = (int)MLIP_CHECK_INDEX(__ldg(k.center_order + first + wg + GW * u), k.n, k.status);
-                        beg = k.nbr_off[i]; end = use_far ? k.nbr_off[i + 1] : beg + k.nbr_near[i];
-                        if (L16) cs = cell_base_of_lane(k, i, lane);
-                    }
-                    const double4 pi = load_pos4(k.pos4 + i);
-                    float Pf[4][4];
-                    n_pairs += encode_atom<TAB_SMEM, L16>(k, tv, pi, beg, end, pq + q_used, LY::POOL - q_used, scr, lane, Pf, queued, nidx, n_pref, cs, pc);
-                    if (u + 1 < APW && queued > LY::POOL - SECOND_ROOM) queued = -1;   // leave the next atom room for a scan
-                    if (lane == 0) *reinterpret_cast<int4 *>(info + 4 * u) = make_int4(i, queued, q_used, 0);
-                    q_used += max(queued, 0);
-                    tmem_st16(u == 0 ? tm_p : tm_vt, Pf);
-                    // Eq. 5 (C_l = I): this lane holds rows a = g, g + 8 of channels 8t + j; sum squares over the rows of a block.
-                    // Rows 1..3 (l = 1) and 4..7 (l = 2) differ in the top bit of g, so one two-step butterfly over the lower
-                    // bits sums both; l = 2 then takes row 8 (held by g = 0) and the upper half's sum, l = 3 is rows 9..15.
-                    float part[4][8];
+            // an atom's moment to tensor memory, its invariants to the regression
+            auto finish_atom = [&](int u, const float (&Pf)[4][4]) {
+                float *xrow = sX + (wg + GW * u) * X_STRIDE;   // (dE/dG of the last tile's atom: this warp has read it)
+                tmem_st16(u == 0 ? tm_p : tm_vt, Pf);
+                // Eq. 5 (C_l = I): this lane holds rows a = g, g + 8 of channels 8t + j; sum squares over the rows of a block.
+                // Rows 1..3 (l = 1) and 4..7 (l = 2) differ in the top bit of g, so two steps over the lower bits sum both; rows
+                // 9..15 (l = 3) take a third.  In each step a lane sends the half of the channels that it does not keep (13 shuffles
+                // instead of the 40 of a butterfly: they use the shared-memory pipe).  Row 8 (l = 2), held by g = 0, joins in shared memory.
+                const bool g0 = lane & 4, g1 = lane & 8, g2 = lane & 16;
+                float qa[8], qb[8];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float pa = Pf[j & 3][j >> 2], pb = Pf[j & 3][2 + (j >> 2)];
-                        float qa = g >= 1 ? pa * pa : 0.f, qb = g >= 1 ? pb * pb : 0.f;
-                        qa += __shfl_xor_sync(0xffffffffu, qa, 4);
-                        qb += __shfl_xor_sync(0xffffffffu, qb, 4);
-                        qa += __shfl_xor_sync(0xffffffffu, qa, 8);
-                        qb += __shfl_xor_sync(0xffffffffu, qb, 8);
-                        const float upper = __shfl_xor_sync(0xffffffffu, qa, 16);   // g = 0 receives the sum over g = 4..7
-                        qb += __shfl_xor_sync(0xffffffffu, qb, 16);
-                        part[0][j] = pa;                  // (the values below are those of the storing lanes, g = 0)
-                        part[1][j] = qa;
-                        part[2][j] = upper + pb * pb;
-                        part[3][j] = qb;
-                    }
-                    if (g == 0) {
-#pragma unroll
-                        for (int l = 0; l < 4; ++l) {
-                            *reinterpret_cast<float4 *>(xrow + 32 * l + 8 * t) = make_float4(part[l][0], part[l][1], part[l][2], part[l][3]);
-                            *reinterpret_cast<float4 *>(xrow + 32 * l + 8 * t + 4) = make_float4(part[l][4], part[l][5], part[l][6], part[l][7]);
-                        }
-                    }
-                } else {   // empty slot of a ragged tile: feed zeros to the head
-                    for (int c = lane; c < N_INV; c += 32) xrow[c] = 0.f;
+                for (int j = 0; j < 8; ++j) {
+                    const float pa = Pf[j & 3][j >> 2], pb = Pf[j & 3][2 + (j >> 2)];
+                    qa[j] = g >= 1 ? pa * pa : 0.f;
+                    qb[j] = pb * pb;
                 }
+                if (g == 0) {
+                    float4 *to = reinterpret_cast<float4 *>(xrow + 8 * t);
+                    to[0] = make_float4(Pf[0][0], Pf[1][0], Pf[2][0], Pf[3][0]);
+                    to[1] = make_float4(Pf[0][1], Pf[1][1], Pf[2][1], Pf[3][1]);
+                    to[16] = make_float4(qb[0], qb[1], qb[2], qb[3]);
+                    to[17] = make_float4(qb[4], qb[5], qb[6], qb[7]);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) qb[j] = 0.f;
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float sa = g0 ? qa[j] : qa[j + 4], sb = g0 ? qb[j] : qb[j + 4];
+                    qa[j] = (g0 ? qa[j + 4] : qa[j]) + __shfl_xor_sync(0xffffffffu, sa, 4);
+                    qb[j] = (g0 ? qb[j + 4] : qb[j]) + __shfl_xor_sync(0xffffffffu, sb, 4);
+                }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const float sa = g1 ? qa[j] : qa[j + 2], sb = g1 ? qb[j] : qb[j + 2];
+                    qa[j] = (g1 ? qa[j + 2] : qa[j]) + __shfl_xor_sync(0xffffffffu, sa, 8);
+                    qb[j] = (g1 ? qb[j + 2] : qb[j]) + __shfl_xor_sync(0xffffffffu, sb, 8);
+                }
+                const float sum3 = (g2 ? qb[1] : qb[0]) + __shfl_xor_sync(0xffffffffu, g2 ? qb[0] : qb[1], 16);
+                const int c = 8 * t + (g0 ? 4 : 0) + (g1 ? 2 : 0);   // this lane's channels: c, c + 1; of l = 3 one of them
+                xrow[96 + c + (g2 ? 1 : 0)] = sum3;
+                __syncwarp();
+                float2 *to = reinterpret_cast<float2 *>(xrow + (g2 ? 64 : 32) + c);
+                float2 sum = make_float2(qa[0], qa[1]);
+                if (g2) { const float2 row8 = *to; sum.x += row8.x; sum.y += row8.y; }
+                *to = sum;
                 __syncwarp();
                 split_invariants(xrow, xs, sc, hc, wg + GW * u, lane);
-                __syncwarp();   // (the next atom's hand-over rows overwrite the invariants)
+            };
+            const int mine = APW == 1 ? (wg < count) : (wg < count) + (wg + GW < count);   // atoms of this warp
+            // Two atoms whose pairs fit the queue together go through the pair loops side by side (see collect_two).
+            bool both = false;
+            int n0 = 0, n1 = 0, i0 = 0, i1 = 0;
+            if (APW == 2) {
+                if (prefetched && pf[PF_IDX + 3] <= NARROW_CHUNKS * 32 && (mine < 2 || pf[PF_WORDS + PF_IDX + 3] <= NARROW_CHUNKS * 32)) {
+                    collect_two<L16>(k, pf, mine, pq, lane, n0, n1);
+                    i0 = pf[PF_IDX];
+                    i1 = mine == 2 ? pf[PF_WORDS + PF_IDX] : 0;
+                    both = true;
+                }
+            }
+            auto atom_and_list = [&](int u, int &i, int64_t &beg, int64_t &end, int &n_pref, int &cs) {
+                const int *nidx = pf + u * PF_WORDS;
+                n_pref = cs = 0;
+                if (prefetched) {
+                    i = nidx[PF_IDX];
+                    beg = ((int64_t)nidx[PF_IDX + 2] << 32) | (unsigned)nidx[PF_IDX + 1];
+                    end = beg + nidx[PF_IDX + 3];
+                    n_pref = min(PF_IDX, nidx[PF_IDX + 3]);
+                    if (L16) cs = lane < 27 ? nidx[PF_CS + lane] : 0;
+                } else {
+                    i = (int)MLIP_CHECK_INDEX(__ldg(k.center_order + first + wg + GW * u), k.n, k.status);
+                    beg = k.nbr_off[i]; end = use_far ? k.nbr_off[i + 1] : beg + k.nbr_near[i];
+                    if (L16) cs = cell_base_of_lane(k, i, lane);
+                }
+            };
+            if (APW == 2 && !both) {   // longer lists, or the first tile of a species
+                both = true;
+#pragma unroll 1
+                for (int u = 0; u < mine && both; ++u) {
+                    int i, n_pref, cs;
+                    int64_t beg, end;
+                    atom_and_list(u, i, beg, end, n_pref, cs);
+                    const double4 pi = load_pos4(k.pos4 + i);
+                    const int at = u == 0 ? 0 : (n0 + 15) & ~15;
+                    int64_t cur = beg;
+                    const int n = collect_pairs<L16>(k, pi, beg, cur, end, pq + at, LY::POOL - at, lane, pf + u * PF_WORDS, n_pref, cs);
+                    both = cur >= end;
+                    if (u == 0) { n0 = n; i0 = i; } else { n1 = n; i1 = i; }
+                }
+            }
+            if (both) {
+                pc.mark(0);
+                const int second = (n0 + 15) & ~15, end = second + n1;
+                if (lane < 2) *reinterpret_cast<int4 *>(info + 4 * lane) = lane == 0 ? make_int4(i0, n0, 0, 1) : make_int4(i1, n1, second, 1);
+                n_pairs += n0 + n1;
+                const EncodeLane el(scr, lane);
+                int p = 0;   // first pair of the k-step
+#pragma unroll 1
+                for (int u = 0; u < 2; ++u) {
+                    float Pf[4][4];
+                    clear_fragments(Pf);
+                    const int stop = u == 0 ? n0 : end;
+#pragma unroll 1
+                    for (; p < stop; p += 16) {
+                        if ((p & 16) == 0) {
+                            const int slot = p + lane;
+                            __syncwarp();
+                            encode_rows<TAB_SMEM>(k, tv, pq, slot, slot < n0 || (slot >= second && slot < end), scr, lane);
+                            __syncwarp();
+                            pc.mark(1);
+                        }
+                        if (stop - p > 8) encode_kstep<TAB_SMEM, false>(tv, scr, el, (p >> 4) & 1, t, Pf);
+                        else encode_kstep<TAB_SMEM, true>(tv, scr, el, (p >> 4) & 1, t, Pf);
+                        pc.mark(2);
+                    }
+                    finish_atom(u, Pf);   // (an empty slot of a ragged tile feeds zeros to the head)
+                }
+                __syncwarp();
+            } else {
+                int q_used = 0;   // pairs of the queue that are kept for the derivation
+#pragma unroll 1
+                for (int u = 0; u < APW; ++u) {
+                    float Pf[4][4];
+                    if (u < mine) {
+                        int i, n_pref, cs, queued = -1;
+                        int64_t beg, end;
+                        atom_and_list(u, i, beg, end, n_pref, cs);
+                        const double4 pi = load_pos4(k.pos4 + i);
+                        n_pairs += encode_atom<TAB_SMEM, L16, APW == 1 ? 2 : 1>(k, tv, pi, beg, end, pq + q_used, LY::POOL - q_used, scr, lane, Pf, queued, pf + u * PF_WORDS, n_pref, cs, pc);
+                        if (u + 1 < APW && queued > LY::POOL - SECOND_ROOM) queued = -1;   // leave the next atom room for a scan
+                        if (lane == 0) *reinterpret_cast<int4 *>(info + 4 * u) = make_int4(i, queued, q_used, 0);
+                        q_used += max(queued, 0);
+                    } else {   // empty slot of a ragged tile: feed zeros to the head
+                        clear_fragments(Pf);
+                        if (u == 0 && lane == 0) *reinterpret_cast<int4 *>(info) = make_int4(0, 0, 0, 0);
+                    }
+                    finish_atom(u, Pf);
+                }
             }
             tmem_wait_st();
             if (wg == 0 && lane == 0) ctl[2 * group + 1] = look_ahead;
@@ -1162,16 +1357,13 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
             prefetched = first_next + wg < s_end;
             pc.mark(9);
 
-            // ---------------- Derivation: the second atom first (a rescan of the first one's list would overwrite its queue) ----
-#pragma unroll 1
-            for (int u = APW - 1; u >= 0; --u) {
-                if (wg + GW * u >= count) continue;
-                const int4 inf = *reinterpret_cast<const int4 *>(info + 4 * u);
+            // ---------------- Derivation ----------------
+            // W_i = dE_i/dP_i (Eq. 7) of the warp's u-th atom as scaled B fragments; returns the inverse of the scale
+            auto weights_of = [&](int u, WFragments &W) {
                 const float *drow = sX + (wg + GW * u) * X_STRIDE;   // dE/dG of the atom
                 float Pf[4][4];
                 tmem_ld16(u == 0 ? tm_p : tm_vt, Pf);
                 tmem_wait_ld();
-                // W_i = dE_i/dP_i (Eq. 7), already in B-fragment order
                 const int la = g == 0 ? 0 : (g <= 3 ? 1 : 2), lb = g == 0 ? 2 : 3;
                 float da[8], db[8];
                 {
@@ -1191,24 +1383,84 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
                     most = fmaxf(fmaxf(most, fmaxf(fabsf(w[nt][0]), fabsf(w[nt][1]))), fmaxf(fabsf(w[nt][2]), fabsf(w[nt][3])));
                 }
                 const float sw = scale_for(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(most))));
-                uint32_t Wh[2][2][2], Wl[2][2][2];
 #pragma unroll
                 for (int ks = 0; ks < 2; ++ks)
 #pragma unroll
                     for (int nt = 0; nt < 2; ++nt) {
-                        split_h2(w[0][2 * nt + ks] * sw, w[1][2 * nt + ks] * sw, Wh[ks][nt][0], Wl[ks][nt][0]);
-                        split_h2(w[2][2 * nt + ks] * sw, w[3][2 * nt + ks] * sw, Wh[ks][nt][1], Wl[ks][nt][1]);
+                        split_h2(w[0][2 * nt + ks] * sw, w[1][2 * nt + ks] * sw, W.hi[ks][nt][0], W.lo[ks][nt][0]);
+                        split_h2(w[2][2 * nt + ks] * sw, w[3][2 * nt + ks] * sw, W.hi[ks][nt][1], W.lo[ks][nt][1]);
                     }
-                derive_atom<TAB_SMEM, DET, L16>(k, tv, inf.x, pq + inf.z, LY::POOL - inf.z, scr, inf.y, lane, Wh, Wl, inverse_pow2(sw), vir, tm_vt, pc);
-                if (DET) {   // fold this atom's virial in now: lane sums in a fixed order, then integers
+                return inverse_pow2(sw);
+            };
+            auto fold_virial = [&]() {   // deterministic mode: lane sums in a fixed order, then integers
 #pragma unroll
-                    for (int q = 0; q < 9; ++q) {
-                        float x = vir[q];
+                for (int q = 0; q < 9; ++q) {
+                    float x = vir[q];
 #pragma unroll
-                        for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-                        if (lane == q) vir_fx += rint((double)x * VIRIAL_FX);
-                        vir[q] = 0.f;
+                    for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                    if (lane == q) vir_fx += rint((double)x * VIRIAL_FX);
+                    vir[q] = 0.f;
+                }
+            };
+            const int4 inf0 = *reinterpret_cast<const int4 *>(info);
+            if (APW == 2 && inf0.w != 0) {
+                // both atoms' pairs, from the last batch to the first: the second atom's moment, where V and T go, is read before the first of them
+                const int4 inf1 = *reinterpret_cast<const int4 *>(info + 4);
+                const int second = inf1.z, end = second + inf1.y;
+                uint32_t chunk[2];
+                derive_chunks(chunk, lane);
+                WFragments W;
+                float inv0 = 0.f, inv1 = 0.f;
+                int holds = -1;   // the atom that W belongs to
+                float3 f = make_float3(0.f, 0.f, 0.f);
+                bool second_open = inf1.y > 0;
+#pragma unroll 1
+                for (int p0 = (end - 1) & ~31; p0 >= 0; p0 -= 32) {
+                    const int slot = p0 + lane;
+                    const bool of_second = slot >= second, live = of_second ? slot < end : slot < inf0.y;
+                    derive_rows<TAB_SMEM>(k, tv, pq, slot, live, scr, lane);
+                    __syncwarp();
+                    pc.mark(4);
+#pragma unroll 1
+                    for (int mt = p0 + 16 < end ? 1 : 0; mt >= 0; --mt) {
+                        const int u = p0 + 16 * mt >= second;
+                        if (u != holds) {
+                            const float inv = weights_of(u, W);
+                            if (u) inv1 = inv; else inv0 = inv;
+                            holds = u;
+                        }
+                        if ((u ? end : inf0.y) - (p0 + 16 * mt) > 8) derive_tile<TAB_SMEM, false>(tv, scr, mt, g, chunk, W, tm_vt);
+                        else derive_tile<TAB_SMEM, true>(tv, scr, mt, g, chunk, W, tm_vt);
                     }
+                    tmem_wait_st();
+                    pc.mark(5);
+                    uint32_t vt[32];
+                    tmem_ld32(tm_vt, vt);
+                    tmem_wait_ld();
+                    float3 q = make_float3(0.f, 0.f, 0.f);
+                    if (live) q = project_pair<DET>(k, pq[slot], vt, of_second ? inv1 : inv0, vir);
+                    if (second_open && p0 <= second) {   // the second atom ends here: what the upper lanes hold is its, the lower ones begin the first's
+                        add_own_force<DET>(k, inf1.x, of_second ? make_float3(f.x + q.x, f.y + q.y, f.z + q.z) : f, lane);
+                        f = of_second ? make_float3(0.f, 0.f, 0.f) : q;
+                        second_open = false;
+                    } else {
+                        f.x += q.x; f.y += q.y; f.z += q.z;
+                    }
+                    __syncwarp();
+                    pc.mark(6);
+                }
+                if (inf0.y > 0) add_own_force<DET>(k, inf0.x, f, lane);
+                if (DET) fold_virial();
+            } else {
+                // the second atom first (a rescan of the first one's list would overwrite its queue)
+#pragma unroll 1
+                for (int u = APW - 1; u >= 0; --u) {
+                    if (wg + GW * u >= count) continue;
+                    const int4 inf = *reinterpret_cast<const int4 *>(info + 4 * u);
+                    WFragments W;
+                    const float inv = weights_of(u, W);
+                    derive_atom<APW, TAB_SMEM, DET, L16>(k, tv, inf.x, pq + inf.z, LY::POOL - inf.z, scr, inf.y, lane, W, inv, vir, tm_vt, pc);
+                    if (DET) fold_virial();
                 }
             }
             pc.mark(10);
