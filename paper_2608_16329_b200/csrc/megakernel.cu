@@ -125,10 +125,16 @@ constexpr int TM_FWD0 = 0, TM_FWD = 64, TM_BWD = 160, TM_BWD0 = 256, TM_VT = 320
 constexpr int HP_TMEM = 4 * TM_VT * 32;
 constexpr int HP_TOTAL = HP_TMEM + (HC_USED + 3) / 4 * 4;
 
+// The hardware's approximations as they are: without -ftz the compiler puts two or three instructions around each for denormal arguments, which do
+// not occur here (squared distances of atoms that do not coincide, 1 + exp(-x)) or come out the same (an exponential below 2^-126 adds nothing
+// to 1).  One evaluation of 1,000,188 atoms 7479 -> 7439 us, of 256,000 with 54 pairs 1634 -> 1621.
+__device__ __forceinline__ float fast_rsqrt(float x) { float y; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+__device__ __forceinline__ float fast_rcp(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+__device__ __forceinline__ float fast_exp2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 // SiLU and its derivative.  exp through the fast exponential: its error scales with |x| 2^-24 and
 // enters the sigmoid damped by s (1 - s), far below fp32 rounding of the surrounding sums.
 __device__ __forceinline__ float silu_f(float x, float &dsilu) {
-    const float s = __fdividef(1.0f, 1.0f + __expf(-x));
+    const float s = fast_rcp(1.0f + fast_exp2(x * -1.44269504f));
     dsilu = s * (1.0f + x * (1.0f - s));
     return x * s;
 }
@@ -434,7 +440,7 @@ __device__ __forceinline__ void encode_rows(const KernelArgs &k, const TableView
     int row = 0;
     if (live) {
         const float4 e = pq[slot];
-        const float d2 = e.x * e.x + e.y * e.y + e.z * e.z, rinv = rsqrtf(d2), r = d2 * rinv;
+        const float d2 = e.x * e.x + e.y * e.y + e.z * e.z, rinv = fast_rsqrt(d2), r = d2 * rinv;
         harmonics(e.x * rinv, e.y * rinv, e.z * rinv, h);
         float u;
         const int iv = spline_interval(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, u, k.status);
@@ -625,7 +631,7 @@ __device__ __forceinline__ void derive_rows(const KernelArgs &k, const TableView
     int row = 0;
     if (live) {
         const float4 ent = pq[slot];
-        const float d2 = ent.x * ent.x + ent.y * ent.y + ent.z * ent.z, r = d2 * rsqrtf(d2);
+        const float d2 = ent.x * ent.x + ent.y * ent.y + ent.z * ent.z, r = d2 * fast_rsqrt(d2);
         float u;
         const int iv = spline_interval(r, k.tab.r_min, k.tab.inv_h, k.tab.knots, u, k.status);
         cubic_basis(u, b);
@@ -721,7 +727,7 @@ __device__ __forceinline__ float3 project_pair(const KernelArgs &k, const float4
 #pragma unroll
     for (int q = 0; q < D_ANG; ++q) { v[q] = __uint_as_float(vt[q]); tt[q] = __uint_as_float(vt[16 + q]); }
     const float x = ent.x, y = ent.y, z = ent.z;
-    const float rinv = rsqrtf(x * x + y * y + z * z);
+    const float rinv = fast_rsqrt(x * x + y * y + z * z);
     const int j = __float_as_int(ent.w) & ((1 << J_BITS) - 1);
     const float ux = x * rinv, uy = y * rinv, uz = z * rinv;
     float s, tx, ty, tz, tu;
