@@ -265,9 +265,10 @@ int mlip_create(mlip_ctx **out, const mlip_config *cfg, const double *enc_w, siz
         if (cudaMallocHost((void **)&c->status_host, sizeof(int)) != cudaSuccess ||
             cudaMallocHost((void **)&c->total_host, sizeof(int64_t)) != cudaSuccess ||
             cudaMallocHost((void **)&c->rebuild_host, sizeof(int)) != cudaSuccess ||
-            cudaMallocHost((void **)&c->build_host, sizeof(int) * mlip_ctx::BUILD_WORDS) != cudaSuccess) {
+            cudaMallocHost((void **)&c->build_host, sizeof(int) * (mlip_ctx::BUILD_WORDS + 1)) != cudaSuccess) {
             rc = MLIP_ERR_CUDA; c->err = "pinned host allocation failed"; break;
         }
+        c->build_host[mlip_ctx::BUILD_WORDS] = 0;
         bool ev_ok = true;
         for (int q = 0; q < mlip_ctx::MARKS; ++q) ev_ok = ev_ok && cudaEventCreate(&c->mark_ev[q]) == cudaSuccess;
         ev_ok = ev_ok && cudaEventCreateWithFlags(&c->check_ev, cudaEventDisableTiming) == cudaSuccess;

@@ -127,7 +127,8 @@ struct mlip_ctx {
     unsigned long long *tile_state = nullptr;   // [tile_words(N)] look-back words of the one-pass build
     int *build_word = nullptr;     // {ticket, private overflow flag, total entries (64 bits)} of the one-pass build, then status, rebuild_flag, far_flag, -, species_start
     float4 *rel_pos = nullptr;     // cell-relative positions of the build in progress
-    int *build_host = nullptr;     // pinned copy
+    int *build_host = nullptr;     // pinned copy, and the ticket of the report that wrote it
+    int reports = 0;
     static constexpr int BUILD_WORDS = 8 + mlip::MAX_SPECIES + 1;
     int64_t nbr_cap = 0, n_entries = 0;
     // scratch
