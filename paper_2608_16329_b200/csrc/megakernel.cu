@@ -125,13 +125,13 @@ constexpr int TM_FWD0 = 0, TM_FWD = 64, TM_BWD = 160, TM_BWD0 = 256, TM_VT = 320
 constexpr int HP_TMEM = 4 * TM_VT * 32;
 constexpr int HP_TOTAL = HP_TMEM + (HC_USED + 3) / 4 * 4;
 
-// The hardware's approximations as they are: without -ftz the compiler puts two or three instructions around each for denormal arguments, which do
-// not occur here (squared distances of atoms that do not coincide, 1 + exp(-x)) or come out the same (an exponential below 2^-126 adds nothing
-// to 1).  One evaluation of 1,000,188 atoms 7479 -> 7439 us, of 256,000 with 54 pairs 1634 -> 1621.
+// The PTX ISA's approximations in their .ftz forms, which take subnormal arguments and results for zero.  Such arguments do not occur here
+// (squared distances of atoms that do not coincide, 1 + exp(-x)) or change nothing (an exponential below 2^-126 adds nothing to 1).
+// One evaluation with rsqrtf, __expf and __fdividef / with these: 1,000,188 atoms 7479 / 7439 us, 256,000 with 54 pairs 1634 / 1621.
 __device__ __forceinline__ float fast_rsqrt(float x) { float y; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ float fast_rcp(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ float fast_exp2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
-// SiLU and its derivative.  exp through the fast exponential: its error scales with |x| 2^-24 and
+// SiLU and its derivative.  exp(-x) as 2^(-x log2 e) through the fast exponential: its error scales with |x| 2^-24 and
 // enters the sigmoid damped by s (1 - s), far below fp32 rounding of the surrounding sums.
 __device__ __forceinline__ float silu_f(float x, float &dsilu) {
     const float s = fast_rcp(1.0f + fast_exp2(x * -1.44269504f));
