@@ -881,7 +881,7 @@ __global__ void __launch_bounds__(LN_THREADS) k_neighbors_lanes(int64_t n, CellG
                             }
                             if (hit) {
                                 const bool near = v < near2;
-                                if (near_at <= far_at) asm volatile("st.shared.u16 [%0], %1;" ::"r"(near ? near_at : far_at), "r"(code + c0 + e));
+                                if (near_at <= far_at) asm volatile("st.shared.u16 [%0], %1;" ::"r"(near ? near_at : far_at), "r"(code + c0 + e) : "memory");
                                 if (near) near_at += 2; else far_at -= 2;
                             }
                         }
@@ -890,9 +890,9 @@ __global__ void __launch_bounds__(LN_THREADS) k_neighbors_lanes(int64_t n, CellG
                         for (int e = 0; e < 8; ++e) {
                             const float v = e & 1 ? d2[e >> 1].y : d2[e >> 1].x;
                             if (OWN) asm volatile("{.reg .pred h, nr, fr; .reg .u32 at; setp.ne.s32 h, %5, %6; setp.le.and.f32 h, %2, %3, h;" MLIP_APPEND
-                                                  : "+r"(near_at), "+r"(far_at) : "f"(v), "f"(rl2_hi), "f"(near2), "r"(code + c0 + e), "r"(self));
+                                                  : "+r"(near_at), "+r"(far_at) : "f"(v), "f"(rl2_hi), "f"(near2), "r"(code + c0 + e), "r"(self) : "memory");
                             else asm volatile("{.reg .pred h, nr, fr; .reg .u32 at; setp.le.f32 h, %2, %3;" MLIP_APPEND
-                                              : "+r"(near_at), "+r"(far_at) : "f"(v), "f"(rl2_hi), "f"(near2), "r"(code + c0 + e));
+                                              : "+r"(near_at), "+r"(far_at) : "f"(v), "f"(rl2_hi), "f"(near2), "r"(code + c0 + e) : "memory");
                         }
                     }
                 }
