@@ -1,0 +1,29 @@
+// Which single traversal builds a system's neighbor lists.  Host arithmetic only: the rule compiles by itself.
+#pragma once
+#include <stdint.h>
+
+#include <algorithm>
+
+namespace mlip {
+
+// One atom or eight, one after the other, to a warp (tiles of 8 / 64 atoms, k_neighbors_onepass), or one to a lane (tiles of 64, k_neighbors_lanes).
+enum class ListForm { WARP_1, WARP_8, LANES };
+constexpr int list_form_tile(ListForm f) { return f == ListForm::WARP_1 ? 8 : 64; }
+
+// One atom to a warp in small systems, where eight traversals one after the other are the kernel's time; from there on one to a lane (grids of three
+// cells per dimension and more, `rel`).  Whole build on the device in us, one atom to a warp / to a lane: 6 species 6,912 atoms 80 / 126, 10,976 101 /
+// 129, 16,384 125 / 128, 32,000 186 / 140; one species 8,192 81 / 113, 16,000 115 / 114, 31,250 164 / 125; three 32,768 176 / 118.
+constexpr int64_t LANES_FROM = 18000;
+// Thinner grids have no form with an atom to a lane: eight to a warp once such tiles fill the SMs.  Two cells across, one atom to a warp / eight: 6 species
+// 19,008 atoms 136 / 194, 26,896 154 / 186, 38,416 195 / 214, 48,400 232 / 303; one species 18,490 114 / 146, 36,000 164 / 165, 47,610 208 / 252.
+constexpr int64_t WARP_8_FROM = 50000;
+
+inline ListForm list_form(int64_t n, bool rel) {
+    if (rel) return n < LANES_FROM ? ListForm::WARP_1 : ListForm::LANES;
+    return n < WARP_8_FROM ? ListForm::WARP_1 : ListForm::WARP_8;
+}
+
+// Look-back words that builds of up to n atoms need, whatever their form.
+inline int64_t list_tile_words(int64_t n) { return std::max(n / 64, std::min(n, WARP_8_FROM) / 8) + 2; }
+
+}  // namespace mlip

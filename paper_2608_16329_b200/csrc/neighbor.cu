@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "list_form.cuh"
 #include "scan.cuh"
 
 namespace mlip {
@@ -648,7 +649,6 @@ __device__ __forceinline__ int onepass_traverse(int64_t i, const CellGrid &g, do
     return cnt;
 }
 
-constexpr int64_t ONEPASS_SMALL = 18000;   // see onepass_per_warp
 constexpr int OP_BUF = 160;   // hits kept per atom in shared memory; a longer list is traversed again straight into global memory
 
 template <bool REL, int PER_WARP, typename ENTRY>
@@ -1156,17 +1156,12 @@ static int refuse_broken_input(mlip_ctx *c, cudaStream_t s) {
     return MLIP_ERR_NONFINITE;
 }
 
-int64_t tile_words(int64_t n) { return std::max(n / OP_TILE, std::min(n, ONEPASS_SMALL) / 8) + 2; }
+int64_t tile_words(int64_t n) { return list_tile_words(n); }
+static_assert(list_form_tile(ListForm::LANES) == OP_TILE, "tiles");
 
-// Atoms per warp of the one-pass traversal (tiles of eight warps): one in small systems, where eight traversals one after the other
-// are the kernel's time; from there on tiles of 64 atoms, eight to a warp or (grids of three cells per dimension and more, k_neighbors_lanes) one to
-// a lane.  Whole build on the device in us, one atom to a warp / to a lane: 6 species 6,912 atoms 80 / 126, 10,976 101 / 129, 16,384 125 / 128, 32,000
-// 186 / 140; one species 8,192 81 / 113, 16,000 115 / 114, 31,250 164 / 125; three 32,768 176 / 118.  Eight atoms to a warp / one to a lane:
-// 6 species 55,296 atoms 317 / 162, 108,000 468 / 271, 1,000,188 2801 / 1379, 8,001,504 21,470 / 9874; three 1,953,125 5406 / 1911; one 65,536
-// 252 / 140.
-static int onepass_per_warp(const mlip_ctx *c) {
-    if (c->lookback_unpublished_tile >= 0 || c->lookback_spin_limit > 0) return 8;   // (diagnostics name 64-atom tiles)
-    return c->n < ONEPASS_SMALL ? 1 : 8;
+static ListForm form_of(const mlip_ctx *c, bool rel) {
+    if (c->lookback_unpublished_tile >= 0 || c->lookback_spin_limit > 0) return rel ? ListForm::LANES : ListForm::WARP_8;   // (diagnostics name 64-atom tiles)
+    return list_form(c->n, rel);
 }
 
 template <bool REL, int PER_WARP, typename ENTRY>
@@ -1218,8 +1213,8 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
     EvalClear clear_forces = eval_clear(c);
     if (rel && clear_forces.force == relpos) { clear_forces.force = nullptr; c->force_cleared = false; }
     c->rel_pos = relpos;
-    const int per_warp = onepass_per_warp(c);
-    const BuildClear clear{c->tile_state, (n + 8 * per_warp - 1) / (8 * per_warp), c->build_word, c->far_flag, c->rebuild_flag};
+    const ListForm form = form_of(c, rel);
+    const BuildClear clear{c->tile_state, (n + list_form_tile(form) - 1) / list_form_tile(form), c->build_word, c->far_flag, c->rebuild_flag};
     const int64_t n_bins = (int64_t)C * g.n_cells;
     if (n <= SMALL_ATOMS && g.n_cells <= SMALL_CELLS && n_bins <= SMALL_BINS) {
         const size_t smem = sizeof(int) * (size_t)(g.n_cells + 1 + n_bins + 1 + n);
@@ -1260,10 +1255,10 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
     if (c->nbr_cap > 0) {
         int *flag = allow_sync_grow ? c->build_word + 1 : c->status;
         int rc = MLIP_OK;
-        if (rel && per_warp == 8) rc = list16 ? launch_lanes(c, nbr16, flag, rl, near2, s) : launch_lanes(c, c->nbr, flag, rl, near2, s);
+        if (form == ListForm::LANES) rc = list16 ? launch_lanes(c, nbr16, flag, rl, near2, s) : launch_lanes(c, c->nbr, flag, rl, near2, s);
         else if (list16) launch_onepass<true, 1, uint16_t>(c, nbr16, flag, rl, near2, s);
         else if (rel) launch_onepass<true, 1, int32_t>(c, c->nbr, flag, rl, near2, s);
-        else per_warp == 1 ? launch_onepass<false, 1, int32_t>(c, c->nbr, flag, rl, near2, s) : launch_onepass<false, 8, int32_t>(c, c->nbr, flag, rl, near2, s);
+        else form == ListForm::WARP_1 ? launch_onepass<false, 1, int32_t>(c, c->nbr, flag, rl, near2, s) : launch_onepass<false, 8, int32_t>(c, c->nbr, flag, rl, near2, s);
         if (rc != MLIP_OK) return rc;
         MLIP_CUDA_TRY(c, cudaGetLastError());
         bool done = true;

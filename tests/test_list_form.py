@@ -1,0 +1,41 @@
+"""Which traversal builds a system's lists: the rule, compiled by itself, against the times that were measured at its lines."""
+import subprocess
+
+import pytest
+
+from conftest import ROOT
+
+PROGRAM = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "list_form.cuh"
+int main(int argc, char **argv) {
+    const int64_t n = atoll(argv[1]);
+    const mlip::ListForm f = mlip::list_form(n, atoi(argv[2]) != 0);
+    printf("%s %lld %lld\n", f == mlip::ListForm::WARP_1 ? "warp 1" : f == mlip::ListForm::WARP_8 ? "warp 8" : "lanes", (long long)((n + mlip::list_form_tile(f) - 1) / mlip::list_form_tile(f)), (long long)mlip::list_tile_words(n));
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    d = tmp_path_factory.mktemp("list_form")
+    (d / "rule.cpp").write_text(PROGRAM)
+    subprocess.check_call(["g++", "-std=c++17", "-I", f"{ROOT}/paper_2608_16329_b200/csrc", "-o", str(d / "rule"), str(d / "rule.cpp")])
+
+    def ask(n, cells):
+        rel = all(c >= 3 for c in cells)
+        form, tiles, words = subprocess.check_output([str(d / "rule"), str(n), str(int(rel))], text=True).strip().rsplit(" ", 2)
+        assert int(tiles) <= int(words)   # every tile has its look-back word
+        return form
+    return ask
+
+
+@pytest.mark.parametrize("n,form", [(1, "warp 1"), (17999, "warp 1"), (18400, "warp 1"), (38416, "warp 1"), (49999, "warp 1"), (50000, "warp 8"), (1000000, "warp 8")])
+def test_grids_of_two_cells_across(rule, n, form):
+    assert rule(n, (2, 60, 60)) == form
+
+
+@pytest.mark.parametrize("n,cells,form", [(17999, (9, 9, 9), "warp 1"), (19652, (8, 8, 8), "lanes"), (8001504, (64, 64, 64), "lanes")])
+def test_condensed_systems(rule, n, cells, form):
+    assert rule(n, cells) == form
