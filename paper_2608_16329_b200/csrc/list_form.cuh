@@ -23,6 +23,17 @@ inline ListForm list_form(int64_t n, bool rel) {
     return n < WARP_8_FROM ? ListForm::WARP_1 : ListForm::WARP_8;
 }
 
+// Row of a lane (k_neighbors_lanes), in entries, a multiple of four: the mean list at the box's density and 30 percent (lattice shells, composition),
+// and where the shared memory of the SMs holds longer rows for all of the tiles at once, those: a list longer than its row is traversed again, and in
+// systems of uneven density many are.  Whole build in us with rows from the mean alone / with these: a crystal of 134-entry lists filling half of its box
+// 19,652 atoms 252 / 124, 55,296 280 / 150, 78,732 352 / 200; a ball of 26,573 238 / 120; filling its box 19,652 129 / 128, 108,000 271 / 271.
+constexpr int LANE_ROW_MOST = 640, LANE_SMEM = 227 * 1024, LANE_SMEM_FIXED = 3 * 1024 + 512;   // per SM; per tile besides the rows (staging, scan, reserved)
+inline int list_lane_row(int64_t n, double mean, int sms) {
+    const int64_t tiles = (n + 63) / 64, per_sm = (tiles + sms - 1) / sms;
+    const int64_t all_at_once = (LANE_SMEM / per_sm - LANE_SMEM_FIXED) / (64 * 2) - 2;
+    return (int)std::min(std::max({(int64_t)(1.3 * mean) + 16, all_at_once, (int64_t)64}), (int64_t)LANE_ROW_MOST) / 4 * 4;
+}
+
 // Look-back words that builds of up to n atoms need, whatever their form.
 inline int64_t list_tile_words(int64_t n) { return std::max(n / 64, std::min(n, WARP_8_FROM) / 8) + 2; }
 

@@ -727,7 +727,12 @@ __global__ void __launch_bounds__(256) k_neighbors_onepass(int64_t n, CellGrid g
 // follow one another along z, so the cells around them are nine columns of (cells spanned + 2) layers; a lane takes part in the
 // three layers around its own cell only.  Each lane meets the candidates in the order of the warp-per-atom traversal, with the same
 // arithmetic, so the lists agree entry by entry.
-// Rows hold 16-bit codes (near hits from the front, far hits from the back); `buf` entries, a multiple of four, from the mean density.
+// Rows hold 16-bit codes (near hits from the front, far hits from the back); `buf` entries, a multiple of four (list_lane_row).  A list that its row may
+// not hold is counted to its end and then traversed a second time, in the same way, straight into its place in the array: systems of uneven density,
+// whose lists are longer than the mean tells, cost no more than with an atom to a warp.  Whole build in us, 8 atoms to a warp / one to a lane:
+// 108,000 atoms filling their box 470 / 271, half of it 472 / 390, a quarter 469 / 414; 1,000,188 in half of their box 2801 / 2212; 97,336 of
+// 274-entry lists in half of theirs 1298 / 768; a ball of 123,161 in 161 Angstrom 445 / 380.  (Rows of 160 entries at least would hold more of those lists,
+// 266 us for the first half-empty box, but fewer tiles fit an SM where lists are short: one species 432,000 atoms 519 / 563.)
 constexpr int LN_WARPS = OP_TILE / 32, LN_THREADS = 32 * LN_WARPS;
 constexpr int LN_SPAN = 4;                          // cells along z that a group of lanes may span: 9 x 6 cells, two to a lane
 constexpr int LN_STAGE = 2 * 3 * 32;                // two chunks of candidates, x, y, z
@@ -791,119 +796,135 @@ __global__ void __launch_bounds__(LN_THREADS) k_neighbors_lanes(int64_t n, CellG
         cx = cell_coord(p.x, g.inv_edge[0], g.n[0]); cy = cell_coord(p.y, g.inv_edge[1], g.n[1]); cz = cell_coord(p.z, g.inv_edge[2], g.n[2]);
     }
     const float rl2_mid = (float)rl2, band = (float)(rl2 * 1.1e-5);
-    // shared-memory addresses of the places for the next near and the next far hit; once they have crossed nothing is stored, only counted
+    // shared-memory addresses of the places for the next near and the next far hit.  Where the two might cross the lane begins its row again: from
+    // there on it counts, and its list is traversed a second time.
     const int row_at = (int)__cvta_generic_to_shared(row), row_end = row_at + 2 * (buf - 1);
-    int near_at = row_at, far_at = row_end;
-    for (unsigned left = __ballot_sync(0xffffffffu, live); left;) {   // groups of lanes with cells along one column
-        const int lead = __ffs(left) - 1;
-        const int X = __shfl_sync(0xffffffffu, cx, lead), Y = __shfl_sync(0xffffffffu, cy, lead), Z = __shfl_sync(0xffffffffu, cz, lead);
-        const bool mine = (left >> lane & 1u) && cx == X && cy == Y && cz - Z < LN_SPAN;   // (atoms come in cell order: cz >= Z)
-        const unsigned group = __ballot_sync(0xffffffffu, mine);
-        left &= ~group;
-        const int layers = __shfl_sync(0xffffffffu, cz, 31 - __clz(group)) - Z + 3, per_column = 65536 / layers + 1;
-        // atom range of the q-th cell of the walk (columns in x, y order, layers Z - 1 .. upwards)
-        auto range = [&](int q, int &b, int &e) {
-            b = e = 0;
-            if (q >= 9 * layers) return;
-            const int col = q * per_column >> 16;
-            int x = X + col / 3 - 1, y = Y + col % 3 - 1, z = Z + (q - col * layers) - 1;
-            x = x < 0 ? x + g.n[0] : (x >= g.n[0] ? x - g.n[0] : x);
-            y = y < 0 ? y + g.n[1] : (y >= g.n[1] ? y - g.n[1] : y);
-            z = z < 0 ? z + g.n[2] : (z >= g.n[2] ? z - g.n[2] : z);
-            const int c = (x * g.n[1] + y) * g.n[2] + z;
-            b = cell_start[c]; e = cell_start[c + 1];
-        };
-        int beg0, end0, beg1, end1;
-        range(lane, beg0, end0);
-        range(lane + 32, beg1, end1);
-        unsigned long long cells = __ballot_sync(0xffffffffu, end0 > beg0) | (unsigned long long)__ballot_sync(0xffffffffu, end1 > beg1) << 32;
-        int q = 0, cell_beg = 0, base = 0, end = 0;   // the chunk being fetched: atoms base .. of cell q
-        auto advance = [&]() {
-            base += 32;
-            if (base < end) return true;
-            if (!cells) return false;
-            q = __ffsll(cells) - 1;
-            cells &= cells - 1;
-            cell_beg = base = __shfl_sync(0xffffffffu, q < 32 ? beg0 : beg1, q & 31);
-            end = __shfl_sync(0xffffffffu, q < 32 ? end0 : end1, q & 31);
-            return true;
-        };
-        const float4 nobody = make_float4(FAR_AWAY, FAR_AWAY, FAR_AWAY, 0.f);
-        bool more = advance();
-        float4 r = more && base + lane < end ? rel[base + lane] : nobody;
-        for (int parity = 0; more; parity ^= 1) {
-            const int col = q * per_column >> 16, dz = Z + (q - col * layers) - 1 - cz, chunk = base, pos = base - cell_beg, m = min(32, end - base);
-            float *st = stage + parity * (LN_STAGE / 2);
-            st[lane] = r.x; st[32 + lane] = r.y; st[64 + lane] = r.z;
-            more = advance();
-            if (more) r = base + lane < end ? rel[base + lane] : nobody;
-            // separation = x_rel(j) + shift, shift = (cell offset) * edge - x_rel(i)
-            const bool in = mine && dz >= -1 && dz <= 1;
-            const float sx = in ? (float)(col / 3 - 1) * edge[0] - ri.x : FAR_AWAY;
-            const float sy = (float)(col % 3 - 1) * edge[1] - ri.y;
-            const float sz = (float)dz * edge[2] - ri.z;
-            const int code = ((3 * col + dz + 1) << L16_SHIFT) + pos;
-            const int self = dz == 0 ? code + (int)(i - chunk) : -1;   // (the central column) the lane's own atom
-            __syncwarp();   // (the buffer before last was read before the last one's barrier)
-            // the hit's code (%5) to the near (%0) or far (%1) place, which moves on; predicate h: hit
+    int near_at = row_at, far_at = row_end, near_lost = 0, lost = 0;   // lost: hits whose places were given to others
+    // second traversal: places in the list itself, of which `fit` are written
+    ENTRY *list = nullptr;
+    int near_next = 0, far_next = 0, fit = 0;
+    auto traverse = [&](auto second_traversal, bool part) {
+        constexpr bool SECOND = decltype(second_traversal)::value;
+        for (unsigned left = __ballot_sync(0xffffffffu, part); left;) {   // groups of lanes with cells along one column
+            const int lead = __ffs(left) - 1;
+            const int X = __shfl_sync(0xffffffffu, cx, lead), Y = __shfl_sync(0xffffffffu, cy, lead), Z = __shfl_sync(0xffffffffu, cz, lead);
+            const bool mine = (left >> lane & 1u) && cx == X && cy == Y && cz - Z < LN_SPAN;   // (atoms come in cell order: cz >= Z)
+            const unsigned group = __ballot_sync(0xffffffffu, mine);
+            left &= ~group;
+            const int layers = __shfl_sync(0xffffffffu, cz, 31 - __clz(group)) - Z + 3, per_column = 65536 / layers + 1;
+            // atom range of the q-th cell of the walk (columns in x, y order, layers Z - 1 .. upwards)
+            auto range = [&](int q, int &b, int &e) {
+                b = e = 0;
+                if (q >= 9 * layers) return;
+                const int col = q * per_column >> 16;
+                int x = X + col / 3 - 1, y = Y + col % 3 - 1, z = Z + (q - col * layers) - 1;
+                x = x < 0 ? x + g.n[0] : (x >= g.n[0] ? x - g.n[0] : x);
+                y = y < 0 ? y + g.n[1] : (y >= g.n[1] ? y - g.n[1] : y);
+                z = z < 0 ? z + g.n[2] : (z >= g.n[2] ? z - g.n[2] : z);
+                const int c = (x * g.n[1] + y) * g.n[2] + z;
+                b = cell_start[c]; e = cell_start[c + 1];
+            };
+            int beg0, end0, beg1, end1;
+            range(lane, beg0, end0);
+            range(lane + 32, beg1, end1);
+            unsigned long long cells = __ballot_sync(0xffffffffu, end0 > beg0) | (unsigned long long)__ballot_sync(0xffffffffu, end1 > beg1) << 32;
+            int q = 0, cell_beg = 0, base = 0, end = 0;   // the chunk being fetched: atoms base .. of cell q
+            auto advance = [&]() {
+                base += 32;
+                if (base < end) return true;
+                if (!cells) return false;
+                q = __ffsll(cells) - 1;
+                cells &= cells - 1;
+                cell_beg = base = __shfl_sync(0xffffffffu, q < 32 ? beg0 : beg1, q & 31);
+                end = __shfl_sync(0xffffffffu, q < 32 ? end0 : end1, q & 31);
+                return true;
+            };
+            const float4 nobody = make_float4(FAR_AWAY, FAR_AWAY, FAR_AWAY, 0.f);
+            bool more = advance();
+            float4 r = more && base + lane < end ? rel[base + lane] : nobody;
+            for (int parity = 0; more; parity ^= 1) {
+                const int col = q * per_column >> 16, dz = Z + (q - col * layers) - 1 - cz, chunk = base, pos = base - cell_beg, m = min(32, end - base);
+                float *st = stage + parity * (LN_STAGE / 2);
+                st[lane] = r.x; st[32 + lane] = r.y; st[64 + lane] = r.z;
+                more = advance();
+                if (more) r = base + lane < end ? rel[base + lane] : nobody;
+                // separation = x_rel(j) + shift, shift = (cell offset) * edge - x_rel(i)
+                const bool in = mine && dz >= -1 && dz <= 1;
+                const float sx = in ? __fmaf_rn((float)(col / 3 - 1), edge[0], -ri.x) : FAR_AWAY;   // (rounded alike in both traversals)
+                const float sy = __fmaf_rn((float)(col % 3 - 1), edge[1], -ri.y);
+                const float sz = __fmaf_rn((float)dz, edge[2], -ri.z);
+                const int code = ((3 * col + dz + 1) << L16_SHIFT) + pos;
+                const int self = dz == 0 ? code + (int)(i - chunk) : -1;   // (the central column) the lane's own atom
+                __syncwarp();   // (the buffer before last was read before the last one's barrier)
+                // the hit's code (%5) to the near (%0) or far (%1) place, which moves on; predicate h: hit
 #define MLIP_APPEND " setp.lt.and.f32 nr, %2, %4, h; setp.ge.and.f32 fr, %2, %4, h; selp.u32 at, %0, %1, nr;" \
                     " @h st.shared.u16 [at], %5; @nr add.s32 %0, %0, 2; @fr sub.s32 %1, %1, 2;}"
-            auto test = [&](auto own_column) {
-                constexpr bool OWN = decltype(own_column)::value;
-                for (int c0 = 0; c0 < m; c0 += 8) {   // (a chunk's places behind its last candidate are out of reach)
-                    float2 d2[4];
+                auto test = [&](auto own_column) {
+                    constexpr bool OWN = decltype(own_column)::value;
+                    for (int c0 = 0; c0 < m; c0 += 8) {   // (a chunk's places behind its last candidate are out of reach)
+                        float2 d2[4];
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const float4 x = *reinterpret_cast<const float4 *>(st + c0 + 4 * h), y = *reinterpret_cast<const float4 *>(st + 32 + c0 + 4 * h),
-                                     z = *reinterpret_cast<const float4 *>(st + 64 + c0 + 4 * h);
-                        d2[2 * h] = pack_norm2(pack_add(make_float2(x.x, x.y), sx), pack_add(make_float2(y.x, y.y), sy), pack_add(make_float2(z.x, z.y), sz));
-                        d2[2 * h + 1] = pack_norm2(pack_add(make_float2(x.z, x.w), sx), pack_add(make_float2(y.z, y.w), sy), pack_add(make_float2(z.z, z.w), sz));
-                    }
-                    float closest = 3.0e38f;   // to the list radius
+                        for (int h = 0; h < 2; ++h) {
+                            const float4 x = *reinterpret_cast<const float4 *>(st + c0 + 4 * h), y = *reinterpret_cast<const float4 *>(st + 32 + c0 + 4 * h),
+                                         z = *reinterpret_cast<const float4 *>(st + 64 + c0 + 4 * h);
+                            d2[2 * h] = pack_norm2(pack_add(make_float2(x.x, x.y), sx), pack_add(make_float2(y.x, y.y), sy), pack_add(make_float2(z.x, z.y), sz));
+                            d2[2 * h + 1] = pack_norm2(pack_add(make_float2(x.z, x.w), sx), pack_add(make_float2(y.z, y.w), sy), pack_add(make_float2(z.z, z.w), sz));
+                        }
+                        float closest = 3.0e38f;   // to the list radius
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float2 off = pack_add(d2[e], -rl2_mid);
-                        closest = fminf(closest, fminf(fabsf(off.x), fabsf(off.y)));
-                    }
-                    if (__any_sync(0xffffffffu, closest <= band || far_at - near_at < 2 * 7)) {
-                        // a candidate within 1e-5 of the list radius, where the exact predicate on the full positions decides, or a row
-                        // that may end among the eight
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 off = pack_add(d2[e], -rl2_mid);
+                            closest = fminf(closest, fminf(fabsf(off.x), fabsf(off.y)));
+                        }
+                        if (!SECOND && far_at - near_at < 2 * 7) {
+                            near_lost += (near_at - row_at) >> 1;
+                            lost += ((near_at - row_at) >> 1) + ((row_end - far_at) >> 1);
+                            near_at = row_at; far_at = row_end;
+                        }
+                        if (SECOND || __any_sync(0xffffffffu, closest <= band)) {
+                            // a candidate within 1e-5 of the list radius: the exact predicate on the full positions decides
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const float v = e & 1 ? d2[e >> 1].y : d2[e >> 1].x;
-                            bool hit = v <= rl2_hi && !(OWN && code + c0 + e == self);
-                            if (hit && v >= rl2_lo) {
-                                const double4 pi = pos4[i], pj = pos4[chunk + c0 + e];
-                                const double ex = min_image(__dsub_rn(pj.x, pi.x), g.box[0], g.half[0]);
-                                const double ey = min_image(__dsub_rn(pj.y, pi.y), g.box[1], g.half[1]);
-                                const double ez = min_image(__dsub_rn(pj.z, pi.z), g.box[2], g.half[2]);
-                                hit = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez)) < rl2;
-                            }
-                            if (hit) {
+                            for (int e = 0; e < 8; ++e) {
+                                const float v = e & 1 ? d2[e >> 1].y : d2[e >> 1].x;
+                                bool hit = v <= rl2_hi && !(OWN && code + c0 + e == self);
+                                if (hit && v >= rl2_lo) {
+                                    const double4 pi = pos4[i], pj = pos4[chunk + c0 + e];
+                                    const double ex = min_image(__dsub_rn(pj.x, pi.x), g.box[0], g.half[0]);
+                                    const double ey = min_image(__dsub_rn(pj.y, pi.y), g.box[1], g.half[1]);
+                                    const double ez = min_image(__dsub_rn(pj.z, pi.z), g.box[2], g.half[2]);
+                                    hit = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez)) < rl2;
+                                }
                                 const bool near = v < near2;
-                                if (near_at <= far_at) asm volatile("st.shared.u16 [%0], %1;" ::"r"(near ? near_at : far_at), "r"(code + c0 + e) : "memory");
-                                if (near) near_at += 2; else far_at -= 2;
+                                if (SECOND) {
+                                    const int at = near ? near_next : far_next;
+                                    if (hit && (unsigned)at < (unsigned)fit) list[at] = (ENTRY)(sizeof(ENTRY) == 4 ? chunk + c0 + e : code + c0 + e);
+                                    near_next += hit && near; far_next -= hit && !near;
+                                } else if (hit) {
+                                    asm volatile("st.shared.u16 [%0], %1;" ::"r"(near ? near_at : far_at), "r"(code + c0 + e) : "memory");
+                                    if (near) near_at += 2; else far_at -= 2;
+                                }
+                            }
+                        } else {   // no branches: few lanes have a hit, and a divergent branch costs more than the instructions it skips
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) {
+                                const float v = e & 1 ? d2[e >> 1].y : d2[e >> 1].x;
+                                if (OWN) asm volatile("{.reg .pred h, nr, fr; .reg .u32 at; setp.ne.s32 h, %5, %6; setp.le.and.f32 h, %2, %3, h;" MLIP_APPEND
+                                                      : "+r"(near_at), "+r"(far_at) : "f"(v), "f"(rl2_hi), "f"(near2), "r"(code + c0 + e), "r"(self) : "memory");
+                                else asm volatile("{.reg .pred h, nr, fr; .reg .u32 at; setp.le.f32 h, %2, %3;" MLIP_APPEND
+                                                  : "+r"(near_at), "+r"(far_at) : "f"(v), "f"(rl2_hi), "f"(near2), "r"(code + c0 + e) : "memory");
                             }
                         }
-                    } else {   // no branches: few lanes have a hit, and a divergent branch costs more than the instructions it skips
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const float v = e & 1 ? d2[e >> 1].y : d2[e >> 1].x;
-                            if (OWN) asm volatile("{.reg .pred h, nr, fr; .reg .u32 at; setp.ne.s32 h, %5, %6; setp.le.and.f32 h, %2, %3, h;" MLIP_APPEND
-                                                  : "+r"(near_at), "+r"(far_at) : "f"(v), "f"(rl2_hi), "f"(near2), "r"(code + c0 + e), "r"(self) : "memory");
-                            else asm volatile("{.reg .pred h, nr, fr; .reg .u32 at; setp.le.f32 h, %2, %3;" MLIP_APPEND
-                                              : "+r"(near_at), "+r"(far_at) : "f"(v), "f"(rl2_hi), "f"(near2), "r"(code + c0 + e) : "memory");
-                        }
                     }
-                }
-            };
+                };
 #undef MLIP_APPEND
-            if (col == 4) test(std::true_type{});
-            else test(std::false_type{});
+                if (col == 4) test(std::true_type{});
+                else test(std::false_type{});
+            }
+            __syncwarp();   // (the next group's first chunk may go where a lane still reads)
         }
-        __syncwarp();   // (the next group's first chunk may go where a lane still reads)
-    }
-    const int cn = (near_at - row_at) >> 1, cnt = cn + ((row_end - far_at) >> 1);   // near hits, hits
+    };
+    traverse(std::false_type{}, live);
+    const int cn = near_lost + ((near_at - row_at) >> 1), cnt = lost + ((near_at - row_at) >> 1) + ((row_end - far_at) >> 1);   // near hits, hits
     s_cnt[32 * warp + lane] = cnt;
     __syncthreads();
     if (warp == 0) tile_offsets<OP_TILE>(tile, s_cnt, s_off, &s_prefix, &s_total, status, tile_state, spin_limit, unpublished_tile, lane);
@@ -915,7 +936,7 @@ __global__ void __launch_bounds__(LN_THREADS) k_neighbors_lanes(int64_t n, CellG
 
     // ---- write the lists: full rows from shared memory ----
     const long long off = s_prefix + s_off[32 * warp + lane];
-    int fit = cnt;   // entries of this list that the array still holds
+    fit = cnt;   // entries of this list that the array still holds
     if (i < n) {
         if (off + cnt > nbr_cap) {
             atomicOr(status, FLAG_NEIGHBOR_OVERFLOW);
@@ -924,16 +945,16 @@ __global__ void __launch_bounds__(LN_THREADS) k_neighbors_lanes(int64_t n, CellG
         nbr_off[i] = off < nbr_cap ? off : nbr_cap;
         nbr_near[i] = cn < fit ? cn : fit;
     }
+    if (__any_sync(0xffffffffu, lost > 0)) {   // lists longer than their rows, straight to their places
+        list = nbr + off; far_next = cnt - 1;
+        traverse(std::true_type{}, lost > 0);
+        if (lost > 0) fit = 0;
+    }
     int cell_of_bases = -1, bases = 0;   // lane q < 27: first atom of the q-th cell around that cell
     for (int a = 0; a < 32; ++a) {
         const int m = __shfl_sync(0xffffffffu, fit, a), all = __shfl_sync(0xffffffffu, cnt, a), near = __shfl_sync(0xffffffffu, cn, a);
-        if (m == 0) continue;   // (atoms beyond the last and ghosts have none either)
+        if (m == 0) continue;   // (written above; atoms beyond the last and ghosts have none either)
         const long long to = __shfl_sync(0xffffffffu, off, a);
-        if (all > buf) {
-            int ignored;
-            onepass_traverse<true, ENTRY, ENTRY>(first + a, g, rl2, edge, rl2_lo, rl2_hi, pos4, rel, cell_start, lane, nbr + to, all - 1, m, near2, ignored);
-            continue;
-        }
         if (sizeof(ENTRY) == 4) {
             const int X = __shfl_sync(0xffffffffu, cx, a), Y = __shfl_sync(0xffffffffu, cy, a), Z = __shfl_sync(0xffffffffu, cz, a);
             const int cell = (X * g.n[1] + Y) * g.n[2] + Z;
@@ -1174,17 +1195,16 @@ static void launch_onepass(mlip_ctx *c, ENTRY *nbr, int *flag, double rl, float 
     c->launches += 1;
 }
 
-// Row of a lane: the mean list at the system's density and 30 percent (lattice shells, composition), in entries.  Longer lists are traversed again.
 static int lanes_row(const mlip_ctx *c, double rl) {
-    const double volume = c->grid.box[0] * c->grid.box[1] * c->grid.box[2], mean = (double)c->n / volume * (4.0 / 3.0 * 3.14159265358979 * rl * rl * rl);
-    return std::min(std::max((int)(1.3 * mean) + 16, 64), 640) / 4 * 4;
+    const double volume = c->grid.box[0] * c->grid.box[1] * c->grid.box[2];
+    return list_lane_row(c->n, (double)c->n / volume * (4.0 / 3.0 * 3.14159265358979 * rl * rl * rl), c->n_sm);
 }
 
 template <typename ENTRY>
 static int launch_lanes(mlip_ctx *c, ENTRY *nbr, int *flag, double rl, float near2, cudaStream_t s) {
     const int spin = c->lookback_spin_limit > 0 ? c->lookback_spin_limit : OP_SPIN, buf = lanes_row(c, rl);
     const size_t smem = ln_smem(buf);
-    if (smem > 40000) MLIP_CUDA_TRY(c, cudaFuncSetAttribute(k_neighbors_lanes<ENTRY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ln_smem(640)));
+    if (smem > 40000) MLIP_CUDA_TRY(c, cudaFuncSetAttribute(k_neighbors_lanes<ENTRY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ln_smem(LANE_ROW_MOST)));
     k_neighbors_lanes<ENTRY><<<(unsigned)((c->n + OP_TILE - 1) / OP_TILE), LN_THREADS, smem, s>>>(
         c->n, c->grid, rl * rl, c->pos4, c->rel_pos, c->cell_start, c->nbr_off, nbr, c->nbr_cap, flag, c->tile_state, c->build_word, c->status, spin,
         c->lookback_unpublished_tile, near2, c->nbr_near, c->user_of, (int32_t)c->n_owned, buf);

@@ -11,6 +11,7 @@ PROGRAM = r"""
 #include "list_form.cuh"
 int main(int argc, char **argv) {
     const int64_t n = atoll(argv[1]);
+    if (argc == 4) { printf("%d\n", mlip::list_lane_row(n, atof(argv[2]), atoi(argv[3]))); return 0; }
     const mlip::ListForm f = mlip::list_form(n, atoi(argv[2]) != 0);
     printf("%s %lld %lld\n", f == mlip::ListForm::WARP_1 ? "warp 1" : f == mlip::ListForm::WARP_8 ? "warp 8" : "lanes", (long long)((n + mlip::list_form_tile(f) - 1) / mlip::list_form_tile(f)), (long long)mlip::list_tile_words(n));
 }
@@ -18,14 +19,18 @@ int main(int argc, char **argv) {
 
 
 @pytest.fixture(scope="module")
-def rule(tmp_path_factory):
+def program(tmp_path_factory):
     d = tmp_path_factory.mktemp("list_form")
     (d / "rule.cpp").write_text(PROGRAM)
     subprocess.check_call(["g++", "-std=c++17", "-I", f"{ROOT}/paper_2608_16329_b200/csrc", "-o", str(d / "rule"), str(d / "rule.cpp")])
+    return str(d / "rule")
 
+
+@pytest.fixture(scope="module")
+def rule(program):
     def ask(n, cells):
         rel = all(c >= 3 for c in cells)
-        form, tiles, words = subprocess.check_output([str(d / "rule"), str(n), str(int(rel))], text=True).strip().rsplit(" ", 2)
+        form, tiles, words = subprocess.check_output([program, str(n), str(int(rel))], text=True).strip().rsplit(" ", 2)
         assert int(tiles) <= int(words)   # every tile has its look-back word
         return form
     return ask
@@ -39,3 +44,13 @@ def test_grids_of_two_cells_across(rule, n, form):
 @pytest.mark.parametrize("n,cells,form", [(17999, (9, 9, 9), "warp 1"), (19652, (8, 8, 8), "lanes"), (8001504, (64, 64, 64), "lanes")])
 def test_condensed_systems(rule, n, cells, form):
     assert rule(n, cells) == form
+
+
+@pytest.mark.parametrize("n,mean,least,most", [(18000, 61.6, 160, 640), (55296, 61.6, 160, 640), (80000, 61.6, 160, 640),   # half-empty boxes of 134-entry lists
+                                               (432000, 80.0, 112, 124), (8001504, 123.2, 168, 180), (8001504, 0.5, 64, 64), (18000, 2000.0, 640, 640)])
+def test_rows_of_the_lanes(program, n, mean, least, most):
+    row = int(subprocess.check_output([program, str(n), str(mean), "148"], text=True))
+    assert least <= row <= most and row % 4 == 0
+    per_sm = ((n + 63) // 64 + 147) // 148
+    if row > max(1.3 * mean + 16, 64):   # longer than the mean asks for: every tile still runs at once
+        assert per_sm * (64 * 2 * (row + 2) + 2 * 2 * 3 * 32 * 4 + 800 + 1024) <= 227 * 1024
