@@ -1182,7 +1182,7 @@ static_assert(list_form_tile(ListForm::LANES) == OP_TILE, "tiles");
 
 static ListForm form_of(const mlip_ctx *c, bool rel) {
     if (c->lookback_unpublished_tile >= 0 || c->lookback_spin_limit > 0) return rel ? ListForm::LANES : ListForm::WARP_8;   // (diagnostics name 64-atom tiles)
-    return list_form(c->n, rel);
+    return list_form(c->n, c->grid.n_cells, rel);
 }
 
 template <bool REL, int PER_WARP, typename ENTRY>
@@ -1276,8 +1276,8 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
         int *flag = allow_sync_grow ? c->build_word + 1 : c->status;
         int rc = MLIP_OK;
         if (form == ListForm::LANES) rc = list16 ? launch_lanes(c, nbr16, flag, rl, near2, s) : launch_lanes(c, c->nbr, flag, rl, near2, s);
-        else if (list16) launch_onepass<true, 1, uint16_t>(c, nbr16, flag, rl, near2, s);
-        else if (rel) launch_onepass<true, 1, int32_t>(c, c->nbr, flag, rl, near2, s);
+        else if (list16) form == ListForm::WARP_1 ? launch_onepass<true, 1, uint16_t>(c, nbr16, flag, rl, near2, s) : launch_onepass<true, 8, uint16_t>(c, nbr16, flag, rl, near2, s);
+        else if (rel) form == ListForm::WARP_1 ? launch_onepass<true, 1, int32_t>(c, c->nbr, flag, rl, near2, s) : launch_onepass<true, 8, int32_t>(c, c->nbr, flag, rl, near2, s);
         else form == ListForm::WARP_1 ? launch_onepass<false, 1, int32_t>(c, c->nbr, flag, rl, near2, s) : launch_onepass<false, 8, int32_t>(c, c->nbr, flag, rl, near2, s);
         if (rc != MLIP_OK) return rc;
         MLIP_CUDA_TRY(c, cudaGetLastError());

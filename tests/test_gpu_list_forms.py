@@ -35,3 +35,22 @@ def build_twice(positions, n, box, list_format=0, C=3, seed=0):
 def test_grids_of_two_cells_across(box, n):
     nl, pot = build_twice(lambda rng: rng.uniform(0, 1, (n, 3)) * np.array(box), n, box)
     assert canonical_equal(nl, *pot.neighbors())
+
+
+# three cells across and more, two to four atoms to a cell: one atom to a warp, eight, and one to a lane
+@pytest.mark.parametrize("box,n", [((400.0, 300.0, 21.5), 18063), ((300.0, 300.0, 21.5), 24063), ((170.0, 170.0, 170.0), 30011), ((280.0, 260.0, 240.0), 100003), ((240.0, 220.0, 210.0), 100003)])
+@pytest.mark.parametrize("list_format", [0, 1])
+def test_few_atoms_to_a_cell(box, n, list_format):
+    nl, pot = build_twice(lambda rng: rng.uniform(0, 1, (n, 3)) * np.array(box), n, box, list_format)
+    assert canonical_equal(nl, *pot.neighbors())
+
+
+@pytest.mark.parametrize("n,edge,list_format", [(100003, 290.0, 0), (100003, 290.0, 1), (60011, 125.0, 0), (60011, 125.0, 1)])
+def test_dense_clusters_among_few_atoms(n, edge, list_format):
+    """A third of the atoms in a ball across the periodic boundary, lists of some hundred entries and more: eight to a warp, one to a lane."""
+    def positions(rng):
+        pos = rng.uniform(0, 1, (n, 3)) * edge
+        pos[:n // 3] = rng.normal(0.0, 14.0, (n // 3, 3))
+        return pos
+    nl, pot = build_twice(positions, n, (edge, edge, edge), list_format)
+    assert canonical_equal(nl, *pot.neighbors())

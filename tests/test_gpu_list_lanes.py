@@ -1,4 +1,4 @@
-"""List builds with one central atom per lane (systems of tens of thousands of atoms): grids of three cells, columns that end inside a tile,
+"""List builds of tens of thousands of atoms, most of them with one central atom per lane: grids of three cells, columns that end inside a tile,
 nearly empty cells, rows that are too short for their list, several tiles' remainders, both list formats, ghosts -- bit for bit against
 the oracle's lists."""
 import numpy as np
@@ -23,7 +23,8 @@ def positions(rng, n, box, clustered):
 
 @pytest.mark.parametrize("box,n,list_format,clustered", [((21.5, 21.5, 60.3), 18001, 0, False),       # 3 x 3 x 8 cells, some 130 atoms to a cell
                                                          ((66.1, 58.7, 50.2), 18000 + 31, 0, False), ((66.1, 58.7, 50.2), 18000 + 33, 1, False),
-                                                         ((400.0, 300.0, 21.5), 18063, 0, False),     # a few atoms to a cell, columns of three cells
+                                                         ((400.0, 300.0, 21.5), 18063, 0, False),     # a few atoms to a cell, columns of three cells: one atom to a warp,
+                                                                                                      # as the clusters below; see test_gpu_list_forms for such with lanes
                                                          ((160.0, 160.0, 160.0), 18240, 1, True)])
 def test_builds_equal_the_oracles_lists(box, n, list_format, clustered):
     import paper_2608_16329_b200 as mlip

@@ -11,8 +11,8 @@ PROGRAM = r"""
 #include "list_form.cuh"
 int main(int argc, char **argv) {
     const int64_t n = atoll(argv[1]);
-    if (argc == 4) { printf("%d\n", mlip::list_lane_row(n, atof(argv[2]), atoi(argv[3]))); return 0; }
-    const mlip::ListForm f = mlip::list_form(n, atoi(argv[2]) != 0);
+    if (argc == 3) { printf("%d\n", mlip::list_lane_row(n, atof(argv[2]), 148)); return 0; }
+    const mlip::ListForm f = mlip::list_form(n, atoll(argv[2]), atoi(argv[3]) != 0);
     printf("%s %lld %lld\n", f == mlip::ListForm::WARP_1 ? "warp 1" : f == mlip::ListForm::WARP_8 ? "warp 8" : "lanes", (long long)((n + mlip::list_form_tile(f) - 1) / mlip::list_form_tile(f)), (long long)mlip::list_tile_words(n));
 }
 """
@@ -29,8 +29,8 @@ def program(tmp_path_factory):
 @pytest.fixture(scope="module")
 def rule(program):
     def ask(n, cells):
-        rel = all(c >= 3 for c in cells)
-        form, tiles, words = subprocess.check_output([program, str(n), str(int(rel))], text=True).strip().rsplit(" ", 2)
+        rel, n_cells = all(c >= 3 for c in cells), cells[0] * cells[1] * cells[2]
+        form, tiles, words = subprocess.check_output([program, str(n), str(n_cells), str(int(rel))], text=True).strip().rsplit(" ", 2)
         assert int(tiles) <= int(words)   # every tile has its look-back word
         return form
     return ask
@@ -46,10 +46,19 @@ def test_condensed_systems(rule, n, cells, form):
     assert rule(n, cells) == form
 
 
+# one atom per cell up to six, and a ball of 85,601 atoms in a wide box
+@pytest.mark.parametrize("n,cells,form", [(20000, (27, 27, 27), "warp 1"), (18500, (18, 18, 18), "warp 1"), (18500, (16, 16, 16), "lanes"), (25000, (23, 23, 23), "warp 1"),
+                                          (25000, (20, 20, 20), "lanes"), (70000, (41, 41, 41), "warp 8"), (70000, (32, 32, 32), "lanes"), (150000, (53, 53, 53), "warp 8"),
+                                          (150000, (36, 36, 36), "lanes"), (300000, (66, 66, 66), "warp 8"), (1000000, (101, 101, 101), "warp 8"), (1000000, (87, 87, 87), "lanes"),
+                                          (85601, (57, 57, 57), "warp 8")])
+def test_sparse_systems(rule, n, cells, form):
+    assert rule(n, cells) == form
+
+
 @pytest.mark.parametrize("n,mean,least,most", [(18000, 61.6, 160, 640), (55296, 61.6, 160, 640), (80000, 61.6, 160, 640),   # half-empty boxes of 134-entry lists
                                                (432000, 80.0, 112, 124), (8001504, 123.2, 168, 180), (8001504, 0.5, 64, 64), (18000, 2000.0, 640, 640)])
 def test_rows_of_the_lanes(program, n, mean, least, most):
-    row = int(subprocess.check_output([program, str(n), str(mean), "148"], text=True))
+    row = int(subprocess.check_output([program, str(n), str(mean)], text=True))
     assert least <= row <= most and row % 4 == 0
     per_sm = ((n + 63) // 64 + 147) // 148
     if row > max(1.3 * mean + 16, 64):   # longer than the mean asks for: every tile still runs at once
