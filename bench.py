@@ -58,7 +58,7 @@ FP64_LANES_PER_SM = 64         # fp64 path: DFMA lanes per SM
 # (dram__bytes_read.sum + dram__bytes_write.sum per atom; the traffic is per-atom, so a launch of N atoms is reported as
 # that figure times N).  The record names the kernel sources it was captured from; a different kernel prints no traffic.
 TRAFFIC_RECORD = os.path.join(ROOT, "profiles", "k_mega_hea6_fcc50.traffic.txt")
-KERNEL_SOURCES = ["megakernel.cu", "pair_math.cuh", "common.cuh"]
+KERNEL_SOURCES = ["megakernel.cuh", "megakernel.cu", "pair_math.cuh", "common.cuh"]
 
 
 def kernel_revision() -> str:
