@@ -125,12 +125,12 @@ struct mlip_ctx {
     bool list16 = false;           // format of the current lists (mlip_config.list_format = 1 on a grid of >= 3 cells per edge)
     int32_t *cell_id = nullptr;    // [N] build-time cell of each atom as packed coordinates, internal order (allocated for list_format = 1)
     unsigned long long *tile_state = nullptr;   // [tile_words(N)] look-back words of the one-pass build
-    int *build_word = nullptr;     // {ticket, private overflow flag, total entries (64 bits)} of the one-pass build, then status, rebuild_flag, far_flag, -, species_start
+    int *build_word = nullptr;     // {ticket, private overflow flag, total entries (64 bits)} of the one-pass build, then status, rebuild_flag, far_flag, number of long lists (LONG_LIST), species_start
     float4 *rel_pos = nullptr;     // cell-relative positions of the build in progress
     int *build_host = nullptr;     // pinned copy, and the ticket of the report that wrote it
     int reports = 0;
     static constexpr int BUILD_WORDS = 8 + mlip::MAX_SPECIES + 1;
-    int64_t nbr_cap = 0, n_entries = 0;
+    int64_t nbr_cap = 0, n_entries = 0, n_long = 0;   // (entries, long lists: of the last synchronising build)
     // scratch
     int64_t *scan_tmp = nullptr;   // block sums for the scans
     int64_t scan_tmp_cap = 0;

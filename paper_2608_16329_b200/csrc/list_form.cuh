@@ -42,6 +42,12 @@ inline int list_lane_row(int64_t n, double mean, int sms) {
     return (int)std::min(std::max({(int64_t)(1.3 * mean) + 16, all_at_once, (int64_t)64}), (int64_t)LANE_ROW_MOST) / 4 * 4;
 }
 
+// Lists whose leading entries (those within r_cut + skin / 2, which evaluations read) are too many for two atoms of a warp to go side by side
+// (launch_megakernel): where more than a tenth of them are, or where the density of the box lets the mean list be a tenth longer.
+constexpr int LONG_LIST = 96;
+inline bool lists_are_long(int64_t n_long, int64_t n_owned) { return 10 * n_long > n_owned; }
+inline bool lists_expected_long(double mean) { return mean > 1.1 * LONG_LIST; }
+
 // Look-back words that builds of up to n atoms need, whatever their form.
 inline int64_t list_tile_words(int64_t n) { return std::max(n / 64, std::min(n, WARP_8_FROM) / 8) + 2; }
 

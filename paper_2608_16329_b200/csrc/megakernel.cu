@@ -3,9 +3,12 @@
 #include <new>
 #include <vector>
 
+#include "list_form.cuh"
 #include "megakernel.cuh"
 
 namespace mlip {
+
+static_assert(LONG_LIST == NARROW_CHUNKS * 32, "lists that two atoms gather together");
 
 // ---------------- host side ----------------
 int table_smem_words(const mlip_ctx *c) { return c->cfg.n_species * (c->cfg.table_knots + 3) * K_RADIAL; }
@@ -114,6 +117,18 @@ __global__ void k_fixed_finish(int64_t n, long long *force_fx, const long long *
     stamp_end(stamp);
 }
 
+// Whether two atoms of a warp go through the pair loops one after the other.  Side by side they are the faster ones where their lists fit the queue
+// together, up to LONG_LIST entries each; with longer ones they are gathered one by one as well, no batch is saved, and from some 110 pairs on
+// warps of both kinds share an SM and wait for each other's instructions.  One evaluation of some 100,000 atoms in us, side by side / one after the
+// other: random positions of 54 pairs an atom 667 / 671, 63 734 / 735, 72 823 / 801, 81 886 / 858, 109 1564 / 1057, 118 2632 / 1203, 163 2131 / 1529; crystals
+// of 42 pairs 494 / 512, 54 574 / 585, 78 846 / 853, 86 995 / 964, 113 1215 / 1153, 131 1506 / 1367, 158 1534 / 1377, 221 2317 / 2123.
+// Asked of the last synchronising build's lists.  Reproducible runs must not depend on when that was: they ask the density of the box.
+static bool long_lists(const mlip_ctx *c) {
+    if (c->cfg.force_mode != 1) return lists_are_long(c->n_long, c->n_owned);
+    const double r = c->cfg.r_cut + 0.5 * c->cfg.skin, volume = c->grid.box[0] * c->grid.box[1] * c->grid.box[2];
+    return lists_expected_long((double)c->n / volume * (4.0 / 3.0 * 3.14159265358979 * r * r * r));
+}
+
 int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     const int64_t n = c->n;
     const bool det = c->cfg.force_mode == 1;
@@ -125,12 +140,10 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     if (c->captured) MLIP_CUDA_TRY(c, cudaMemsetAsync(blk.use, 0, LAUNCH_CLEAR_BYTES, s));
     const bool in_smem = tables_fit_smem(c);
     const int tab_words = in_smem ? table_smem_words(c) : 0;
-    // instantiations: {one, two atoms per warp, two with tables in global memory}
-    // x floating-point / integer scatter x int32 / 16-bit lists
-    static const MegaKernel kernels[3][4] = {{mega_one(false, false), mega_one(false, true), mega_one(true, false), mega_one(true, true)},
-                                             {mega_two(false), mega_two(true), mega_two_fixed(false), mega_two_fixed(true)},
-                                             {mega_two_global(false, false), mega_two_global(false, true), mega_two_global(true, false), mega_two_global(true, true)}};
-    const int shape = !in_smem ? 2 : n >= ONE_PER_WARP_BELOW_ATOMS ? 1 : 0;
+    const int shape = in_smem && n < ONE_PER_WARP_BELOW_ATOMS ? 0 : long_lists(c) ? 2 : 1;   // one atom per warp, two side by side, two one after the other
+    auto kernel_of = [&](int shape, bool list16) {
+        return shape == 0 ? mega_one(det, list16) : shape == 2 ? mega_apart(in_smem, det, list16) : !in_smem ? mega_two_global(det, list16) : det ? mega_two_fixed(list16) : mega_two(list16);
+    };
     const int apw = shape == 0 ? 1 : 2;
     const size_t smem_bytes = sizeof(float) * (size_t)((apw == 1 ? Layout<1>::FIXED : Layout<2>::FIXED) + tab_words);
     const int C = c->cfg.n_species, tile_atoms = GW * apw;
@@ -138,12 +151,13 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     for (int q = 0; q < C; ++q) all += tiles[q] = (c->species_host[q + 1] - c->species_host[q] + tile_atoms - 1) / tile_atoms;
     const int blocks = (int)std::min<int64_t>(all, (int64_t)c->n_sm);
     if (!c->kernel_ready) {
-        // A limit of the kernels, shared by every context of the process: the same whatever this one's tables need.
-        for (int q = 0; q < 12; ++q) {
-            const int most = q < 8 ? SMEM_LIMIT_WORDS : Layout<2>::FIXED;
-            cudaError_t e = cudaFuncSetAttribute((const void *)kernels[q / 4][q % 4], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(float) * most);
-            if (e != cudaSuccess) { c->err = std::string("fused kernel shared memory: ") + cudaGetErrorString(e); return MLIP_ERR_CUDA; }
-        }
+        // A limit of the kernels, shared by every context of the process: the same whatever this one's tables need.  Those that this context may launch.
+        for (int q = in_smem ? 0 : 1; q < 3; ++q)
+            for (int compact = 0; compact <= (c->cfg.list_format == 1); ++compact) {
+                const cudaError_t e = cudaFuncSetAttribute((const void *)kernel_of(q, compact), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           (int)sizeof(float) * (in_smem ? SMEM_LIMIT_WORDS : Layout<2>::FIXED));
+                if (e != cudaSuccess) { c->err = std::string("fused kernel shared memory: ") + cudaGetErrorString(e); return MLIP_ERR_CUDA; }
+            }
         c->kernel_ready = true;
     }
     KernelArgs k;
@@ -177,7 +191,7 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     }
     k.stamp = timed_begin(c, MARK_KERNEL, s);
     k.early = !c->lists_fresh;   // (the kernel reads the lists before it waits)
-    MLIP_CUDA_TRY(c, launch_after_if(k.early, kernels[shape][(det ? 2 : 0) + (c->list16 ? 1 : 0)], blocks, NW * 32, smem_bytes, s, k, tab_words));
+    MLIP_CUDA_TRY(c, launch_after_if(k.early, kernel_of(shape, c->list16), blocks, NW * 32, smem_bytes, s, k, tab_words));
     c->lists_fresh = c->force_cleared = false;
     set_eval_block(c, blk.use);
     if (det) {

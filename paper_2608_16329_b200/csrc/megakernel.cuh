@@ -525,7 +525,8 @@ __device__ __forceinline__ void clear_fragments(float (&Pf)[4][4]) {
 // One atom on its own: returns the number of pairs and the moment as accumulator fragments.
 // `queued` returns the number of pairs left in the queue when the whole list fitted in one round
 // (the derivation then reuses them), or -1.
-// (UNROLL = 2, tiles of one atom per warp: two k-steps side by side and no half ones, the chain through a tile being their time)
+// (UNROLL = 2, kernels without atoms side by side: two k-steps side by side and no half ones.  With one atom per warp the chain through a tile is the
+// time; with two, 97,336 atoms of 158 pairs 1397 us an evaluation with half steps one by one, 1377 so.)
 template <bool TAB_SMEM, bool L16, int UNROLL>
 __device__ __forceinline__ int encode_atom(const KernelArgs &k, const TableView &tv, const double4 &pi, int64_t beg, int64_t end,
                                            float4 *pq, int cap, float *stage, int lane, float (&Pf)[4][4], int &queued, const int *sidx, int n_pref,
@@ -762,7 +763,7 @@ __device__ __forceinline__ void derive_chunks(uint32_t (&chunk)[2], int lane) {
 }
 
 // One atom on its own.
-template <int APW, bool TAB_SMEM, bool DET, bool L16>
+template <bool SIDE, bool TAB_SMEM, bool DET, bool L16>
 __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView &tv, int i,
                                             float4 *pq, int cap, float *scr, int queued, int lane, const WFragments &W, float w_scale_inv,
                                             float (&vir)[9], uint32_t tm_vt, PhaseClock &pc) {
@@ -777,7 +778,7 @@ __device__ __forceinline__ void derive_atom(const KernelArgs &k, const TableView
         const int nmt = (n + 15) >> 4;
 #pragma unroll 1
         for (int mt = 0; mt < nmt; ++mt) {
-            if (APW == 1 || n - 16 * mt > 8) derive_tile<TAB_SMEM, false>(tv, scr, mt, lane >> 2, chunk, W, tm_vt);
+            if (!SIDE || n - 16 * mt > 8) derive_tile<TAB_SMEM, false>(tv, scr, mt, lane >> 2, chunk, W, tm_vt);
             else derive_tile<TAB_SMEM, true>(tv, scr, mt, lane >> 2, chunk, W, tm_vt);
         }
         tmem_wait_st();
@@ -1063,8 +1064,10 @@ __device__ __forceinline__ void head_tile(const KernelArgs &k, const float *xs, 
 }
 
 constexpr int TOTALS = 9 + 16 + 1;   // per warp at the end: virial, E_i sums of up to 16 lanes, pairs
-template <int APW, bool TAB_SMEM, bool DET, bool L16>
+// SIDE: a warp's two atoms go through the pair loops side by side where their pairs fit its queue together.
+template <int APW, bool SIDE, bool TAB_SMEM, bool DET, bool L16>
 __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ KernelArgs k, int tab_words) {
+    static_assert(APW == 2 || !SIDE, "two atoms side by side");
     extern __shared__ __align__(128) float smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     using LY = Layout<APW>;
@@ -1256,7 +1259,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
             // Two atoms whose pairs fit the queue together go through the pair loops side by side (see collect_two).
             bool both = false;
             int n0 = 0, n1 = 0, i0 = 0, i1 = 0;
-            if (APW == 2) {
+            if (SIDE) {
                 if (prefetched && pf[PF_IDX + 3] <= NARROW_CHUNKS * 32 && (mine < 2 || pf[PF_WORDS + PF_IDX + 3] <= NARROW_CHUNKS * 32)) {
                     collect_two<L16>(k, pf, mine, pq, lane, n0, n1);
                     i0 = pf[PF_IDX];
@@ -1279,7 +1282,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
                     if (L16) cs = cell_base_of_lane(k, i, lane);
                 }
             };
-            if (APW == 2 && !both) {   // longer lists, or the first tile of a species
+            if (SIDE && !both) {   // longer lists, or the first tile of a species
                 both = true;
 #pragma unroll 1
                 for (int u = 0; u < mine && both; ++u) {
@@ -1332,7 +1335,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
                         int64_t beg, end;
                         atom_and_list(u, i, beg, end, n_pref, cs);
                         const double4 pi = load_pos4(k.pos4 + i);
-                        n_pairs += encode_atom<TAB_SMEM, L16, APW == 1 ? 2 : 1>(k, tv, pi, beg, end, pq + q_used, LY::POOL - q_used, scr, lane, Pf, queued, pf + u * PF_WORDS, n_pref, cs, pc);
+                        n_pairs += encode_atom<TAB_SMEM, L16, SIDE ? 1 : 2>(k, tv, pi, beg, end, pq + q_used, LY::POOL - q_used, scr, lane, Pf, queued, pf + u * PF_WORDS, n_pref, cs, pc);
                         if (u + 1 < APW && queued > LY::POOL - SECOND_ROOM) queued = -1;   // leave the next atom room for a scan
                         if (lane == 0) *reinterpret_cast<int4 *>(info + 4 * u) = make_int4(i, queued, q_used, 0);
                         q_used += max(queued, 0);
@@ -1406,7 +1409,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
                 }
             };
             const int4 inf0 = *reinterpret_cast<const int4 *>(info);
-            if (APW == 2 && inf0.w != 0) {
+            if (SIDE && inf0.w != 0) {
                 // both atoms' pairs, from the last batch to the first: the second atom's moment, where V and T go, is read before the first of them
                 const int4 inf1 = *reinterpret_cast<const int4 *>(info + 4);
                 const int second = inf1.z, end = second + inf1.y;
@@ -1462,7 +1465,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
                     const int4 inf = *reinterpret_cast<const int4 *>(info + 4 * u);
                     WFragments W;
                     const float inv = weights_of(u, W);
-                    derive_atom<APW, TAB_SMEM, DET, L16>(k, tv, inf.x, pq + inf.z, LY::POOL - inf.z, scr, inf.y, lane, W, inv, vir, tm_vt, pc);
+                    derive_atom<SIDE, TAB_SMEM, DET, L16>(k, tv, inf.x, pq + inf.z, LY::POOL - inf.z, scr, inf.y, lane, W, inv, vir, tm_vt, pc);
                     if (DET) fold_virial();
                 }
             }
@@ -1519,9 +1522,10 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
 // integer scatter of two atoms per warp is the better one beside the kernels of one (19,652 atoms 199 us, on its own 202), the kernels with tables in
 // global memory beside those with tables in shared memory (eight species, compact lists, 108,000 atoms 958 us, on their own 978).
 using MegaKernel = void (*)(KernelArgs, int);
-MegaKernel mega_one(bool det, bool list16);          // one atom per warp
-MegaKernel mega_two_fixed(bool list16);              // two atoms per warp, integer scatter
-MegaKernel mega_two(bool list16);                    // two atoms per warp, floating-point scatter
-MegaKernel mega_two_global(bool det, bool list16);   // two atoms per warp, tables in global memory
+MegaKernel mega_one(bool det, bool list16);                      // one atom per warp
+MegaKernel mega_two_fixed(bool list16);                          // two atoms per warp, side by side; integer scatter
+MegaKernel mega_two(bool list16);                                // floating-point scatter
+MegaKernel mega_two_global(bool det, bool list16);               // tables in global memory
+MegaKernel mega_apart(bool in_smem, bool det, bool list16);      // two atoms per warp, one after the other (launch_megakernel)
 
 }  // namespace mlip

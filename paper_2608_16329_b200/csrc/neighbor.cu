@@ -39,7 +39,8 @@ __device__ __forceinline__ OUT list_entry(int j, int it, int cell_beg) {
     return (OUT)j;
 }
 
-// What a build clears on its way: the look-back words, {ticket, overflow, total} of the one-pass traversal, and the two flags.
+constexpr int LONG_WORD = 7;   // of build_word: lists with more than LONG_LIST near entries
+// What a build clears on its way: the look-back words, {ticket, overflow, total} and the long lists of the one-pass traversal, and the two flags.
 struct BuildClear {
     unsigned long long *tile_state;
     int64_t n_words;       // <= number of atoms
@@ -56,6 +57,7 @@ __global__ void k_cell_id(const double *__restrict__ pos, const int32_t *__restr
     if (i < clear.n_words) clear.tile_state[i] = 0;
     if (i == 0) {
         for (int q = 0; q < 4; ++q) clear.build_word[q] = 0;
+        clear.build_word[LONG_WORD] = 0;
         *clear.far_flag = 0; *clear.rebuild_flag = 0;
     }
     double4 p;
@@ -218,6 +220,7 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_bin_small(const double *__res
     for (int q = threadIdx.x; q < clear.n_words; q += SMALL_THREADS) clear.tile_state[q] = 0;
     if (threadIdx.x == 0) {
         for (int q = 0; q < 4; ++q) clear.build_word[q] = 0;
+        clear.build_word[LONG_WORD] = 0;
         *clear.far_flag = 0; *clear.rebuild_flag = 0;
     }
     __syncthreads();
@@ -688,6 +691,11 @@ __global__ void __launch_bounds__(256) k_neighbors_onepass(int64_t n, CellGrid g
 
     // ---- offsets: scan inside the tile, look back over the tiles before it ----
     if (warp == 0) tile_offsets<TILE_ATOMS>(tile, s_cnt, s_off, &s_prefix, &s_total, status, tile_state, spin_limit, unpublished_tile, lane);
+    if (warp == 1) {
+        unsigned longer = __popc(__ballot_sync(0xffffffffu, lane < TILE_ATOMS && s_near[lane] > LONG_LIST));
+        if (TILE_ATOMS > 32) longer += __popc(__ballot_sync(0xffffffffu, s_near[(lane + 32) % OP_TILE] > LONG_LIST));
+        if (lane == 0 && longer) atomicAdd(build_word + LONG_WORD, (int)longer);
+    }
     __syncthreads();
     const long long tile_off = s_prefix;
     if (first + TILE_ATOMS >= n && threadIdx.x == 0) {   // the last tile closes the offsets
@@ -945,6 +953,8 @@ __global__ void __launch_bounds__(LN_THREADS) k_neighbors_lanes(int64_t n, CellG
         nbr_off[i] = off < nbr_cap ? off : nbr_cap;
         nbr_near[i] = cn < fit ? cn : fit;
     }
+    const unsigned longer = __ballot_sync(0xffffffffu, cn > LONG_LIST);
+    if (lane == 0 && longer) atomicAdd(build_word + LONG_WORD, __popc(longer));
     if (__any_sync(0xffffffffu, lost > 0)) {   // lists longer than their rows, straight to their places
         list = nbr + off; far_next = cnt - 1;
         traverse(std::true_type{}, lost > 0);
@@ -1168,6 +1178,13 @@ static int read_build_words(mlip_ctx *c, cudaStream_t s) {
     return MLIP_OK;
 }
 
+// Long lists after a counting pass (the single traversal counts them on its way).
+__global__ void k_count_long(int64_t n, const int32_t *__restrict__ nbr_near, int *count) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int longer = __syncthreads_count(i < n && nbr_near[i] > LONG_LIST);
+    if (threadIdx.x == 0 && longer) atomicAdd(count, longer);
+}
+
 // A synchronising build that met a non-finite or out-of-box position, a species out of range or an over-full cell: the
 // list kernels have not run, so there is nothing to size a list from.  Reports it now and clears the flag.
 static int refuse_broken_input(mlip_ctx *c, cudaStream_t s) {
@@ -1289,7 +1306,7 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
             int64_t total;
             memcpy(&total, c->build_host + 2, sizeof total);
             done = c->build_host[1] == 0 && total <= c->nbr_cap;
-            if (done) c->n_entries = total;
+            if (done) { c->n_entries = total; c->n_long = c->build_host[LONG_WORD]; }
         }
         if (done) {
             mark_end(c, MARK_BUILD, s);
@@ -1303,12 +1320,16 @@ int launch_build(mlip_ctx *c, bool allow_sync_grow, const double *pos, const int
     c->launches += 1 + exclusive_scan<int32_t, int64_t>(c->nbr_count, c->nbr_off, n, c->scan_tmp, s);
     MLIP_CUDA_TRY(c, cudaGetLastError());
     if (allow_sync_grow) {
+        MLIP_CUDA_TRY(c, cudaMemsetAsync(c->build_word + LONG_WORD, 0, sizeof(int), s));
+        k_count_long<<<blocks_for(n, 256), 256, 0, s>>>(n, c->nbr_near, c->build_word + LONG_WORD);
+        c->launches += 1;
         MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->total_host, c->nbr_off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
         MLIP_CUDA_TRY(c, cudaMemcpyAsync(c->build_host, c->build_word, sizeof(int) * mlip_ctx::BUILD_WORDS, cudaMemcpyDeviceToHost, s));
         MLIP_CUDA_TRY(c, cudaStreamSynchronize(s));
         if (c->build_host[4] & FLAG_NONFINITE) return refuse_broken_input(c, s);
         memcpy(c->species_host, c->build_host + 8, sizeof c->species_host);
         c->n_entries = *c->total_host;
+        c->n_long = c->build_host[LONG_WORD];
         if (c->n_entries > c->nbr_cap) {
             int64_t want = c->n_entries + c->n_entries / 8 + 1024;
             if (c->nbr) { cudaFree(c->nbr); c->resident -= entry_bytes * c->nbr_cap; c->nbr = nullptr; c->nbr_cap = 0; }

@@ -1,0 +1,87 @@
+"""Fused kernel, two atoms per warp, on both sides of the line between atoms side by side and one after the other (long_lists): systems in which some or most
+lists are too long for two atoms to share the pair queue, in every form of the kernel, against the oracle; and the time per pair."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def two_phases(rng, dense_layers, spacing, sparse_layers):
+    """A simple cubic crystal of the given spacing (1.7: some 185 pairs an atom) beside one of 2.9 (some 37), as slabs across the box."""
+    w = 30 * spacing
+    dense = wl.lattice_sites((dense_layers, 30, 30), spacing, wl._SC_BASIS)
+    m = int(w / 2.9)
+    sparse = wl.lattice_sites((sparse_layers, m, m), 2.9, wl._SC_BASIS) * [1.0, w / (2.9 * m), w / (2.9 * m)]
+    sparse[:, 0] += dense_layers * spacing + 1.5
+    box = np.array([dense_layers * spacing + 1.5 + sparse_layers * 2.9, w, w])
+    pos = np.concatenate([dense, sparse]) + rng.normal(0.0, 0.05, (len(dense) + len(sparse), 3))
+    pos -= np.floor(pos / box) * box
+    pos[pos >= box] = 0.0
+    return np.ascontiguousarray(pos), box
+
+
+def liquid(rng, cells, density):
+    """A simple cubic lattice shaken by up to a fifth of its spacing."""
+    a = density ** (-1.0 / 3.0)
+    pos = wl.lattice_sites((cells,) * 3, a, wl._SC_BASIS) + rng.uniform(-0.2 * a, 0.2 * a, (cells ** 3, 3))
+    box = np.full(3, cells * a)
+    return np.ascontiguousarray(pos - np.floor(pos / box) * box), box
+
+
+# 6 percent of the atoms in the dense slab (side by side, the dense ones not), 60 percent (one after the other, the sparse ones too), all; liquids of 72 and of 118 pairs
+STRUCTURES = {"some": lambda rng: two_phases(rng, 2, 1.7, 90), "most": lambda rng: two_phases(rng, 9, 1.7, 20), "all": lambda rng: two_phases(rng, 14, 1.7, 1),
+              "liquid 72": lambda rng: liquid(rng, 24, 0.08), "liquid 118": lambda rng: liquid(rng, 24, 0.13)}
+
+
+@pytest.mark.parametrize("structure,C,list_format,force_mode", [("some", 3, 0, 0), ("some", 3, 1, 0), ("some", 3, 0, 1), ("some", 8, 0, 0), ("most", 3, 0, 0), ("most", 3, 1, 0), ("most", 8, 0, 0),
+                                                                ("most", 8, 1, 1), ("all", 3, 0, 1), ("all", 8, 0, 1), ("liquid 72", 3, 0, 0), ("liquid 118", 3, 0, 0),
+                                                                ("liquid 118", 3, 0, 1), ("liquid 118", 8, 1, 0)])
+def test_long_lists_match_the_oracle(structure, C, list_format, force_mode):
+    """Tolerances: those of the order-one workloads, forces relative to their RMS where that exceeds 1 eV/Angstrom (see test_gpu_pair_counts).  Eight species: tables
+    in global memory."""
+    import paper_2608_16329_b200 as mlip
+    rng = np.random.default_rng(len(structure) + C)
+    pos, box = STRUCTURES[structure](rng)
+    assert len(pos) >= 12000   # two atoms per warp
+    species = rng.integers(0, C, len(pos)).astype(np.int32)
+    enc, head = wl.make_weights(C, seed=78, enc_out_scale=0.05, head_out_scale=0.1)
+    pot = mlip.Potential(C, 6.0, 1.0, enc, head, np.full(C, 50.0), list_format=list_format, force_mode=force_mode)
+    pot.build_neighbors(pos, species, box)
+    out = pot.compute(want_e_atom=True)
+    pot.sync_status()
+    ref = oracle.evaluate(oracle.Model(C, 6.0, enc, head), pos, species, box)
+    scale = max(1.0, float(np.sqrt((ref["forces"] ** 2).sum(1).mean())))
+    assert abs(float(out["energy"].cpu()) - ref["energy"]) <= 1e-6 * abs(ref["energy"])
+    assert np.abs(out["forces"].cpu().numpy() - ref["forces"]).max() <= 1e-4 * scale
+    assert np.abs(out["e_atom"].cpu().numpy() - ref["e_atom"]).max() <= 2e-5 * max(1.0, np.abs(ref["e_atom"]).max())
+    assert np.abs(out["virial"].cpu().numpy().ravel() - np.asarray(ref["virial"]).ravel()).max() <= 1e-5 * np.abs(ref["virial"]).max()
+    if force_mode:   # once more, bit for bit: which tiles were prefetched differs from run to run
+        again = pot.compute(want_e_atom=True)
+        assert all(np.array_equal(out[k].cpu().numpy(), again[k].cpu().numpy()) for k in ("energy", "forces", "virial"))
+
+
+def test_a_pair_costs_no_more_where_there_are_many():
+    """Device time per pair of random positions of 118 pairs an atom against 45: 0.8 times.  (Two atoms of a warp tried side by side first: 1.7.)"""
+    import paper_2608_16329_b200 as mlip
+    import torch
+    cost = []
+    for density in (0.05, 0.13):
+        box = np.full(3, (100000 / density) ** (1.0 / 3.0))
+        pos = np.random.default_rng(1).uniform(0.0, 1.0, (100000, 3)) * box
+        enc, head = wl.make_weights(3, seed=78, enc_out_scale=0.05, head_out_scale=0.3)
+        pot = mlip.Potential(3, 6.0, 1.0, enc, head, np.full(3, 50.0), table_tol=1.0)
+        pot.build_neighbors(pos, np.random.default_rng(2).integers(0, 3, len(pos)).astype(np.int32), box)
+        best = 1e9
+        for _ in range(8):
+            begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            begin.record()
+            for _ in range(4):
+                pot.compute()
+            end.record()
+            torch.cuda.synchronize()
+            best = min(best, begin.elapsed_time(end))
+        cost.append(best / mlip.mlip_get_counters(pot.ctx)["pairs_in_cutoff"])
+    assert cost[1] < 1.2 * cost[0], cost

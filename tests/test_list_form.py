@@ -11,6 +11,7 @@ PROGRAM = r"""
 #include "list_form.cuh"
 int main(int argc, char **argv) {
     const int64_t n = atoll(argv[1]);
+    if (argc == 5) { printf("%d %d\n", mlip::lists_are_long(n, atoll(argv[2])), mlip::lists_expected_long(atof(argv[3]))); return 0; }
     if (argc == 3) { printf("%d\n", mlip::list_lane_row(n, atof(argv[2]), 148)); return 0; }
     const mlip::ListForm f = mlip::list_form(n, atoll(argv[2]), atoi(argv[3]) != 0);
     printf("%s %lld %lld\n", f == mlip::ListForm::WARP_1 ? "warp 1" : f == mlip::ListForm::WARP_8 ? "warp 8" : "lanes", (long long)((n + mlip::list_form_tile(f) - 1) / mlip::list_form_tile(f)), (long long)mlip::list_tile_words(n));
@@ -63,3 +64,9 @@ def test_rows_of_the_lanes(program, n, mean, least, most):
     per_sm = ((n + 63) // 64 + 147) // 148
     if row > max(1.3 * mean + 16, 64):   # longer than the mean asks for: every tile still runs at once
         assert per_sm * (64 * 2 * (row + 2) + 2 * 2 * 3 * 32 * 4 + 800 + 1024) <= 227 * 1024
+
+
+# lists of more than 96 leading entries among all; the mean at the box's density: alloy of 134 entries (99 within 6.5 Angstrom), liquids of 0.08, 0.1 and 0.13 atoms per cubic Angstrom
+@pytest.mark.parametrize("n_long,n,mean,by_count,by_density", [(0, 100000, 98.6, 0, 0), (10000, 100000, 92.0, 0, 0), (10001, 100000, 115.0, 1, 1), (100000, 100000, 150.0, 1, 1), (0, 0, 0.0, 0, 0)])
+def test_atoms_one_after_the_other(program, n_long, n, mean, by_count, by_density):
+    assert subprocess.check_output([program, str(n_long), str(n), str(mean), "-"], text=True).split() == [str(by_count), str(by_density)]
