@@ -33,15 +33,20 @@ def test_builds_equal_the_oracles_lists(box, n, list_format, clustered):
     C = 3
     enc, head = wl.make_weights(C, seed=1, enc_hidden=8, enc_layers=1)
     pot = mlip.Potential(C, 6.0, 1.0, enc, head, np.ones(C), table_tol=1.0, enc_hidden=8, enc_layers=1, list_format=list_format)
-    for trial in range(2):   # the first build has no array yet, the second takes the single traversal
+    launches = [mlip.mlip_get_counters(pot.ctx)["launches"]]
+    for trial in range(2):   # the first build has no array yet, the second takes the single traversal: no scan and no filling kernel behind it
         pos = positions(rng, n, box, clustered)
         species = rng.integers(0, C, n).astype(np.int32)
         pot.build_neighbors(pos, species, box)
+        launches.append(mlip.mlip_get_counters(pot.ctx)["launches"])
+    assert launches[2] - launches[1] < launches[1] - launches[0]
     nl = oracle.neighbors(pos, species, C, box, 7.0)
     assert canonical_equal(nl, *pot.neighbors())
     # a domain with ghosts: the last third has no lists of its own, and the others' stay what they are
     owned = 2 * n // 3
+    before = mlip.mlip_get_counters(pot.ctx)["launches"]
     pot.build_neighbors(pos, species, box, n_owned=owned)
+    assert mlip.mlip_get_counters(pot.ctx)["launches"] - before == launches[2] - launches[1]
     seg, nbr = pot.neighbors()
     seg, nbr = np.asarray(seg.cpu()), np.asarray(nbr.cpu())
     assert (seg[owned * C:] == seg[-1]).all()
