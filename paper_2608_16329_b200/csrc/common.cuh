@@ -33,7 +33,7 @@ enum : int {
 };
 
 // Range-checked build (-DMLIP_DEBUG_BOUNDS): every index that the fused kernels and the export take from a list or an
-// order array is compared with its array's size before it is used; an index out of range raises FLAG_BOUNDS and is
+// order array, and every place and entry that lanes write to a list, is compared with its array's size before it is used; an index out of range raises FLAG_BOUNDS and is
 // replaced by 0, so the access still happens inside the array.  Stands in for a memory checker on the kernels' gathers.
 #ifdef MLIP_DEBUG_BOUNDS
 #define MLIP_CHECK_INDEX(idx, size, status) (((unsigned long long)(idx) < (unsigned long long)(size)) ? (idx) : (atomicOr((status), FLAG_BOUNDS), 0))

@@ -810,7 +810,9 @@ __global__ void __launch_bounds__(LN_THREADS) k_neighbors_lanes(int64_t n, CellG
     int near_at = row_at, far_at = row_end, near_lost = 0, lost = 0;   // lost: hits whose places were given to others
     // second traversal: places in the list itself, of which `fit` are written
     ENTRY *list = nullptr;
+    long long off = 0;   // of the list
     int near_next = 0, far_next = 0, fit = 0;
+    int *bounds = const_cast<int *>(global_status);   // (range-checked builds only write it)
     auto traverse = [&](auto second_traversal, bool part) {
         constexpr bool SECOND = decltype(second_traversal)::value;
         for (unsigned left = __ballot_sync(0xffffffffu, part); left;) {   // groups of lanes with cells along one column
@@ -896,7 +898,7 @@ __global__ void __launch_bounds__(LN_THREADS) k_neighbors_lanes(int64_t n, CellG
                                 const float v = e & 1 ? d2[e >> 1].y : d2[e >> 1].x;
                                 bool hit = v <= rl2_hi && !(OWN && code + c0 + e == self);
                                 if (hit && v >= rl2_lo) {
-                                    const double4 pi = pos4[i], pj = pos4[chunk + c0 + e];
+                                    const double4 pi = pos4[i], pj = pos4[MLIP_CHECK_INDEX(chunk + c0 + e, n, bounds)];
                                     const double ex = min_image(__dsub_rn(pj.x, pi.x), g.box[0], g.half[0]);
                                     const double ey = min_image(__dsub_rn(pj.y, pi.y), g.box[1], g.half[1]);
                                     const double ez = min_image(__dsub_rn(pj.z, pi.z), g.box[2], g.half[2]);
@@ -905,7 +907,7 @@ __global__ void __launch_bounds__(LN_THREADS) k_neighbors_lanes(int64_t n, CellG
                                 const bool near = v < near2;
                                 if (SECOND) {
                                     const int at = near ? near_next : far_next;
-                                    if (hit && (unsigned)at < (unsigned)fit) list[at] = (ENTRY)(sizeof(ENTRY) == 4 ? chunk + c0 + e : code + c0 + e);
+                                    if (hit && (unsigned)at < (unsigned)fit) list[MLIP_CHECK_INDEX(off + at, nbr_cap, bounds) - off] = (ENTRY)(sizeof(ENTRY) == 4 ? chunk + c0 + e : code + c0 + e);
                                     near_next += hit && near; far_next -= hit && !near;
                                 } else if (hit) {
                                     asm volatile("st.shared.u16 [%0], %1;" ::"r"(near ? near_at : far_at), "r"(code + c0 + e) : "memory");
@@ -943,7 +945,7 @@ __global__ void __launch_bounds__(LN_THREADS) k_neighbors_lanes(int64_t n, CellG
     }
 
     // ---- write the lists: full rows from shared memory ----
-    const long long off = s_prefix + s_off[32 * warp + lane];
+    off = s_prefix + s_off[32 * warp + lane];
     fit = cnt;   // entries of this list that the array still holds
     if (i < n) {
         if (off + cnt > nbr_cap) {
@@ -984,7 +986,7 @@ __global__ void __launch_bounds__(LN_THREADS) k_neighbors_lanes(int64_t n, CellG
             const int e = e0 + lane, code = e < m ? src[e < near ? e : e + (buf - all)] : 0;
             int entry = code;
             if (sizeof(ENTRY) == 4) entry = __shfl_sync(0xffffffffu, bases, code >> L16_SHIFT) + (code & L16_MASK);
-            if (e < m) nbr[to + e] = (ENTRY)entry;
+            if (e < m) nbr[MLIP_CHECK_INDEX(to + e, nbr_cap, bounds)] = (ENTRY)MLIP_CHECK_INDEX(entry, sizeof(ENTRY) == 4 ? n : 27ll << L16_SHIFT, bounds);
         }
     }
 }
