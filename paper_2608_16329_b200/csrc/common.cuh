@@ -155,7 +155,8 @@ struct mlip_ctx {
     double *stage_out = nullptr;   // [10]
     int64_t stage_cap = 0;
 
-    bool built = false, forces_current = false, kernel_ready = false;
+    bool built = false, forces_current = false;
+    int kernel_ready = 0;          // fused kernels whose shared-memory limit this context has set, a bit each (fp64: whether)
     size_t table_bytes = 0;
     int64_t step = 0;
     int64_t launches = 0;

@@ -141,24 +141,20 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     const bool in_smem = tables_fit_smem(c);
     const int tab_words = in_smem ? table_smem_words(c) : 0;
     const int shape = in_smem && n < ONE_PER_WARP_BELOW_ATOMS ? 0 : long_lists(c) ? 2 : 1;   // one atom per warp, two side by side, two one after the other
-    auto kernel_of = [&](int shape, bool list16) {
-        return shape == 0 ? mega_one(det, list16) : shape == 2 ? mega_apart(in_smem, det, list16) : !in_smem ? mega_two_global(det, list16) : det ? mega_two_fixed(list16) : mega_two(list16);
-    };
     const int apw = shape == 0 ? 1 : 2;
     const size_t smem_bytes = sizeof(float) * (size_t)((apw == 1 ? Layout<1>::FIXED : Layout<2>::FIXED) + tab_words);
     const int C = c->cfg.n_species, tile_atoms = GW * apw;
     int64_t tiles[MAX_SPECIES], all = 0;
     for (int q = 0; q < C; ++q) all += tiles[q] = (c->species_host[q + 1] - c->species_host[q] + tile_atoms - 1) / tile_atoms;
     const int blocks = (int)std::min<int64_t>(all, (int64_t)c->n_sm);
-    if (!c->kernel_ready) {
-        // A limit of the kernels, shared by every context of the process: the same whatever this one's tables need.  Those that this context may launch.
-        for (int q = in_smem ? 0 : 1; q < 3; ++q)
-            for (int compact = 0; compact <= (c->cfg.list_format == 1); ++compact) {
-                const cudaError_t e = cudaFuncSetAttribute((const void *)kernel_of(q, compact), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                           (int)sizeof(float) * (in_smem ? SMEM_LIMIT_WORDS : Layout<2>::FIXED));
-                if (e != cudaSuccess) { c->err = std::string("fused kernel shared memory: ") + cudaGetErrorString(e); return MLIP_ERR_CUDA; }
-            }
-        c->kernel_ready = true;
+    const MegaKernel kernel = shape == 0 ? mega_one(det, c->list16) : shape == 2 ? mega_apart(in_smem, det, c->list16) : !in_smem ? mega_two_global(det, c->list16)
+                            : det ? mega_two_fixed(c->list16) : mega_two(c->list16);
+    const int ready = 1 << (2 * shape + (c->list16 ? 1 : 0));
+    if (!(c->kernel_ready & ready)) {
+        // A limit of the kernel, shared by every context of the process: the same whatever this one's tables need.
+        const cudaError_t e = cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(float) * (in_smem ? SMEM_LIMIT_WORDS : Layout<2>::FIXED));
+        if (e != cudaSuccess) { c->err = std::string("fused kernel shared memory: ") + cudaGetErrorString(e); return MLIP_ERR_CUDA; }
+        c->kernel_ready |= ready;
     }
     KernelArgs k;
     k.n = n; k.n_species = c->cfg.n_species; k.grid = c->grid; k.rc2 = c->cfg.r_cut * c->cfg.r_cut; k.tab = c->tab;
@@ -191,7 +187,7 @@ int launch_megakernel(mlip_ctx *c, cudaStream_t s) {
     }
     k.stamp = timed_begin(c, MARK_KERNEL, s);
     k.early = !c->lists_fresh;   // (the kernel reads the lists before it waits)
-    MLIP_CUDA_TRY(c, launch_after_if(k.early, kernel_of(shape, c->list16), blocks, NW * 32, smem_bytes, s, k, tab_words));
+    MLIP_CUDA_TRY(c, launch_after_if(k.early, kernel, blocks, NW * 32, smem_bytes, s, k, tab_words));
     c->lists_fresh = c->force_cleared = false;
     set_eval_block(c, blk.use);
     if (det) {

@@ -696,7 +696,7 @@ static cudaError_t launch_shape(mlip_ctx *c, F64Args &k, cudaStream_t s) {
             e = cudaMemcpyToSymbol(c_ang_q, q, sizeof q);
             if (e != cudaSuccess) return e;
         }
-        c->kernel_ready = true;
+        c->kernel_ready = 1;
     }
     const int per_sm = f64_ctas_per_sm<K, LMAX, BASIS>();
     const int64_t tiles_max = (k.n + F64_TILE - 1) / F64_TILE + k.n_species;

@@ -200,7 +200,7 @@ int build_tables(mlip_ctx *c, const double *enc_w_host, size_t n_enc) {
     else MLIP_CUDA_TRY(c, cudaMalloc(&c->table, coef_bytes));
     c->table_bytes = coef_bytes;
     c->resident += coef_bytes;
-    c->kernel_ready = false;
+    c->kernel_ready = 0;
     MLIP_CUDA_TRY(c, cudaMemcpy(w, enc_w_host, sizeof(double) * n_enc, cudaMemcpyHostToDevice));
     MLIP_CUDA_TRY(c, cudaMemset(stats, 0, sizeof(unsigned long long) * 4));
 

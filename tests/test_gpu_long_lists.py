@@ -85,3 +85,28 @@ def test_a_pair_costs_no_more_where_there_are_many():
             best = min(best, begin.elapsed_time(end))
         cost.append(best / mlip.mlip_get_counters(pot.ctx)["pairs_in_cutoff"])
     assert cost[1] < 1.2 * cost[0], cost
+
+
+@pytest.mark.parametrize("cells,spacing", [(10, 2.2), (24, 2.2), (24, 1.8)])   # one atom per warp, two side by side, two one after the other
+def test_a_first_evaluation_can_be_captured(cells, spacing):
+    """The kernel's shared-memory limit is set by the first evaluation that launches it, inside a capture too."""
+    import paper_2608_16329_b200 as mlip
+    import torch
+    rng = np.random.default_rng(cells)
+    pos = wl.lattice_sites((cells,) * 3, spacing, wl._SC_BASIS) + rng.normal(0.0, 0.05, (cells ** 3, 3))
+    box = np.full(3, cells * spacing)
+    pos -= np.floor(pos / box) * box
+    pos[pos >= box] = 0.0
+    enc, head = wl.make_weights(2, seed=78, enc_out_scale=0.05, head_out_scale=0.3)
+    pot = mlip.Potential(2, 6.0, 1.0, enc, head, np.full(2, 50.0))
+    pot.build_neighbors(pos, rng.integers(0, 2, len(pos)).astype(np.int32), box)
+    forces = torch.zeros(len(pos), 3, dtype=torch.float32, device=pot.device)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        mlip.mlip_compute(pot.ctx, None, forces, None, None)
+    graph.replay()
+    torch.cuda.synchronize()
+    captured = forces.clone()
+    eager = pot.compute()["forces"]
+    scale = float(torch.sqrt((eager ** 2).sum(1).mean()))
+    assert float((captured - eager).abs().max()) <= 1e-5 * max(1.0, scale)   # (sums in another order)
