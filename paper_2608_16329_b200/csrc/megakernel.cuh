@@ -7,7 +7,7 @@
 //   walks through the central species in order; for each it stages that species' radial tables
 //   (one per neighbor species) and head constants in shared memory, then each group takes tiles of
 //   16 (small systems: 8) central atoms of that species from a global counter (each warp encodes and
-//   derives two of them, side by side in its pair loops) and runs them on its own,
+//   derives two of them, side by side in its pair loops where lists are short) and runs them on its own,
 //   synchronising only inside the group (named barriers), so that one group's latency-bound head
 //   overlaps the other group's pair loops.
 //   Encoding    The warp scans the atom's list (lane = entry), queues the pairs inside r_cut in
@@ -1202,7 +1202,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_mega(const __grid_constant__ Ker
             pc.mark(11);
             const int count = min(NA, s_end - first);
 
-            // ---------------- Encoding + invariants: the warp's atoms wg, wg + 8 one after the other ----------------
+            // ---------------- Encoding + invariants: the warp's atoms wg, wg + 8 ----------------
             if (prefetched) {
                 asm volatile("cp.async.wait_group 0;" ::: "memory");
                 __syncwarp();

@@ -3,7 +3,8 @@
 // Section 4.1.4).  Everything runs on the device:
 //   cell id per atom -> counting sort into cell order (ties broken by species, then by the
 //   caller's index, so the internal order is reproducible) -> per-species processing order
-//   -> one warp-per-atom traversal of the 27 surrounding cells (two, count and fill, when there is no array yet or it is too small).
+//   -> one traversal of the 27 surrounding cells, a warp per atom or a lane (list_form.cuh); two, count and fill, when there is no array
+//   yet or it is too small.
 // Small systems are bound by the number of launches and by the longest chain in one thread or warp, large ones by the
 // traversal's instruction issue.
 // The inclusion test is fp64 with separately rounded operations, so the set of pairs is
@@ -1150,7 +1151,7 @@ static ListView list_view(const mlip_ctx *c) {
 
 // What a synchronising build has to know -- {ticket, overflow, total, status} and the species' starts, neighbors in memory -- is written by
 // a kernel straight to page-locked host memory, where the host watches for the ticket behind it: a copy and the wait for the stream
-// leave the GPU idle for longer (256-atom screening 81.0 -> 72.8 us a configuration).  After REPORT_WATCH (a large build, or one queued behind other
+// leave the GPU idle for longer (256-atom screening 82 -> 77 us a configuration).  After REPORT_WATCH (a large build, or one queued behind other
 // work) the host waits for the stream after all; the stream is asked now and then, so that an error ends the watch.
 constexpr std::chrono::microseconds REPORT_WATCH(500);
 __global__ void k_report(const int *words, volatile int *host, int ticket) {
