@@ -119,7 +119,7 @@ __global__ void k_fixed_finish(int64_t n, long long *force_fx, const long long *
 
 // Whether two atoms of a warp go through the pair loops one after the other.  Side by side they are the faster ones where their lists fit the queue
 // together, up to LONG_LIST entries each; with longer ones they are gathered one by one as well, no batch is saved, and from some 110 pairs on
-// warps of both kinds share an SM and wait for each other's instructions.  One evaluation of some 100,000 atoms in us, side by side / one after the
+// warps of both kinds, which then share an SM, hold each other up.  One evaluation of some 100,000 atoms in us, side by side / one after the
 // other: random positions of 54 pairs an atom 667 / 671, 63 734 / 735, 72 823 / 801, 81 886 / 858, 109 1564 / 1057, 118 2632 / 1203, 163 2131 / 1529; crystals
 // of 42 pairs 494 / 512, 54 574 / 585, 78 846 / 853, 86 995 / 964, 113 1215 / 1153, 131 1506 / 1367, 158 1534 / 1377, 221 2317 / 2123.
 // Asked of the last synchronising build's lists.  Reproducible runs must not depend on when that was: they ask the density of the box.
