@@ -813,7 +813,7 @@ __global__ void __launch_bounds__(LN_THREADS) k_neighbors_lanes(int64_t n, CellG
     ENTRY *list = nullptr;
     long long off = 0;   // of the list
     int near_next = 0, far_next = 0, fit = 0;
-    int *bounds = const_cast<int *>(global_status);   // (range-checked builds only write it)
+    [[maybe_unused]] int *bounds = const_cast<int *>(global_status);   // (range-checked builds only write it)
     auto traverse = [&](auto second_traversal, bool part) {
         constexpr bool SECOND = decltype(second_traversal)::value;
         for (unsigned left = __ballot_sync(0xffffffffu, part); left;) {   // groups of lanes with cells along one column
